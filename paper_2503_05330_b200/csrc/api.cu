@@ -12,7 +12,7 @@ constexpr size_t kAlign = 256;
 inline size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
 struct Layout {
-  size_t tok, pq, len, rec, status, index, q_fp, q_mode, q_reserved, q_off, q_cursor, match_cursor, g_nscan, g_trim, matches;
+  size_t tok, pq, len, rec, status, index, q_fp, q_mode, q_reserved, q_off, q_cursor, match_cursor, g_nscan, g_trim, a_plan, matches;
   size_t w_ctl, w_desc, w_pred, w_edge, w_tab, w_key, w_item, b_ent, b_ctl, bp_todo;
   bool wide_on;
   uint64_t w_slots;
@@ -74,6 +74,7 @@ Layout make_layout(const sdms_config* c) {
   l.match_cursor = take(8);
   l.g_nscan = take((size_t)c->num_groups * 4);
   l.g_trim = take((size_t)c->num_groups * 4);
+  l.a_plan = take(P * 8);
   l.matches = take((size_t)mc * 4);
   l.x_draft_tok = take(P * D * 4); l.x_draft_len = take(P * 4);
   l.x_node_tok = take(P * D * B * 4); l.x_node_S = take(P * D * B * 8); l.x_node_cnt = take(P * D * B * 4);
@@ -256,6 +257,7 @@ int sdms_create(const sdms_config* cfg, void* d_workspace, size_t bytes, sdms_ct
   d.q_reserved = (int32_t*)(w + lay.q_reserved); d.q_off = (int32_t*)(w + lay.q_off);
   d.match_cursor = (unsigned long long*)(w + lay.match_cursor);
   d.q_cursor = (int32_t*)(w + lay.q_cursor); d.g_nscan = (int32_t*)(w + lay.g_nscan); d.g_trim = (int32_t*)(w + lay.g_trim);
+  d.a_plan = (int2*)(w + lay.a_plan);
   d.matches = (int32_t*)(w + lay.matches);
   ctx->x_draft_tok = (int32_t*)(w + lay.x_draft_tok); ctx->x_draft_len = (int32_t*)(w + lay.x_draft_len);
   d.x_node_tok = (int32_t*)(w + lay.x_node_tok); d.x_node_S = (int64_t*)(w + lay.x_node_S);
@@ -297,6 +299,7 @@ int sdms_append(sdms_ctx* ctx, const int32_t* d_tokens, const float* d_logprobs,
   if (!ctx || !d_tokens || !d_logprobs || !d_counts || row_width < 1) return SDMS_ERR_INVALID_ARG;
   cudaStream_t st = (cudaStream_t)stream;
   ctx->built = false;
+  if (row_width >= kBulkAppendFrom) ++ctx->launches;   // two launches
   return timed(ctx, SDMS_KERNEL_APPEND, st,
                [&] { return launch_append(ctx->dev, d_tokens, d_logprobs, d_counts, row_width, st); });
 }

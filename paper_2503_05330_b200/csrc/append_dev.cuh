@@ -104,6 +104,31 @@ __device__ void index_insert(const Dev& s, int g, int n, uint64_t h, uint32_t lp
   *st |= SDMS_STATUS_INDEX_FULL;
 }
 
+// The same for thousands of inserts at a time, where throughput counts and not the latency of one: the bucket's head
+// is read before any atomic, so that an occurrence of a known n-gram costs one atomic (the heads of popular n-grams
+// take thousands of them, one after the other) and a bucket of another n-gram costs none.
+__device__ __forceinline__ void index_insert_bulk(const Dev& s, int g, int n, uint64_t h, uint32_t lpos, uint32_t* st) {
+  uint32_t* table = index_table(s, g, n);
+  const uint32_t fp = gram_fp(h);
+  uint32_t b = gram_bucket(h, s.table_cap);
+  for (uint32_t probe = 0; probe < s.table_cap; ++probe) {
+    uint32_t* bucket = table + (size_t)b * kBucketWords;
+    unsigned long long* head = reinterpret_cast<unsigned long long*>(bucket);
+    unsigned long long old = __ldcg(head);
+    if (old == 0ull) {
+      old = atomicCAS(head, 0ull, (1ull << 32) | fp);
+      if (old == 0ull) { bucket[2] = lpos; return; }
+    }
+    if ((uint32_t)old == fp) {
+      const uint32_t slot = (uint32_t)(atomicAdd(head, 1ull << 32) >> 32);
+      if (slot < (uint32_t)kInlineSlots) bucket[2 + slot] = lpos;
+      return;
+    }
+    b = (b + 1) & (s.table_cap - 1);
+  }
+  *st |= SDMS_STATUS_INDEX_FULL;
+}
+
 // Block-cooperative append of n validated tokens to path p whose length is len0.  rec is the
 // path's record as it was before the call (shared memory): rec[1 + t] = token at len0 - 1 - t.
 // Also writes the path's new record and length (and a copy of the record to rec_out, shared

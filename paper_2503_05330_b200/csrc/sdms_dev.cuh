@@ -68,6 +68,7 @@ struct Dev {
   int32_t* q_cursor;                   // [P] matches written
   unsigned long long* match_cursor;    // match slots handed to scan queries by the probe; zero between builds
   int32_t* g_nscan;                    // [G] queries of the prompt that need the scan; zero between builds
+  int2* a_plan;                        // [P] an append of wide rows: tokens the path held before, tokens it takes
   int32_t* g_trim;                     // [G] a path of the prompt was trimmed: its index is rebuilt
   int32_t* matches;                    // [match_cap] global positions j*L+e
   // device-wide aggregation of queries with many matches (dag_wide.cu); w_slots = 0: not in use

@@ -75,6 +75,30 @@ def test_append_clamping_and_status_bits():
     pair.build_and_compare(2)
 
 
+@pytest.mark.parametrize("width", [63, 64, 65, 255, 256, 257, 511, 512, 513, 1100])
+def test_append_of_wide_rows(width):
+    # rows around the widths at which an append takes its two launches and a chunk ends: a second row behind a first one
+    # (n-grams across the seam), counts at and around the row's end, tokens outside the vocabulary in different chunks
+    N, V, k_max = 5, 40, 6
+    L = 2 * width + 3
+    pair = Pair(1, N, L, V, k_max, 4, alpha=0.5)
+    tokens, lps = synth.small_random(N, 3 * width, V, 4100 + width)
+    pair.append(tokens[:, :width], lps[:, :width], np.array([width, 0, 5, width // 2, 1]), expect_status=0)
+    pair.check_history()
+    pair.build_and_compare(k_max)
+    row, lp = tokens[:, width:2 * width].copy(), lps[:, width:2 * width].copy()
+    row[3, width - 2] = V                             # the path keeps what came before
+    row[4, min(width - 1, 300)] = -1
+    lp[2, 7] = np.nan
+    pair.append(row, lp, np.array([width, width + 1, width - 1, width, width]), expect_status=0x01 | 0x04 | 0x08)
+    pair.check_history()
+    for k in range(1, k_max + 1):
+        pair.build_and_compare(k)
+    pair.append(tokens[:, 2 * width:], lps[:, 2 * width:], np.array([width, 0, 0, 3, 0]), expect_status=0x02)   # past the capacity
+    pair.check_history()
+    pair.build_and_compare(3)
+
+
 def test_empty_and_degenerate_states():
     # nothing appended yet, then a single token per path, then k larger than some paths
     pair = Pair(2, 3, 16, 5, 3, 3, B=2, Ke=2)
