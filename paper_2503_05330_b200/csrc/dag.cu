@@ -7,14 +7,12 @@
 // and cnt of nodes and edges are integer sums, so the order of accumulation
 // (atomics, warp shuffles) cannot change a result.
 //
-// Two ways through, both per query path in one CTA:
-//   dag_small (M <= 32 matches, the common case): lane m owns candidate m and
-//     each WARP owns a layer, so all layers aggregate at the same time.  Lanes
-//     with the same follower token (__match_any_sync) form a node, lanes that
-//     also share the previous token form an edge; sums run over the lanes of a
-//     group, ranks over the group leaders, and each layer also decides the best
-//     way out of every source node.  One barrier, then one warp walks the layers
-//     by looking those decisions up.
+// Ways through, all per query path in one CTA:
+//   dag_walk_warp (M <= 32 matches, the common case) and dag_walk (up to thousands): the greedy draft alone.  Node
+//     sums of all layers first, side by side, then the walk, then the weights of the edges taken.
+//   dag_small (M <= 32; export, tree pool, layer-wise search): lane m owns candidate m and each WARP owns a
+//     layer.  Lanes with the same follower token (__match_any_sync) form a node, lanes that also share the previous
+//     token form an edge; sums run over the lanes of a group, ranks over the group leaders.
 //   dag_block (any M): layers in sequence.  Followers are staged in shared memory
 //     when they fit; every candidate adds into a shared-memory hash table keyed
 //     by token (32-bit atomics with explicit carry).  Unstaged fan-out past the
@@ -148,6 +146,7 @@ struct Smem {
   int* kept; int* r_nedge; int* r_outdeg;
   int* st_tok; int* st_pq;                      // staged followers [m*D + d-1], token -1 = past the path's end
   int* list;                                    // fused kernel: first kListCap matches
+  int pool_words;                               // words from st_tok on (at least kPoolWords): one pool for the aggregations
 };
 
 constexpr int kMaxWarps = 32;
@@ -172,6 +171,12 @@ __device__ Smem carve(unsigned char* base) {
     m.t_S = p8; p8 += kMaxWarps * 32;
   }
   int* p4 = reinterpret_cast<int*>(p8);
+  if (!EXPORT) {
+    unsigned bytes;
+    asm volatile("mov.u32 %0, %%dynamic_smem_size;" : "=r"(bytes));
+    m.list = p4; p4 += kListCap;
+    m.pool_words = (int)(bytes >> 2) - kListCap;
+  }
   m.st_tok = p4; p4 += kStageWords;
   m.st_pq = p4; p4 += kStageWords;
   m.n_key = p4; p4 += CAP;
@@ -182,8 +187,9 @@ __device__ Smem carve(unsigned char* base) {
   m.n_call = reinterpret_cast<unsigned*>(p4); p4 += CAP;
   m.n_ccur = reinterpret_cast<unsigned*>(p4); p4 += CAP;
   m.n_touch = p4; p4 += CAP;
-  m.list = p4; p4 += kListCap;
   if (EXPORT) {
+    m.list = p4; p4 += kListCap;
+    m.pool_words = 0;
     m.e_key = p4; p4 += CAP;
     m.e_Slo = reinterpret_cast<unsigned*>(p4); p4 += CAP;
     m.e_Shi = reinterpret_cast<unsigned*>(p4); p4 += CAP;
@@ -974,6 +980,384 @@ __device__ void dag_layers(const Dev& s, const Smem& sm, int i, int M, const int
   if (tid == 0) draft_len[i] = emitted;
 }
 
+// ---- the greedy walk (search modes 0 and 2) -----------------------------------------------------------
+// One CTA is bound here by how many dependent instructions follow one another (4.3 cycles each, 33 for a shared load, 50 to
+// 70 for a taken or divergent branch): so items are handled in fixed batches of registers, without branches in between.
+
+// Largest value of the warp (values are >= 0), in every lane: 57 cycles.
+__device__ __forceinline__ u64 warp_max64(u64 x) {
+  const unsigned hi = (unsigned)(x >> 32), top = __reduce_max_sync(FULL, hi);
+  const unsigned lo = __reduce_max_sync(FULL, hi == top ? (unsigned)x : 0u);
+  return (u64)top << 32 | lo;
+}
+__device__ __forceinline__ u64 max64(u64 a, u64 b) { return a > b ? a : b; }
+
+// M <= 32: lane m of a warp holds candidate m.  A warp per layer fetches the followers and forms every candidate's node
+// sum (a broadcast read of the layer's row: 32 compares, where __match_any_sync on distinct tokens takes 364 cycles);
+// one warp walks.  Where all candidates on a node go on with the same token nothing is compared.
+constexpr int kRow = 36;                 // words per layer: 16-byte aligned, rows on different banks
+
+__device__ void dag_walk_warp(const Dev& s, int i, int M, const int32_t* mlist, const int32_t* plen, int poff,
+                              int32_t* draft_tok, int32_t* draft_len, float* draft_score, float* draft_edge_w) {
+  // (shared memory is named here and not passed in, so that every access is known to be to shared memory: atomics
+  // through a generic pointer cost several hundred cycles each)
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5, D = s.D;
+  int* const row_v = reinterpret_cast<int*>(smem_raw) + kListCap;     // [d - 1][kRow] token, -1: the candidate has ended
+  int* const row_p = row_v + kRow * SDMS_MAX_DRAFT;
+  unsigned* const row_lo = reinterpret_cast<unsigned*>(row_p + kRow * SDMS_MAX_DRAFT);     // node sum of the candidate's token
+  unsigned* const row_hi = row_lo + kRow * SDMS_MAX_DRAFT;
+  unsigned* const row_c = row_hi + kRow * SDMS_MAX_DRAFT;
+  if (warp < D) {
+    int gpos = 0, n_m = 0;
+    if (lane < M) {
+      gpos = mlist[lane];
+      const int j = path_of(s, gpos);
+      n_m = min(D, plen[j - poff] - 1 - (gpos - j * s.L));
+    }
+    for (int d = warp + 1; d <= D; d += nwarps) {
+      const int v = d <= n_m ? ldm(s.tok + gpos + d) : -1, p = d <= n_m ? ldm(s.pq + gpos + d) : 0;
+      int* const rv = row_v + (d - 1) * kRow;
+      int* const rp = row_p + (d - 1) * kRow;
+      rv[lane] = v; rp[lane] = p;
+      __syncwarp();
+      u64 S = 0;
+      unsigned c = 0;
+#pragma unroll 2
+      for (int x = 0; x < M; x += 4) {
+        const int4 tv = *reinterpret_cast<const int4*>(rv + x), tp = *reinterpret_cast<const int4*>(rp + x);
+        if (tv.x == v) { S += (unsigned)tp.x; ++c; }
+        if (tv.y == v) { S += (unsigned)tp.y; ++c; }
+        if (tv.z == v) { S += (unsigned)tp.z; ++c; }
+        if (tv.w == v) { S += (unsigned)tp.w; ++c; }
+      }
+      row_lo[(d - 1) * kRow + lane] = (unsigned)S; row_hi[(d - 1) * kRow + lane] = (unsigned)(S >> 32);
+      row_c[(d - 1) * kRow + lane] = c;
+    }
+  }
+  __syncthreads();
+  if (warp != 0) return;
+  auto sum_at = [&](int d, int x) { return ((u64)row_hi[(d - 1) * kRow + x] << 32) | row_lo[(d - 1) * kRow + x]; };
+  unsigned from = __ballot_sync(FULL, lane < M);       // candidates on the current node
+  int emitted = 0;
+  int my_tok = -1, my_src = 0;                         // lane d - 1 keeps what was decided for layer d
+  unsigned my_node = 0u, my_edge = 0u;
+  int v = row_v[lane];
+#pragma unroll 1
+  for (int d = 1; d <= D; ++d) {
+    const int v_next = d < D ? row_v[d * kRow + lane] : -1;
+    const bool on = (from >> lane & 1u) && v >= 0;
+    const unsigned succ = __ballot_sync(FULL, on);
+    if (succ == 0u) break;
+    int src = __ffs(succ) - 1;
+    int tok = __shfl_sync(FULL, v, src);
+    if (__ballot_sync(FULL, on && v != tok)) {         // several successors: the heaviest
+      src = warp_arg_first(on, eq5_weight(s.alpha, sum_at(d, lane), row_c[(d - 1) * kRow + lane]), v);
+      tok = __shfl_sync(FULL, v, src);
+    }
+    const unsigned node = __ballot_sync(FULL, v == tok);
+    if (lane == d - 1) { my_tok = tok; my_src = src; my_node = node; my_edge = node & from; }
+    from = node; v = v_next;
+    emitted = d;
+  }
+  if (lane < D) {
+    u64 S = 0, Se = 0;
+    if (lane < emitted) {
+      S = Se = sum_at(lane + 1, my_src);
+      if (my_edge != my_node) {
+        Se = 0;
+        for (unsigned rem = my_edge; rem; rem &= rem - 1u) Se += (unsigned)row_p[lane * kRow + __ffs(rem) - 1];
+      }
+    }
+    const size_t at = (size_t)i * D + lane;
+    draft_tok[at] = my_tok;
+    if (draft_score) draft_score[at] = my_tok >= 0 ? (float)eq5_weight(s.alpha, S, __popc(my_node)) : 0.0f;
+    if (draft_edge_w) draft_edge_w[at] = my_tok >= 0 ? (float)eq5_weight(s.alpha, Se, __popc(my_edge)) : 0.0f;
+  }
+  if (lane == 0) draft_len[i] = emitted;
+}
+
+// More candidates.  As many layers at once as fit shared memory (all of them up to a hundred-odd candidates), a table per
+// layer, all (candidate, layer) items side by side, four of a thread's at a time:
+//   sums   an item claims the slot of its token in the layer's table and adds its probability; it notes the slot
+//   keys   the slot becomes the item's key: its node's weight and its token in one word that orders by weight, then by
+//          smaller token (PACKED: with alpha = 1 the weight is the sum itself; else weight and token stay apart)
+//   walk   per layer the largest key among the candidates on the current node, four candidates per lane: one warp, and no
+//          barrier, up to 128 candidates; a layer's rows do not depend on the walk and are fetched a layer ahead
+constexpr int kWideFrom = 64;            // matches from which a query of a large prompt goes to the wide pass: 64 here 20 us, there 29-35 us a launch that
+                                         // other queries need anyway; 1000 here 60 us
+constexpr int kWalkMaxCap = 8192;        // most slots of a layer's table
+
+struct WalkPlan { int cap, stride, layers; bool packed; };    // slots per table, words per row of items, layers per round
+// layers = 0: does not fit
+__device__ __forceinline__ WalkPlan walk_plan(const Dev& s, int M, int pool_words) {
+  WalkPlan w;
+  w.cap = 64;
+  while (7 * w.cap < 8 * M) w.cap *= 2;                // at most 7/8 full
+  w.stride = ((M + 31) & ~31) + 4;
+  // sum (30 bits and those of the number of candidates) and token side by side in 64 bits
+  w.packed = s.alpha == 1.0 && (32 - __clz(M)) + (32 - __clz(s.V)) + 30 <= 64;
+  const int per_layer = (w.packed ? 3 : 4) * (w.stride + w.cap), room = pool_words - w.stride;
+  w.layers = w.cap > kWalkMaxCap || room < per_layer ? 0 : s.D * per_layer <= room ? s.D : room / per_layer;
+  return w;
+}
+
+template <bool PACKED>
+__device__ void dag_walk(const Dev& s, const WalkPlan w, int i, int M, const int32_t* mlist, const int32_t* plen,
+                         int poff, int root, int32_t* draft_tok, int32_t* draft_len, float* draft_score,
+                         float* draft_edge_w) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ u64 sh_best[2][kMaxWarps];
+  __shared__ int sh_tok[2][kMaxWarps];
+  __shared__ unsigned sh_e[SDMS_MAX_DRAFT][3];          // walk by several warps: edge sum (lower 16 bits, rest), count
+  __shared__ int sh_cur;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5, D = s.D;
+  const int cap = w.cap, mask = cap - 1, shift = __clz(cap) + 1, stride = w.stride;
+  const int all = w.layers * cap, items = w.layers * stride;
+  int* const keys = reinterpret_cast<int*>(smem_raw) + kListCap;                 // tables, every array: [layer of the round][slot]
+  unsigned* const sum_lo = reinterpret_cast<unsigned*>(keys + all);
+  unsigned* const sum_hi = sum_lo + all;
+  unsigned* const cnt = sum_hi + all;                   // not packed
+  unsigned* const row_prev = reinterpret_cast<unsigned*>(keys + (PACKED ? 3 : 4) * all);     // last layer's tokens of the round before
+  unsigned* const rows_t = row_prev + stride;           // items, every array: [layer][candidate]: token, -1: has ended; packed: then lower key word
+  unsigned* const rows_p = rows_t + items;              // probability
+  unsigned* const rows_h = rows_p + items;              // slot, then upper key word
+  unsigned* const rows_l = PACKED ? rows_t : rows_h + items;                     // lower key word
+  // the token of an item as the walk compares it: packed, its complement in the lower bits of the key (0: has ended)
+  const int tok_bits = 32 - __clz(s.V);
+  const unsigned tok_mask = PACKED ? (1u << tok_bits) - 1u : ~0u;
+  auto code_of = [&](int tok) { return PACKED ? ~(unsigned)tok & tok_mask : (unsigned)tok; };
+  const int walkers = min(nwarps, (M + 127) >> 7), width = walkers * 32;
+
+  if (tid < D) { sh_e[tid][0] = 0u; sh_e[tid][1] = 0u; sh_e[tid][2] = 0u; }
+  // lane d - 1 of warp 0 keeps what layer d comes to
+  int my_tok = -1;
+  u64 my_key = 0ull;
+  unsigned my_e0 = 0u, my_e1 = 0u, my_e2 = 0u;
+  int cur = root, emitted = 0;
+#pragma unroll 1
+  for (int d0 = 1; d0 <= D; d0 += w.layers) {
+    const int nl = min(w.layers, D - d0 + 1);
+    const int lN = nl > 1 ? 32 - __clz(nl - 1) : 0, nN = 1 << lN;       // items are numbered m << lN | layer: no division
+    {
+      int4* const z = reinterpret_cast<int4*>(keys);
+      const int key_end = all / 4, end = key_end * (PACKED ? 3 : 4);
+      for (int x = tid; x < key_end; x += blockDim.x) z[x] = make_int4(-1, -1, -1, -1);
+      for (int x = key_end + tid; x < end; x += blockDim.x) z[x] = make_int4(0, 0, 0, 0);
+    }
+    // the followers: four entries of a thread are asked for before the first is stored
+#pragma unroll 1
+    for (int x0 = tid; x0 < (M << lN); x0 += 4 * blockDim.x) {
+      int gpos[4], left[4], tk[4], pr[4];
+#pragma unroll
+      for (int r = 0; r < 4; ++r) gpos[r] = mlist[min((x0 + r * (int)blockDim.x) >> lN, M - 1)];
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        const int j = path_of(s, gpos[r]);
+        left[r] = plen[j - poff] - 1 - (gpos[r] - j * s.L);              // followers of the match
+      }
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        const int l = (x0 + r * (int)blockDim.x) & (nN - 1);
+        const bool on = d0 + l <= left[r] && l < nl;
+        tk[r] = -1; pr[r] = 0;
+        if (on) { tk[r] = ldm(s.tok + gpos[r] + d0 + l); pr[r] = ldm(s.pq + gpos[r] + d0 + l); }
+      }
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        const int x = x0 + r * (int)blockDim.x, m = x >> lN, l = x & (nN - 1);
+        if (m < M && l < nl) { rows_t[l * stride + m] = (unsigned)tk[r]; rows_p[l * stride + m] = (unsigned)pr[r]; }
+      }
+    }
+    __syncthreads();
+    const int ntask = ((M + 31) >> 5) << lN;            // a warp takes 32 candidates of one layer
+    // sums
+#pragma unroll 1
+    for (int t0 = warp; t0 < ntask; t0 += 4 * nwarps) {
+      int v[4], at[4], k[4], slot[4];                   // slot: within all layers' tables
+      unsigned p[4];
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        const int t = t0 + r * nwarps, l = t & (nN - 1), m = ((t >> lN) << 5) + lane;
+        const bool in = t < ntask && l < nl && m < M;
+        at[r] = in ? l * stride + m : -1;
+        v[r] = in ? (int)rows_t[at[r]] : -1;
+        p[r] = in ? rows_p[at[r]] : 0u;
+        slot[r] = (in ? l * cap : 0) + (int)(((unsigned)v[r] * 2654435761u) >> shift);
+      }
+#pragma unroll
+      for (int r = 0; r < 4; ++r) k[r] = *(volatile int*)&keys[slot[r]];
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+        if (k[r] == -1 && v[r] >= 0) k[r] = atomicCAS(&keys[slot[r]], -1, v[r]);
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+#pragma unroll 1
+        while (v[r] >= 0 && k[r] != -1 && k[r] != v[r]) {                // ends: more slots than candidates
+          slot[r] = (slot[r] & ~mask) | ((slot[r] + 1) & mask);
+          k[r] = atomicCAS(&keys[slot[r]], -1, v[r]);
+        }
+      }
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        if (v[r] >= 0) {
+          atomicAdd(&sum_lo[slot[r]], p[r] & 0xffffu);
+          atomicAdd(&sum_hi[slot[r]], p[r] >> 16);
+          if (!PACKED) atomicAdd(&cnt[slot[r]], 1u);
+        }
+        if (at[r] >= 0) rows_h[at[r]] = (unsigned)slot[r];
+      }
+    }
+    __syncthreads();
+    // keys
+#pragma unroll 1
+    for (int t0 = warp; t0 < ntask; t0 += 4 * nwarps) {
+      int at[4], v[4], sl[4];
+      u64 key[4];
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        const int t = t0 + r * nwarps, l = t & (nN - 1), m = ((t >> lN) << 5) + lane;
+        const bool in = t < ntask && l < nl && m < M;
+        at[r] = in ? l * stride + m : -1;
+        v[r] = in ? (int)rows_t[at[r]] : -1;
+        sl[r] = in ? (int)rows_h[at[r]] : 0;
+      }
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        const u64 S = ((u64)sum_hi[sl[r]] << 16) + sum_lo[sl[r]];
+        key[r] = PACKED ? S << tok_bits | (~(unsigned)v[r] & tok_mask) : (u64)__double_as_longlong(eq5_weight(s.alpha, S, cnt[sl[r]]));
+        if (v[r] < 0) key[r] = 0ull;
+      }
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+        if (at[r] >= 0) { rows_h[at[r]] = (unsigned)(key[r] >> 32); rows_l[at[r]] = (unsigned)key[r]; }
+    }
+    __syncthreads();
+    // walk
+    if (tid < width) {
+      unsigned u[4], t[4], h[4], lw[4], p[4];           // tokens of the layer before, of this one, key words, probabilities
+      // candidates m0 + r * width at layer l; behind the last one: has ended
+      auto fetch = [&](int l, int m0) {
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          const int m = m0 + r * width, at = l * stride + min(m, M - 1);
+          const bool in = m < M;
+          t[r] = rows_t[at]; h[r] = rows_h[at]; p[r] = rows_p[at];
+          lw[r] = PACKED ? 0u : rows_l[at];
+          if (!in) { t[r] = PACKED ? 0u : ~0u; h[r] = 0u; }
+        }
+      };
+      auto fetch_before = [&](int l, int m0) {          // (row_prev lies in front of the rows)
+#pragma unroll
+        for (int r = 0; r < 4; ++r) u[r] = rows_t[l * stride + min(m0 + r * width, M - 1) - stride];
+      };
+      const bool one = M <= 4 * width;                  // a thread's candidates fit its registers
+      fetch(0, tid);
+      if (d0 > 1) fetch_before(0, tid);
+#pragma unroll 1
+      for (int l = 0; l < nl; ++l) {
+        const int d = d0 + l;
+        const bool first = d == 1;                      // every first token follows the root
+        const unsigned from = code_of(cur);
+        u64 best = 0ull;
+        int tok = INT_MAX;                              // not packed: smallest token of that weight
+        auto consider = [&]() {
+#pragma unroll
+          for (int r = 0; r < 4; ++r) {
+            const bool on = first || (u[r] & tok_mask) == from;
+            if (PACKED) {
+              best = max64(best, on ? (u64)h[r] << 32 | t[r] : 0ull);
+            } else {
+              const u64 key = (u64)h[r] << 32 | lw[r];
+              const bool better = on && (int)t[r] >= 0 && (tok == INT_MAX || key > best || (key == best && (int)t[r] < tok));
+              best = better ? key : best; tok = better ? (int)t[r] : tok;
+            }
+          }
+        };
+        consider();
+        if (!one) {
+#pragma unroll 1
+          for (int m0 = tid + 4 * width; m0 - tid < M; m0 += 4 * width) {
+            fetch(l, m0);
+            if (!first) fetch_before(l, m0);
+            consider();
+          }
+        }
+        if (PACKED) {
+          best = warp_max64(best);
+        } else {
+          const u64 mine = tok == INT_MAX ? 0ull : best;
+          best = warp_max64(mine);
+          tok = (int)__reduce_min_sync(FULL, tok != INT_MAX && mine == best ? (unsigned)tok : (unsigned)INT_MAX);
+        }
+        if (walkers > 1) {
+          if (lane == 0) { sh_best[l & 1][warp] = best; sh_tok[l & 1][warp] = tok; }
+          asm volatile("bar.sync 1, %0;" ::"r"(width) : "memory");
+          const u64 b = lane < walkers ? sh_best[l & 1][lane] : 0ull;
+          const int bt = lane < walkers ? sh_tok[l & 1][lane] : INT_MAX;
+          best = warp_max64(PACKED || bt != INT_MAX ? b : 0ull);
+          if (!PACKED) tok = (int)__reduce_min_sync(FULL, bt != INT_MAX && b == best ? (unsigned)bt : (unsigned)INT_MAX);
+        }
+        if (PACKED ? best == 0ull : tok == INT_MAX) { cur = -1; break; }   // no successor: the draft ends here
+        if (PACKED) tok = (int)(~(unsigned)best & tok_mask);
+        // weight of the edge taken
+        const unsigned want = code_of(tok);
+        unsigned e0 = 0u, e1 = 0u, e2 = 0u;
+        auto weigh = [&]() {
+#pragma unroll
+          for (int r = 0; r < 4; ++r) {
+            const bool on = (t[r] & tok_mask) == want && (first || (u[r] & tok_mask) == from);
+            e0 += on ? p[r] & 0xffffu : 0u; e1 += on ? p[r] >> 16 : 0u; e2 += on;
+          }
+        };
+        if (one) {
+          weigh();
+#pragma unroll
+          for (int r = 0; r < 4; ++r) u[r] = t[r];
+        } else {
+#pragma unroll 1
+          for (int m0 = tid; m0 - tid < M; m0 += 4 * width) {
+            fetch(l, m0);
+            if (!first) fetch_before(l, m0);
+            weigh();
+          }
+        }
+        if (l + 1 < nl) {
+          fetch(l + 1, tid);                            // in flight during the sums below
+          if (!one) fetch_before(l + 1, tid);
+        }
+        e0 = __reduce_add_sync(FULL, e0); e1 = __reduce_add_sync(FULL, e1); e2 = __reduce_add_sync(FULL, e2);
+        if (walkers > 1) {
+          if (lane < 3 && e2 != 0u) atomicAdd(&sh_e[d - 1][lane], lane == 0 ? e0 : lane == 1 ? e1 : e2);
+        }
+        if (lane == d - 1) { my_tok = tok; my_key = best; my_e0 = e0; my_e1 = e1; my_e2 = e2; }
+        cur = tok; emitted = d;
+      }
+      if (tid == 0) sh_cur = cur;
+    }
+    if (d0 + nl <= D) {
+      __syncthreads();
+      cur = sh_cur;
+      if (cur < 0) break;                               // (the same for everybody)
+      for (int m = tid; m < M; m += blockDim.x) row_prev[m] = rows_t[(nl - 1) * stride + m];
+      __syncthreads();
+    }
+  }
+  if (walkers > 1) __syncthreads();                     // the edge sums are complete
+  if (warp == 0) {
+    if (lane < D) {
+      if (walkers > 1) { my_e0 = sh_e[lane][0]; my_e1 = sh_e[lane][1]; my_e2 = sh_e[lane][2]; }
+      const size_t at = (size_t)i * D + lane;
+      const bool on = my_tok >= 0;
+      draft_tok[at] = my_tok;
+      if (draft_score)
+        draft_score[at] = !on ? 0.0f : PACKED ? (float)eq5_weight(1.0, my_key >> tok_bits, 0u) : (float)__longlong_as_double((long long)my_key);
+      if (draft_edge_w) draft_edge_w[at] = on ? (float)eq5_weight(PACKED ? 1.0 : s.alpha, ((u64)my_e1 << 16) + my_e0, my_e2) : 0.0f;
+    }
+    if (lane == 0) draft_len[i] = emitted;
+  }
+}
+
 // ---- best path instead of the greedy walk (search mode 2) ------------------------------------------
 // best(d, v) = w(d, v) + max over the successors v' of v of best(d + 1, v')  (0 for no successor), w the
 // node's Eq. 5 in-weight; the draft follows, from the root, the successor with the largest best(), ties
@@ -1212,6 +1596,18 @@ __device__ __forceinline__ void dag_phase(const Dev& s, const Smem& sm, int i, i
       atomicOr(s.status, SDMS_STATUS_SEARCH_FALLBACK);
     }
   }
+  if (!EXPORT && s.pool == 0 && s.mode != 1) {
+    if (M <= 32) {
+      dag_walk_warp(s, i, M, mlist, plen, poff, draft_tok, draft_len, draft_score, draft_edge_w);
+      return;
+    }
+    const WalkPlan w = walk_plan(s, M, sm.pool_words);
+    if (w.layers > 0) {
+      if (w.packed) dag_walk<true>(s, w, i, M, mlist, plen, poff, root, draft_tok, draft_len, draft_score, draft_edge_w);
+      else dag_walk<false>(s, w, i, M, mlist, plen, poff, root, draft_tok, draft_len, draft_score, draft_edge_w);
+      return;
+    }
+  }
   if (!EXPORT && s.pool == 2) list_pool(s, i, M, mlist, plen, poff, draft_tok, draft_len, draft_score, draft_edge_w);
   else if (M <= 32) dag_small<EXPORT>(s, sm, i, M, mlist, plen, poff, root, draft_tok, draft_len, draft_score, draft_edge_w);
   else if (!EXPORT && s.pool == 0 && M * s.D <= kStageWords && layers_in_round_ok(M, s.D))
@@ -1261,7 +1657,7 @@ __global__ void __launch_bounds__(kDagThreads, EXPORT ? 1 : 2) dag_kernel(Dev s,
     __syncthreads();
   }
   // more matches than a warp holds: all SMs share the work (the pass that follows this kernel)
-  if (!EXPORT && s.pool == 0 && s.mode != 2 && Mk > 32 && wide_register(s, i, Mk)) return;
+  if (!EXPORT && s.pool == 0 && s.mode != 2 && Mk > kWideFrom && wide_register(s, i, Mk)) return;
   dag_phase<EXPORT>(s, sm, i, Mk, mlist, sh_len, g * s.N, root, draft_tok, draft_len, draft_score, draft_edge_w);
 }
 
@@ -1624,6 +2020,14 @@ __global__ void __launch_bounds__(kFusedThreads, 1) step_kernel(Dev s, int k, in
 
 }  // namespace
 
+// Dynamic shared memory of the single-launch kernels.  A CTA has its SM to itself (registers), so prompts with room for
+// thousands of matches take what the walk over them can use; small prompts keep the cache.
+constexpr size_t kBigPool = 200 * 1024;
+constexpr long long kBigPoolFrom = 32768;             // tokens of a prompt
+static size_t fused_smem_bytes(const Dev& s) {
+  return (long long)s.N * s.L >= kBigPoolFrom ? kBigPool : dag_smem_bytes<false>();
+}
+
 cudaError_t dag_kernel_setup() {
   cudaError_t e = cudaFuncSetAttribute(dag_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)dag_smem_bytes<false>());
@@ -1631,16 +2035,14 @@ cudaError_t dag_kernel_setup() {
     e = cudaFuncSetAttribute(dag_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)dag_smem_bytes<true>());
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(build_fused_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)dag_smem_bytes<false>());
+    e = cudaFuncSetAttribute(build_fused_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBigPool);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(build_fused_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)dag_smem_bytes<false>());
+    e = cudaFuncSetAttribute(build_fused_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBigPool);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(step_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dag_smem_bytes<false>());
+    e = cudaFuncSetAttribute(step_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBigPool);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(step_kernel<false>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(step_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dag_smem_bytes<false>());
+    e = cudaFuncSetAttribute(step_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBigPool);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(step_kernel<true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   return e;
 }
@@ -1649,7 +2051,7 @@ namespace {
 void step_launch_config(const Dev& s, cudaStream_t stream, cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr) {
   *cfg = cudaLaunchConfig_t{};
   cfg->gridDim = dim3(s.P); cfg->blockDim = dim3(kFusedThreads);
-  cfg->dynamicSmemBytes = dag_smem_bytes<false>(); cfg->stream = stream;
+  cfg->dynamicSmemBytes = fused_smem_bytes(s); cfg->stream = stream;
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = s.N; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -1700,7 +2102,7 @@ int build_cluster_size(const Dev& s) {
   for (int c = 8; c >= 2; --c) {
     if (s.N % c) continue;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(s.P); cfg.blockDim = dim3(kFusedThreads); cfg.dynamicSmemBytes = dag_smem_bytes<false>();
+    cfg.gridDim = dim3(s.P); cfg.blockDim = dim3(kFusedThreads); cfg.dynamicSmemBytes = fused_smem_bytes(s);
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = c; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
@@ -1715,11 +2117,11 @@ int build_cluster_size(const Dev& s) {
 cudaError_t launch_build_fused(const Dev& s, int k_hi, int k_lo, int32_t* draft_tok, int32_t* draft_len,
                                float* draft_score, float* draft_edge_w, int32_t* used_k, cudaStream_t stream) {
   if (s.build_cluster <= 1 || k_lo != k_hi)
-    return launch_overlapped(build_fused_kernel<false, false>, dim3(s.P), dim3(kFusedThreads), dag_smem_bytes<false>(), stream,
+    return launch_overlapped(build_fused_kernel<false, false>, dim3(s.P), dim3(kFusedThreads), fused_smem_bytes(s), stream,
                              s, k_hi, k_lo, draft_tok, draft_len, draft_score, draft_edge_w, used_k, 0);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(s.P); cfg.blockDim = dim3(kFusedThreads);
-  cfg.dynamicSmemBytes = dag_smem_bytes<false>(); cfg.stream = stream;
+  cfg.dynamicSmemBytes = fused_smem_bytes(s); cfg.stream = stream;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = s.build_cluster; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
