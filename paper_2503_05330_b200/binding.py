@@ -122,24 +122,24 @@ def sdms_host_pointer(t) -> int:
 def _dp(t):
     """Pointer the kernels can use: a CUDA tensor's own, or the device-side address of a page-locked
     host tensor that the library has verified (None -> NULL)."""
+    # plain ints: ctypes turns them into void* itself (a c_void_p made here costs 0.2 us, for seven pointers a step)
     if t is None:
         return None
     assert t.is_contiguous()
-    if t.is_cuda:
-        return C.c_void_p(t.data_ptr())
     key = t.data_ptr()
+    if t.is_cuda:
+        return key
     if key not in _mapped:
         _mapped[key] = sdms_host_pointer(t)
-    return C.c_void_p(_mapped[key])
+    return _mapped[key]
 
 
 def _sp(stream):
     """cudaStream_t of a torch stream (None: the current one) or of a raw handle given as int."""
-    if isinstance(stream, int):
-        return C.c_void_p(stream)
     if stream is None:
-        stream = torch.cuda.current_stream()
-    return C.c_void_p(stream.cuda_stream)
+        # the handle itself: 0.3 us, where building the torch.cuda.Stream object around it takes 3.5 us a call
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    return stream if isinstance(stream, int) else stream.cuda_stream
 
 
 # ---- the C entry points, one to one ------------------------------------------
