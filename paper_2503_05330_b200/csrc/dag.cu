@@ -1676,6 +1676,85 @@ __device__ __forceinline__ bool window_head_equal(const int32_t* at, int k, cons
   return true;
 }
 
+// Is some window of k - 1, k or k + 1 tokens (at least one) that ends at `at` = row + e within one edit of q[0 .. k)?
+// With a = common prefix and b = common suffix (each at most the shorter length) of q and the window: iff a + b >= the
+// longer length - 1.  The window's tokens are compared with q at three offsets, one bit per token; all loads are independent.
+__device__ __forceinline__ bool one_edit_end(const int32_t* at, int e, const int32_t* q, int k) {
+  unsigned same = 0u, shorter = 0u, longer = 0u;       // bit t: the token t before the end equals q[k - 1 - t], q[k - 2 - t], q[k - t]
+#pragma unroll 4
+  for (int t = 0; t <= k; ++t) {
+    const int x = t <= e ? ldm(at - t) : -1;
+    same |= (unsigned)(t < k && x == q[max(k - 1 - t, 0)]) << t;
+    shorter |= (unsigned)(t + 1 < k && x == q[max(k - 2 - t, 0)]) << t;
+    longer |= (unsigned)(t > 0 && x == q[k - t]) << t;
+  }
+  const int b = __ffs(~same) - 1;                      // common suffix of q and the path's end (the same for every window)
+  auto ok = [&](int n, unsigned mask) {
+    if (n < 1 || n > e + 1) return false;
+    const int a = __clz(~(mask << (32 - n)));          // bits n - 1, n - 2, ...: the common prefix
+    return min(a, min(k, n)) + min(b, min(k, n)) >= max(k, n) - 1;
+  };
+  return ok(k, same) || ok(k - 1, shorter) || ok(k + 1, longer);
+}
+
+// All positions of the other paths of prompt g that match the query q[0 .. k) of its path `own`: emit(position).  The
+// prompt's rows lie one behind the other, so any row length is read in 16-byte chunks, eight of a thread's in flight.  A
+// position is looked at more closely only if its own token and the one before it allow it (the neighbouring lane or the
+// same chunk has that token).  FUZZY (one edit): the token at the end or the one before it is one of the query's last two.
+template <bool FUZZY, class Emit>
+__device__ __forceinline__ void scan_prompt(const Dev& s, int g, int own, int k, const int32_t* q, const int32_t* plen, Emit emit) {
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int row0 = g * s.N, lo = row0 * s.L, hi = lo + s.N * s.L, a0 = lo & ~3, total = (hi - a0 + 3) >> 2;
+  const int4* const t4 = reinterpret_cast<const int4*>(s.tok) + (a0 >> 2);
+  const int last = q[k - 1], before_last = k >= 2 ? q[k - 2] : -1;
+  constexpr int kBatch = 8;
+#pragma unroll 1
+  for (int base = 0; base < total; base += kBatch * (int)blockDim.x) {       // same trip count for every thread
+    int4 w[kBatch];
+    int left0[kBatch];
+#pragma unroll
+    for (int r = 0; r < kBatch; ++r) {
+      const int x = base + r * (int)blockDim.x + tid, at = a0 + 4 * x;
+      w[r] = make_int4(-1, -1, -1, -1); left0[r] = -1;
+      if (x >= total) continue;
+      const int j = path_of(s, at), e = at - j * s.L, jn = j - row0;
+      // nothing of the chunk's first row can match (its end, the query's own path), and no other row begins in it
+      const bool dead = jn < 0 || jn == own || e > plen[jn] - 2;
+      if (dead && e + 3 < s.L) continue;
+      w[r] = ldm(t4 + x);
+      if (lane == 0 && at > lo && k >= 2) left0[r] = ldm(s.tok + at - 1);
+    }
+    unsigned cand = 0;                                                       // bit 4 r + u: position u of chunk r is a candidate
+#pragma unroll
+    for (int r = 0; r < kBatch; ++r) {
+      int left = __shfl_up_sync(FULL, w[r].w, 1);
+      if (lane == 0) left = left0[r];
+      const int v[5] = {left, w[r].x, w[r].y, w[r].z, w[r].w};
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const bool ok = FUZZY ? k < 2 || v[u + 1] == last || v[u + 1] == before_last || v[u] == last || v[u] == before_last
+                              : v[u + 1] == last && (k < 2 || v[u] == before_last);
+        cand |= (unsigned)ok << (4 * r + u);
+      }
+    }
+    // one copy of the code that looks closer, run once per candidate
+    while (cand) {
+      const int bit = __ffs(cand) - 1;
+      cand &= cand - 1;
+      const int at = a0 + 4 * (base + (bit >> 2) * (int)blockDim.x + tid) + (bit & 3);
+      const int j = path_of(s, at), e = at - j * s.L, jn = j - row0;
+      if (jn < 0 || jn >= s.N || jn == own || e > plen[jn] - 2) continue;
+      if (FUZZY) {
+        if (k >= 2 && !one_edit_end(s.tok + at, e, q, k)) continue;
+      } else {
+        if (e < k - 1) continue;
+        if (k >= 3 && !window_head_equal(s.tok + at, k, q)) continue;
+      }
+      emit(at);
+    }
+  }
+}
+
 // ---- a thread-block cluster shares the scan of its prompt ------------------------------------------
 // In the single-launch build every query that its index bucket cannot answer streams the other paths
 // of the prompt; with many such queries the same histories cross the chip once per query.  When the
@@ -1712,7 +1791,7 @@ __device__ void shared_scan(const Dev& s, int g, int k, int nq, const int32_t (*
   const int tid = threadIdx.x;
   const int32_t* gtok = s.tok + (size_t)g * s.N * s.L;
   const int pos0 = g * s.N * s.L, slice = s.N * s.L;
-  const int per = s.L >> 2, total = s.N * per;
+  const int total = s.N * (s.L >> 2);
   const int4* g4 = reinterpret_cast<const int4*>(gtok);
   const int lo = (int)((long long)total * crank / csize), hi = (int)((long long)total * (crank + 1) / csize);
   constexpr int kBatch = 8;
@@ -1722,7 +1801,7 @@ __device__ void shared_scan(const Dev& s, int g, int k, int nq, const int32_t (*
 #pragma unroll
     for (int r = 0; r < kBatch; ++r) {
       const int x = base + r * blockDim.x + tid;
-      jn[r] = x < hi ? x / per : -1;
+      jn[r] = x < hi ? path_of(s, 4 * x) : -1;
       e0[r] = jn[r] >= 0 ? 4 * x - jn[r] * s.L : 0;
       e_hi[r] = jn[r] >= 0 ? sh_len[jn[r]] - 2 : -1;
       w[r] = make_int4(-1, -1, -1, -1);
@@ -1869,99 +1948,14 @@ __device__ void build_phase(const Dev& s, const Smem& sm, int k_hi, int k_lo, in
       for (int x = tid; x < min(M, kListCap); x += blockDim.x) sm.list[x] = __ldcg(my_matches + x);
       if (tid == 0) sh_M = M;
     }
-  } else if (mode == Q_SCAN && s.eps > 0) {
-    // Eq. 4 with tolerance 1.  A window s' is within one edit of the query q iff, with a = their common
-    // prefix and b = their common suffix (each at most the shorter length), a + b >= max(|q|, |s'|) - 1.
-    // For the windows that end at e, b is shared; a is looked at only as far as it can still decide.
-    const int32_t* gtok = s.tok + (size_t)g * s.N * s.L;
-    for (int jn = 0; jn < s.N; ++jn) {
-      if (g * s.N + jn == i) continue;
-      const int32_t* row = gtok + (size_t)jn * s.L;
-      const int e_hi = sh_len[jn] - 2;
-      for (int e = tid; e <= e_hi; e += blockDim.x) {
-        int b = 0;
-        while (b < k && b <= e && ldm(row + e - b) == sh_q[k - 1 - b]) ++b;
-        bool found = false;
-        for (int n = max(1, k - 1); n <= k + 1 && !found; ++n) {
-          if (e - n + 1 < 0) break;
-          const int shorter = min(k, n), need = max(k, n) - 1 - min(b, shorter);
-          if (need <= 0) { found = true; break; }
-          if (need > shorter) continue;
-          int a = 0;
-          while (a < need && ldm(row + e - n + 1 + a) == sh_q[a]) ++a;
-          found = a >= need;
-        }
-        if (found) {
-          const int at = atomicAdd(&sh_M, 1);
-          const int pos = (g * s.N + jn) * s.L + e;
-          if (at < kListCap) sm.list[at] = pos;
-          my_matches[at] = pos;
-        }
-      }
-    }
   } else if (mode == Q_SCAN) {
-    // every other path of the prompt, all loads independent of each other:
-    // compare the last token of the query first, the rest of the window on a hit
-    const int last = sh_q[k - 1];
-    const int32_t* gtok = s.tok + (size_t)g * s.N * s.L;
-    const int own = i - g * s.N;
-    const int pos0 = g * s.N * s.L;
-    if ((s.L & 3) == 0) {
-      // 16-byte chunks, chunk x = path x / per, tokens 4 * (x % per) ..; a thread keeps eight loads in flight.
-      // A position passes on to the full comparison only if the token before it fits as well: that token
-      // sits in the same chunk or in the neighbouring lane's, so the filter costs no dependent load.
-      const int per = s.L >> 2, total = s.N * per;
-      const int4* g4 = reinterpret_cast<const int4*>(gtok);
-      const int before_last = k >= 2 ? sh_q[k - 2] : -1;
-      constexpr int kBatch = 8;
-      for (int base = 0; base < total; base += kBatch * blockDim.x) {       // same trip count for every thread
-        int4 w[kBatch];
-        int e0[kBatch], e_hi[kBatch];
-#pragma unroll
-        for (int r = 0; r < kBatch; ++r) {
-          const int x = base + r * blockDim.x + tid;
-          const int jn = x < total ? x / per : own;
-          e0[r] = 4 * x - jn * s.L;                                   // 4 * (x % per)
-          e_hi[r] = jn != own ? sh_len[jn] - 2 : -1;                  // last position with a follower
-          w[r] = make_int4(-1, -1, -1, -1);
-          if (e0[r] <= e_hi[r]) w[r] = ldm(g4 + x);
-        }
-        unsigned cand = 0;                                            // bit 4 r + u: position u of chunk r is a candidate
-#pragma unroll
-        for (int r = 0; r < kBatch; ++r) {
-          const int left = __shfl_up_sync(FULL, w[r].w, 1);           // last token of the chunk before this one
-          const int v[5] = {left, w[r].x, w[r].y, w[r].z, w[r].w};
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const bool ok = v[u + 1] == last && e0[r] + u >= k - 1 && e0[r] + u <= e_hi[r] &&
-                            (k < 2 || v[u] == before_last || (u == 0 && (tid & 31) == 0));
-            cand |= (unsigned)ok << (4 * r + u);
-          }
-        }
-        // one copy of the code that looks closer, run once per candidate
-        while (cand) {
-          const int bit = __ffs(cand) - 1;
-          cand &= cand - 1;
-          const int at = 4 * (base + (bit >> 2) * (int)blockDim.x + tid) + (bit & 3);   // position within the prompt
-          if (k >= 2 && (bit & 3) == 0 && (tid & 31) == 0 && ldm(gtok + at - 1) != before_last) continue;
-          if (k >= 3 && !window_head_equal(gtok + at, k, sh_q)) continue;
-          const int n = atomicAdd(&sh_M, 1);
-          if (n < kListCap) sm.list[n] = pos0 + at;
-          my_matches[n] = pos0 + at;
-        }
-      }
-    } else {
-      const int total = s.N * s.L;
-      for (int x = tid; x < total; x += blockDim.x) {
-        const int jn = x / s.L, e = x - jn * s.L;
-        if (jn == own || e < k - 1 || e > sh_len[jn] - 2) continue;
-        if (ldm(gtok + x) != last) continue;
-        if (k >= 2 && (ldm(gtok + x - 1) != sh_q[k - 2] || !window_head_equal(gtok + x, k, sh_q))) continue;
-        const int n = atomicAdd(&sh_M, 1);
-        if (n < kListCap) sm.list[n] = pos0 + x;
-        my_matches[n] = pos0 + x;
-      }
-    }
+    auto emit = [&](int pos) {
+      const int n = atomicAdd(&sh_M, 1);
+      if (n < kListCap) sm.list[n] = pos;
+      my_matches[n] = pos;
+    };
+    if (s.eps > 0) scan_prompt<true>(s, g, i - g * s.N, k, sh_q, sh_len, emit);
+    else scan_prompt<false>(s, g, i - g * s.N, k, sh_q, sh_len, emit);
   }
   __syncthreads();
   if (sh_M > 0 || k <= k_lo) break;

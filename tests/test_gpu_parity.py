@@ -99,6 +99,42 @@ def test_append_of_wide_rows(width):
     pair.build_and_compare(3)
 
 
+@pytest.mark.parametrize("eps", [0, 1])
+@pytest.mark.parametrize("L", [5, 61, 62, 63, 64, 129])
+def test_single_launch_scan_of_any_row_length(L, eps):
+    # several prompts one behind the other: rows that start at every offset from a 16-byte boundary, paths of every
+    # length up to full (a full path is searched but does not search), chunks that reach over a row's end
+    G, N, V, k_max = 3, 3, 3, 4
+    tokens, lps = synth.small_random(G * N, L, V, 6200 + L)
+    pair = Pair(G, N, L, V, min(k_max, L - 1), 4, alpha=0.5, eps=eps)
+    assert pair.g.step_is_single_launch()
+    lens = np.array([L, L - 1, L - 2, max(L - 3, 1), L // 2, 1, 0, L - 1, L - 4], np.int32)
+    pair.append(tokens, lps, lens, expect_status=0)
+    for k in range(1, min(k_max, L - 1) + 1):
+        pair.build_and_compare(k)
+
+
+@pytest.mark.parametrize("M", [31, 32, 33, 127, 128, 129, 600])
+@pytest.mark.parametrize("alpha", [1.0, 0.5])
+def test_walk_at_the_edges_of_its_forms(M, alpha):
+    # one query with exactly M matches (a marker token nowhere else), followers over a small alphabet with a heavy-tailed
+    # draw: one warp to 32, one warp's registers to 128, several warps and several rounds of layers beyond
+    V, D, k = 50, 9, 1
+    step = D + 2
+    L = 2 + ((M + 1) // 2 + 1) * step
+    rng = np.random.default_rng(7000 + M)
+    tokens = 1 + np.minimum((rng.random((3, L)) ** 3 * (V - 1)).astype(np.int32), V - 2)
+    lps = -rng.exponential(0.5, (3, L)).astype(np.float32)
+    at = [(p, 1 + m * step) for m in range((M + 1) // 2) for p in (1, 2)][:M]
+    for p, x in at:
+        tokens[p, x] = 0
+    tokens[0, L - 3] = 0
+    pair = Pair(1, 3, L, V, k, D, alpha=alpha)
+    pair.append(tokens, lps, np.array([L - 2, L - 1, L - 1]), expect_status=0)
+    tok, ln = pair.build_and_compare(k)
+    assert len(pair.o.matches(0)) == M and ln[0] > 0
+
+
 def test_empty_and_degenerate_states():
     # nothing appended yet, then a single token per path, then k larger than some paths
     pair = Pair(2, 3, 16, 5, 3, 3, B=2, Ke=2)
