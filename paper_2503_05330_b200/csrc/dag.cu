@@ -1676,27 +1676,6 @@ __device__ __forceinline__ bool window_head_equal(const int32_t* at, int k, cons
   return true;
 }
 
-// Is some window of k - 1, k or k + 1 tokens (at least one) that ends at `at` = row + e within one edit of q[0 .. k)?
-// With a = common prefix and b = common suffix (each at most the shorter length) of q and the window: iff a + b >= the
-// longer length - 1.  The window's tokens are compared with q at three offsets, one bit per token; all loads are independent.
-__device__ __forceinline__ bool one_edit_end(const int32_t* at, int e, const int32_t* q, int k) {
-  unsigned same = 0u, shorter = 0u, longer = 0u;       // bit t: the token t before the end equals q[k - 1 - t], q[k - 2 - t], q[k - t]
-#pragma unroll 4
-  for (int t = 0; t <= k; ++t) {
-    const int x = t <= e ? ldm(at - t) : -1;
-    same |= (unsigned)(t < k && x == q[max(k - 1 - t, 0)]) << t;
-    shorter |= (unsigned)(t + 1 < k && x == q[max(k - 2 - t, 0)]) << t;
-    longer |= (unsigned)(t > 0 && x == q[k - t]) << t;
-  }
-  const int b = __ffs(~same) - 1;                      // common suffix of q and the path's end (the same for every window)
-  auto ok = [&](int n, unsigned mask) {
-    if (n < 1 || n > e + 1) return false;
-    const int a = __clz(~(mask << (32 - n)));          // bits n - 1, n - 2, ...: the common prefix
-    return min(a, min(k, n)) + min(b, min(k, n)) >= max(k, n) - 1;
-  };
-  return ok(k, same) || ok(k - 1, shorter) || ok(k + 1, longer);
-}
-
 // All positions of the other paths of prompt g that match the query q[0 .. k) of its path `own`: emit(position).  The
 // prompt's rows lie one behind the other, so any row length is read in 16-byte chunks, eight of a thread's in flight.  A
 // position is looked at more closely only if its own token and the one before it allow it (the neighbouring lane or the

@@ -4,7 +4,7 @@
 // within edit distance 1 of the query; each position counts once.  Index counts say nothing about how
 // many such positions there are, so the match slices are sized by counting first:
 //   fuzzy_prepare  every path with a query (k tokens, not full) is marked for scanning, counters zeroed
-//   fuzzy_scan     (count) one CTA per 1024-token tile of one path j: positions that can end a match of
+//   fuzzy_scan     (count) one CTA per 512-token tile of one path j: positions that can end a match of
 //                  ANY query of the prompt are picked out by a bit table, then tested against every query
 //   fuzzy_alloc    slices handed out from the match list by the counts
 //   fuzzy_scan     (fill) the same scan writes the positions
@@ -17,15 +17,16 @@
 // a bit that some query set for q[k-1] or q[k-2].  With k = 1 every position is within one substitution
 // of every query and nothing is filtered.
 //
-// The test.  With a = common prefix and b = common suffix of q and a window s' (each at most the shorter
-// length), the edit distance is at most 1 iff a + b >= max(|q|, |s'|) - 1.
+// The test: one_edit_end, for the pairs of candidate and query that the two tokens at the candidate's end do not rule
+// out.  A scan of 96 x 3000 tokens took 84 us with every pair tested, 55 with the pairs sorted out first but tested where they
+// turned up (one or two lanes of a warp at a time), 20.5 with the pairs queued per warp.
 #include "sdms_internal.h"
 
 namespace sdms {
 
 namespace {
 
-constexpr int kFzTile = 1024;
+constexpr int kFzTile = 512;                       // 96 x 3000 tokens: 20.5 us a scan, with 256 21, with 1024 28.5 (too few CTAs)
 constexpr int kFzThreads = 256;
 constexpr int kFzHalo = SDMS_MAX_K + 1;            // tokens in front of a tile that a window may reach
 constexpr int kFzBits = 65536;
@@ -61,31 +62,17 @@ __global__ void __launch_bounds__(256) fuzzy_alloc_kernel(Dev s) {
   }
 }
 
-// Is some window that ends at position e of `row` (tokens row[0 .. e]) within one edit of q[0 .. k)?
-__device__ __forceinline__ bool one_edit_end(const int32_t* row, int e, const int32_t* q, int k) {
-  int b = 0;
-  while (b < k && b <= e && row[e - b] == q[k - 1 - b]) ++b;
-  for (int n = max(1, k - 1); n <= k + 1; ++n) {
-    if (e - n + 1 < 0) break;
-    const int shorter = min(k, n), need = max(k, n) - 1 - min(b, shorter);
-    if (need <= 0) return true;
-    if (need > shorter) continue;
-    int a = 0;
-    while (a < need && row[e - n + 1 + a] == q[a]) ++a;
-    if (a >= need) return true;
-  }
-  return false;
-}
-
 template <bool FILL>
 __global__ void __launch_bounds__(kFzThreads) fuzzy_scan_kernel(Dev s, int k, int tiles) {
   __shared__ int32_t sh_tok[kFzHalo + kFzTile];            // sh_tok[kFzHalo + x] = token at t0 + x
   __shared__ uint32_t sh_bits[kFzBits / 32];
   __shared__ int32_t sh_q[kFzQueries][SDMS_MAX_K];
-  __shared__ int32_t sh_qi[kFzQueries];
+  __shared__ int32_t sh_qi[kFzQueries], sh_last[kFzQueries], sh_before[kFzQueries];   // its path, last token, the one before
+  __shared__ int sh_count[kFzQueries];
+  __shared__ int sh_pair[kFzThreads / 32][64];             // per warp: pairs that wait to be tested, position << 8 | query
   __shared__ int sh_cand[kFzTile];
   __shared__ int sh_ncand, sh_nq;
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int j = blockIdx.x / tiles, t0 = (blockIdx.x - j * tiles) * kFzTile;
   const int g = j / s.N, len_j = s.len[j];
   const int e_hi = min(t0 + kFzTile - 1, len_j - 2);        // last position of the tile with a follower
@@ -137,25 +124,54 @@ __global__ void __launch_bounds__(kFzThreads) fuzzy_scan_kernel(Dev s, int k, in
       const int i = g * s.N + n;
       if (i == j || s.q_mode[i] != Q_SCAN) continue;
       const int at = atomicAdd(&sh_nq, 1);
-      sh_qi[at] = i;
+      sh_qi[at] = i; sh_count[at] = 0;
       const int32_t* rec = s.rec + (size_t)i * kRecWords;
       for (int t = 0; t < k; ++t) sh_q[at][t] = rec[k - t];   // oldest token first
+      sh_last[at] = rec[1]; sh_before[at] = k >= 2 ? rec[2] : rec[1];
     }
     __syncthreads();
     const int nq = sh_nq;
-    for (int x = tid; x < ncand * nq; x += blockDim.x) {
-      const int c = x / nq, q = x - c * nq;
-      const int pos = sh_cand[c];                              // position t0 + pos
-      // the window may reach kFzHalo tokens in front of the tile; what lies before the path's start is -1
-      const int reach = min(t0 + pos, kFzHalo + pos);          // tokens available before (and at) the position, minus one
-      if (!one_edit_end(sh_tok + kFzHalo + pos - reach, reach, sh_q[q], k)) continue;
-      const int i = sh_qi[q];
-      if (FILL) {
-        const int at = atomicAdd(&s.q_cursor[i], 1);
-        if (at < s.q_reserved[i]) s.matches[(size_t)s.q_off[i] + at] = j * s.L + t0 + pos;
-      } else {
-        atomicAdd(&s.q_reserved[i], 1);
+    // A warp per candidate, its lanes over the queries: the two tokens at the candidate's end decide almost always.  Pairs
+    // that pass are queued and tested 32 at a time, so that no lane tests while the others wait.
+    int waiting = 0;                                           // the same in every lane
+    auto test = [&](int take) {
+      __syncwarp();
+      waiting -= take;
+      if (lane < take) {
+        const int pair = sh_pair[warp][waiting + lane], pos = pair >> 8, q = pair & 255;
+        if (k < 2 || one_edit_end(sh_tok + kFzHalo + pos, t0 + pos, sh_q[q], k)) {
+          if (FILL) {
+            const int i = sh_qi[q], n = atomicAdd(&s.q_cursor[i], 1);
+            if (n < s.q_reserved[i]) s.matches[(size_t)s.q_off[i] + n] = j * s.L + t0 + pos;
+          } else {
+            atomicAdd(&sh_count[q], 1);
+          }
+        }
       }
+      __syncwarp();
+    };
+    for (int c = warp; c < ncand; c += kFzThreads / 32) {
+      const int pos = sh_cand[c];                              // position t0 + pos; what lies before the path's start is -1
+      const int32_t end = sh_tok[kFzHalo + pos], before_end = sh_tok[kFzHalo + pos - 1];
+      for (int q0 = 0; q0 < nq; q0 += 32) {
+        const int q = q0 + lane;
+        bool pass = q < nq;
+        if (pass && k >= 2) {
+          const int32_t a = sh_last[q], b = sh_before[q];
+          pass = end == a || end == b || before_end == a || before_end == b;
+        }
+        const unsigned who = __ballot_sync(0xffffffffu, pass);
+        if (who == 0u) continue;
+        if (pass) sh_pair[warp][waiting + __popc(who & ((1u << lane) - 1u))] = pos << 8 | q;
+        waiting += __popc(who);
+        if (waiting >= 32) test(32);
+      }
+    }
+    if (waiting) test(waiting);
+    if (!FILL) {
+      __syncthreads();
+      for (int q = tid; q < nq; q += blockDim.x)
+        if (sh_count[q]) atomicAdd(&s.q_reserved[sh_qi[q]], sh_count[q]);
     }
   }
 }

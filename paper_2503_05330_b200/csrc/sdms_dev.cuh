@@ -127,6 +127,27 @@ __device__ __forceinline__ double eq5_weight(double alpha, unsigned long long S,
   return __dadd_rn(t1, t2);
 }
 
+// Is some window of k - 1, k or k + 1 tokens (at least one) that ends at `at` = row + e within one edit of q[0 .. k)?
+// With a = common prefix and b = common suffix (each at most the shorter length) of q and the window: iff a + b >= the
+// longer length - 1.  The window's tokens are compared with q at three offsets, one bit per token; all loads are independent.
+__device__ __forceinline__ bool one_edit_end(const int32_t* at, int e, const int32_t* q, int k) {
+  unsigned same = 0u, shorter = 0u, longer = 0u;       // bit t: the token t before the end equals q[k - 1 - t], q[k - 2 - t], q[k - t]
+#pragma unroll 4
+  for (int t = 0; t <= k; ++t) {
+    const int x = t <= e ? at[-t] : -1;
+    same |= (unsigned)(t < k && x == q[max(k - 1 - t, 0)]) << t;
+    shorter |= (unsigned)(t + 1 < k && x == q[max(k - 2 - t, 0)]) << t;
+    longer |= (unsigned)(t > 0 && x == q[k - t]) << t;
+  }
+  const int b = __ffs(~same) - 1;                      // common suffix of q and the path's end (the same for every window)
+  auto ok = [&](int n, unsigned mask) {
+    if (n < 1 || n > e + 1) return false;
+    const int a = __clz(~(mask << (32 - n)));          // bits n - 1, n - 2, ...: the common prefix
+    return min(a, min(k, n)) + min(b, min(k, n)) >= max(k, n) - 1;
+  };
+  return ok(k, same) || ok(k - 1, shorter) || ok(k + 1, longer);
+}
+
 // Programmatic dependent launch: a kernel launched with launch_overlapped() may be scheduled while
 // the kernel before it on the stream is still draining.  grid_wait() returns once that kernel has
 // completed and its writes are visible; everything that touches memory comes after it.
