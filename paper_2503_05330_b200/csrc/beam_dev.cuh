@@ -172,4 +172,163 @@ __device__ __forceinline__ void beams_of_query(const Dev& s, int i, int M, const
   for (size_t x = tid; x < ((size_t)D << lcap) * stride; x += blockDim.x) ze[x] = make_uint4(0u, 0u, 0u, 0u);
 }
 
+// The same for pools whose tables fit shared memory (a hundred-odd matches), by one CTA.  Layers from the last to the
+// first; most nodes carry one candidate, and such a node's list is its successor's with its own weight added: a thread
+// each.  A node with several candidates is worked out by a warp: its lanes hold the candidates, every rank is an arg-max
+// over the best continuation that each candidate's next node has left.  Bound by dependent shared-memory accesses; over
+// tables in global memory (two rounds of L2 atomics and a barrier per layer and rank) 139 us for 30 matches, D = 8, B = 4.
+struct BeamPlan { int cap, stride; };    // slots per layer's table, words per row of items; cap = 0: does not fit
+__device__ __forceinline__ BeamPlan beam_plan(int M, int D, int B, unsigned bytes) {
+  BeamPlan w;
+  w.cap = 64;
+  while (7 * w.cap < 8 * M && w.cap < (1 << 20)) w.cap *= 2;
+  w.stride = (M + 31) & ~31;
+  const long long need = (long long)D * (w.cap * (20ll + 16 * B) + w.stride * 8ll) + 4ll * w.cap;
+  if (need > (long long)bytes) w.cap = 0;
+  return w;
+}
+
+__device__ __forceinline__ u64 beam_warp_max(u64 x) {
+  const unsigned hi = (unsigned)(x >> 32), top = __reduce_max_sync(FULL, hi);
+  const unsigned lo = __reduce_max_sync(FULL, hi == top ? (unsigned)x : 0u);
+  return (u64)top << 32 | lo;
+}
+
+__device__ __forceinline__ void beams_in_shared(const Dev& s, const BeamPlan w, int M, const int32_t* list, int B, int32_t* beam_tok,
+                                                int32_t* beam_len, float* beam_value) {
+  extern __shared__ __align__(16) unsigned char beam_smem[];
+  __shared__ BeamEnt sh_root[SDMS_MAX_BEAMS];
+  __shared__ int sh_n[2];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5, D = s.D;
+  const int cap = w.cap, mask = cap - 1, shift = __clz(cap) + 1, stride = w.stride, all = D * cap;
+  BeamEnt* const ent = reinterpret_cast<BeamEnt*>(beam_smem);          // [layer][slot][rank]
+  int* const key = reinterpret_cast<int*>(ent + (size_t)all * B);      // [layer][slot]
+  unsigned* const lo = reinterpret_cast<unsigned*>(key + all);         // sums of the lower 16 bits, of the rest, count
+  unsigned* const hi = lo + all;
+  unsigned* const cnt = hi + all;
+  int* const own = reinterpret_cast<int*>(cnt + all);                  // a candidate of the node
+  int* const tok = own + all;                                          // [layer][candidate], -1: has ended
+  int* const slot = tok + D * stride;
+  int* const todo = slot + D * stride;                                 // [cap] nodes of the layer with several candidates
+
+  for (int x = tid; x < all; x += blockDim.x) { key[x] = -1; lo[x] = 0u; hi[x] = 0u; cnt[x] = 0u; }
+  if (tid < 2) sh_n[tid] = 0;
+  __syncthreads();
+  // candidates' followers into the tables: a warp takes 32 candidates of one layer
+  const int nchunk = stride >> 5;
+  for (int t = warp, l = 0, c = warp; t < D * nchunk; t += nwarps, c += nwarps) {
+    while (c >= nchunk) { c -= nchunk; ++l; }
+    const int m = c * 32 + lane;
+    int v = -1;
+    unsigned p = 0u;
+    if (m < M) {
+      const int gpos = list[m], j = path_of(s, gpos);
+      if (l + 1 <= __ldg(s.len + j) - 1 - (gpos - j * s.L)) { v = __ldg(s.tok + gpos + l + 1); p = (unsigned)__ldg(s.pq + gpos + l + 1); }
+    }
+    int sl = 0;
+    if (v >= 0) {
+      unsigned h = ((unsigned)v * 2654435761u) >> shift;
+      int k;
+#pragma unroll 1
+      while (true) {                                                   // ends: more slots than candidates
+        k = atomicCAS(&key[l * cap + h], -1, v);
+        if (k == -1 || k == v) break;
+        h = (h + 1) & mask;
+      }
+      sl = (int)h;
+      if (k == -1) own[l * cap + h] = m;
+      atomicAdd(&lo[l * cap + h], p & 0xffffu);
+      atomicAdd(&hi[l * cap + h], p >> 16);
+      atomicAdd(&cnt[l * cap + h], 1u);
+    }
+    tok[l * stride + m] = v; slot[l * stride + m] = sl;
+  }
+  __syncthreads();
+  // the B best continuations among what the candidates with `on` set have at layer l + 1, each with w_u added (add); lane 0
+  // writes them to `to`; false: none of them goes on
+  auto merge = [&](int l, int at, bool add, double w_u, BeamEnt* to) -> bool {       // at: the node's slot at layer l, -1: the root
+    BeamEnt prev{~0ull, ~0ull};
+    for (int r = 0; r < B; ++r) {
+      u64 bv = 0ull, bn = 0ull;
+      for (int m = lane; m < M; m += 32) {
+        if (at >= 0 && (tok[l * stride + m] < 0 || slot[l * stride + m] != at)) continue;
+        const int vn = l + 1 < D ? tok[(l + 1) * stride + m] : -1;
+        if (vn < 0) continue;
+        const int sn = slot[(l + 1) * stride + m];
+        const BeamEnt* const theirs = ent + ((size_t)(l + 1) * cap + sn) * B;
+        for (int j = 0; j < B; ++j) {                                  // best first: the first that is still left is the offer
+          const BeamEnt e = theirs[j];
+          if (e.next == 0ull) break;
+          const u64 val = add ? (u64)__double_as_longlong(__dadd_rn(w_u, __longlong_as_double((long long)e.value))) : e.value;
+          const u64 nx = beam_next((uint32_t)vn, j, sn);
+          if (r > 0 && !beam_after(val, nx, prev)) continue;
+          if (bn == 0ull || val > bv || (val == bv && nx > bn)) { bv = val; bn = nx; }
+          break;
+        }
+      }
+      const unsigned any = __ballot_sync(FULL, bn != 0ull);
+      if (any == 0u) {
+        if (r == 0) return false;
+        if (lane == 0) for (int x = r; x < B; ++x) to[x] = BeamEnt{0ull, 0ull};
+        return true;
+      }
+      prev.value = beam_warp_max(bn ? bv : 0ull);
+      prev.next = beam_warp_max(bn && bv == prev.value ? bn : 0ull);
+      if (lane == 0) to[r] = prev;
+    }
+    return true;
+  };
+  auto weight = [&](int x) { return eq5_weight(s.alpha, ((u64)hi[x] << 16) + lo[x], cnt[x]); };
+#pragma unroll 1
+  for (int l = D - 1; l >= 0; --l) {
+    for (int x = tid; x < cap; x += blockDim.x) {
+      const int at = l * cap + x;
+      if (key[at] < 0) continue;
+      if (cnt[at] > 1u) { todo[atomicAdd(&sh_n[l & 1], 1)] = x; continue; }
+      const double w_u = weight(at);
+      BeamEnt* const mine = ent + (size_t)at * B;
+      const int m = own[at], vn = l + 1 < D ? tok[(l + 1) * stride + m] : -1;
+      if (vn < 0) {
+        for (int r = 0; r < B; ++r) mine[r] = r == 0 ? BeamEnt{(u64)__double_as_longlong(w_u), kBeamLeaf} : BeamEnt{0ull, 0ull};
+        continue;
+      }
+      const int sn = slot[(l + 1) * stride + m];
+      const BeamEnt* const theirs = ent + ((size_t)(l + 1) * cap + sn) * B;
+      for (int r = 0; r < B; ++r) {
+        const BeamEnt e = theirs[r];
+        mine[r] = e.next == 0ull ? BeamEnt{0ull, 0ull}
+                                 : BeamEnt{(u64)__double_as_longlong(__dadd_rn(w_u, __longlong_as_double((long long)e.value))),
+                                           beam_next((uint32_t)vn, r, sn)};
+      }
+    }
+    __syncthreads();
+    const int n = sh_n[l & 1];
+    if (tid == 0) sh_n[(l & 1) ^ 1] = 0;
+    for (int q = warp; q < n; q += nwarps) {
+      const int x = todo[q], at = l * cap + x;
+      const double w_u = weight(at);
+      BeamEnt* const mine = ent + (size_t)at * B;
+      if (!merge(l, x, true, w_u, mine) && lane == 0)                  // a leaf: its only continuation is to stop
+        for (int r = 0; r < B; ++r) mine[r] = r == 0 ? BeamEnt{(u64)__double_as_longlong(w_u), kBeamLeaf} : BeamEnt{0ull, 0ull};
+    }
+    __syncthreads();
+  }
+  if (warp != 0) return;
+  if (!merge(-1, -1, false, 0.0, sh_root) && lane == 0)
+    for (int r = 0; r < B; ++r) sh_root[r] = BeamEnt{0ull, 0ull};
+  __syncwarp();
+  if (lane < B) {
+    BeamEnt e = sh_root[lane];
+    int len = 0;
+    beam_value[lane] = e.next != 0ull ? (float)__longlong_as_double((long long)e.value) : 0.0f;
+    for (int d = 0; d < D && e.next != 0ull && e.next != kBeamLeaf; ++d) {
+      const int rank = 7 - (int)((e.next >> 24) & 7u), sl = (int)(e.next & 0xffffffu);
+      beam_tok[lane * D + len++] = (int32_t)~(uint32_t)(e.next >> 32);
+      e = ent[((size_t)d * cap + sl) * B + rank];
+    }
+    for (int d = len; d < D; ++d) beam_tok[lane * D + d] = -1;
+    beam_len[lane] = len;
+  }
+}
+
 }  // namespace sdms

@@ -8,9 +8,13 @@ namespace sdms {
 
 namespace {
 
+constexpr int kBeamSmem = 200 * 1024;                 // shared memory of a CTA: one per SM
+
 __global__ void __launch_bounds__(kWideThreads, 1) beam_kernel(Dev s, int B, int32_t* __restrict__ beam_tok,
                                                                int32_t* __restrict__ beam_len,
                                                                float* __restrict__ beam_value) {
+  grid_wait();
+  grid_release();
   __shared__ long long sh_first;
   const int i = blockIdx.x, tid = threadIdx.x, D = s.D;
   int32_t* const my_tok = beam_tok + (size_t)i * B * D;
@@ -32,6 +36,12 @@ __global__ void __launch_bounds__(kWideThreads, 1) beam_kernel(Dev s, int B, int
   if (sh_first < 0) {                                  // no match, or no room: no beam
     for (int x = tid; x < B * D; x += blockDim.x) my_tok[x] = -1;
     if (tid < B) { beam_len[(size_t)i * B + tid] = 0; beam_value[(size_t)i * B + tid] = 0.0f; }
+    return;
+  }
+  // (the room in the table area decides who is served, also where the work is done in shared memory)
+  const BeamPlan w = beam_plan(M, D, B, kBeamSmem);
+  if (w.cap) {
+    beams_in_shared(s, w, M, s.matches + s.q_off[i], B, my_tok, beam_len + (size_t)i * B, beam_value + (size_t)i * B);
     return;
   }
   beams_of_query(s, i, M, s.matches + s.q_off[i], (unsigned)sh_first, lcap, B, my_tok, beam_len + (size_t)i * B,
@@ -73,6 +83,11 @@ __global__ void __launch_bounds__(kWideThreads, 1) best_path_fix_kernel(Dev s, i
 
 }  // namespace
 
+// Called when a context is created, with its device current.
+cudaError_t beam_kernel_setup() {
+  return cudaFuncSetAttribute(beam_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kBeamSmem);
+}
+
 cudaError_t launch_best_path_fix(const Dev& s, int32_t* draft_tok, int32_t* draft_len, float* draft_score,
                                  float* draft_edge_w, cudaStream_t stream) {
   cudaError_t e = cudaMemsetAsync(s.b_ctl + 1, 0, 8, stream);
@@ -85,8 +100,7 @@ cudaError_t launch_beams(const Dev& s, int B, int32_t* beam_tok, int32_t* beam_l
                          cudaStream_t stream) {
   cudaError_t e = cudaMemsetAsync(s.b_ctl, 0, 8, stream);
   if (e != cudaSuccess) return e;
-  beam_kernel<<<s.P, kWideThreads, 0, stream>>>(s, B, beam_tok, beam_len, beam_value);
-  return cudaGetLastError();
+  return launch_overlapped(beam_kernel, dim3(s.P), dim3(kWideThreads), kBeamSmem, stream, s, B, beam_tok, beam_len, beam_value);
 }
 
 }  // namespace sdms

@@ -53,5 +53,6 @@ cudaError_t launch_best_path_fix(const Dev& s, int32_t* draft_tok, int32_t* draf
                                  float* draft_edge_w, cudaStream_t stream);
 cudaError_t dag_kernel_setup();
 cudaError_t scan_kernel_setup();
+cudaError_t beam_kernel_setup();
 
 }  // namespace sdms

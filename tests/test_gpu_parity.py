@@ -129,10 +129,11 @@ def test_walk_at_the_edges_of_its_forms(M, alpha):
     for p, x in at:
         tokens[p, x] = 0
     tokens[0, L - 3] = 0
-    pair = Pair(1, 3, L, V, k, D, alpha=alpha)
+    pair = Pair(1, 3, L, V, k, D, alpha=alpha, max_beams=3)
     pair.append(tokens, lps, np.array([L - 2, L - 1, L - 1]), expect_status=0)
     tok, ln = pair.build_and_compare(k)
     assert len(pair.o.matches(0)) == M and ln[0] > 0
+    pair.beams_and_compare(3, paths=[0])              # in shared memory up to 129 of these, over the table area for 600
 
 
 def test_empty_and_degenerate_states():
