@@ -9,10 +9,11 @@ using namespace sdms;
 namespace {
 
 constexpr size_t kAlign = 256;
+constexpr size_t kEpochIndexBytes = 16 << 20;   // index from which a reset counts epochs instead of clearing: 16 MiB clear in 4 us
 inline size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
 struct Layout {
-  size_t tok, pq, len, rec, status, index, q_fp, q_mode, q_reserved, q_off, q_cursor, match_cursor, g_nscan, g_trim, a_plan, matches;
+  size_t tok, pq, len, rec, status, index, q_fp, q_mode, q_reserved, q_off, q_cursor, match_cursor, g_nscan, g_trim, a_plan, matches, e_ctl;
   size_t w_ctl, w_desc, w_pred, w_edge, w_tab, w_key, w_item, b_ent, b_ctl, bp_todo;
   bool wide_on;
   uint64_t w_slots;
@@ -76,6 +77,7 @@ Layout make_layout(const sdms_config* c) {
   l.g_trim = take((size_t)c->num_groups * 4);
   l.a_plan = take(P * 8);
   l.matches = take((size_t)mc * 4);
+  l.e_ctl = take(8);
   l.x_draft_tok = take(P * D * 4); l.x_draft_len = take(P * 4);
   l.x_node_tok = take(P * D * B * 4); l.x_node_S = take(P * D * B * 8); l.x_node_cnt = take(P * D * B * 4);
   l.x_node_count = take(P * D * 4);
@@ -249,6 +251,7 @@ int sdms_create(const sdms_config* cfg, void* d_workspace, size_t bytes, sdms_ct
   d.eps = cfg->epsilon;
   d.pool = cfg->pool_mode;
   d.R = cfg->max_matches_per_path;
+  d.epochs = lay.q_fp - lay.index >= kEpochIndexBytes;
   ctx->step_fits = false;                        // decided below, once the kernels' attributes are set
   unsigned char* w = ctx->ws;
   d.tok = (int32_t*)(w + lay.tok); d.pq = (int32_t*)(w + lay.pq); d.len = (int32_t*)(w + lay.len); d.rec = (int32_t*)(w + lay.rec);
@@ -257,7 +260,7 @@ int sdms_create(const sdms_config* cfg, void* d_workspace, size_t bytes, sdms_ct
   d.q_reserved = (int32_t*)(w + lay.q_reserved); d.q_off = (int32_t*)(w + lay.q_off);
   d.match_cursor = (unsigned long long*)(w + lay.match_cursor);
   d.q_cursor = (int32_t*)(w + lay.q_cursor); d.g_nscan = (int32_t*)(w + lay.g_nscan); d.g_trim = (int32_t*)(w + lay.g_trim);
-  d.a_plan = (int2*)(w + lay.a_plan);
+  d.a_plan = (int2*)(w + lay.a_plan); d.e_ctl = (uint32_t*)(w + lay.e_ctl);
   d.matches = (int32_t*)(w + lay.matches);
   ctx->x_draft_tok = (int32_t*)(w + lay.x_draft_tok); ctx->x_draft_len = (int32_t*)(w + lay.x_draft_len);
   d.x_node_tok = (int32_t*)(w + lay.x_node_tok); d.x_node_S = (int64_t*)(w + lay.x_node_S);
@@ -281,9 +284,14 @@ int sdms_reset(sdms_ctx* ctx, void* stream) {
   cudaStream_t st = (cudaStream_t)stream;
   // the path store need not be cleared: lengths say what is valid
   const Layout& l = ctx->lay;
-  if (cudaMemsetAsync(ctx->ws + l.len, 0, l.matches - l.len, st) != cudaSuccess) return SDMS_ERR_CUDA;
   ctx->built = false;
-  return SDMS_OK;
+  // a large index is not cleared: its buckets go out of date with the epoch
+  if (ctx->dev.epochs) {
+    ++ctx->launches;
+    return launch_reset(ctx->dev, ctx->ws + l.len, l.index - l.len, ctx->ws + l.q_fp, l.matches - l.q_fp, l.q_fp - l.index, st) ==
+                   cudaSuccess ? SDMS_OK : SDMS_ERR_CUDA;
+  }
+  return cudaMemsetAsync(ctx->ws + l.len, 0, l.matches - l.len, st) == cudaSuccess ? SDMS_OK : SDMS_ERR_CUDA;
 }
 
 int sdms_destroy(sdms_ctx* ctx) {

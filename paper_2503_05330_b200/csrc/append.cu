@@ -98,13 +98,14 @@ __global__ void __launch_bounds__(kPlanThreads) append_plan_kernel(Dev s, const 
 // at x0 + t (shared memory).
 __device__ __forceinline__ void insert_positions(const Dev& s, int p, int n, int x0, int x1, const int32_t* win, uint32_t* st) {
   const int g = p / s.N;
+  const uint32_t epoch = epoch_of(s.rec[(size_t)p * kRecWords + kRecEpoch]);
   const uint32_t lbase = (uint32_t)(p - g * s.N) * (uint32_t)s.L;
   for (int x = x0 + (int)threadIdx.x; x < x1; x += kBulkThreads) {
     if (x + 1 < n) continue;
     uint64_t h = gram_init(n);
     const int32_t* q = win + kHalo - n + (x - x0);
     for (int t = 0; t < n; ++t) h = gram_step(h, q[t]);
-    index_insert_bulk(s, g, n, gram_final(h), lbase + (uint32_t)x, st);
+    index_insert<true>(s, g, n, gram_final(h), lbase + (uint32_t)x, epoch, st);
   }
 }
 
@@ -157,6 +158,28 @@ __global__ void __launch_bounds__(128) accept_kernel(Dev s, const int32_t* __res
   accept_commit_phase(s, blockIdx.x, draft_tok, draft_len, sampled, sampled_lp, accept_len);
 }
 
+// sdms_reset of a large index: lengths, records and the small state between `a` / `b` and their ends become zero, the
+// records get the next epoch.  Only when the epochs run out (every 255th time) the index is cleared.
+__global__ void __launch_bounds__(256) reset_kernel(Dev s, uint4* a, size_t a_words, uint4* b, size_t b_words, size_t index_words) {
+  grid_wait();
+  grid_release();
+  const uint32_t next = *(volatile uint32_t*)s.e_ctl + 1u < 255u ? *(volatile uint32_t*)s.e_ctl + 1u : 0u;
+  const size_t first = (size_t)blockIdx.x * blockDim.x + threadIdx.x, step = (size_t)gridDim.x * blockDim.x;
+  const size_t rec0 = reinterpret_cast<uint4*>(s.rec) - a, rec1 = rec0 + (size_t)s.P * kRecWords / 4;
+  for (size_t x = first; x < a_words; x += step) {
+    const bool tail = x >= rec0 && x < rec1 && (x - rec0) % (kRecWords / 4) == kRecWords / 4 - 1;
+    a[x] = make_uint4(0u, 0u, 0u, tail ? next : 0u);
+  }
+  for (size_t x = first; x < b_words; x += step) b[x] = make_uint4(0u, 0u, 0u, 0u);
+  if (next == 0u)
+    for (size_t x = first; x < index_words; x += step) reinterpret_cast<uint4*>(s.index)[x] = make_uint4(0u, 0u, 0u, 0u);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    if (atomicAdd(&s.e_ctl[1], 1u) == gridDim.x - 1) { s.e_ctl[1] = 0u; s.e_ctl[0] = next; }      // everybody has read it
+  }
+}
+
 // sdms_trim, first launch: path p keeps its newest keep[p] tokens, moved to the front of its store.
 __global__ void __launch_bounds__(128) trim_shift_kernel(Dev s, const int32_t* __restrict__ keep) {
   grid_wait();
@@ -183,7 +206,7 @@ __global__ void __launch_bounds__(128) trim_shift_kernel(Dev s, const int32_t* _
   }
   int32_t* rec = s.rec + (size_t)p * kRecWords;
   if (threadIdx.x == 0) { s.len[p] = want; rec[0] = want; s.g_trim[p / s.N] = 1; }
-  if (threadIdx.x >= 1 && threadIdx.x < kRecWords && (int)threadIdx.x > want) rec[threadIdx.x] = 0;   // tokens that are gone
+  if (threadIdx.x >= 1 && threadIdx.x <= SDMS_MAX_K && (int)threadIdx.x > want) rec[threadIdx.x] = 0;   // tokens that are gone
 }
 
 // Second launch: the tables of the prompts that changed become empty.
@@ -217,6 +240,13 @@ __global__ void __launch_bounds__(kBulkThreads, 8) trim_reindex_kernel(Dev s, in
 }
 
 }  // namespace
+
+cudaError_t launch_reset(const Dev& s, void* a, size_t a_bytes, void* b, size_t b_bytes, size_t index_bytes, cudaStream_t stream) {
+  const size_t words = (a_bytes + b_bytes) / 16;
+  const unsigned ctas = (unsigned)(words < 148 * 256 ? (words + 255) / 256 : 148 * 4);
+  return launch_overlapped(reset_kernel, dim3(ctas), dim3(256), 0, stream, s, static_cast<uint4*>(a), a_bytes / 16, static_cast<uint4*>(b),
+                           b_bytes / 16, index_bytes / 16);
+}
 
 namespace {
 // Positions per CTA of the kernels that index rows of `width` positions of every path: few, short CTAs where the device

@@ -1858,7 +1858,8 @@ __device__ void build_phase(const Dev& s, const Smem& sm, int k_hi, int k_lo, in
       uint64_t h = gram_init(nx);
       for (int t = 0; t < k; ++t) { const int32_t x = ldm(rec + k - t); sh_q[t] = x; if (t >= k - nx) h = gram_step(h, x); }
       h = gram_final(h);
-      fp = gram_fp(h);
+      const uint32_t epoch = epoch_of(ldm(rec + kRecEpoch));
+      fp = index_tag(h, epoch);
       const uint32_t* table = index_table(s, g, nx);
       uint32_t b = gram_bucket(h, s.table_cap);
       for (uint32_t probe = 0; probe < s.table_cap; ++probe) {
@@ -1870,7 +1871,7 @@ __device__ void build_phase(const Dev& s, const Smem& sm, int k_hi, int k_lo, in
           mode = count <= (uint32_t)kInlineSlots ? Q_INLINE : Q_SCAN;
           break;
         }
-        if (lo.x == 0u) break;
+        if (bucket_empty(lo.x, epoch)) break;
         b = (b + 1) & (s.table_cap - 1);
       }
     }

@@ -86,7 +86,7 @@ __global__ void __launch_bounds__(kProbeWarps * 32) probe_kernel(Dev s, int k, i
     }
     fp = gram_fp(gram_final(h));
     hx = gram_final(hx);
-    const uint32_t want = gram_fp(hx);
+    const uint32_t epoch = epoch_of(__shfl_sync(FULL_MASK, mine, kRecEpoch)), want = index_tag(hx, epoch);
     const uint32_t* table = index_table(s, g, nx);
     uint32_t b = gram_bucket(hx, s.table_cap);
     int found = -1;                                              // lane that holds the bucket's first word
@@ -98,7 +98,7 @@ __global__ void __launch_bounds__(kProbeWarps * 32) probe_kernel(Dev s, int k, i
       for (int r = 0; r < 4 && found < 0 && !end; ++r) {
         const uint32_t w0 = __shfl_sync(FULL_MASK, word, 8 * r);
         if (w0 == want) found = 8 * r;
-        else if (w0 == 0u) end = true;
+        else if (bucket_empty(w0, epoch)) end = true;
       }
       if (end) break;
       b = (b + 4) & (s.table_cap - 1);

@@ -22,6 +22,7 @@ cudaError_t launch_overlapped(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
 constexpr int kBulkAppendFrom = 64;   // row width from which an append is two launches (plan, many CTAs per path)
 cudaError_t launch_append(const Dev& s, const int32_t* tokens, const float* logprobs, const int32_t* counts,
                           int row_width, cudaStream_t stream);
+cudaError_t launch_reset(const Dev& s, void* a, size_t a_bytes, void* b, size_t b_bytes, size_t index_bytes, cudaStream_t stream);
 cudaError_t launch_accept(const Dev& s, const int32_t* draft_tok, const int32_t* draft_len,
                           const int32_t* sampled, const float* sampled_lp, int32_t* accept_len,
                           cudaStream_t stream);

@@ -136,6 +136,35 @@ def test_walk_at_the_edges_of_its_forms(M, alpha):
     pair.beams_and_compare(3, paths=[0])              # in shared memory up to 129 of these, over the table area for 600
 
 
+@pytest.mark.parametrize("N,L", [(16, 1024), (64, 2048)])
+def test_reset_leaves_nothing_behind(N, L):
+    # an index that is cleared and one whose buckets go out of date: more resets than there are epochs, other streams
+    # after each; buckets of every age are met by appends of both widths, by steps and by a trim
+    V, k_max, D = 30, 3, 4
+    pair = Pair(1, N, L, V, k_max, D, max_append=D)
+    for it in range(262):
+        pair.g.reset()
+        if it not in (0, 1, 2, 100, 253, 254, 255, 256, 261):
+            tok, lp = synth.small_random(N, 70, 2000, 300 + it)           # many different n-grams, to age the buckets
+            pair.g.append(harness.t32(tok, pair.dev), harness.t32(lp, pair.dev), harness.t32(np.full(N, 70, np.int32), pair.dev))
+            continue
+        from oracle import Oracle
+        pair.o = Oracle(1, N, L, V, D)
+        tok, lp = synth.small_random(N, 160, V, 900 + it)
+        pair.append(tok[:, :100], lp[:, :100], np.full(N, 100), expect_status=0)
+        pair.append(tok[:, 100:120], lp[:, 100:120], np.full(N, 20), expect_status=0)
+        for k in (3, 2):
+            _, ln = pair.build_and_compare(k, check_dag=False)
+        d_tok, d_ln, _, _ = pair.o.drafts()
+        sm, slp = synth.sampled_window(tok, lp, pair.o.lengths(), D + 1)
+        pair.o.accept_commit(d_tok, d_ln, sm, slp, D)
+        pair.g.accept(harness.t32(sm, pair.dev), harness.t32(slp, pair.dev))
+        pair.build_and_compare(3, check_dag=False)
+        pair.trim(np.full(N, 60, np.int32))
+        pair.check_history()
+        pair.build_and_compare(2, check_dag=False)
+
+
 def test_empty_and_degenerate_states():
     # nothing appended yet, then a single token per path, then k larger than some paths
     pair = Pair(2, 3, 16, 5, 3, 3, B=2, Ke=2)
