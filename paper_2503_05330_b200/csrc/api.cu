@@ -97,7 +97,7 @@ Layout make_layout(const sdms_config* c) {
   }
   l.w_slots = (l.wide_on || (stride > 0 && wide > 0)) ? (uint64_t)wide / slot_bytes : 0;
   l.w_ctl = take((size_t)kWideCtlWords * 8);
-  l.b_ctl = take(16);
+  l.b_ctl = take(32);
   l.bp_todo = take(P * 4);
   l.w_desc = take(l.wide_on ? (size_t)kMaxWide * 16 : 0);
   l.w_pred = take(l.wide_on ? (size_t)kMaxWide * SDMS_MAX_DRAFT * sizeof(WidePred) : 0);

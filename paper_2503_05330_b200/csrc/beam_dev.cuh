@@ -172,19 +172,21 @@ __device__ __forceinline__ void beams_of_query(const Dev& s, int i, int M, const
   for (size_t x = tid; x < ((size_t)D << lcap) * stride; x += blockDim.x) ze[x] = make_uint4(0u, 0u, 0u, 0u);
 }
 
-// The same for pools whose tables fit shared memory (a hundred-odd matches), by one CTA.  Layers from the last to the
-// first; most nodes carry one candidate, and such a node's list is its successor's with its own weight added: a thread
-// each.  A node with several candidates is worked out by a warp: its lanes hold the candidates, every rank is an arg-max
-// over the best continuation that each candidate's next node has left.  Bound by dependent shared-memory accesses; over
-// tables in global memory (two rounds of L2 atomics and a barrier per layer and rank) 139 us for 30 matches, D = 8, B = 4.
-struct BeamPlan { int cap, stride; };    // slots per layer's table, words per row of items; cap = 0: does not fit
+// The same by one CTA with the node tables in shared memory (pools up to several hundred matches), the continuation lists
+// there too if they fit, else in the table area.  Layers from the last to the first.  Most nodes carry one candidate, and
+// such a node's list is its successor's with its own weight added: a thread each.  A node with several candidates is worked
+// out by a warp: a lane per candidate holds the best continuation that its next node has left, and every rank is an arg-max
+// over the lanes.  With more candidates than lanes the B best next nodes are found first, by the heads of their lists: no
+// other one can contribute.  Bound by dependent accesses; with everything in the table area (two rounds of L2 atomics and a
+// barrier per layer and rank) 139 us for 30 matches, 570 us for 760, D = 8, B = 4.
+struct BeamPlan { int cap, stride; bool lists; };    // slots per layer's table (0: does not fit), items per row, lists in shared memory
 __device__ __forceinline__ BeamPlan beam_plan(int M, int D, int B, unsigned bytes) {
   BeamPlan w;
-  w.cap = 64;
-  while (7 * w.cap < 8 * M && w.cap < (1 << 20)) w.cap *= 2;
+  w.cap = 1 << beam_lcap(min(M, 1 << 20));
   w.stride = (M + 31) & ~31;
-  const long long need = (long long)D * (w.cap * (20ll + 16 * B) + w.stride * 8ll) + 4ll * w.cap;
-  if (need > (long long)bytes) w.cap = 0;
+  const long long tables = (long long)D * (w.cap * 16ll + w.stride * 2ll) + w.cap * 6ll + w.stride * 2ll;
+  w.lists = tables + (long long)D * w.cap * B * 16 <= (long long)bytes;
+  if (tables > (long long)bytes || M >= 0xffff) w.cap = 0;
   return w;
 }
 
@@ -194,38 +196,43 @@ __device__ __forceinline__ u64 beam_warp_max(u64 x) {
   return (u64)top << 32 | lo;
 }
 
-__device__ __forceinline__ void beams_in_shared(const Dev& s, const BeamPlan w, int M, const int32_t* list, int B, int32_t* beam_tok,
-                                                int32_t* beam_len, float* beam_value) {
+// ent0: the path's lists in the table area, ent_stride entries per slot (used if !SHARED_LISTS; left zero).  want0, score0,
+// edge0: as for beams_of_query.
+template <bool SHARED_LISTS>
+__device__ __forceinline__ void beams_in_shared(const Dev& s, const BeamPlan w, int M, const int32_t* list, int B, BeamEnt* ent0,
+                                                int ent_stride, int32_t* beam_tok, int32_t* beam_len, float* beam_value,
+                                                bool want0 = false, float* score0 = nullptr, float* edge0 = nullptr) {
   extern __shared__ __align__(16) unsigned char beam_smem[];
   __shared__ BeamEnt sh_root[SDMS_MAX_BEAMS];
-  __shared__ int sh_n[2];
+  __shared__ int sh_n, sh_members, sh_blen, sh_bslot[SDMS_MAX_DRAFT];
+  __shared__ unsigned sh_be[SDMS_MAX_DRAFT][3];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5, D = s.D;
   const int cap = w.cap, mask = cap - 1, shift = __clz(cap) + 1, stride = w.stride, all = D * cap;
-  BeamEnt* const ent = reinterpret_cast<BeamEnt*>(beam_smem);          // [layer][slot][rank]
-  int* const key = reinterpret_cast<int*>(ent + (size_t)all * B);      // [layer][slot]
-  unsigned* const lo = reinterpret_cast<unsigned*>(key + all);         // sums of the lower 16 bits, of the rest, count
+  const int es = SHARED_LISTS ? B : ent_stride;
+  BeamEnt* const ent = SHARED_LISTS ? reinterpret_cast<BeamEnt*>(beam_smem) : ent0;          // [layer][slot][rank]
+  int* const key = reinterpret_cast<int*>(beam_smem + (SHARED_LISTS ? (size_t)all * B * 16 : 0));   // [layer][slot] token, -1: free
+  unsigned* const lo = reinterpret_cast<unsigned*>(key + all);         // sums of the lower 16 bits, of the rest
   unsigned* const hi = lo + all;
-  unsigned* const cnt = hi + all;
-  int* const own = reinterpret_cast<int*>(cnt + all);                  // a candidate of the node
-  int* const tok = own + all;                                          // [layer][candidate], -1: has ended
-  int* const slot = tok + D * stride;
-  int* const todo = slot + D * stride;                                 // [cap] nodes of the layer with several candidates
+  unsigned* const cw = hi + all;                                       // a candidate of the node << 16 | count
+  int* const start = reinterpret_cast<int*>(cw + all);                 // [slot] of the layer at hand: where its members are listed
+  unsigned short* const todo = reinterpret_cast<unsigned short*>(start + cap);           // its nodes with several candidates
+  unsigned short* const member = todo + cap;                           // [stride] candidates, node by node
+  unsigned short* const slot = member + stride;                        // [layer][candidate], 0xffff: has ended
+  constexpr int kEnded = 0xffff;
 
-  for (int x = tid; x < all; x += blockDim.x) { key[x] = -1; lo[x] = 0u; hi[x] = 0u; cnt[x] = 0u; }
-  if (tid < 2) sh_n[tid] = 0;
+  for (int x = tid; x < all; x += blockDim.x) { key[x] = -1; lo[x] = 0u; hi[x] = 0u; cw[x] = 0u; }
   __syncthreads();
   // candidates' followers into the tables: a warp takes 32 candidates of one layer
   const int nchunk = stride >> 5;
   for (int t = warp, l = 0, c = warp; t < D * nchunk; t += nwarps, c += nwarps) {
     while (c >= nchunk) { c -= nchunk; ++l; }
     const int m = c * 32 + lane;
-    int v = -1;
+    int v = -1, sl = kEnded;
     unsigned p = 0u;
     if (m < M) {
       const int gpos = list[m], j = path_of(s, gpos);
       if (l + 1 <= __ldg(s.len + j) - 1 - (gpos - j * s.L)) { v = __ldg(s.tok + gpos + l + 1); p = (unsigned)__ldg(s.pq + gpos + l + 1); }
     }
-    int sl = 0;
     if (v >= 0) {
       unsigned h = ((unsigned)v * 2654435761u) >> shift;
       int k;
@@ -236,98 +243,148 @@ __device__ __forceinline__ void beams_in_shared(const Dev& s, const BeamPlan w, 
         h = (h + 1) & mask;
       }
       sl = (int)h;
-      if (k == -1) own[l * cap + h] = m;
       atomicAdd(&lo[l * cap + h], p & 0xffffu);
       atomicAdd(&hi[l * cap + h], p >> 16);
-      atomicAdd(&cnt[l * cap + h], 1u);
+      atomicAdd(&cw[l * cap + h], k == -1 ? (unsigned)m << 16 | 1u : 1u);
     }
-    tok[l * stride + m] = v; slot[l * stride + m] = sl;
+    slot[l * stride + m] = (unsigned short)sl;
   }
   __syncthreads();
-  // the B best continuations among what the candidates with `on` set have at layer l + 1, each with w_u added (add); lane 0
-  // writes them to `to`; false: none of them goes on
-  auto merge = [&](int l, int at, bool add, double w_u, BeamEnt* to) -> bool {       // at: the node's slot at layer l, -1: the root
-    BeamEnt prev{~0ull, ~0ull};
-    for (int r = 0; r < B; ++r) {
-      u64 bv = 0ull, bn = 0ull;
-      for (int m = lane; m < M; m += 32) {
-        if (at >= 0 && (tok[l * stride + m] < 0 || slot[l * stride + m] != at)) continue;
-        const int vn = l + 1 < D ? tok[(l + 1) * stride + m] : -1;
-        if (vn < 0) continue;
-        const int sn = slot[(l + 1) * stride + m];
-        const BeamEnt* const theirs = ent + ((size_t)(l + 1) * cap + sn) * B;
-        for (int j = 0; j < B; ++j) {                                  // best first: the first that is still left is the offer
-          const BeamEnt e = theirs[j];
-          if (e.next == 0ull) break;
-          const u64 val = add ? (u64)__double_as_longlong(__dadd_rn(w_u, __longlong_as_double((long long)e.value))) : e.value;
-          const u64 nx = beam_next((uint32_t)vn, j, sn);
-          if (r > 0 && !beam_after(val, nx, prev)) continue;
-          if (bn == 0ull || val > bv || (val == bv && nx > bn)) { bv = val; bn = nx; }
-          break;
+  auto weight = [&](int x) { return eq5_weight(s.alpha, ((u64)hi[x] << 16) + lo[x], cw[x] & 0xffffu); };
+  struct Offer { u64 val, nx; };
+  // what next node sn of layer l + 1 has to offer at rank j (nothing: nx = 0)
+  auto offer_of = [&](int l, int sn, int j, bool add, double w_u) {
+    Offer o{0ull, 0ull};
+    if (sn == kEnded || j >= B) return o;
+    const BeamEnt e = ent[((size_t)(l + 1) * cap + sn) * es + j];
+    if (e.next == 0ull) return o;
+    o.val = add ? (u64)__double_as_longlong(__dadd_rn(w_u, __longlong_as_double((long long)e.value))) : e.value;
+    o.nx = beam_next((uint32_t)key[(l + 1) * cap + sn], j, sn);
+    return o;
+  };
+  // The B best continuations of the n candidates cand(0 .. n - 1) at layer l (-1: the root), w_u added to each (add), written
+  // to `to` by lane 0; false: none of them goes on.
+  auto merge = [&](int l, int n, auto cand, bool add, double w_u, BeamEnt* to) -> bool {
+    auto next_of = [&](int x) { return l + 1 < D ? (int)slot[(l + 1) * stride + cand(x)] : kEnded; };
+    int sn = kEnded;                                                   // this lane's next node
+    if (n <= 32) {
+      if (lane < n) sn = next_of(lane);
+    } else {
+      Offer prev{~0ull, ~0ull};
+      for (int r = 0; r < B; ++r) {
+        Offer best{0ull, 0ull};
+#pragma unroll 4
+        for (int x = lane; x < n; x += 32) {
+          const Offer o = offer_of(l, next_of(x), 0, add, w_u);
+          const bool after = o.val < prev.val || (o.val == prev.val && o.nx < prev.nx);
+          if (o.nx != 0ull && after && (o.val > best.val || (o.val == best.val && o.nx > best.nx))) best = o;
         }
+        prev.val = beam_warp_max(best.val);
+        prev.nx = beam_warp_max(best.val == prev.val ? best.nx : 0ull);
+        if (prev.nx == 0ull) break;
+        if (lane == r) sn = (int)(prev.nx & 0xffffffu);
       }
-      const unsigned any = __ballot_sync(FULL, bn != 0ull);
-      if (any == 0u) {
+    }
+    int j = 0;
+    Offer mine = offer_of(l, sn, 0, add, w_u);
+    for (int r = 0; r < B; ++r) {
+      const u64 val = beam_warp_max(mine.val), nx = beam_warp_max(mine.val == val ? mine.nx : 0ull);
+      if (nx == 0ull) {
         if (r == 0) return false;
         if (lane == 0) for (int x = r; x < B; ++x) to[x] = BeamEnt{0ull, 0ull};
         return true;
       }
-      prev.value = beam_warp_max(bn ? bv : 0ull);
-      prev.next = beam_warp_max(bn && bv == prev.value ? bn : 0ull);
-      if (lane == 0) to[r] = prev;
+      if (lane == 0) to[r] = BeamEnt{val, nx};
+      if (mine.val == val && mine.nx == nx) mine = offer_of(l, sn, ++j, add, w_u);      // (every lane with this next node)
     }
     return true;
   };
-  auto weight = [&](int x) { return eq5_weight(s.alpha, ((u64)hi[x] << 16) + lo[x], cnt[x]); };
 #pragma unroll 1
   for (int l = D - 1; l >= 0; --l) {
+    if (tid == 0) { sh_n = 0; sh_members = 0; }
+    __syncthreads();
     for (int x = tid; x < cap; x += blockDim.x) {
       const int at = l * cap + x;
       if (key[at] < 0) continue;
-      if (cnt[at] > 1u) { todo[atomicAdd(&sh_n[l & 1], 1)] = x; continue; }
-      const double w_u = weight(at);
-      BeamEnt* const mine = ent + (size_t)at * B;
-      const int m = own[at], vn = l + 1 < D ? tok[(l + 1) * stride + m] : -1;
-      if (vn < 0) {
-        for (int r = 0; r < B; ++r) mine[r] = r == 0 ? BeamEnt{(u64)__double_as_longlong(w_u), kBeamLeaf} : BeamEnt{0ull, 0ull};
+      const unsigned c = cw[at];
+      if ((c & 0xffffu) > 1u) {
+        todo[atomicAdd(&sh_n, 1)] = (unsigned short)x;
+        start[x] = atomicAdd(&sh_members, (int)(c & 0xffffu));
         continue;
       }
-      const int sn = slot[(l + 1) * stride + m];
-      const BeamEnt* const theirs = ent + ((size_t)(l + 1) * cap + sn) * B;
-      for (int r = 0; r < B; ++r) {
-        const BeamEnt e = theirs[r];
-        mine[r] = e.next == 0ull ? BeamEnt{0ull, 0ull}
-                                 : BeamEnt{(u64)__double_as_longlong(__dadd_rn(w_u, __longlong_as_double((long long)e.value))),
-                                           beam_next((uint32_t)vn, r, sn)};
+      const double w_u = weight(at);
+      BeamEnt* const mine = ent + (size_t)at * es;
+      const int sn = l + 1 < D ? (int)slot[(l + 1) * stride + (c >> 16)] : kEnded;
+      if (sn == kEnded) mine[0] = BeamEnt{(u64)__double_as_longlong(w_u), kBeamLeaf};    // a leaf: its only continuation is to stop
+      for (int r = sn == kEnded ? 1 : 0; r < B; ++r) {
+        const Offer o = offer_of(l, sn, r, true, w_u);
+        mine[r] = BeamEnt{o.val, o.nx};
       }
     }
     __syncthreads();
-    const int n = sh_n[l & 1];
-    if (tid == 0) sh_n[(l & 1) ^ 1] = 0;
-    for (int q = warp; q < n; q += nwarps) {
-      const int x = todo[q], at = l * cap + x;
-      const double w_u = weight(at);
-      BeamEnt* const mine = ent + (size_t)at * B;
-      if (!merge(l, x, true, w_u, mine) && lane == 0)                  // a leaf: its only continuation is to stop
-        for (int r = 0; r < B; ++r) mine[r] = r == 0 ? BeamEnt{(u64)__double_as_longlong(w_u), kBeamLeaf} : BeamEnt{0ull, 0ull};
+    const int n = sh_n;
+    if (n > 0) {
+      for (int m = tid; m < M; m += blockDim.x) {
+        const int x = slot[l * stride + m];
+        if (x != kEnded && (cw[l * cap + x] & 0xffffu) > 1u) member[atomicAdd(&start[x], 1)] = (unsigned short)m;
+      }
+      __syncthreads();
+      for (int q = warp; q < n; q += nwarps) {
+        const int x = todo[q], at = l * cap + x, cnt = (int)(cw[at] & 0xffffu);
+        const unsigned short* const mem = member + start[x] - cnt;     // (start has moved to the end)
+        const double w_u = weight(at);
+        BeamEnt* const mine = ent + (size_t)at * es;
+        if (!merge(l, cnt, [&](int y) { return (int)mem[y]; }, true, w_u, mine) && lane == 0)
+          for (int r = 0; r < B; ++r) mine[r] = r == 0 ? BeamEnt{(u64)__double_as_longlong(w_u), kBeamLeaf} : BeamEnt{0ull, 0ull};
+      }
+      __syncthreads();
     }
-    __syncthreads();
   }
-  if (warp != 0) return;
-  if (!merge(-1, -1, false, 0.0, sh_root) && lane == 0)
-    for (int r = 0; r < B; ++r) sh_root[r] = BeamEnt{0ull, 0ull};
-  __syncwarp();
-  if (lane < B) {
-    BeamEnt e = sh_root[lane];
-    int len = 0;
-    beam_value[lane] = e.next != 0ull ? (float)__longlong_as_double((long long)e.value) : 0.0f;
-    for (int d = 0; d < D && e.next != 0ull && e.next != kBeamLeaf; ++d) {
-      const int rank = 7 - (int)((e.next >> 24) & 7u), sl = (int)(e.next & 0xffffffu);
-      beam_tok[lane * D + len++] = (int32_t)~(uint32_t)(e.next >> 32);
-      e = ent[((size_t)d * cap + sl) * B + rank];
+  if (warp == 0) {
+    if (!merge(-1, M, [](int y) { return y; }, false, 0.0, sh_root) && lane == 0)
+      for (int r = 0; r < B; ++r) sh_root[r] = BeamEnt{0ull, 0ull};
+    __syncwarp();
+    if (lane < B) {
+      BeamEnt e = sh_root[lane];
+      int len = 0;
+      beam_value[lane] = e.next != 0ull ? (float)__longlong_as_double((long long)e.value) : 0.0f;
+      for (int d = 0; d < D && e.next != 0ull && e.next != kBeamLeaf; ++d) {
+        const int rank = 7 - (int)((e.next >> 24) & 7u), sl = (int)(e.next & 0xffffffu);
+        if (lane == 0) sh_bslot[len] = sl;
+        beam_tok[lane * D + len++] = (int32_t)~(uint32_t)(e.next >> 32);
+        e = ent[((size_t)d * cap + sl) * es + rank];
+      }
+      if (lane == 0) sh_blen = len;
+      for (int d = len; d < D; ++d) beam_tok[lane * D + d] = -1;
+      beam_len[lane] = len;
     }
-    for (int d = len; d < D; ++d) beam_tok[lane * D + d] = -1;
-    beam_len[lane] = len;
+  }
+  if (want0) {
+    // node weights of the first beam, and of the edges it takes: a warp per layer
+    if (tid < SDMS_MAX_DRAFT) { sh_be[tid][0] = 0u; sh_be[tid][1] = 0u; sh_be[tid][2] = 0u; }
+    __syncthreads();
+    const int len = sh_blen;
+    if (score0 && tid < D) score0[tid] = tid < len ? (float)weight(tid * cap + sh_bslot[tid]) : 0.0f;
+    if (edge0) {
+      for (int l = warp; l < len; l += nwarps) {
+        unsigned e0 = 0u, e1 = 0u, e2 = 0u;
+        for (int m = lane; m < M; m += 32) {
+          if (slot[l * stride + m] != sh_bslot[l] || (l > 0 && slot[(l - 1) * stride + m] != sh_bslot[l - 1])) continue;
+          const unsigned p = (unsigned)__ldg(s.pq + list[m] + l + 1);
+          e0 += p & 0xffffu; e1 += p >> 16; ++e2;
+        }
+        e0 = __reduce_add_sync(FULL, e0); e1 = __reduce_add_sync(FULL, e1); e2 = __reduce_add_sync(FULL, e2);
+        if (lane == 0) { sh_be[l][0] = e0; sh_be[l][1] = e1; sh_be[l][2] = e2; }
+      }
+      __syncthreads();
+      if (tid < D) edge0[tid] = tid < len ? (float)eq5_weight(s.alpha, ((u64)sh_be[tid][1] << 16) + sh_be[tid][0], sh_be[tid][2]) : 0.0f;
+    }
+  }
+  if (!SHARED_LISTS) {                                                  // leave the lists as they were found
+    __syncthreads();
+    for (int x = tid; x < all; x += blockDim.x)
+      if (key[x] >= 0)
+        for (int r = 0; r < B; ++r) ent[(size_t)x * es + r] = BeamEnt{0ull, 0ull};
   }
 }
 

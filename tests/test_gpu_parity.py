@@ -114,7 +114,7 @@ def test_single_launch_scan_of_any_row_length(L, eps):
         pair.build_and_compare(k)
 
 
-@pytest.mark.parametrize("M", [31, 32, 33, 127, 128, 129, 600])
+@pytest.mark.parametrize("M", [31, 32, 33, 127, 128, 129, 600, 1500])
 @pytest.mark.parametrize("alpha", [1.0, 0.5])
 def test_walk_at_the_edges_of_its_forms(M, alpha):
     # one query with exactly M matches (a marker token nowhere else), followers over a small alphabet with a heavy-tailed
@@ -133,7 +133,7 @@ def test_walk_at_the_edges_of_its_forms(M, alpha):
     pair.append(tokens, lps, np.array([L - 2, L - 1, L - 1]), expect_status=0)
     tok, ln = pair.build_and_compare(k)
     assert len(pair.o.matches(0)) == M and ln[0] > 0
-    pair.beams_and_compare(3, paths=[0])              # in shared memory up to 129 of these, over the table area for 600
+    pair.beams_and_compare(3, paths=[0])              # in shared memory up to 129 of these, lists in the table area for 600, all there for 1500
 
 
 @pytest.mark.parametrize("N,L", [(16, 1024), (64, 2048)])
