@@ -14,7 +14,7 @@ inline size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
 struct Layout {
   size_t tok, pq, len, rec, status, index, q_fp, q_mode, q_reserved, q_off, q_cursor, match_cursor, g_nscan, g_trim, a_plan, matches, e_ctl;
-  size_t w_ctl, w_desc, w_pred, w_edge, w_tab, w_key, w_item, b_ent, b_ctl, bp_todo;
+  size_t w_ctl, w_desc, w_done, w_tab, w_key, w_item, b_ent, b_ctl, bp_todo;
   bool wide_on;
   uint64_t w_slots;
   size_t x_draft_tok, x_draft_len, x_node_tok, x_node_S, x_node_cnt, x_node_count, x_edge_dst, x_edge_S, x_edge_cnt, x_out_degree;
@@ -100,8 +100,7 @@ Layout make_layout(const sdms_config* c) {
   l.b_ctl = take(32);
   l.bp_todo = take(P * 4);
   l.w_desc = take(l.wide_on ? (size_t)kMaxWide * 16 : 0);
-  l.w_pred = take(l.wide_on ? (size_t)kMaxWide * SDMS_MAX_DRAFT * sizeof(WidePred) : 0);
-  l.w_edge = take(l.wide_on ? (size_t)kMaxWide * SDMS_MAX_DRAFT * 8 : 0);
+  l.w_done = take(l.wide_on ? (size_t)kMaxWide * 4 : 0);
   l.w_tab = take((size_t)l.w_slots * sizeof(WideSlot));
   l.w_key = take((size_t)l.w_slots * 4);
   l.w_item = take((size_t)l.w_slots * 4);
@@ -268,7 +267,7 @@ int sdms_create(const sdms_config* cfg, void* d_workspace, size_t bytes, sdms_ct
   d.x_edge_dst = (int32_t*)(w + lay.x_edge_dst); d.x_edge_S = (int64_t*)(w + lay.x_edge_S);
   d.x_edge_cnt = (int32_t*)(w + lay.x_edge_cnt); d.x_out_degree = (int32_t*)(w + lay.x_out_degree);
   d.w_ctl = (unsigned long long*)(w + lay.w_ctl); d.w_desc = (int4*)(w + lay.w_desc);
-  d.w_pred = (WidePred*)(w + lay.w_pred); d.w_edge = (unsigned long long*)(w + lay.w_edge);
+  d.w_done = (int*)(w + lay.w_done);
   d.w_tab = (WideSlot*)(w + lay.w_tab); d.w_key = (uint32_t*)(w + lay.w_key); d.w_item = (int32_t*)(w + lay.w_item);
   d.w_grid = lay.wide_on ? wide_kernel_grid() : 0;   // 0 (also without cooperative launch on this device): one thread block per query
   d.w_slots = lay.w_slots;

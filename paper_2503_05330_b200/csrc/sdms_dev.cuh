@@ -22,15 +22,13 @@ constexpr int kFusedMaxTokens = 131072; // largest N*L a CTA scans on its own
 constexpr int kMaxWide = 1024;          // queries one build can hand to the device-wide aggregation pass
 constexpr int kWideSumShift = 47;       // packed node sums: count in the upper 17 bits, sum of probabilities below
 constexpr int kWideMaxMatches = (1 << 17) - 1;   // so that both parts of a packed sum fit
-constexpr int kWideBarrierWays = 8;     // grid-barrier arrivals are spread over this many counters ...
-constexpr int kWideBarrierAt = 16, kWideBarrierStride = 16;   // ... at w_ctl[16], [32], ...: a 128-byte line each
-constexpr int kWideCtlWords = kWideBarrierAt + kWideBarrierWays * kWideBarrierStride;
+constexpr int kWideCtlWords = 3;
 
 // Q_DONE: a back-off build on a large prompt has found this path's matches at a longer suffix length
 enum QueryMode : int32_t { Q_NONE = 0, Q_INLINE = 1, Q_SCAN = 2, Q_DONE = 3 };
 constexpr int kRoundBackoff = 1, kRoundNotFirst = 2, kRoundLast = 4;   // flags of one round of such a build
 
-// One slot of a wide query's node table of one layer (32 bytes, one sector).  All-zero = empty.  The keys
+// One slot of a node table of one layer in the table area (32 bytes, one sector; beams).  All-zero = empty.  The keys
 // (token + 1) that the probing looks at lie in an array of their own, eight to a sector.
 struct WideSlot {
   uint32_t tok1;                 // token + 1, written by whoever claimed the slot
@@ -40,7 +38,6 @@ struct WideSlot {
   unsigned long long succ;       // ~token << 32 | slot of the successor with that weight and the smallest token; 0 = none
 };
 struct BeamEnt;
-struct WidePred { unsigned long long succ_w, succ; };   // the same two words for the root (and, in mode 1, for each layer)
 
 // Everything a kernel needs, passed by value.
 struct Dev {
@@ -76,10 +73,9 @@ struct Dev {
   int32_t* g_trim;                     // [G] a path of the prompt was trimmed: its index is rebuilt
   int32_t* matches;                    // [match_cap] global positions j*L+e
   // device-wide aggregation of queries with many matches (dag_wide.cu); w_slots = 0: not in use
-  unsigned long long* w_ctl;           // [kWideCtlWords] queries registered, slots handed out, -, end of the slots in use; barrier counters
-  int4* w_desc;                        // [kMaxWide] query path, matches, log2 of the slots per layer, first slot
-  WidePred* w_pred;                    // [kMaxWide][SDMS_MAX_DRAFT]
-  unsigned long long* w_edge;          // [kMaxWide][SDMS_MAX_DRAFT] packed sums of the edges the draft takes
+  unsigned long long* w_ctl;           // [kWideCtlWords] queries registered, slots handed out, tasks handed out beyond the first of each CTA
+  int4* w_desc;                        // [kMaxWide] query path, matches, first slot, -
+  int* w_done;                         // [kMaxWide] layers of the query that are done; zero between builds
   WideSlot* w_tab;                     // [w_slots]
   uint32_t* w_key;                     // [w_slots] token + 1 of the node in the slot, 0 = free
   int32_t* w_item;                     // [w_slots] per (layer, match): slot of the item's token in the layer's table

@@ -4,24 +4,19 @@
 
 namespace sdms {
 
-// log2 of the slots of one layer's node table: a power of two above 5/2 of the matches.  A layer in which
-// every candidate is a node of its own fills at most 40 % of it: the whole grid waits for the unluckiest
-// lane of a pass, that is for the fullest eight-key sector of all tables (every claimer that meets
-// somebody else's token there pays another round trip), and how full that sector is grows quickly with the fill.
-__device__ __forceinline__ int wide_lcap(int M) {
-  int l = 6;
-  while ((1ll << l) < (5ll * M) / 2 + 1) ++l;
-  return l;
+// Room (in table slots of 32 bytes) that a query with M matches takes: weight and token of every (match, layer).
+__device__ __forceinline__ unsigned long long wide_slots(const Dev& s, int M) {
+  return ((unsigned long long)M * s.D * 12 + sizeof(WideSlot) - 1) / sizeof(WideSlot);
 }
 
-// The same for the one-CTA-per-path beam kernel, which nobody waits for: above 5/4 of the matches.
+// log2 of the slots of one layer's node table in the table area (beams): a power of two above 5/4 of the matches.
 __device__ __forceinline__ int beam_lcap(int M) {
   int l = 6;
   while ((1ll << l) < (long long)M + (M >> 2) + 1) ++l;
   return l;
 }
 
-// Called by every thread of the query's CTA.  Reserves table slots for all D layers and enters the
+// Called by every thread of the query's CTA.  Reserves room for all D layers and enters the
 // query in the list the wide pass works through; false (for all threads) if the pass is not in use,
 // the list is full or the slots have run out - the caller then aggregates the query itself.
 __device__ __forceinline__ bool wide_register(const Dev& s, int i, int M) {
@@ -29,26 +24,19 @@ __device__ __forceinline__ bool wide_register(const Dev& s, int i, int M) {
   if (s.w_grid == 0 || M > kWideMaxMatches) return false;
   if (threadIdx.x == 0) {
     int q = -1;
-    const int lcap = wide_lcap(M);
-    const unsigned long long need = (unsigned long long)s.D << lcap;
+    const unsigned long long need = wide_slots(s, M);
     const unsigned long long first = atomicAdd(&s.w_ctl[1], need);
     if (first + need <= s.w_slots) {
       const unsigned long long n = atomicAdd(&s.w_ctl[0], 1ull);
       if (n < (unsigned long long)kMaxWide) {
         q = (int)n;
-        s.w_desc[q] = make_int4(i, M, lcap, (int)(unsigned)first);
-        atomicMax(&s.w_ctl[3], first + need);
+        s.w_desc[q] = make_int4(i, M, (int)(unsigned)first, 0);
       }
     }
     sh_wide_q = q;
   }
   __syncthreads();
-  const int q = sh_wide_q;
-  if (q >= 0 && threadIdx.x < SDMS_MAX_DRAFT) {
-    s.w_pred[(size_t)q * SDMS_MAX_DRAFT + threadIdx.x] = WidePred{0ull, 0ull};
-    s.w_edge[(size_t)q * SDMS_MAX_DRAFT + threadIdx.x] = 0ull;
-  }
-  return q >= 0;
+  return sh_wide_q >= 0;
 }
 
 
