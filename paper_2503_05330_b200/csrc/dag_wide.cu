@@ -22,8 +22,9 @@ namespace sdms {
 
 namespace {
 
-constexpr int kWideSmem = 196608;                    // a task's table: 16384 slots of three words, 12288 of four
-constexpr int kWideTableMatches = 14336;             // candidates per table: 7/8 of 16384 if all their tokens differ
+constexpr int kWideSlots = 16384;                    // most slots of a task's table (half of them where counts are kept too)
+constexpr int kWideSmem = kWideSlots * 12;
+constexpr int kWideTableMatches = 16384;             // candidates per table
 constexpr int kWideWarps = kWideThreads / 32;
 constexpr int kSortFrom = 256;                       // more queries than this balance without an order
 
@@ -65,10 +66,63 @@ __device__ __forceinline__ int wide_classes(int M) {
 }
 __device__ __forceinline__ unsigned wide_class(int v) { return ((unsigned)v * 0x85ebca6bu) >> 8; }
 
-// Layer d of a query, tokens of class `cls` of `classes`: node sums, then every candidate's token and node weight.
-__device__ __forceinline__ void wide_sums(const Dev& s, const int4 de, int d, unsigned cls, unsigned classes) {
+// The table of one layer in shared memory.
+struct WideTable { int* key; unsigned* lo; unsigned* hi; unsigned* cnt; int mask, shift; };   // sums of the lower 15 bits, of the rest, counts
+__device__ __forceinline__ WideTable wide_table(unsigned char* smem, int cap) {
+  WideTable t;
+  t.key = reinterpret_cast<int*>(smem);
+  t.lo = reinterpret_cast<unsigned*>(t.key + cap); t.hi = t.lo + cap; t.cnt = t.hi + cap;
+  t.mask = cap - 1; t.shift = __clz(cap) + 1;
+  return t;
+}
+__device__ __forceinline__ void wide_table_empty(unsigned char* smem, int cap, bool counts) {
+  int4* const z = reinterpret_cast<int4*>(smem);
+  const int k4 = cap / 4, end = (counts ? 4 : 3) * k4;
+  for (int x = threadIdx.x; x < k4; x += kWideThreads) z[x] = make_int4(-1, -1, -1, -1);
+  for (int x = k4 + threadIdx.x; x < end; x += kWideThreads) z[x] = make_int4(0, 0, 0, 0);
+}
+// Slot of token v, claimed if need be; -1: the table is full.
+__device__ __forceinline__ int wide_claim(const WideTable& t, int v, int cap) {
+  unsigned h = ((unsigned)v * 2654435761u) >> t.shift;
+#pragma unroll 1
+  for (int probe = 0; probe < cap; ++probe) {
+    int k = *(volatile int*)&t.key[h];
+    if (k == -1) k = atomicCAS(&t.key[h], -1, v);
+    if (k == -1 || k == v) return (int)h;
+    h = (h + 1) & t.mask;
+  }
+  return -1;
+}
+__device__ __forceinline__ void wide_add(const WideTable& t, int h, unsigned p, bool counts) {
+  atomicAdd(&t.lo[h], p & 0x7fffu);
+  atomicAdd(&t.hi[h], p >> 15);
+  if (counts) atomicAdd(&t.cnt[h], 1u);
+}
+__device__ __forceinline__ u64 wide_weight(const Dev& s, const WideTable& t, int h, bool counts) {
+  const u64 S = ((u64)t.hi[h] << 15) + t.lo[h];
+  return counts ? (u64)__double_as_longlong(eq5_weight(s.alpha, S, t.cnt[h])) : S;
+}
+// Followers d of candidates m0, m0 + kWideThreads, ...: token (-1: none) and probability, all requests on their way together.
+template <int N>
+__device__ __forceinline__ void wide_gather(const Dev& s, const int32_t* list, int M, int d, int m0, int (&v)[N], unsigned (&p)[N]) {
+  int gpos[N];
+#pragma unroll
+  for (int r = 0; r < N; ++r) gpos[r] = __ldg(list + min(m0 + r * kWideThreads, M - 1));
+#pragma unroll
+  for (int r = 0; r < N; ++r) {
+    const int j = path_of(s, gpos[r]);
+    const bool on = m0 + r * kWideThreads < M && gpos[r] - j * s.L + d <= __ldg(s.len + j) - 1;
+    v[r] = -1; p[r] = 0u;
+    if (on) { v[r] = __ldg(s.tok + gpos[r] + d); p[r] = (unsigned)__ldg(s.pq + gpos[r] + d); }
+  }
+}
+
+// Layer d of a query with at most N * CH * kWideThreads candidates: node sums, then every candidate's token and node weight.
+// The slots stay in registers in between.  false: more distinct tokens than slots, nothing is done.
+template <int N, int CH>
+__device__ __forceinline__ bool wide_sums_kept(const Dev& s, const int4 de, int d) {
   extern __shared__ __align__(16) unsigned char wide_smem[];
-  __shared__ int sh_over;
+  __shared__ int sh_full;
   const int tid = threadIdx.x, M = de.y;
   const int32_t* const list = s.matches + s.q_off[de.x];
   const WideItems items = wide_items(s, de.z, M);
@@ -76,155 +130,159 @@ __device__ __forceinline__ void wide_sums(const Dev& s, const int4 de, int d, un
   int* const tok = items.tok + (size_t)(d - 1) * M;
   const bool counts = s.alpha != 1.0;                  // with alpha = 1 a weight does not depend on the count
   int cap = 64;
-  const int most = counts ? 8192 : 16384;              // slots that fit
-  while (cap < most && 7ll * cap < 8ll * M) cap *= 2;
-  const int mask = cap - 1, shift = __clz(cap) + 1;
-  int* const key = reinterpret_cast<int*>(wide_smem);
-  unsigned* const lo = reinterpret_cast<unsigned*>(key + cap);         // sums of the lower 15 bits, of the rest, counts
-  unsigned* const hi = lo + cap;
-  unsigned* const cnt = hi + cap;
-  const int rounds = (M + kWideThreads - 1) / kWideThreads;
-  // Almost always one pass.  A table that turns out too small is done again in sub-classes.
+  while (cap < (counts ? kWideSlots / 2 : kWideSlots) && 7 * cap < 8 * M) cap *= 2;
+  const WideTable t = wide_table(wide_smem, cap);
+  if (tid == 0) sh_full = 0;
+  int v[N];
+  unsigned p[N];
+  wide_gather<N>(s, list, M, d, tid, v, p);            // on its way while the table is emptied
+  wide_table_empty(wide_smem, cap, counts);
+  __syncthreads();
+  int slot[CH][N];
+#pragma unroll
+  for (int c = 0; c < CH; ++c) {
+    const int m0 = c * N * kWideThreads + tid;
+    if (c > 0) wide_gather<N>(s, list, M, d, m0, v, p);
+#pragma unroll
+    for (int r = 0; r < N; ++r) {
+      const int m = m0 + r * kWideThreads;
+      if (m < M) tok[m] = v[r];
+      slot[c][r] = -1;
+      if (v[r] < 0) continue;
+      slot[c][r] = wide_claim(t, v[r], cap);
+      if (slot[c][r] < 0) sh_full = 1;
+      else wide_add(t, slot[c][r], p[r], counts);
+    }
+  }
+  __syncthreads();
+  if (sh_full) return false;                           // (the same for everybody)
+#pragma unroll
+  for (int c = 0; c < CH; ++c)
+#pragma unroll
+    for (int r = 0; r < N; ++r)
+      if (slot[c][r] >= 0) weight[(c * N + r) * kWideThreads + tid] = wide_weight(s, t, slot[c][r], counts);
+  return true;
+}
+
+// The same for any number of candidates, tokens of class `cls` of `classes`; the followers are fetched twice.  Almost always
+// one pass; a table that turns out too small is done again in sub-classes.
+__device__ __forceinline__ void wide_sums_any(const Dev& s, const int4 de, int d, unsigned cls, unsigned classes) {
+  extern __shared__ __align__(16) unsigned char wide_smem[];
+  __shared__ int sh_over;
+  const int tid = threadIdx.x, M = de.y;
+  const int32_t* const list = s.matches + s.q_off[de.x];
+  const WideItems items = wide_items(s, de.z, M);
+  u64* const weight = items.weight + (size_t)(d - 1) * M;
+  int* const tok = items.tok + (size_t)(d - 1) * M;
+  const bool counts = s.alpha != 1.0;
+  const int cap = counts ? kWideSlots / 2 : kWideSlots;
+  const WideTable t = wide_table(wide_smem, cap);
   unsigned subs = 1;
 #pragma unroll 1
   for (unsigned sub = 0; sub < subs; ++sub) {
     const unsigned all_classes = classes * subs, mine = cls + classes * sub;
     if (tid == 0) sh_over = 0;
-    {
-      int4* const z = reinterpret_cast<int4*>(wide_smem);
-      const int k4 = cap / 4, end = (counts ? 4 : 3) * k4;
-      for (int x = tid; x < k4; x += kWideThreads) z[x] = make_int4(-1, -1, -1, -1);
-      for (int x = k4 + tid; x < end; x += kWideThreads) z[x] = make_int4(0, 0, 0, 0);
-    }
+    wide_table_empty(wide_smem, cap, counts);
     __syncthreads();
 #pragma unroll 1
-    for (int r0 = 0; r0 < rounds; r0 += 4) {
-      int gpos[4], v[4];
-      unsigned p[4];
-#pragma unroll
-      for (int r = 0; r < 4; ++r) gpos[r] = __ldg(list + min((r0 + r) * kWideThreads + tid, M - 1));
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const int j = path_of(s, gpos[r]);
-        const bool on = (r0 + r) * kWideThreads + tid < M && gpos[r] - j * s.L + d <= __ldg(s.len + j) - 1;
-        v[r] = -1; p[r] = 0u;
-        if (on) { v[r] = __ldg(s.tok + gpos[r] + d); p[r] = (unsigned)__ldg(s.pq + gpos[r] + d); }
-      }
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const int m = (r0 + r) * kWideThreads + tid;
-        if (cls == 0u && sub == 0u && m < M) tok[m] = v[r];
-        if (v[r] < 0 || (wide_class(v[r]) & (all_classes - 1u)) != mine) continue;
-        unsigned h = ((unsigned)v[r] * 2654435761u) >> shift;
-        int probe = 0;
+    for (int sweep = 0; sweep < 2; ++sweep) {
 #pragma unroll 1
-        for (; probe < cap; ++probe) {
-          int k = *(volatile int*)&key[h];
-          if (k == -1) k = atomicCAS(&key[h], -1, v[r]);
-          if (k == -1 || k == v[r]) break;
-          h = (h + 1) & mask;
+      for (int m0 = tid; m0 - tid < M; m0 += 8 * kWideThreads) {
+        int v[8];
+        unsigned p[8];
+        wide_gather<8>(s, list, M, d, m0, v, p);
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+          const int m = m0 + r * kWideThreads;
+          if (sweep == 0 && cls == 0u && sub == 0u && m < M) tok[m] = v[r];
+          if (v[r] < 0 || (wide_class(v[r]) & (all_classes - 1u)) != mine) continue;
+          const int h = wide_claim(t, v[r], cap);
+          if (h < 0) sh_over = 1;
+          else if (sweep == 0) wide_add(t, h, p[r], counts);
+          else weight[m] = wide_weight(s, t, h, counts);
         }
-        if (probe == cap) { sh_over = 1; continue; }
-        atomicAdd(&lo[h], p[r] & 0x7fffu);
-        atomicAdd(&hi[h], p[r] >> 15);
-        if (counts) atomicAdd(&cnt[h], 1u);
       }
+      __syncthreads();
+      if (sh_over) break;                              // (the same for everybody; only sweep 0 claims)
     }
-    __syncthreads();
-    if (sh_over) {                                     // (the same for everybody)
+    if (sh_over) {
       __syncthreads();
       subs *= 2; sub = ~0u;
-      continue;
     }
-#pragma unroll 1
-    for (int r0 = 0; r0 < rounds; r0 += 4) {
-      int gpos[4], v[4];
-#pragma unroll
-      for (int r = 0; r < 4; ++r) gpos[r] = __ldg(list + min((r0 + r) * kWideThreads + tid, M - 1));
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {                    // the same followers again: near, and cheaper than keeping their slots
-        const int j = path_of(s, gpos[r]);
-        const bool on = (r0 + r) * kWideThreads + tid < M && gpos[r] - j * s.L + d <= __ldg(s.len + j) - 1;
-        v[r] = on ? __ldg(s.tok + gpos[r] + d) : -1;
-      }
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        if (v[r] < 0 || (wide_class(v[r]) & (all_classes - 1u)) != mine) continue;
-        unsigned h = ((unsigned)v[r] * 2654435761u) >> shift;
-        while (key[h] != v[r]) h = (h + 1) & mask;
-        const u64 S = ((u64)hi[h] << 15) + lo[h];
-        weight[(r0 + r) * kWideThreads + tid] = counts ? (u64)__double_as_longlong(eq5_weight(s.alpha, S, cnt[h])) : S;
-      }
-    }
-    __syncthreads();
   }
 }
 
-// The walk over a query whose layers are all done.  Pass d chooses the token of layer d and adds up the edge that the token of
-// layer d - 1 was reached by.
+__device__ __forceinline__ void wide_sums(const Dev& s, const int4 de, int d, unsigned cls, unsigned classes) {
+  const int M = de.y;
+  bool done = false;
+  if (M <= 4 * kWideThreads) done = wide_sums_kept<4, 1>(s, de, d);
+  else if (M <= 32 * kWideThreads) done = wide_sums_kept<8, 4>(s, de, d);
+  if (!done) { __syncthreads(); wide_sums_any(s, de, d, cls, classes); }
+}
+
+// The walk over a query whose layers are all done.  N > 0: at most N candidates per thread; their tokens of the layer before
+// stay in registers, and with AHEAD a layer's tokens and weights are asked for a layer ahead.  N = 0: any number.
+template <int N, bool AHEAD>
 __device__ __forceinline__ void wide_walk(const Dev& s, const int4 de, int32_t* __restrict__ draft_tok, int32_t* __restrict__ draft_len,
                                           float* __restrict__ draft_score, float* __restrict__ draft_edge_w) {
   __shared__ u64 sh_best[2][kWideWarps];
   __shared__ int sh_tok[2][kWideWarps];
+  __shared__ int sh_draft[SDMS_MAX_DRAFT];
   __shared__ unsigned sh_e[SDMS_MAX_DRAFT][3];
+  constexpr int B = N > 0 ? N : 8;                     // candidates of a thread in flight
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, D = s.D, i = de.x, M = de.y;
   const int32_t* const list = s.matches + s.q_off[i];
   const WideItems items = wide_items(s, de.z, M);
-  if (tid < SDMS_MAX_DRAFT) { sh_e[tid][0] = 0u; sh_e[tid][1] = 0u; sh_e[tid][2] = 0u; }
-  __syncthreads();
-  int my_tok = -1, emitted = 0, cur = -1, before = -1;  // lane d - 1 of warp 0 keeps what layer d comes to
+  if (tid < SDMS_MAX_DRAFT) { sh_e[tid][0] = 0u; sh_e[tid][1] = 0u; sh_e[tid][2] = 0u; sh_draft[tid] = -1; }
+  int my_tok = -1, cur = -1;                           // lane d - 1 of warp 0 keeps what layer d comes to
   u64 my_weight = 0ull;
-  bool walking = true;
+  int t[B], u[B];
+  u64 w[AHEAD ? B : 1];
+  auto fetch = [&](int d, int m0) {
+#pragma unroll
+    for (int r = 0; r < B; ++r) {
+      const int m = m0 + r * kWideThreads;
+      t[r] = m < M ? __ldcg(items.tok + (size_t)(d - 1) * M + m) : -1;
+      if (AHEAD) w[r] = m < M ? ld_u64(items.weight + (size_t)(d - 1) * M + m) : 0ull;
+    }
+  };
+  if (N > 0) fetch(1, tid);
+  int emitted = 0;
 #pragma unroll 1
-  for (int d = 1; walking && d <= D + 1; ++d) {
-    const int* const row_t = items.tok + (size_t)(d - 1) * M;
-    const u64* const row_w = items.weight + (size_t)(d - 1) * M;
+  for (int d = 1; d <= D; ++d) {
     u64 best = 0ull;
     int tok = INT_MAX;
-    unsigned e0 = 0u, e1 = 0u, e2 = 0u;
 #pragma unroll 1
-    for (int m0 = tid; m0 < M; m0 += 4 * kWideThreads) {
-      int t[4], u[4], uu[4];
-      u64 w[4];
-      unsigned p[4];
+    for (int m0 = tid; m0 - tid < (N > 0 ? 1 : M); m0 += B * kWideThreads) {
+      if (N == 0) {
+        fetch(d, m0);
 #pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const int m = m0 + r * kWideThreads;
-        t[r] = -1; u[r] = -1; uu[r] = -1;
-        if (m < M) {
-          if (d <= D) t[r] = __ldcg(row_t + m);
-          if (d > 1) u[r] = __ldcg(row_t + m - M);
-          if (d > 2) uu[r] = __ldcg(row_t + m - 2 * (size_t)M);
-        }
+        for (int r = 0; r < B; ++r) u[r] = d > 1 && m0 + r * kWideThreads < M ? __ldcg(items.tok + (size_t)(d - 2) * M + m0 + r * kWideThreads) : -1;
+      }
+      int q[B];
+      u64 ww[B];
+#pragma unroll
+      for (int r = 0; r < B; ++r) {
+        q[r] = d == 1 || s.mode == 1 || u[r] == cur ? t[r] : -1;                 // -1: not on the current node
+        ww[r] = AHEAD ? w[AHEAD ? r : 0] : q[r] >= 0 ? ld_u64(items.weight + (size_t)(d - 1) * M + m0 + r * kWideThreads) : 0ull;
       }
 #pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const int m = m0 + r * kWideThreads;
-        const bool on = t[r] >= 0 && (d == 1 || s.mode == 1 || u[r] == cur);
-        const bool edge = d > 1 && u[r] == cur && (d == 2 || uu[r] == before) && m < M;
-        w[r] = 0ull; p[r] = ~0u;
-        if (on) w[r] = ld_u64(row_w + m);
-        else t[r] = -1;
-        if (edge) p[r] = (unsigned)__ldg(s.pq + __ldg(list + m) + d - 1);
-      }
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const bool better = t[r] >= 0 && (tok == INT_MAX || w[r] > best || (w[r] == best && t[r] < tok));
-        best = better ? w[r] : best; tok = better ? t[r] : tok;
-        const bool edge = p[r] != ~0u;
-        e0 += edge ? p[r] & 0x7fffu : 0u; e1 += edge ? p[r] >> 15 : 0u; e2 += edge;
+      for (int r = 0; r < B; ++r) {
+        const bool better = q[r] >= 0 && (tok == INT_MAX || ww[r] > best || (ww[r] == best && q[r] < tok));
+        best = better ? ww[r] : best; tok = better ? q[r] : tok;
       }
     }
-    if (d > 1 && __any_sync(FULL, e2 != 0u)) {
-      e0 = __reduce_add_sync(FULL, e0); e1 = __reduce_add_sync(FULL, e1); e2 = __reduce_add_sync(FULL, e2);
-      if (lane < 3) atomicAdd(&sh_e[d - 2][lane], lane == 0 ? e0 : lane == 1 ? e1 : e2);
+    if (N > 0) {
+#pragma unroll
+      for (int r = 0; r < B; ++r) u[r] = t[r];
+      if (AHEAD && d < D) fetch(d + 1, tid);           // arrives during the reduction
     }
-    if (d > D) break;
     {
       const u64 top = warp_max64(best);
       tok = (int)__reduce_min_sync(FULL, best == top ? (unsigned)tok : (unsigned)INT_MAX);
       if (lane == 0) { sh_best[d & 1][warp] = top; sh_tok[d & 1][warp] = tok; }
     }
+    if (N > 0 && !AHEAD && d < D) fetch(d + 1, tid);
     __syncthreads();
     {
       const u64 b = lane < kWideWarps ? sh_best[d & 1][lane] : 0ull;
@@ -233,13 +291,38 @@ __device__ __forceinline__ void wide_walk(const Dev& s, const int4 de, int32_t* 
       // (a node of weight zero is still a node: what counts is whether there is a token)
       tok = (int)__reduce_min_sync(FULL, b == best ? (unsigned)bt : (unsigned)INT_MAX);
     }
-    walking = tok != INT_MAX;
-    if (walking) {
-      if (lane == d - 1) { my_tok = tok; my_weight = best; }
-      before = cur; cur = tok; emitted = d;
+    if (tok == INT_MAX) break;                         // no successor: the draft ends here
+    if (lane == d - 1) { my_tok = tok; my_weight = best; }
+    if (tid == 0) sh_draft[d - 1] = tok;
+    cur = tok; emitted = d;
+  }
+  __syncthreads();
+  // weights of the edges taken: a warp takes 128 candidates of one layer at a time
+  const int chunks = (M + 127) >> 7;
+#pragma unroll 1
+  for (int x = warp, l = 0, c = warp; x < emitted * chunks; x += kWideWarps, c += kWideWarps) {
+    while (c >= chunks) { c -= chunks; ++l; }
+    const int want = sh_draft[l], from = l > 0 ? sh_draft[l - 1] : -1;
+    int a[4], b[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const int m = c * 128 + r * 32 + lane;
+      a[r] = m < M ? __ldcg(items.tok + (size_t)l * M + m) : -1;
+      b[r] = l > 0 && m < M ? __ldcg(items.tok + (size_t)(l - 1) * M + m) : -1;
+    }
+    unsigned e0 = 0u, e1 = 0u, e2 = 0u;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      if (a[r] != want || b[r] != from) continue;
+      const unsigned p = (unsigned)__ldg(s.pq + __ldg(list + c * 128 + r * 32 + lane) + l + 1);
+      e0 += p & 0x7fffu; e1 += p >> 15; ++e2;
+    }
+    if (__any_sync(FULL, e2 != 0u)) {
+      e0 = __reduce_add_sync(FULL, e0); e1 = __reduce_add_sync(FULL, e1); e2 = __reduce_add_sync(FULL, e2);
+      if (lane < 3) atomicAdd(&sh_e[l][lane], lane == 0 ? e0 : lane == 1 ? e1 : e2);
     }
   }
-  __syncthreads();                                     // the edge sums are complete
+  __syncthreads();
   if (warp == 0) {
     if (lane < D) {
       const size_t at = (size_t)i * D + lane;
@@ -254,6 +337,7 @@ __device__ __forceinline__ void wide_walk(const Dev& s, const int4 de, int32_t* 
     if (lane == 0) draft_len[i] = emitted;
   }
   if (s.beam_stride > 0) {                             // the beams want the table area empty
+    __syncthreads();
     uint4* const z = reinterpret_cast<uint4*>(s.w_tab + (unsigned)de.z);
     for (size_t x = tid; x < (size_t)wide_slots(s, M) * 2; x += kWideThreads) z[x] = make_uint4(0u, 0u, 0u, 0u);
   }
@@ -346,7 +430,11 @@ dag_wide_kernel(Dev s, int32_t* __restrict__ draft_tok, int32_t* __restrict__ dr
       __threadfence();
     }
     __syncthreads();
-    if (sh_last) wide_walk(s, de, draft_tok, draft_len, draft_score, draft_edge_w);
+    if (sh_last) {
+      if (de.y <= 4 * kWideThreads) wide_walk<4, true>(s, de, draft_tok, draft_len, draft_score, draft_edge_w);
+      else if (de.y <= 16 * kWideThreads) wide_walk<16, false>(s, de, draft_tok, draft_len, draft_score, draft_edge_w);
+      else wide_walk<0, false>(s, de, draft_tok, draft_len, draft_score, draft_edge_w);
+    }
     task = sh_task;
     __syncthreads();
   }
