@@ -2,18 +2,21 @@
 // single-launch build, spread over the whole device.
 //
 // One CTA that aggregates a query of thousands of matches by itself takes hundreds of microseconds while the other SMs idle,
-// so dag_kernel hands such queries over (wide_register).  Here every (query, layer) pair is a task of its own: a CTA gathers
-// the layer's followers, sums them up per token in a hash table in its shared memory and leaves, for every candidate, its
-// token and its node's weight in the table area of the workspace.  The CTA that completes the last layer of a query then
-// walks it: per layer one coalesced sweep over the candidates' tokens, the weights only of those on the current node.
-// Nobody waits for anybody: tasks come from a counter, heavy queries first.  Sums are integers and every choice has a tie
-// rule, so the order in which things happen cannot show in a result.
+// so dag_kernel hands such queries over (wide_register).  Here every (query, layer) pair is a task of its own, done by one CTA
+// in its shared memory:
+//   sums    the layer's followers are gathered and summed up per token in a hash table
+//   offers  a second table, by the token of the layer before: the heaviest node among its successors, found in three 32-bit
+//           maxima (upper and lower word of the weight, then the smaller token), and the sums of the edge to it
+// Every candidate gets its token, its node's weight and, as the best successor of the node it comes from, the index of one
+// candidate on it.  The CTA that completes the last layer of a query then walks it: one dependent load per layer.  Nobody
+// waits for anybody: tasks come from a counter, heavy queries first.  Sums are integers and every choice has a tie rule, so the
+// order in which things happen cannot show in a result.
 //
-// What bounds it: a task the gather (one 32-byte sector per follower and SM at a time) and the shared-memory atomics, both
-// around 1.3 cycles per candidate; the walk one round trip to L2 and one barrier per layer.  The form before this one kept all
-// nodes in tables in global memory and passed over all items five times with grid barriers in between: 32 us for one query
-// of 200 matches and D = 16, 165 us for 12 000 matches, and room for a quarter of the 420 000 matches of 16 prompts of 128 x
-// 4096 tokens, whose heaviest queries then kept one CTA each busy for 1.2 ms.
+// What bounds a task: the gather (a 32-byte sector per follower) and the shared-memory atomics.  The forms before: all nodes
+// in tables in global memory and five passes over all items with grid barriers in between took 32 us for one query of 200
+// matches and D = 16, 165 us for 12 000 matches, and had room for a quarter of the 420 000 matches of 16 prompts of 128 x 4096
+// tokens, whose heaviest queries then kept one CTA each busy for 1.2 ms; sums by tasks as here but a walk that swept over the
+// candidates layer by layer left 1.0 us of one SM per thousand candidates and layer at the end.
 #include <climits>
 #include "sdms_internal.h"
 #include "wide_dev.cuh"
@@ -24,8 +27,8 @@ namespace {
 
 constexpr int kWideSlots = 16384;                    // most slots of a task's table (half of them where counts are kept too)
 constexpr int kWideSmem = kWideSlots * 12;
-constexpr int kWideTableMatches = 16384;             // candidates per table
-constexpr int kWideWarps = kWideThreads / 32;
+constexpr int kWideHalf = kWideSlots / 2;              // slots where an entry takes up to 24 bytes
+constexpr int kWideProbes = 256;
 constexpr int kSortFrom = 256;                       // more queries than this balance without an order
 
 __device__ __forceinline__ u64 ld_u64(const u64* p) { return __ldcg(p); }
@@ -45,24 +48,22 @@ __global__ void wait_timeout_kernel(Dev s, long long cycles) {
   if (threadIdx.x == 0 && !wait_for_count(s.b_ctl + 1, ~0ull, cycles)) atomicOr(s.status, SDMS_STATUS_TIMEOUT);
 }
 
-__device__ __forceinline__ u64 warp_max64(u64 x) {
-  const unsigned hi = (unsigned)(x >> 32), top = __reduce_max_sync(FULL, hi);
-  const unsigned lo = __reduce_max_sync(FULL, hi == top ? (unsigned)x : 0u);
-  return (u64)top << 32 | lo;
-}
-
-// Where a query's candidates leave their nodes: weights [D][M], then tokens [D][M] (-1: the candidate has ended).
-struct WideItems { u64* weight; int* tok; };
+// What the tasks leave for a query, per (layer, candidate): the best successor of the node that the candidate was on at the
+// layer before (a candidate on that successor; -1: none), and for candidates that are named so what the draft says of them
+// (score, weight of the edge from the node before).  Until a task is done it keeps node weights and slots there.
+struct WideItems { u64* out; int* succ; };
 __device__ __forceinline__ WideItems wide_items(const Dev& s, int first, int M) {
-  u64* const w = reinterpret_cast<u64*>(s.w_tab + (unsigned)first);
-  return WideItems{w, reinterpret_cast<int*>(w + (size_t)s.D * M)};
+  WideItems w;
+  w.out = reinterpret_cast<u64*>(s.w_tab + (unsigned)first);
+  w.succ = reinterpret_cast<int*>(w.out + (size_t)s.D * M);
+  return w;
 }
-
-// Number of tables (a power of two) that the tokens of a layer are dealt out to by their hash.
-__device__ __forceinline__ int wide_classes(int M) {
-  int c = 1;
-  while ((long long)c * kWideTableMatches < M) c *= 2;
-  return c;
+// Follower d of candidate m, which has one.
+__device__ __forceinline__ int wide_token(const Dev& s, const int32_t* list, int m, int d) { return __ldg(s.tok + __ldg(list + m) + d); }
+__device__ __forceinline__ u64 wide_out(const Dev& s, u64 weight, u64 edge_sum, unsigned edge_count) {
+  const float score = s.alpha == 1.0 ? (float)eq5_weight(1.0, weight, 0u) : (float)__longlong_as_double((long long)weight);
+  const float edge = s.mode == 1 ? 0.0f : (float)eq5_weight(s.alpha, edge_sum, edge_count);
+  return (u64)__float_as_uint(edge) << 32 | __float_as_uint(score);
 }
 __device__ __forceinline__ unsigned wide_class(int v) { return ((unsigned)v * 0x85ebca6bu) >> 8; }
 
@@ -81,11 +82,11 @@ __device__ __forceinline__ void wide_table_empty(unsigned char* smem, int cap, b
   for (int x = threadIdx.x; x < k4; x += kWideThreads) z[x] = make_int4(-1, -1, -1, -1);
   for (int x = k4 + threadIdx.x; x < end; x += kWideThreads) z[x] = make_int4(0, 0, 0, 0);
 }
-// Slot of token v, claimed if need be; -1: the table is full.
-__device__ __forceinline__ int wide_claim(const WideTable& t, int v, int cap) {
+// Slot of token v, claimed if need be; -1: the table is full, or as good as (a full table is not searched to its end).
+__device__ __forceinline__ int wide_claim(const WideTable& t, int v) {
   unsigned h = ((unsigned)v * 2654435761u) >> t.shift;
 #pragma unroll 1
-  for (int probe = 0; probe < cap; ++probe) {
+  for (int probe = 0; probe < kWideProbes; ++probe) {
     int k = *(volatile int*)&t.key[h];
     if (k == -1) k = atomicCAS(&t.key[h], -1, v);
     if (k == -1 || k == v) return (int)h;
@@ -117,20 +118,20 @@ __device__ __forceinline__ void wide_gather(const Dev& s, const int32_t* list, i
   }
 }
 
-// Layer d of a query with at most N * CH * kWideThreads candidates: node sums, then every candidate's token and node weight.
-// The slots stay in registers in between.  false: more distinct tokens than slots, nothing is done.
-template <int N, int CH>
-__device__ __forceinline__ bool wide_sums_kept(const Dev& s, const int4 de, int d) {
+// Layer d of a query with at most N * CH * kWideThreads candidates.  Slots and tokens stay in registers, with KEEP weights too
+// (else they are read again from where they were left).  false: more distinct tokens than slots, nothing is done.
+template <int N, int CH, bool KEEP>
+__device__ __forceinline__ bool wide_layer(const Dev& s, const int4 de, int d) {
   extern __shared__ __align__(16) unsigned char wide_smem[];
   __shared__ int sh_full;
+  static_assert(N * CH <= 32, "one bit per candidate");
   const int tid = threadIdx.x, M = de.y;
   const int32_t* const list = s.matches + s.q_off[de.x];
   const WideItems items = wide_items(s, de.z, M);
-  u64* const weight = items.weight + (size_t)(d - 1) * M;
-  int* const tok = items.tok + (size_t)(d - 1) * M;
+  u64* const weight = items.out + (size_t)(d - 1) * M;
   const bool counts = s.alpha != 1.0;                  // with alpha = 1 a weight does not depend on the count
   int cap = 64;
-  while (cap < (counts ? kWideSlots / 2 : kWideSlots) && 7 * cap < 8 * M) cap *= 2;
+  while (cap < (counts ? kWideHalf : kWideSlots) && 7 * cap < 8 * M) cap *= 2;
   const WideTable t = wide_table(wide_smem, cap);
   if (tid == 0) sh_full = 0;
   int v[N];
@@ -138,18 +139,20 @@ __device__ __forceinline__ bool wide_sums_kept(const Dev& s, const int4 de, int 
   wide_gather<N>(s, list, M, d, tid, v, p);            // on its way while the table is emptied
   wide_table_empty(wide_smem, cap, counts);
   __syncthreads();
+  // ---- sums
   int slot[CH][N];
+  int kt[CH][N];                                       // tokens and weights
+  u64 kw[KEEP ? CH : 1][N];
 #pragma unroll
   for (int c = 0; c < CH; ++c) {
     const int m0 = c * N * kWideThreads + tid;
     if (c > 0) wide_gather<N>(s, list, M, d, m0, v, p);
 #pragma unroll
     for (int r = 0; r < N; ++r) {
-      const int m = m0 + r * kWideThreads;
-      if (m < M) tok[m] = v[r];
+      kt[c][r] = v[r];
       slot[c][r] = -1;
       if (v[r] < 0) continue;
-      slot[c][r] = wide_claim(t, v[r], cap);
+      slot[c][r] = wide_claim(t, v[r]);
       if (slot[c][r] < 0) sh_full = 1;
       else wide_add(t, slot[c][r], p[r], counts);
     }
@@ -159,182 +162,338 @@ __device__ __forceinline__ bool wide_sums_kept(const Dev& s, const int4 de, int 
 #pragma unroll
   for (int c = 0; c < CH; ++c)
 #pragma unroll
+    for (int r = 0; r < N; ++r) {
+      if (KEEP) kw[KEEP ? c : 0][r] = 0ull;
+      if (slot[c][r] < 0) continue;
+      const u64 w = wide_weight(s, t, slot[c][r], counts);
+      if (KEEP) kw[KEEP ? c : 0][r] = w;
+      else weight[(c * N + r) * kWideThreads + tid] = w;
+    }
+  __syncthreads();
+  // ---- offers.  slot becomes that of the node before (-1: the candidate was not on one)
+  const bool single = d == 1 || s.mode == 1;           // all successors of the root / of no node in particular
+  for (int x = tid; x < (single ? 1 : cap); x += kWideThreads) { t.key[x] = -1; t.lo[x] = 0u; t.hi[x] = 0u; }
+  __syncthreads();
+  unsigned alive = 0u, best = 0u, named = 0u;         // bit c * N + r: has a token; is on the best successor; is the one that is named
+#pragma unroll
+  for (int c = 0; c < CH; ++c) {
+    const int m0 = c * N * kWideThreads + tid;
+    if (!single) wide_gather<N>(s, list, M, d - 1, m0, v, p);
+#pragma unroll
+    for (int r = 0; r < N; ++r) {
+      const int m = m0 + r * kWideThreads;
+      alive |= (unsigned)(slot[c][r] >= 0) << (c * N + r);
+      slot[c][r] = m >= M || (!single && v[r] < 0) ? -1 : single ? 0 : wide_claim(t, v[r]);
+      if (!single && m < M && v[r] >= 0 && slot[c][r] < 0) sh_full = 1;
+    }
+  }
+  __syncthreads();
+  if (sh_full) return false;
+  auto weight_of = [&](int c, int r) { return KEEP ? kw[KEEP ? c : 0][r] : weight[(c * N + r) * kWideThreads + tid]; };
+#pragma unroll
+  for (int c = 0; c < CH; ++c)
+#pragma unroll
     for (int r = 0; r < N; ++r)
-      if (slot[c][r] >= 0) weight[(c * N + r) * kWideThreads + tid] = wide_weight(s, t, slot[c][r], counts);
+      if (alive >> (c * N + r) & 1u) {
+        const unsigned x = (unsigned)(weight_of(c, r) >> 32);
+        if (*(volatile unsigned*)&t.hi[slot[c][r]] < x) atomicMax(&t.hi[slot[c][r]], x);
+      }
+  __syncthreads();
+#pragma unroll
+  for (int c = 0; c < CH; ++c)
+#pragma unroll
+    for (int r = 0; r < N; ++r)
+      if (alive >> (c * N + r) & 1u) {
+        const u64 w = weight_of(c, r);
+        if (t.hi[slot[c][r]] == (unsigned)(w >> 32) && *(volatile unsigned*)&t.lo[slot[c][r]] < (unsigned)w) atomicMax(&t.lo[slot[c][r]], (unsigned)w);
+      }
+  __syncthreads();
+#pragma unroll
+  for (int c = 0; c < CH; ++c)
+#pragma unroll
+    for (int r = 0; r < N; ++r)
+      if (alive >> (c * N + r) & 1u) {
+        const u64 w = weight_of(c, r);
+        best |= (unsigned)(t.hi[slot[c][r]] == (unsigned)(w >> 32) && t.lo[slot[c][r]] == (unsigned)w) << (c * N + r);
+      }
+  __syncthreads();
+  for (int x = tid; x < (single ? 1 : cap); x += kWideThreads) { t.hi[x] = 0u; t.lo[x] = ~0u; }
+  __syncthreads();
+#pragma unroll
+  for (int c = 0; c < CH; ++c)
+#pragma unroll
+    for (int r = 0; r < N; ++r)
+      if (best >> (c * N + r) & 1u) {
+        const unsigned x = ~(unsigned)kt[c][r];   // the smallest token is the largest complement
+        if (*(volatile unsigned*)&t.hi[slot[c][r]] < x) atomicMax(&t.hi[slot[c][r]], x);
+      }
+  __syncthreads();
+#pragma unroll
+  for (int c = 0; c < CH; ++c)
+#pragma unroll
+    for (int r = 0; r < N; ++r)
+      if (best >> (c * N + r) & 1u) {
+        if (t.hi[slot[c][r]] == ~(unsigned)kt[c][r]) t.lo[slot[c][r]] = (unsigned)((c * N + r) * kWideThreads + tid);   // any one of them
+        else best &= ~(1u << (c * N + r));
+      }
+  __syncthreads();
+  int* const succ = items.succ + (size_t)(d - 1) * M;
+#pragma unroll
+  for (int c = 0; c < CH; ++c)
+#pragma unroll
+    for (int r = 0; r < N; ++r)
+      if (slot[c][r] >= 0) {
+        const int m = (c * N + r) * kWideThreads + tid, to = (int)t.lo[slot[c][r]];
+        succ[m] = to;
+        named |= (unsigned)(to == m) << (c * N + r);
+      }
+  __syncthreads();
+  for (int x = tid; x < (single ? 1 : cap); x += kWideThreads) { t.hi[x] = 0u; t.lo[x] = 0u; t.key[x] = 0; }
+  __syncthreads();
+  // the edge to the best successor: in layer-wise search it counts only for candidates that were on the winner's own node, which
+  // is not known here: the walk adds it up
+  if (s.mode != 1) {
+    unsigned lo = 0u, hi = 0u;
+#pragma unroll
+    for (int c = 0; c < CH; ++c)
+#pragma unroll
+      for (int r = 0; r < N; ++r)
+        if (best >> (c * N + r) & 1u) {
+          const unsigned q = (unsigned)__ldg(s.pq + __ldg(list + (c * N + r) * kWideThreads + tid) + d);
+          if (single) { lo += q & 0x7fffu; hi += q >> 15; }
+          else {
+            atomicAdd(&t.lo[slot[c][r]], q & 0x7fffu);
+            atomicAdd(&t.hi[slot[c][r]], q >> 15);
+            atomicAdd(&t.key[slot[c][r]], 1);
+          }
+        }
+    if (single) {                                      // one edge for all
+      lo = __reduce_add_sync(FULL, lo); hi = __reduce_add_sync(FULL, hi);
+      const unsigned n = __reduce_add_sync(FULL, (unsigned)__popc(best));
+      if ((tid & 31) == 0 && n) { atomicAdd(&t.lo[0], lo); atomicAdd(&t.hi[0], hi); atomicAdd(&t.key[0], (int)n); }
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int c = 0; c < CH; ++c)
+#pragma unroll
+    for (int r = 0; r < N; ++r)
+      if (named >> (c * N + r) & 1u) {
+        const int x = slot[c][r], m = (c * N + r) * kWideThreads + tid;
+        const u64 w = weight_of(c, r);
+        weight[m] = wide_out(s, w, ((u64)t.hi[x] << 15) + t.lo[x], (unsigned)t.key[x]);
+      }
   return true;
 }
 
-// The same for any number of candidates, tokens of class `cls` of `classes`; the followers are fetched twice.  Almost always
-// one pass; a table that turns out too small is done again in sub-classes.
-__device__ __forceinline__ void wide_sums_any(const Dev& s, const int4 de, int d, unsigned cls, unsigned classes) {
+// The same for any number of candidates and of distinct tokens: what is known of a candidate stays in global memory, and tokens
+// are dealt out by their hash to as many classes, one after the other, as their tables need to fit.
+__device__ __forceinline__ void wide_layer_any(const Dev& s, const int4 de, int d) {
   extern __shared__ __align__(16) unsigned char wide_smem[];
   __shared__ int sh_over;
+  constexpr int N = 8;
+  constexpr u64 kEnded = ~0ull;                        // no weight
   const int tid = threadIdx.x, M = de.y;
   const int32_t* const list = s.matches + s.q_off[de.x];
   const WideItems items = wide_items(s, de.z, M);
-  u64* const weight = items.weight + (size_t)(d - 1) * M;
-  int* const tok = items.tok + (size_t)(d - 1) * M;
-  const bool counts = s.alpha != 1.0;
-  const int cap = counts ? kWideSlots / 2 : kWideSlots;
-  const WideTable t = wide_table(wide_smem, cap);
-  unsigned subs = 1;
+  u64* const weight = items.out + (size_t)(d - 1) * M;
+  int* const succ = items.succ + (size_t)(d - 1) * M;  // -2 - slot while a candidate's class is being worked on
+  const bool counts = s.alpha != 1.0, single = d == 1 || s.mode == 1;
+  // A sweep over this thread's candidates, N in flight: f(candidate, slot, weight, r) for those that have a slot, of the
+  // candidates with `tokens` (filled in by then: those that pass `want(slot, weight)`).
+  int token[N];
+  auto sweep = [&](auto&& want, auto&& f) {
 #pragma unroll 1
-  for (unsigned sub = 0; sub < subs; ++sub) {
-    const unsigned all_classes = classes * subs, mine = cls + classes * sub;
-    if (tid == 0) sh_over = 0;
-    wide_table_empty(wide_smem, cap, counts);
-    __syncthreads();
-#pragma unroll 1
-    for (int sweep = 0; sweep < 2; ++sweep) {
-#pragma unroll 1
-      for (int m0 = tid; m0 - tid < M; m0 += 8 * kWideThreads) {
-        int v[8];
-        unsigned p[8];
-        wide_gather<8>(s, list, M, d, m0, v, p);
+    for (int m0 = tid; m0 < M; m0 += N * kWideThreads) {
+      int h[N], at[N];
+      u64 w[N];
 #pragma unroll
-        for (int r = 0; r < 8; ++r) {
+      for (int r = 0; r < N; ++r) {
+        const int m = min(m0 + r * kWideThreads, M - 1);
+        h[r] = m0 + r * kWideThreads < M ? -2 - __ldcg(succ + m) : -1;
+        w[r] = ld_u64(weight + m);
+        at[r] = __ldg(list + m);
+      }
+#pragma unroll
+      for (int r = 0; r < N; ++r) token[r] = h[r] >= 0 && want(h[r], w[r]) ? __ldg(s.tok + at[r] + d) : -1;
+#pragma unroll
+      for (int r = 0; r < N; ++r)
+        if (h[r] >= 0) f(m0 + r * kWideThreads, h[r], w[r], token[r]);
+    }
+  };
+  auto none = [](int, u64) { return false; };
+  unsigned classes = 1;
+  while ((long long)classes * (kWideHalf / 4 * 3) < M) classes *= 2;
+  for (;; classes *= 2) {                              // again with smaller classes if a table has run over
+    __syncthreads();
+    if (tid == 0) sh_over = 0;
+    // ---- sums
+    const WideTable t = wide_table(wide_smem, counts ? kWideHalf : kWideSlots);
+#pragma unroll 1
+    for (unsigned cls = 0; cls < classes; ++cls) {
+      wide_table_empty(wide_smem, t.mask + 1, counts);
+      __syncthreads();
+#pragma unroll 1
+      for (int m0 = tid; m0 < M; m0 += N * kWideThreads) {
+        int v[N];
+        unsigned p[N];
+        wide_gather<N>(s, list, M, d, m0, v, p);
+#pragma unroll
+        for (int r = 0; r < N; ++r) {
           const int m = m0 + r * kWideThreads;
-          if (sweep == 0 && cls == 0u && sub == 0u && m < M) tok[m] = v[r];
-          if (v[r] < 0 || (wide_class(v[r]) & (all_classes - 1u)) != mine) continue;
-          const int h = wide_claim(t, v[r], cap);
-          if (h < 0) sh_over = 1;
-          else if (sweep == 0) wide_add(t, h, p[r], counts);
-          else weight[m] = wide_weight(s, t, h, counts);
+          if (m >= M) continue;
+          const bool mine = v[r] >= 0 && (wide_class(v[r]) & (classes - 1)) == cls;
+          const int h = mine ? wide_claim(t, v[r]) : -1;
+          if (h >= 0) wide_add(t, h, p[r], counts);
+          else if (mine) sh_over = 1;
+          succ[m] = -2 - h;
+          if (v[r] < 0) weight[m] = kEnded;
         }
       }
       __syncthreads();
-      if (sh_over) break;                              // (the same for everybody; only sweep 0 claims)
-    }
-    if (sh_over) {
+      if (sh_over) break;                              // (the same for everybody)
+      sweep(none, [&](int m, int h, u64, int) { weight[m] = wide_weight(s, t, h, counts); });
       __syncthreads();
-      subs *= 2; sub = ~0u;
     }
+    if (sh_over) continue;
+    // ---- offers
+    WideTable u;
+    u.key = reinterpret_cast<int*>(wide_smem);
+    unsigned* const hi = reinterpret_cast<unsigned*>(u.key + kWideHalf);
+    unsigned* const lo = hi + kWideHalf;
+    unsigned* const nt = lo + kWideHalf;               // complement of the token: the smallest token has the largest
+    unsigned* const cnt = nt + kWideHalf;
+    int* const one = reinterpret_cast<int*>(cnt + kWideHalf);          // a candidate on the best successor
+    u.lo = lo; u.hi = hi; u.cnt = cnt; u.mask = kWideHalf - 1; u.shift = __clz(kWideHalf) + 1;
+    const int used = single ? 1 : kWideHalf;
+#pragma unroll 1
+    for (unsigned cls = 0; cls < (single ? 1u : classes); ++cls) {
+      for (int x = tid; x < used; x += kWideThreads) { u.key[x] = -1; hi[x] = 0u; lo[x] = 0u; nt[x] = 0u; cnt[x] = 0u; one[x] = -1; }
+      __syncthreads();
+#pragma unroll 1
+      for (int m0 = tid; m0 < M; m0 += N * kWideThreads) {
+        int v[N];
+        unsigned p[N];
+        u64 w[N];
+        if (!single) wide_gather<N>(s, list, M, d - 1, m0, v, p);
+#pragma unroll
+        for (int r = 0; r < N; ++r) w[r] = ld_u64(weight + min(m0 + r * kWideThreads, M - 1));
+#pragma unroll
+        for (int r = 0; r < N; ++r) {
+          const int m = m0 + r * kWideThreads;
+          if (m >= M) continue;
+          const bool mine = single || (v[r] >= 0 && (wide_class(v[r]) & (classes - 1)) == cls);
+          if (!mine) {
+            if (cls == 0) succ[m] = -1;                // (what an earlier class has found stays)
+            continue;
+          }
+          const int h = single ? 0 : wide_claim(u, v[r]);
+          if (h < 0) { sh_over = 1; continue; }
+          succ[m] = -2 - h;
+          const unsigned x = (unsigned)(w[r] >> 32);
+          if (w[r] != kEnded && *(volatile unsigned*)&hi[h] < x) atomicMax(&hi[h], x);
+        }
+      }
+      __syncthreads();
+      if (sh_over) break;
+      sweep(none, [&](int, int h, u64 w, int) {
+        if (w != kEnded && hi[h] == (unsigned)(w >> 32) && *(volatile unsigned*)&lo[h] < (unsigned)w) atomicMax(&lo[h], (unsigned)w);
+      });
+      __syncthreads();
+      auto heaviest = [&](int h, u64 w) { return w != kEnded && hi[h] == (unsigned)(w >> 32) && lo[h] == (unsigned)w; };
+      sweep(heaviest, [&](int, int h, u64, int v) {
+        if (v >= 0 && *(volatile unsigned*)&nt[h] < ~(unsigned)v) atomicMax(&nt[h], ~(unsigned)v);
+      });
+      __syncthreads();
+      sweep(heaviest, [&](int m, int h, u64, int v) {
+        if (v >= 0 && nt[h] == ~(unsigned)v) one[h] = m;               // any one of them
+      });
+      __syncthreads();
+      sweep(heaviest, [&](int m, int h, u64, int v) {
+        if (v >= 0 && nt[h] == ~(unsigned)v) return;
+        succ[m] = one[h];                              // not on it, and done
+      });
+      __syncthreads();
+      for (int x = tid; x < used; x += kWideThreads) { hi[x] = 0u; lo[x] = 0u; }
+      __syncthreads();
+      unsigned a = 0u, b = 0u, n = 0u;                 // the root's edge is added up in registers
+      sweep(none, [&](int m, int h, u64, int) {
+        if (s.mode == 1) return;
+        const unsigned q = (unsigned)__ldg(s.pq + __ldg(list + m) + d);
+        if (single) { a += q & 0x7fffu; b += q >> 15; ++n; }
+        else { atomicAdd(&lo[h], q & 0x7fffu); atomicAdd(&hi[h], q >> 15); atomicAdd(&cnt[h], 1u); }
+      });
+      if (n) { atomicAdd(&lo[0], a); atomicAdd(&hi[0], b); atomicAdd(&cnt[0], n); }
+      __syncthreads();
+      sweep(none, [&](int m, int h, u64 w, int) {
+        const int to = one[h];
+        succ[m] = to;
+        if (to == m) weight[m] = wide_out(s, w, ((u64)hi[h] << 15) + lo[h], cnt[h]);
+      });
+      __syncthreads();
+    }
+    if (!sh_over) return;
   }
 }
 
-__device__ __forceinline__ void wide_sums(const Dev& s, const int4 de, int d, unsigned cls, unsigned classes) {
+__device__ __forceinline__ void wide_task(const Dev& s, const int4 de, int d) {
   const int M = de.y;
-  bool done = false;
-  if (M <= 4 * kWideThreads) done = wide_sums_kept<4, 1>(s, de, d);
-  else if (M <= 32 * kWideThreads) done = wide_sums_kept<8, 4>(s, de, d);
-  if (!done) { __syncthreads(); wide_sums_any(s, de, d, cls, classes); }
+  if (M <= 4 * kWideThreads ? wide_layer<4, 1, true>(s, de, d)
+      : M <= 16 * kWideThreads ? wide_layer<8, 2, true>(s, de, d)
+      : M <= 32 * kWideThreads && wide_layer<8, 4, false>(s, de, d)) return;
+  wide_layer_any(s, de, d);
 }
 
-// The walk over a query whose layers are all done.  N > 0: at most N candidates per thread; their tokens of the layer before
-// stay in registers, and with AHEAD a layer's tokens and weights are asked for a layer ahead.  N = 0: any number.
-template <int N, bool AHEAD>
-__device__ __forceinline__ void wide_walk(const Dev& s, const int4 de, int32_t* __restrict__ draft_tok, int32_t* __restrict__ draft_len,
-                                          float* __restrict__ draft_score, float* __restrict__ draft_edge_w) {
-  __shared__ u64 sh_best[2][kWideWarps];
-  __shared__ int sh_tok[2][kWideWarps];
+// ---- the walk over a query whose layers are all done: one dependent load per layer --------------------------------
+struct WideOut { int32_t* tok; int32_t* len; float* score; float* edge_w; };
+
+__device__ __forceinline__ void wide_walk(const Dev& s, const int4 de, const WideOut out) {
   __shared__ int sh_draft[SDMS_MAX_DRAFT];
-  __shared__ unsigned sh_e[SDMS_MAX_DRAFT][3];
-  constexpr int B = N > 0 ? N : 8;                     // candidates of a thread in flight
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, D = s.D, i = de.x, M = de.y;
+  __shared__ unsigned sh_e[SDMS_MAX_DRAFT][3];         // layer-wise search: edge sums (lower 15 bits, rest) and counts
+  static_assert(SDMS_MAX_DRAFT <= 32, "a lane per layer");
+  const int tid = threadIdx.x, D = s.D, i = de.x, M = de.y;
   const int32_t* const list = s.matches + s.q_off[i];
   const WideItems items = wide_items(s, de.z, M);
-  if (tid < SDMS_MAX_DRAFT) { sh_e[tid][0] = 0u; sh_e[tid][1] = 0u; sh_e[tid][2] = 0u; sh_draft[tid] = -1; }
-  int my_tok = -1, cur = -1;                           // lane d - 1 of warp 0 keeps what layer d comes to
-  u64 my_weight = 0ull;
-  int t[B], u[B];
-  u64 w[AHEAD ? B : 1];
-  auto fetch = [&](int d, int m0) {
-#pragma unroll
-    for (int r = 0; r < B; ++r) {
-      const int m = m0 + r * kWideThreads;
-      t[r] = m < M ? __ldcg(items.tok + (size_t)(d - 1) * M + m) : -1;
-      if (AHEAD) w[r] = m < M ? ld_u64(items.weight + (size_t)(d - 1) * M + m) : 0ull;
-    }
-  };
-  if (N > 0) fetch(1, tid);
-  int emitted = 0;
-#pragma unroll 1
-  for (int d = 1; d <= D; ++d) {
-    u64 best = 0ull;
-    int tok = INT_MAX;
-#pragma unroll 1
-    for (int m0 = tid; m0 - tid < (N > 0 ? 1 : M); m0 += B * kWideThreads) {
-      if (N == 0) {
-        fetch(d, m0);
-#pragma unroll
-        for (int r = 0; r < B; ++r) u[r] = d > 1 && m0 + r * kWideThreads < M ? __ldcg(items.tok + (size_t)(d - 2) * M + m0 + r * kWideThreads) : -1;
-      }
-      int q[B];
-      u64 ww[B];
-#pragma unroll
-      for (int r = 0; r < B; ++r) {
-        q[r] = d == 1 || s.mode == 1 || u[r] == cur ? t[r] : -1;                 // -1: not on the current node
-        ww[r] = AHEAD ? w[AHEAD ? r : 0] : q[r] >= 0 ? ld_u64(items.weight + (size_t)(d - 1) * M + m0 + r * kWideThreads) : 0ull;
-      }
-#pragma unroll
-      for (int r = 0; r < B; ++r) {
-        const bool better = q[r] >= 0 && (tok == INT_MAX || ww[r] > best || (ww[r] == best && q[r] < tok));
-        best = better ? ww[r] : best; tok = better ? q[r] : tok;
-      }
-    }
-    if (N > 0) {
-#pragma unroll
-      for (int r = 0; r < B; ++r) u[r] = t[r];
-      if (AHEAD && d < D) fetch(d + 1, tid);           // arrives during the reduction
-    }
-    {
-      const u64 top = warp_max64(best);
-      tok = (int)__reduce_min_sync(FULL, best == top ? (unsigned)tok : (unsigned)INT_MAX);
-      if (lane == 0) { sh_best[d & 1][warp] = top; sh_tok[d & 1][warp] = tok; }
-    }
-    if (N > 0 && !AHEAD && d < D) fetch(d + 1, tid);
+  if (s.mode == 1 && out.edge_w) {                     // the edges are known only now
+    if (tid < 32) { sh_draft[tid] = -1; sh_e[tid][0] = 0u; sh_e[tid][1] = 0u; sh_e[tid][2] = 0u; }
     __syncthreads();
-    {
-      const u64 b = lane < kWideWarps ? sh_best[d & 1][lane] : 0ull;
-      const int bt = lane < kWideWarps ? sh_tok[d & 1][lane] : INT_MAX;
-      best = warp_max64(b);
-      // (a node of weight zero is still a node: what counts is whether there is a token)
-      tok = (int)__reduce_min_sync(FULL, b == best ? (unsigned)bt : (unsigned)INT_MAX);
+    if (tid < D) { const int at = __ldcg(items.succ + (size_t)tid * M); if (at >= 0) sh_draft[tid] = wide_token(s, list, at, tid + 1); }
+    __syncthreads();
+    for (int m = tid; m < M; m += kWideThreads) {
+      const int g = __ldg(list + m), j = path_of(s, g), n = min(D, __ldg(s.len + j) - 1 - (g - j * s.L));
+      bool on = true;                                  // this candidate is on the draft's node so far
+      for (int l = 0; l < n && sh_draft[l] >= 0; ++l) {
+        const bool here = __ldg(s.tok + g + l + 1) == sh_draft[l];
+        if (on && here) {
+          const unsigned q = (unsigned)__ldg(s.pq + g + l + 1);
+          atomicAdd(&sh_e[l][0], q & 0x7fffu); atomicAdd(&sh_e[l][1], q >> 15); atomicAdd(&sh_e[l][2], 1u);
+        }
+        on = here;
+      }
     }
-    if (tok == INT_MAX) break;                         // no successor: the draft ends here
-    if (lane == d - 1) { my_tok = tok; my_weight = best; }
-    if (tid == 0) sh_draft[d - 1] = tok;
-    cur = tok; emitted = d;
+    __syncthreads();
   }
-  __syncthreads();
-  // weights of the edges taken: a warp takes 128 candidates of one layer at a time
-  const int chunks = (M + 127) >> 7;
+  if (tid < 32) {
+    int at = __ldcg(items.succ), emitted = 0, mine = -1;               // every candidate of layer 1 names the root's best
 #pragma unroll 1
-  for (int x = warp, l = 0, c = warp; x < emitted * chunks; x += kWideWarps, c += kWideWarps) {
-    while (c >= chunks) { c -= chunks; ++l; }
-    const int want = sh_draft[l], from = l > 0 ? sh_draft[l - 1] : -1;
-    int a[4], b[4];
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      const int m = c * 128 + r * 32 + lane;
-      a[r] = m < M ? __ldcg(items.tok + (size_t)l * M + m) : -1;
-      b[r] = l > 0 && m < M ? __ldcg(items.tok + (size_t)(l - 1) * M + m) : -1;
+    for (int d = 1; d <= D && at >= 0; ++d) {
+      if (tid == d - 1) mine = at;
+      emitted = d;
+      at = d < D ? __ldcg(items.succ + (size_t)d * M + at) : -1;
     }
-    unsigned e0 = 0u, e1 = 0u, e2 = 0u;
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      if (a[r] != want || b[r] != from) continue;
-      const unsigned p = (unsigned)__ldg(s.pq + __ldg(list + c * 128 + r * 32 + lane) + l + 1);
-      e0 += p & 0x7fffu; e1 += p >> 15; ++e2;
+    if (tid < D) {
+      const size_t x = (size_t)i * D + tid, y = (size_t)tid * M + max(mine, 0);
+      const bool on = mine >= 0;
+      const int v = on ? wide_token(s, list, mine, tid + 1) : -1;
+      const u64 o = ld_u64(items.out + y);
+      out.tok[x] = v;
+      if (out.score) out.score[x] = on ? __uint_as_float((unsigned)o) : 0.0f;
+      if (out.edge_w)
+        out.edge_w[x] = !on ? 0.0f
+                        : s.mode == 1 ? (float)eq5_weight(s.alpha, ((u64)sh_e[tid][1] << 15) + sh_e[tid][0], sh_e[tid][2])
+                                      : __uint_as_float((unsigned)(o >> 32));
     }
-    if (__any_sync(FULL, e2 != 0u)) {
-      e0 = __reduce_add_sync(FULL, e0); e1 = __reduce_add_sync(FULL, e1); e2 = __reduce_add_sync(FULL, e2);
-      if (lane < 3) atomicAdd(&sh_e[l][lane], lane == 0 ? e0 : lane == 1 ? e1 : e2);
-    }
-  }
-  __syncthreads();
-  if (warp == 0) {
-    if (lane < D) {
-      const size_t at = (size_t)i * D + lane;
-      const bool on = my_tok >= 0;
-      draft_tok[at] = my_tok;
-      if (draft_score)
-        draft_score[at] = !on ? 0.0f : s.alpha == 1.0 ? (float)eq5_weight(1.0, my_weight, 0u)
-                                                      : (float)__longlong_as_double((long long)my_weight);
-      if (draft_edge_w)
-        draft_edge_w[at] = on ? (float)eq5_weight(s.alpha, ((u64)sh_e[lane][1] << 15) + sh_e[lane][0], sh_e[lane][2]) : 0.0f;
-    }
-    if (lane == 0) draft_len[i] = emitted;
+    if (tid == 0) out.len[i] = emitted;
   }
   if (s.beam_stride > 0) {                             // the beams want the table area empty
     __syncthreads();
@@ -351,12 +510,10 @@ dag_wide_kernel(Dev s, int32_t* __restrict__ draft_tok, int32_t* __restrict__ dr
   if (registered == 0) return;
   const int nq = (int)(registered < (u64)kMaxWide ? registered : (u64)kMaxWide);
   __shared__ int4 sh_desc[kMaxWide];
-  __shared__ int sh_base[kMaxWide + 1];                // first task of each query
-  __shared__ int sh_warp[kWideWarps];
   __shared__ int sh_task, sh_last;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, D = s.D;
+  const int tid = threadIdx.x, D = s.D;
   static_assert(kMaxWide == 2 * kWideThreads, "two list entries per thread");
-  // the list of queries, the largest first, and by a prefix sum the first task of each
+  // the list of queries, the largest first
   {
     int4 de[2];
     int rank[2];
@@ -389,52 +546,24 @@ dag_wide_kernel(Dev s, int32_t* __restrict__ draft_tok, int32_t* __restrict__ dr
         if (2 * tid + r < nq) sh_desc[2 * tid + r].w = 2 * tid + r;
     }
     __syncthreads();
-    int c[2];
-#pragma unroll
-    for (int r = 0; r < 2; ++r) c[r] = 2 * tid + r < nq ? D * wide_classes(sh_desc[2 * tid + r].y) : 0;
-    int x = c[0] + c[1];
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) { const int y = __shfl_up_sync(FULL, x, o); if (lane >= o) x += y; }
-    if (lane == 31) sh_warp[warp] = x;
-    __syncthreads();
-    if (warp == 0) {
-      int w = lane < kWideWarps ? sh_warp[lane] : 0;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) { const int y = __shfl_up_sync(FULL, w, o); if (lane >= o) w += y; }
-      if (lane < kWideWarps) sh_warp[lane] = w;
-    }
-    __syncthreads();
-    const int ahead = (warp ? sh_warp[warp - 1] : 0) + x - c[0] - c[1];
-    sh_base[2 * tid] = ahead;
-    sh_base[2 * tid + 1] = ahead + c[0];
-    if (tid == kWideThreads - 1) sh_base[kMaxWide] = ahead + c[0] + c[1];
-    __syncthreads();
   }
-  const int tasks = sh_base[nq];
+  const int tasks = nq * D;
   int task = blockIdx.x;                               // the first one without asking
 #pragma unroll 1
   while (task < tasks) {
-    int a = 0, b = nq;                                 // sh_base[a] <= task < sh_base[b]
-    while (b - a > 1) { const int mid = (a + b) >> 1; if (sh_base[mid] <= task) a = mid; else b = mid; }
-    const int4 de = sh_desc[a];
-    const int classes = wide_classes(de.y), part = task - sh_base[a];
-    wide_sums(s, de, part / classes + 1, (unsigned)(part % classes), (unsigned)classes);
+    const int4 de = sh_desc[task / D];
+    wide_task(s, de, task % D + 1);
     // done with it: its results are out before it is counted, and whoever counts the last one has seen all of them
     __threadfence();
     __syncthreads();
     if (tid == 0) {
       sh_task = (int)gridDim.x + (int)atomicAdd(&s.w_ctl[2], 1ull);
-      const int total = D * classes;
-      sh_last = atomicAdd(&s.w_done[de.w], 1) == total - 1;
+      sh_last = atomicAdd(&s.w_done[de.w], 1) == D - 1;
       if (sh_last) s.w_done[de.w] = 0;                 // the next build finds it at zero
       __threadfence();
     }
     __syncthreads();
-    if (sh_last) {
-      if (de.y <= 4 * kWideThreads) wide_walk<4, true>(s, de, draft_tok, draft_len, draft_score, draft_edge_w);
-      else if (de.y <= 16 * kWideThreads) wide_walk<16, false>(s, de, draft_tok, draft_len, draft_score, draft_edge_w);
-      else wide_walk<0, false>(s, de, draft_tok, draft_len, draft_score, draft_edge_w);
-    }
+    if (sh_last) wide_walk(s, de, WideOut{draft_tok, draft_len, draft_score, draft_edge_w});
     task = sh_task;
     __syncthreads();
   }

@@ -4,7 +4,7 @@
 
 namespace sdms {
 
-// Room (in table slots of 32 bytes) that a query with M matches takes: weight and token of every (match, layer).
+// Room (in table slots of 32 bytes) that a query with M matches takes: 12 bytes for every (match, layer).
 __device__ __forceinline__ unsigned long long wide_slots(const Dev& s, int M) {
   return ((unsigned long long)M * s.D * 12 + sizeof(WideSlot) - 1) / sizeof(WideSlot);
 }
