@@ -27,8 +27,13 @@ namespace {
 
 constexpr int kWideSlots = 16384;                    // most slots of a task's table (half of them where counts are kept too)
 constexpr int kWideSmem = kWideSlots * 12;
-constexpr int kWideHalf = kWideSlots / 2;              // slots where an entry takes up to 24 bytes
-constexpr int kWideProbes = 256;
+// Most candidates of a query whose layers are one CTA's each: a table is at most 7/8 full.
+__device__ __forceinline__ int wide_alone(const Dev& s) { return (s.alpha != 1.0 ? kWideSlots / 2 : kWideSlots) / 8 * 7; }
+#ifndef SPREAD
+#define SPREAD 1
+#endif
+constexpr int kWideSpread = SPREAD;
+constexpr int kWideWarps = kWideThreads / 32;
 constexpr int kSortFrom = 256;                       // more queries than this balance without an order
 
 __device__ __forceinline__ u64 ld_u64(const u64* p) { return __ldcg(p); }
@@ -82,11 +87,11 @@ __device__ __forceinline__ void wide_table_empty(unsigned char* smem, int cap, b
   for (int x = threadIdx.x; x < k4; x += kWideThreads) z[x] = make_int4(-1, -1, -1, -1);
   for (int x = k4 + threadIdx.x; x < end; x += kWideThreads) z[x] = make_int4(0, 0, 0, 0);
 }
-// Slot of token v, claimed if need be; -1: the table is full, or as good as (a full table is not searched to its end).
+// Slot of token v, claimed if need be; -1: the table is full.
 __device__ __forceinline__ int wide_claim(const WideTable& t, int v) {
   unsigned h = ((unsigned)v * 2654435761u) >> t.shift;
 #pragma unroll 1
-  for (int probe = 0; probe < kWideProbes; ++probe) {
+  for (int probe = 0; probe <= t.mask; ++probe) {
     int k = *(volatile int*)&t.key[h];
     if (k == -1) k = atomicCAS(&t.key[h], -1, v);
     if (k == -1 || k == v) return (int)h;
@@ -103,27 +108,26 @@ __device__ __forceinline__ u64 wide_weight(const Dev& s, const WideTable& t, int
   const u64 S = ((u64)t.hi[h] << 15) + t.lo[h];
   return counts ? (u64)__double_as_longlong(eq5_weight(s.alpha, S, t.cnt[h])) : S;
 }
-// Followers d of candidates m0, m0 + kWideThreads, ...: token (-1: none) and probability, all requests on their way together.
-template <int N>
+// Followers d of candidates m0, m0 + T, ...: token (-1: none) and probability, all requests on their way together.
+template <int N, int T = kWideThreads>
 __device__ __forceinline__ void wide_gather(const Dev& s, const int32_t* list, int M, int d, int m0, int (&v)[N], unsigned (&p)[N]) {
   int gpos[N];
 #pragma unroll
-  for (int r = 0; r < N; ++r) gpos[r] = __ldg(list + min(m0 + r * kWideThreads, M - 1));
+  for (int r = 0; r < N; ++r) gpos[r] = __ldg(list + min(m0 + r * T, M - 1));
 #pragma unroll
   for (int r = 0; r < N; ++r) {
     const int j = path_of(s, gpos[r]);
-    const bool on = m0 + r * kWideThreads < M && gpos[r] - j * s.L + d <= __ldg(s.len + j) - 1;
+    const bool on = m0 + r * T < M && gpos[r] - j * s.L + d <= __ldg(s.len + j) - 1;
     v[r] = -1; p[r] = 0u;
     if (on) { v[r] = __ldg(s.tok + gpos[r] + d); p[r] = (unsigned)__ldg(s.pq + gpos[r] + d); }
   }
 }
 
 // Layer d of a query with at most N * CH * kWideThreads candidates.  Slots and tokens stay in registers, with KEEP weights too
-// (else they are read again from where they were left).  false: more distinct tokens than slots, nothing is done.
+// (else they are read again from where they were left).
 template <int N, int CH, bool KEEP>
-__device__ __forceinline__ bool wide_layer(const Dev& s, const int4 de, int d) {
+__device__ __forceinline__ void wide_layer(const Dev& s, const int4 de, int d) {
   extern __shared__ __align__(16) unsigned char wide_smem[];
-  __shared__ int sh_full;
   static_assert(N * CH <= 32, "one bit per candidate");
   const int tid = threadIdx.x, M = de.y;
   const int32_t* const list = s.matches + s.q_off[de.x];
@@ -131,9 +135,8 @@ __device__ __forceinline__ bool wide_layer(const Dev& s, const int4 de, int d) {
   u64* const weight = items.out + (size_t)(d - 1) * M;
   const bool counts = s.alpha != 1.0;                  // with alpha = 1 a weight does not depend on the count
   int cap = 64;
-  while (cap < (counts ? kWideHalf : kWideSlots) && 7 * cap < 8 * M) cap *= 2;
+  while (7 * cap < 8 * M) cap *= 2;
   const WideTable t = wide_table(wide_smem, cap);
-  if (tid == 0) sh_full = 0;
   int v[N];
   unsigned p[N];
   wide_gather<N>(s, list, M, d, tid, v, p);            // on its way while the table is emptied
@@ -153,12 +156,10 @@ __device__ __forceinline__ bool wide_layer(const Dev& s, const int4 de, int d) {
       slot[c][r] = -1;
       if (v[r] < 0) continue;
       slot[c][r] = wide_claim(t, v[r]);
-      if (slot[c][r] < 0) sh_full = 1;
-      else wide_add(t, slot[c][r], p[r], counts);
+      wide_add(t, slot[c][r], p[r], counts);
     }
   }
   __syncthreads();
-  if (sh_full) return false;                           // (the same for everybody)
 #pragma unroll
   for (int c = 0; c < CH; ++c)
 #pragma unroll
@@ -184,11 +185,9 @@ __device__ __forceinline__ bool wide_layer(const Dev& s, const int4 de, int d) {
       const int m = m0 + r * kWideThreads;
       alive |= (unsigned)(slot[c][r] >= 0) << (c * N + r);
       slot[c][r] = m >= M || (!single && v[r] < 0) ? -1 : single ? 0 : wide_claim(t, v[r]);
-      if (!single && m < M && v[r] >= 0 && slot[c][r] < 0) sh_full = 1;
     }
   }
   __syncthreads();
-  if (sh_full) return false;
   auto weight_of = [&](int c, int r) { return KEEP ? kw[KEEP ? c : 0][r] : weight[(c * N + r) * kWideThreads + tid]; };
 #pragma unroll
   for (int c = 0; c < CH; ++c)
@@ -283,171 +282,244 @@ __device__ __forceinline__ bool wide_layer(const Dev& s, const int4 de, int d) {
         const u64 w = weight_of(c, r);
         weight[m] = wide_out(s, w, ((u64)t.hi[x] << 15) + t.lo[x], (unsigned)t.key[x]);
       }
-  return true;
-}
-
-// The same for any number of candidates and of distinct tokens: what is known of a candidate stays in global memory, and tokens
-// are dealt out by their hash to as many classes, one after the other, as their tables need to fit.
-__device__ __forceinline__ void wide_layer_any(const Dev& s, const int4 de, int d) {
-  extern __shared__ __align__(16) unsigned char wide_smem[];
-  __shared__ int sh_over;
-  constexpr int N = 8;
-  constexpr u64 kEnded = ~0ull;                        // no weight
-  const int tid = threadIdx.x, M = de.y;
-  const int32_t* const list = s.matches + s.q_off[de.x];
-  const WideItems items = wide_items(s, de.z, M);
-  u64* const weight = items.out + (size_t)(d - 1) * M;
-  int* const succ = items.succ + (size_t)(d - 1) * M;  // -2 - slot while a candidate's class is being worked on
-  const bool counts = s.alpha != 1.0, single = d == 1 || s.mode == 1;
-  // A sweep over this thread's candidates, N in flight: f(candidate, slot, weight, r) for those that have a slot, of the
-  // candidates with `tokens` (filled in by then: those that pass `want(slot, weight)`).
-  int token[N];
-  auto sweep = [&](auto&& want, auto&& f) {
-#pragma unroll 1
-    for (int m0 = tid; m0 < M; m0 += N * kWideThreads) {
-      int h[N], at[N];
-      u64 w[N];
-#pragma unroll
-      for (int r = 0; r < N; ++r) {
-        const int m = min(m0 + r * kWideThreads, M - 1);
-        h[r] = m0 + r * kWideThreads < M ? -2 - __ldcg(succ + m) : -1;
-        w[r] = ld_u64(weight + m);
-        at[r] = __ldg(list + m);
-      }
-#pragma unroll
-      for (int r = 0; r < N; ++r) token[r] = h[r] >= 0 && want(h[r], w[r]) ? __ldg(s.tok + at[r] + d) : -1;
-#pragma unroll
-      for (int r = 0; r < N; ++r)
-        if (h[r] >= 0) f(m0 + r * kWideThreads, h[r], w[r], token[r]);
-    }
-  };
-  auto none = [](int, u64) { return false; };
-  unsigned classes = 1;
-  while ((long long)classes * (kWideHalf / 4 * 3) < M) classes *= 2;
-  for (;; classes *= 2) {                              // again with smaller classes if a table has run over
-    __syncthreads();
-    if (tid == 0) sh_over = 0;
-    // ---- sums
-    const WideTable t = wide_table(wide_smem, counts ? kWideHalf : kWideSlots);
-#pragma unroll 1
-    for (unsigned cls = 0; cls < classes; ++cls) {
-      wide_table_empty(wide_smem, t.mask + 1, counts);
-      __syncthreads();
-#pragma unroll 1
-      for (int m0 = tid; m0 < M; m0 += N * kWideThreads) {
-        int v[N];
-        unsigned p[N];
-        wide_gather<N>(s, list, M, d, m0, v, p);
-#pragma unroll
-        for (int r = 0; r < N; ++r) {
-          const int m = m0 + r * kWideThreads;
-          if (m >= M) continue;
-          const bool mine = v[r] >= 0 && (wide_class(v[r]) & (classes - 1)) == cls;
-          const int h = mine ? wide_claim(t, v[r]) : -1;
-          if (h >= 0) wide_add(t, h, p[r], counts);
-          else if (mine) sh_over = 1;
-          succ[m] = -2 - h;
-          if (v[r] < 0) weight[m] = kEnded;
-        }
-      }
-      __syncthreads();
-      if (sh_over) break;                              // (the same for everybody)
-      sweep(none, [&](int m, int h, u64, int) { weight[m] = wide_weight(s, t, h, counts); });
-      __syncthreads();
-    }
-    if (sh_over) continue;
-    // ---- offers
-    WideTable u;
-    u.key = reinterpret_cast<int*>(wide_smem);
-    unsigned* const hi = reinterpret_cast<unsigned*>(u.key + kWideHalf);
-    unsigned* const lo = hi + kWideHalf;
-    unsigned* const nt = lo + kWideHalf;               // complement of the token: the smallest token has the largest
-    unsigned* const cnt = nt + kWideHalf;
-    int* const one = reinterpret_cast<int*>(cnt + kWideHalf);          // a candidate on the best successor
-    u.lo = lo; u.hi = hi; u.cnt = cnt; u.mask = kWideHalf - 1; u.shift = __clz(kWideHalf) + 1;
-    const int used = single ? 1 : kWideHalf;
-#pragma unroll 1
-    for (unsigned cls = 0; cls < (single ? 1u : classes); ++cls) {
-      for (int x = tid; x < used; x += kWideThreads) { u.key[x] = -1; hi[x] = 0u; lo[x] = 0u; nt[x] = 0u; cnt[x] = 0u; one[x] = -1; }
-      __syncthreads();
-#pragma unroll 1
-      for (int m0 = tid; m0 < M; m0 += N * kWideThreads) {
-        int v[N];
-        unsigned p[N];
-        u64 w[N];
-        if (!single) wide_gather<N>(s, list, M, d - 1, m0, v, p);
-#pragma unroll
-        for (int r = 0; r < N; ++r) w[r] = ld_u64(weight + min(m0 + r * kWideThreads, M - 1));
-#pragma unroll
-        for (int r = 0; r < N; ++r) {
-          const int m = m0 + r * kWideThreads;
-          if (m >= M) continue;
-          const bool mine = single || (v[r] >= 0 && (wide_class(v[r]) & (classes - 1)) == cls);
-          if (!mine) {
-            if (cls == 0) succ[m] = -1;                // (what an earlier class has found stays)
-            continue;
-          }
-          const int h = single ? 0 : wide_claim(u, v[r]);
-          if (h < 0) { sh_over = 1; continue; }
-          succ[m] = -2 - h;
-          const unsigned x = (unsigned)(w[r] >> 32);
-          if (w[r] != kEnded && *(volatile unsigned*)&hi[h] < x) atomicMax(&hi[h], x);
-        }
-      }
-      __syncthreads();
-      if (sh_over) break;
-      sweep(none, [&](int, int h, u64 w, int) {
-        if (w != kEnded && hi[h] == (unsigned)(w >> 32) && *(volatile unsigned*)&lo[h] < (unsigned)w) atomicMax(&lo[h], (unsigned)w);
-      });
-      __syncthreads();
-      auto heaviest = [&](int h, u64 w) { return w != kEnded && hi[h] == (unsigned)(w >> 32) && lo[h] == (unsigned)w; };
-      sweep(heaviest, [&](int, int h, u64, int v) {
-        if (v >= 0 && *(volatile unsigned*)&nt[h] < ~(unsigned)v) atomicMax(&nt[h], ~(unsigned)v);
-      });
-      __syncthreads();
-      sweep(heaviest, [&](int m, int h, u64, int v) {
-        if (v >= 0 && nt[h] == ~(unsigned)v) one[h] = m;               // any one of them
-      });
-      __syncthreads();
-      sweep(heaviest, [&](int m, int h, u64, int v) {
-        if (v >= 0 && nt[h] == ~(unsigned)v) return;
-        succ[m] = one[h];                              // not on it, and done
-      });
-      __syncthreads();
-      for (int x = tid; x < used; x += kWideThreads) { hi[x] = 0u; lo[x] = 0u; }
-      __syncthreads();
-      unsigned a = 0u, b = 0u, n = 0u;                 // the root's edge is added up in registers
-      sweep(none, [&](int m, int h, u64, int) {
-        if (s.mode == 1) return;
-        const unsigned q = (unsigned)__ldg(s.pq + __ldg(list + m) + d);
-        if (single) { a += q & 0x7fffu; b += q >> 15; ++n; }
-        else { atomicAdd(&lo[h], q & 0x7fffu); atomicAdd(&hi[h], q >> 15); atomicAdd(&cnt[h], 1u); }
-      });
-      if (n) { atomicAdd(&lo[0], a); atomicAdd(&hi[0], b); atomicAdd(&cnt[0], n); }
-      __syncthreads();
-      sweep(none, [&](int m, int h, u64 w, int) {
-        const int to = one[h];
-        succ[m] = to;
-        if (to == m) weight[m] = wide_out(s, w, ((u64)hi[h] << 15) + lo[h], cnt[h]);
-      });
-      __syncthreads();
-    }
-    if (!sh_over) return;
-  }
 }
 
 __device__ __forceinline__ void wide_task(const Dev& s, const int4 de, int d) {
   const int M = de.y;
-  if (M <= 4 * kWideThreads ? wide_layer<4, 1, true>(s, de, d)
-      : M <= 16 * kWideThreads ? wide_layer<8, 2, true>(s, de, d)
-      : M <= 32 * kWideThreads && wide_layer<8, 4, false>(s, de, d)) return;
-  wide_layer_any(s, de, d);
+  if (M <= 4 * kWideThreads) wide_layer<4, 1, true>(s, de, d);
+  else if (M <= 16 * kWideThreads) wide_layer<8, 2, true>(s, de, d);
+  else wide_layer<7, 4, false>(s, de, d);
 }
 
-// ---- the walk over a query whose layers are all done: one dependent load per layer --------------------------------
+// ---- larger queries: sums only, one task per class of tokens ------------------------------------------------------
+// What those tasks leave, in the place of WideItems: weights, and tokens in rows that start on 16 bytes.
+struct WideRows { u64* weight; int* tok; int pitch; };
+__device__ __forceinline__ WideRows wide_rows(const Dev& s, int first, int M) {
+  WideRows w;
+  w.pitch = wide_pitch(M);
+  w.weight = reinterpret_cast<u64*>(s.w_tab + (unsigned)first);
+  w.tok = reinterpret_cast<int*>(w.weight + (size_t)s.D * w.pitch);
+  return w;
+}
+// Classes (a power of two): tables at most 7/8 full.
+__device__ __forceinline__ int wide_classes(const Dev& s, int M) {
+  if (M <= wide_alone(s)) return 1;
+  int c = 2;
+  while ((long long)c * (wide_alone(s) / kWideSpread) < M) c *= 2;
+  return c;
+}
+// Weights of the nodes of layer d with tokens of class `cls`.  A table that overruns all the same is done again in sub-classes.
+__device__ __forceinline__ void wide_sums(const Dev& s, const int4 de, int d, unsigned cls, unsigned classes) {
+  extern __shared__ __align__(16) unsigned char wide_smem[];
+  __shared__ int sh_over;
+  constexpr int N = 16;
+  const int tid = threadIdx.x, M = de.y;
+  const int32_t* const list = s.matches + s.q_off[de.x];
+  const WideRows rows = wide_rows(s, de.z, M);
+  u64* const weight = rows.weight + (size_t)(d - 1) * rows.pitch;
+  int* const tok = rows.tok + (size_t)(d - 1) * rows.pitch;
+  const bool counts = s.alpha != 1.0;
+  const int cap = counts ? kWideSlots / 2 : kWideSlots;
+  const WideTable t = wide_table(wide_smem, cap);
+  unsigned subs = 1;
+#pragma unroll 1
+  for (unsigned sub = 0; sub < subs; ++sub) {
+    const unsigned others = classes * subs - 1u, mine = cls + classes * sub;
+    if (tid == 0) sh_over = 0;
+    wide_table_empty(wide_smem, cap, counts);
+    __syncthreads();
+#pragma unroll 1
+    for (int m0 = tid; m0 < M; m0 += N * kWideThreads) {
+      int v[N];
+      unsigned p[N];
+      wide_gather<N>(s, list, M, d, m0, v, p);
+#pragma unroll
+      for (int r = 0; r < N; ++r) {
+        const int m = m0 + r * kWideThreads;
+        if (m < M) tok[m] = v[r];                      // (all classes write the same)
+        if (v[r] < 0 || (wide_class(v[r]) & others) != mine) continue;
+        const int h = wide_claim(t, v[r]);
+        if (h < 0) sh_over = 1;
+        else wide_add(t, h, p[r], counts);
+      }
+    }
+    __syncthreads();
+    if (sh_over) {                                     // (the same for everybody)
+      __syncthreads();
+      subs *= 2; sub = ~0u;
+      continue;
+    }
+#pragma unroll 1
+    for (int m0 = tid; m0 < M; m0 += N * kWideThreads) {
+      int v[N];
+#pragma unroll
+      for (int r = 0; r < N; ++r) v[r] = m0 + r * kWideThreads < M ? __ldcg(tok + m0 + r * kWideThreads) : -1;
+#pragma unroll
+      for (int r = 0; r < N; ++r)
+        if (v[r] >= 0 && (wide_class(v[r]) & others) == mine) weight[m0 + r * kWideThreads] = wide_weight(s, t, wide_claim(t, v[r]), counts);
+    }
+    __syncthreads();
+  }
+}
+
+// ---- the walk over a query whose layers are all done --------------------------------------------------------------
 struct WideOut { int32_t* tok; int32_t* len; float* score; float* edge_w; };
 
-__device__ __forceinline__ void wide_walk(const Dev& s, const int4 de, const WideOut out) {
+__device__ __forceinline__ u64 warp_max64(u64 x) {
+  const unsigned hi = (unsigned)(x >> 32), top = __reduce_max_sync(FULL, hi);
+  const unsigned lo = __reduce_max_sync(FULL, hi == top ? (unsigned)x : 0u);
+  return (u64)top << 32 | lo;
+}
+struct WideWalk {                        // what the walk over rows keeps in shared memory
+  u64 best[2][kWideWarps];
+  int tok[2][kWideWarps];
+  int draft[SDMS_MAX_DRAFT];
+  u64 weight[SDMS_MAX_DRAFT];
+  unsigned e[SDMS_MAX_DRAFT][3];         // edge sums: lower 15 bits, rest, count
+  int hits[2], edges;
+};
+// One candidate more on the edge that the draft takes into layer l + 1.
+__device__ __forceinline__ void walk_edge(const Dev& s, WideWalk& sh, const int32_t* list, int m, int l) {
+  const unsigned p = (unsigned)__ldg(s.pq + __ldg(list + m) + l + 1);
+  atomicAdd(&sh.e[l][0], p & 0x7fffu); atomicAdd(&sh.e[l][1], p >> 15); atomicAdd(&sh.e[l][2], 1u);
+}
+
+// Sums only: layer by layer the candidates on the current node are picked from its row into a list in shared memory (whose
+// length does not depend on M, and is short for most nodes), their successors compared, and the candidates on the edge taken
+// put aside to be weighed at the end.  A list that overflows, and layer 1, where all are on the root, go over the rows instead.
+__device__ __forceinline__ void wide_walk_rows(const Dev& s, const int4 de, const WideOut out) {
+  extern __shared__ __align__(16) unsigned char wide_smem[];
+  __shared__ WideWalk sh;
+  constexpr int B = 8, kHits = kWideSmem / 8, kEdges = kWideSmem / 16;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, D = s.D, i = de.x, M = de.y;
+  const int32_t* const list = s.matches + s.q_off[i];
+  const WideRows rows = wide_rows(s, de.z, M);
+  int* const hit = reinterpret_cast<int*>(wide_smem);
+  int2* const edge = reinterpret_cast<int2*>(hit + kHits);             // (candidate, layer - 1)
+  if (tid < SDMS_MAX_DRAFT) { sh.e[tid][0] = 0u; sh.e[tid][1] = 0u; sh.e[tid][2] = 0u; }
+  if (tid == 0) { sh.hits[0] = 0; sh.hits[1] = 0; sh.edges = 0; }
+  __syncthreads();
+  int cur = -1, emitted = 0;
+#pragma unroll 1
+  for (int d = 1; d <= D; ++d) {
+    const int* const row = rows.tok + (size_t)(d - 1) * rows.pitch;
+    const int* const before = row - rows.pitch;
+    const u64* const row_w = rows.weight + (size_t)(d - 1) * rows.pitch;
+    const bool all = d == 1 || s.mode == 1;            // successors of the root / of no node in particular
+    if (!all) {
+#pragma unroll 1
+      for (int x0 = 4 * tid; x0 < M; x0 += B * 4 * kWideThreads) {
+        int4 u[B];
+#pragma unroll
+        for (int r = 0; r < B; ++r) {
+          const int x = x0 + r * 4 * kWideThreads;
+          u[r] = x < M ? __ldcg(reinterpret_cast<const int4*>(before + x)) : make_int4(-1, -1, -1, -1);
+          if (x + 1 >= M) u[r].y = -1;
+          if (x + 2 >= M) u[r].z = -1;
+          if (x + 3 >= M) u[r].w = -1;
+        }
+        unsigned on = 0u;
+#pragma unroll
+        for (int r = 0; r < B; ++r)
+          on |= ((unsigned)(u[r].x == cur) | (unsigned)(u[r].y == cur) << 1 | (unsigned)(u[r].z == cur) << 2 | (unsigned)(u[r].w == cur) << 3) << (4 * r);
+        if (on == 0u) continue;
+        int at = atomicAdd(&sh.hits[d & 1], __popc(on));
+        for (; on && at < kHits; on &= on - 1u, ++at) {
+          const int bit = __ffs(on) - 1;
+          hit[at] = x0 + (bit >> 2) * 4 * kWideThreads + (bit & 3);
+        }
+      }
+      __syncthreads();
+    }
+    const int hits = all ? M : sh.hits[d & 1];
+    const bool listed = !all && hits <= kHits;
+    const int n = listed ? hits : M;
+    if (tid == 0) sh.hits[(d + 1) & 1] = 0;
+    // the best successor
+    u64 best = 0ull;
+    int tok = INT_MAX;
+#pragma unroll 1
+    for (int x0 = tid; x0 < n; x0 += B * kWideThreads) {
+      int t[B];
+      u64 w[B];
+#pragma unroll
+      for (int r = 0; r < B; ++r) {
+        const int x = x0 + r * kWideThreads, m = x >= n ? 0 : listed ? hit[x] : x;
+        t[r] = x < n ? __ldcg(row + m) : -1;
+        w[r] = x < n ? ld_u64(row_w + m) : 0ull;
+        if (!all && !listed && x < n && __ldcg(before + m) != cur) t[r] = -1;
+      }
+#pragma unroll
+      for (int r = 0; r < B; ++r) {
+        // (a node of weight zero is still a node: what counts is whether there is a token)
+        const bool better = t[r] >= 0 && (tok == INT_MAX || w[r] > best || (w[r] == best && t[r] < tok));
+        best = better ? w[r] : best; tok = better ? t[r] : tok;
+      }
+    }
+    {
+      const u64 top = warp_max64(best);
+      tok = (int)__reduce_min_sync(FULL, best == top ? (unsigned)tok : (unsigned)INT_MAX);
+      if (lane == 0) { sh.best[d & 1][warp] = top; sh.tok[d & 1][warp] = tok; }
+      __syncthreads();
+      const u64 b = lane < kWideWarps ? sh.best[d & 1][lane] : 0ull;
+      const int bt = lane < kWideWarps ? sh.tok[d & 1][lane] : INT_MAX;
+      best = warp_max64(b);
+      tok = (int)__reduce_min_sync(FULL, b == best ? (unsigned)bt : (unsigned)INT_MAX);
+    }
+    if (tok == INT_MAX) break;                         // no successor: the draft ends here
+    // the candidates on the edge to it
+#pragma unroll 1
+    for (int x0 = tid; x0 < n; x0 += B * kWideThreads) {
+      unsigned on = 0u;
+#pragma unroll
+      for (int r = 0; r < B; ++r) {
+        const int x = x0 + r * kWideThreads, m = x >= n ? 0 : listed ? hit[x] : x;
+        const bool here = x < n && __ldcg(row + m) == tok && (listed || d == 1 || __ldcg(before + m) == cur);
+        on |= (unsigned)here << r;
+      }
+      if (on == 0u) continue;
+      int at = atomicAdd(&sh.edges, __popc(on));
+      for (; on; on &= on - 1u, ++at) {
+        const int x = x0 + (__ffs(on) - 1) * kWideThreads, m = listed ? hit[x] : x;
+        if (at < kEdges) edge[at] = make_int2(m, d - 1);
+        else walk_edge(s, sh, list, m, d - 1);
+      }
+    }
+    if (tid == 0) { sh.draft[d - 1] = tok; sh.weight[d - 1] = best; }
+    cur = tok; emitted = d;
+    __syncthreads();                                   // before the next layer's list
+  }
+  __syncthreads();
+  const int n = min(sh.edges, kEdges);
+#pragma unroll 1
+  for (int x0 = tid; x0 < n; x0 += 4 * kWideThreads) {
+    unsigned p[4];
+    int l[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const int2 e = edge[min(x0 + r * kWideThreads, n - 1)];
+      l[r] = e.y;
+      p[r] = (unsigned)__ldg(s.pq + __ldg(list + e.x) + e.y + 1);
+    }
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+      if (x0 + r * kWideThreads < n) { atomicAdd(&sh.e[l[r]][0], p[r] & 0x7fffu); atomicAdd(&sh.e[l[r]][1], p[r] >> 15); atomicAdd(&sh.e[l[r]][2], 1u); }
+  }
+  __syncthreads();
+  if (tid < D) {
+    const size_t x = (size_t)i * D + tid;
+    const bool on = tid < emitted;
+    out.tok[x] = on ? sh.draft[tid] : -1;
+    if (out.score)
+      out.score[x] = !on ? 0.0f : s.alpha == 1.0 ? (float)eq5_weight(1.0, sh.weight[tid], 0u)
+                                                 : (float)__longlong_as_double((long long)sh.weight[tid]);
+    if (out.edge_w) out.edge_w[x] = on ? (float)eq5_weight(s.alpha, ((u64)sh.e[tid][1] << 15) + sh.e[tid][0], sh.e[tid][2]) : 0.0f;
+  }
+  if (tid == 0) out.len[i] = emitted;
+}
+// Successors known: one dependent load per layer.
+
+__device__ __forceinline__ void wide_walk_known(const Dev& s, const int4 de, const WideOut out) {
   __shared__ int sh_draft[SDMS_MAX_DRAFT];
   __shared__ unsigned sh_e[SDMS_MAX_DRAFT][3];         // layer-wise search: edge sums (lower 15 bits, rest) and counts
   static_assert(SDMS_MAX_DRAFT <= 32, "a lane per layer");
@@ -495,10 +567,15 @@ __device__ __forceinline__ void wide_walk(const Dev& s, const int4 de, const Wid
     }
     if (tid == 0) out.len[i] = emitted;
   }
+}
+
+__device__ __forceinline__ void wide_walk(const Dev& s, const int4 de, const WideOut out) {
+  if (de.y <= wide_alone(s)) wide_walk_known(s, de, out);
+  else wide_walk_rows(s, de, out);
   if (s.beam_stride > 0) {                             // the beams want the table area empty
     __syncthreads();
     uint4* const z = reinterpret_cast<uint4*>(s.w_tab + (unsigned)de.z);
-    for (size_t x = tid; x < (size_t)wide_slots(s, M) * 2; x += kWideThreads) z[x] = make_uint4(0u, 0u, 0u, 0u);
+    for (size_t x = threadIdx.x; x < (size_t)wide_slots(s, de.y) * 2; x += kWideThreads) z[x] = make_uint4(0u, 0u, 0u, 0u);
   }
 }
 
@@ -510,10 +587,12 @@ dag_wide_kernel(Dev s, int32_t* __restrict__ draft_tok, int32_t* __restrict__ dr
   if (registered == 0) return;
   const int nq = (int)(registered < (u64)kMaxWide ? registered : (u64)kMaxWide);
   __shared__ int4 sh_desc[kMaxWide];
+  __shared__ int sh_base[kMaxWide + 1];                // first task of each query
+  __shared__ int sh_warp[kWideWarps];
   __shared__ int sh_task, sh_last;
-  const int tid = threadIdx.x, D = s.D;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, D = s.D;
   static_assert(kMaxWide == 2 * kWideThreads, "two list entries per thread");
-  // the list of queries, the largest first
+  // the list of queries, the largest first, and by a prefix sum the first task of each
   {
     int4 de[2];
     int rank[2];
@@ -546,19 +625,44 @@ dag_wide_kernel(Dev s, int32_t* __restrict__ draft_tok, int32_t* __restrict__ dr
         if (2 * tid + r < nq) sh_desc[2 * tid + r].w = 2 * tid + r;
     }
     __syncthreads();
+    int c[2];
+#pragma unroll
+    for (int r = 0; r < 2; ++r) c[r] = 2 * tid + r < nq ? D * wide_classes(s, sh_desc[2 * tid + r].y) : 0;
+    int x = c[0] + c[1];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) { const int y = __shfl_up_sync(FULL, x, o); if (lane >= o) x += y; }
+    if (lane == 31) sh_warp[warp] = x;
+    __syncthreads();
+    if (warp == 0) {
+      int w = lane < kWideWarps ? sh_warp[lane] : 0;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) { const int y = __shfl_up_sync(FULL, w, o); if (lane >= o) w += y; }
+      if (lane < kWideWarps) sh_warp[lane] = w;
+    }
+    __syncthreads();
+    const int ahead = (warp ? sh_warp[warp - 1] : 0) + x - c[0] - c[1];
+    sh_base[2 * tid] = ahead;
+    sh_base[2 * tid + 1] = ahead + c[0];
+    if (tid == kWideThreads - 1) sh_base[kMaxWide] = ahead + c[0] + c[1];
+    __syncthreads();
   }
-  const int tasks = nq * D;
+  const int tasks = sh_base[nq];
   int task = blockIdx.x;                               // the first one without asking
 #pragma unroll 1
   while (task < tasks) {
-    const int4 de = sh_desc[task / D];
-    wide_task(s, de, task % D + 1);
+    int a = 0, b = nq;                                 // sh_base[a] <= task < sh_base[b]
+    while (b - a > 1) { const int mid = (a + b) >> 1; if (sh_base[mid] <= task) a = mid; else b = mid; }
+    const int4 de = sh_desc[a];
+    const int classes = wide_classes(s, de.y), part = task - sh_base[a];
+    if (de.y <= wide_alone(s)) wide_task(s, de, part + 1);
+    else wide_sums(s, de, part / classes + 1, (unsigned)(part % classes), (unsigned)classes);
     // done with it: its results are out before it is counted, and whoever counts the last one has seen all of them
     __threadfence();
     __syncthreads();
     if (tid == 0) {
       sh_task = (int)gridDim.x + (int)atomicAdd(&s.w_ctl[2], 1ull);
-      sh_last = atomicAdd(&s.w_done[de.w], 1) == D - 1;
+      const int total = D * classes;
+      sh_last = atomicAdd(&s.w_done[de.w], 1) == total - 1;
       if (sh_last) s.w_done[de.w] = 0;                 // the next build finds it at zero
       __threadfence();
     }

@@ -5,8 +5,9 @@
 namespace sdms {
 
 // Room (in table slots of 32 bytes) that a query with M matches takes: 12 bytes for every (match, layer).
+__device__ __forceinline__ int wide_pitch(int M) { return (M + 3) & ~3; }
 __device__ __forceinline__ unsigned long long wide_slots(const Dev& s, int M) {
-  return ((unsigned long long)M * s.D * 12 + sizeof(WideSlot) - 1) / sizeof(WideSlot);
+  return ((unsigned long long)wide_pitch(M) * s.D * 12 + sizeof(WideSlot) - 1) / sizeof(WideSlot);
 }
 
 // log2 of the slots of one layer's node table in the table area (beams): a power of two above 5/4 of the matches.
