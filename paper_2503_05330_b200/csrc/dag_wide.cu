@@ -376,28 +376,22 @@ struct WideWalk {                        // what the walk over rows keeps in sha
   int draft[SDMS_MAX_DRAFT];
   u64 weight[SDMS_MAX_DRAFT];
   unsigned e[SDMS_MAX_DRAFT][3];         // edge sums: lower 15 bits, rest, count
-  int hits[2], edges;
+  int hits[2];
 };
-// One candidate more on the edge that the draft takes into layer l + 1.
-__device__ __forceinline__ void walk_edge(const Dev& s, WideWalk& sh, const int32_t* list, int m, int l) {
-  const unsigned p = (unsigned)__ldg(s.pq + __ldg(list + m) + l + 1);
-  atomicAdd(&sh.e[l][0], p & 0x7fffu); atomicAdd(&sh.e[l][1], p >> 15); atomicAdd(&sh.e[l][2], 1u);
-}
 
 // Sums only: layer by layer the candidates on the current node are picked from its row into a list in shared memory (whose
-// length does not depend on M, and is short for most nodes), their successors compared, and the candidates on the edge taken
-// put aside to be weighed at the end.  A list that overflows, and layer 1, where all are on the root, go over the rows instead.
+// length does not depend on M, and is short for most nodes), their successors compared and the candidates on the edge
+// taken weighed.  A list that overflows, and layer 1, where all are on the root, go over the rows instead.
 __device__ __forceinline__ void wide_walk_rows(const Dev& s, const int4 de, const WideOut out) {
   extern __shared__ __align__(16) unsigned char wide_smem[];
   __shared__ WideWalk sh;
-  constexpr int B = 8, kHits = kWideSmem / 8, kEdges = kWideSmem / 16;
+  constexpr int B = 8, kHits = kWideSmem / 4;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, D = s.D, i = de.x, M = de.y;
   const int32_t* const list = s.matches + s.q_off[i];
   const WideRows rows = wide_rows(s, de.z, M);
   int* const hit = reinterpret_cast<int*>(wide_smem);
-  int2* const edge = reinterpret_cast<int2*>(hit + kHits);             // (candidate, layer - 1)
   if (tid < SDMS_MAX_DRAFT) { sh.e[tid][0] = 0u; sh.e[tid][1] = 0u; sh.e[tid][2] = 0u; }
-  if (tid == 0) { sh.hits[0] = 0; sh.hits[1] = 0; sh.edges = 0; }
+  if (tid == 0) { sh.hits[0] = 0; sh.hits[1] = 0; }
   __syncthreads();
   int cur = -1, emitted = 0;
 #pragma unroll 1
@@ -468,42 +462,30 @@ __device__ __forceinline__ void wide_walk_rows(const Dev& s, const int4 de, cons
     }
     if (tok == INT_MAX) break;                         // no successor: the draft ends here
     // the candidates on the edge to it
+    unsigned lo = 0u, hi = 0u, count = 0u;
 #pragma unroll 1
     for (int x0 = tid; x0 < n; x0 += B * kWideThreads) {
-      unsigned on = 0u;
+      bool on[B];
+      int m[B];
+      unsigned p[B];
 #pragma unroll
       for (int r = 0; r < B; ++r) {
-        const int x = x0 + r * kWideThreads, m = x >= n ? 0 : listed ? hit[x] : x;
-        const bool here = x < n && __ldcg(row + m) == tok && (listed || d == 1 || __ldcg(before + m) == cur);
-        on |= (unsigned)here << r;
+        const int x = x0 + r * kWideThreads;
+        m[r] = x >= n ? 0 : listed ? hit[x] : x;
+        on[r] = x < n && __ldcg(row + m[r]) == tok && (all ? d == 1 || __ldcg(before + m[r]) == cur : listed || __ldcg(before + m[r]) == cur);
       }
-      if (on == 0u) continue;
-      int at = atomicAdd(&sh.edges, __popc(on));
-      for (; on; on &= on - 1u, ++at) {
-        const int x = x0 + (__ffs(on) - 1) * kWideThreads, m = listed ? hit[x] : x;
-        if (at < kEdges) edge[at] = make_int2(m, d - 1);
-        else walk_edge(s, sh, list, m, d - 1);
-      }
+#pragma unroll
+      for (int r = 0; r < B; ++r) m[r] = on[r] ? __ldg(list + m[r]) : 0;
+#pragma unroll
+      for (int r = 0; r < B; ++r) p[r] = on[r] ? (unsigned)__ldg(s.pq + m[r] + d) : 0u;
+#pragma unroll
+      for (int r = 0; r < B; ++r) { lo += p[r] & 0x7fffu; hi += p[r] >> 15; count += on[r]; }
     }
+    lo = __reduce_add_sync(FULL, lo); hi = __reduce_add_sync(FULL, hi); count = __reduce_add_sync(FULL, count);
+    if (lane == 0 && count) { atomicAdd(&sh.e[d - 1][0], lo); atomicAdd(&sh.e[d - 1][1], hi); atomicAdd(&sh.e[d - 1][2], count); }
     if (tid == 0) { sh.draft[d - 1] = tok; sh.weight[d - 1] = best; }
     cur = tok; emitted = d;
     __syncthreads();                                   // before the next layer's list
-  }
-  __syncthreads();
-  const int n = min(sh.edges, kEdges);
-#pragma unroll 1
-  for (int x0 = tid; x0 < n; x0 += 4 * kWideThreads) {
-    unsigned p[4];
-    int l[4];
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      const int2 e = edge[min(x0 + r * kWideThreads, n - 1)];
-      l[r] = e.y;
-      p[r] = (unsigned)__ldg(s.pq + __ldg(list + e.x) + e.y + 1);
-    }
-#pragma unroll
-    for (int r = 0; r < 4; ++r)
-      if (x0 + r * kWideThreads < n) { atomicAdd(&sh.e[l[r]][0], p[r] & 0x7fffu); atomicAdd(&sh.e[l[r]][1], p[r] >> 15); atomicAdd(&sh.e[l[r]][2], 1u); }
   }
   __syncthreads();
   if (tid < D) {
