@@ -83,12 +83,12 @@ Layout make_layout(const sdms_config* c) {
   l.x_node_count = take(P * D * 4);
   l.x_edge_dst = take(P * D * B * Ke * 4); l.x_edge_S = take(P * D * B * Ke * 8);
   l.x_edge_cnt = take(P * D * B * Ke * 4); l.x_out_degree = take(P * D * B * 4);
-  // node tables in global memory: the device-wide aggregation of large prompts and the beams.  A slot:
-  // 32 bytes of sums, 4 of key, 4 per (match, layer) item, 16 per kept continuation
+  // table area: the device-wide aggregation of large prompts (32 bytes per slot) and the beams' node tables, whose slots have
+  // 32 bytes of sums, 4 of key, 4 per (match, layer) item and 16 per kept continuation
   const int64_t group_tokens = (int64_t)c->paths_per_group * c->capacity;
   const bool fused = group_tokens <= kFusedMaxTokens && (int64_t)P * group_tokens <= mc;
   const int64_t stride = c->max_beams > 0 ? c->max_beams : (c->search_mode == 2 ? 1 : 0);   // continuations kept per node
-  const int64_t slot_bytes = 40 + 16 * stride;
+  const int64_t slot_bytes = stride > 0 ? 40 + 16 * stride : 32;
   l.wide_on = !fused && c->wide_table_bytes >= 0;
   int64_t wide = c->wide_table_bytes;
   if (wide == 0) {
@@ -102,8 +102,8 @@ Layout make_layout(const sdms_config* c) {
   l.w_desc = take(l.wide_on ? (size_t)kMaxWide * 16 : 0);
   l.w_done = take(l.wide_on ? (size_t)kMaxWide * 4 : 0);
   l.w_tab = take((size_t)l.w_slots * sizeof(WideSlot));
-  l.w_key = take((size_t)l.w_slots * 4);
-  l.w_item = take((size_t)l.w_slots * 4);
+  l.w_key = take(stride > 0 ? (size_t)l.w_slots * 4 : 0);
+  l.w_item = take(stride > 0 ? (size_t)l.w_slots * 4 : 0);
   l.b_ent = take((size_t)l.w_slots * 16 * stride);
   l.total = o;
   return l;

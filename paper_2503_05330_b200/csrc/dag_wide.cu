@@ -25,14 +25,7 @@ namespace sdms {
 
 namespace {
 
-constexpr int kWideSlots = 16384;                    // most slots of a task's table (half of them where counts are kept too)
 constexpr int kWideSmem = kWideSlots * 12;
-// Most candidates of a query whose layers are one CTA's each: a table is at most 7/8 full.
-__device__ __forceinline__ int wide_alone(const Dev& s) { return (s.alpha != 1.0 ? kWideSlots / 2 : kWideSlots) / 8 * 7; }
-#ifndef SPREAD
-#define SPREAD 1
-#endif
-constexpr int kWideSpread = SPREAD;
 constexpr int kWideWarps = kWideThreads / 32;
 constexpr int kSortFrom = 256;                       // more queries than this balance without an order
 
@@ -53,18 +46,22 @@ __global__ void wait_timeout_kernel(Dev s, long long cycles) {
   if (threadIdx.x == 0 && !wait_for_count(s.b_ctl + 1, ~0ull, cycles)) atomicOr(s.status, SDMS_STATUS_TIMEOUT);
 }
 
-// What the tasks leave for a query, per (layer, candidate): the best successor of the node that the candidate was on at the
-// layer before (a candidate on that successor; -1: none), and for candidates that are named so what the draft says of them
-// (score, weight of the edge from the node before).  Until a task is done it keeps node weights and slots there.
-struct WideItems { u64* out; int* succ; };
+// What is kept for a query, in rows of `pitch` entries, one for every layer:
+//   tok    the candidates' followers (-1: ended), from dag_rows_kernel
+//   out    first their probabilities (32 bits each, the first half of the row), then node weights, in the end for those
+//          candidates that are named by others what the draft says of them (score, weight of the edge from the node before)
+//   succ   the best successor of the node that the candidate was on at the layer before (a candidate on it; -1: none).  Queries
+//          of more than wide_alone() matches have no such row.
+struct WideItems { u64* out; int* tok; int* succ; int pitch; };
 __device__ __forceinline__ WideItems wide_items(const Dev& s, int first, int M) {
   WideItems w;
+  w.pitch = wide_pitch(M);
+  const size_t n = (size_t)s.D * w.pitch;
   w.out = reinterpret_cast<u64*>(s.w_tab + (unsigned)first);
-  w.succ = reinterpret_cast<int*>(w.out + (size_t)s.D * M);
+  w.tok = reinterpret_cast<int*>(w.out + n);
+  w.succ = w.tok + n;
   return w;
 }
-// Follower d of candidate m, which has one.
-__device__ __forceinline__ int wide_token(const Dev& s, const int32_t* list, int m, int d) { return __ldg(s.tok + __ldg(list + m) + d); }
 __device__ __forceinline__ u64 wide_out(const Dev& s, u64 weight, u64 edge_sum, unsigned edge_count) {
   const float score = s.alpha == 1.0 ? (float)eq5_weight(1.0, weight, 0u) : (float)__longlong_as_double((long long)weight);
   const float edge = s.mode == 1 ? 0.0f : (float)eq5_weight(s.alpha, edge_sum, edge_count);
@@ -108,18 +105,64 @@ __device__ __forceinline__ u64 wide_weight(const Dev& s, const WideTable& t, int
   const u64 S = ((u64)t.hi[h] << 15) + t.lo[h];
   return counts ? (u64)__double_as_longlong(eq5_weight(s.alpha, S, t.cnt[h])) : S;
 }
-// Followers d of candidates m0, m0 + T, ...: token (-1: none) and probability, all requests on their way together.
-template <int N, int T = kWideThreads>
-__device__ __forceinline__ void wide_gather(const Dev& s, const int32_t* list, int M, int d, int m0, int (&v)[N], unsigned (&p)[N]) {
-  int gpos[N];
+// Entries m0, m0 + kWideThreads, ... of a row (`none` where there is no candidate).
+template <int N>
+__device__ __forceinline__ void wide_row(const int* row, int M, int m0, int none, int (&v)[N]) {
 #pragma unroll
-  for (int r = 0; r < N; ++r) gpos[r] = __ldg(list + min(m0 + r * T, M - 1));
+  for (int r = 0; r < N; ++r) v[r] = m0 + r * kWideThreads < M ? __ldcg(row + m0 + r * kWideThreads) : none;
+}
+
+// ---- the followers of all candidates, layer by layer ---------------------------------------------------------------
+// A candidate's followers lie next to each other in the store, a task wants one of each candidate.  Fetched by the tasks, each
+// layer and each step on its own, they were 3 to 4 sectors of 32 bytes per (candidate, layer), and those were what a task
+// waited for (40 of the 90 K cycles of a layer of 7300 candidates).  Here a thread reads a candidate's followers and
+// probabilities, 16 aligned bytes at a time, and lays them out in rows.
+constexpr int kRowThreads = 256;
+__device__ __forceinline__ int4 shifted(int4 a, int4 b, int off) {      // words off .. off + 3 of a, b
+  if (off & 2) { a.x = a.z; a.y = a.w; a.z = b.x; a.w = b.y; b.x = b.z; }
+  if (off & 1) { a.x = a.y; a.y = a.z; a.z = a.w; a.w = b.x; }
+  return a;
+}
+__global__ void __launch_bounds__(kRowThreads) dag_rows_kernel(Dev s) {
+  grid_wait();                                         // scheduled while dag_kernel drains; its list is complete from here on
+  const u64 registered = ld_u64(&s.w_ctl[0]);
+  const int nq = (int)(registered < (u64)kMaxWide ? registered : (u64)kMaxWide);
+  __shared__ int4 sh_desc[kMaxWide];
+  for (int q = threadIdx.x; q < nq; q += kRowThreads) sh_desc[q] = __ldcg(&s.w_desc[q]);
+  __syncthreads();
+  int skip = blockIdx.x;                               // chunks of kRowThreads candidates until this CTA's next one
+#pragma unroll 1
+  for (int q = 0; q < nq; ++q) {
+    const int4 de = sh_desc[q];
+    const int M = de.y, chunks = (M + kRowThreads - 1) / kRowThreads;
+    for (; skip < chunks; skip += gridDim.x) {
+      const int m = skip * kRowThreads + threadIdx.x;
+      if (m >= M) continue;
+      const WideItems items = wide_items(s, de.z, M);
+      const int g = __ldg(s.matches + s.q_off[de.x] + m), j = path_of(s, g);
+      const int n = min(s.D, __ldg(s.len + j) - 1 - (g - j * s.L));    // followers
+      const int off = (g + 1) & 3;
+      const int4* const st = reinterpret_cast<const int4*>(s.tok) + ((g + 1) >> 2);
+      const int4* const sp = reinterpret_cast<const int4*>(s.pq) + ((g + 1) >> 2);
+      int4 a = make_int4(0, 0, 0, 0), b = a, c = a, e = a;             // 16 bytes of tokens and the next 16, the same of probabilities
+      if (n > 0) { a = __ldg(st); c = __ldg(sp); }
+      int* tok = items.tok + m;
+      int* p = reinterpret_cast<int*>(items.out) + m;
+#pragma unroll 1
+      for (int l = 0, x = 1; l < s.D; l += 4, ++x) {
+        if (4 * x - off < n) { b = __ldg(st + x); e = __ldg(sp + x); } // (only what holds a follower)
+        const int4 v = shifted(a, b, off), q4 = shifted(c, e, off);
+        a = b; c = e;
+        const int vs[4] = {v.x, v.y, v.z, v.w}, ps[4] = {q4.x, q4.y, q4.z, q4.w};
 #pragma unroll
-  for (int r = 0; r < N; ++r) {
-    const int j = path_of(s, gpos[r]);
-    const bool on = m0 + r * T < M && gpos[r] - j * s.L + d <= __ldg(s.len + j) - 1;
-    v[r] = -1; p[r] = 0u;
-    if (on) { v[r] = __ldg(s.tok + gpos[r] + d); p[r] = (unsigned)__ldg(s.pq + gpos[r] + d); }
+        for (int y = 0; y < 4; ++y)
+          if (l + y < s.D) {
+            *tok = l + y < n ? vs[y] : -1; *p = ps[y];
+            tok += items.pitch; p += 2 * items.pitch;
+          }
+      }
+    }
+    skip -= chunks;
   }
 }
 
@@ -132,14 +175,16 @@ __device__ __forceinline__ void wide_layer(const Dev& s, const int4 de, int d) {
   const int tid = threadIdx.x, M = de.y;
   const int32_t* const list = s.matches + s.q_off[de.x];
   const WideItems items = wide_items(s, de.z, M);
-  u64* const weight = items.out + (size_t)(d - 1) * M;
+  u64* const weight = items.out + (size_t)(d - 1) * items.pitch;
+  const int* const row = items.tok + (size_t)(d - 1) * items.pitch;
+  const int* const row_p = reinterpret_cast<const int*>(weight);
   const bool counts = s.alpha != 1.0;                  // with alpha = 1 a weight does not depend on the count
   int cap = 64;
   while (7 * cap < 8 * M) cap *= 2;
   const WideTable t = wide_table(wide_smem, cap);
-  int v[N];
-  unsigned p[N];
-  wide_gather<N>(s, list, M, d, tid, v, p);            // on its way while the table is emptied
+  int v[N], p[N];
+  wide_row<N>(row, M, tid, -1, v);                     // on its way while the table is emptied
+  wide_row<N>(row_p, M, tid, 0, p);
   wide_table_empty(wide_smem, cap, counts);
   __syncthreads();
   // ---- sums
@@ -149,7 +194,7 @@ __device__ __forceinline__ void wide_layer(const Dev& s, const int4 de, int d) {
 #pragma unroll
   for (int c = 0; c < CH; ++c) {
     const int m0 = c * N * kWideThreads + tid;
-    if (c > 0) wide_gather<N>(s, list, M, d, m0, v, p);
+    if (c > 0) { wide_row<N>(row, M, m0, -1, v); wide_row<N>(row_p, M, m0, 0, p); }
 #pragma unroll
     for (int r = 0; r < N; ++r) {
       kt[c][r] = v[r];
@@ -179,7 +224,7 @@ __device__ __forceinline__ void wide_layer(const Dev& s, const int4 de, int d) {
 #pragma unroll
   for (int c = 0; c < CH; ++c) {
     const int m0 = c * N * kWideThreads + tid;
-    if (!single) wide_gather<N>(s, list, M, d - 1, m0, v, p);
+    if (!single) wide_row<N>(row - items.pitch, M, m0, -1, v);
 #pragma unroll
     for (int r = 0; r < N; ++r) {
       const int m = m0 + r * kWideThreads;
@@ -236,7 +281,7 @@ __device__ __forceinline__ void wide_layer(const Dev& s, const int4 de, int d) {
         else best &= ~(1u << (c * N + r));
       }
   __syncthreads();
-  int* const succ = items.succ + (size_t)(d - 1) * M;
+  int* const succ = items.succ + (size_t)(d - 1) * items.pitch;
 #pragma unroll
   for (int c = 0; c < CH; ++c)
 #pragma unroll
@@ -258,7 +303,8 @@ __device__ __forceinline__ void wide_layer(const Dev& s, const int4 de, int d) {
 #pragma unroll
       for (int r = 0; r < N; ++r)
         if (best >> (c * N + r) & 1u) {
-          const unsigned q = (unsigned)__ldg(s.pq + __ldg(list + (c * N + r) * kWideThreads + tid) + d);
+          const int m = (c * N + r) * kWideThreads + tid;
+          const unsigned q = (unsigned)(KEEP ? __ldcg(row_p + m) : __ldg(s.pq + __ldg(list + m) + d));
           if (single) { lo += q & 0x7fffu; hi += q >> 15; }
           else {
             atomicAdd(&t.lo[slot[c][r]], q & 0x7fffu);
@@ -292,20 +338,11 @@ __device__ __forceinline__ void wide_task(const Dev& s, const int4 de, int d) {
 }
 
 // ---- larger queries: sums only, one task per class of tokens ------------------------------------------------------
-// What those tasks leave, in the place of WideItems: weights, and tokens in rows that start on 16 bytes.
-struct WideRows { u64* weight; int* tok; int pitch; };
-__device__ __forceinline__ WideRows wide_rows(const Dev& s, int first, int M) {
-  WideRows w;
-  w.pitch = wide_pitch(M);
-  w.weight = reinterpret_cast<u64*>(s.w_tab + (unsigned)first);
-  w.tok = reinterpret_cast<int*>(w.weight + (size_t)s.D * w.pitch);
-  return w;
-}
 // Classes (a power of two): tables at most 7/8 full.
 __device__ __forceinline__ int wide_classes(const Dev& s, int M) {
   if (M <= wide_alone(s)) return 1;
   int c = 2;
-  while ((long long)c * (wide_alone(s) / kWideSpread) < M) c *= 2;
+  while ((long long)c * wide_alone(s) < M) c *= 2;
   return c;
 }
 // Weights of the nodes of layer d with tokens of class `cls`.  A table that overruns all the same is done again in sub-classes.
@@ -315,9 +352,9 @@ __device__ __forceinline__ void wide_sums(const Dev& s, const int4 de, int d, un
   constexpr int N = 16;
   const int tid = threadIdx.x, M = de.y;
   const int32_t* const list = s.matches + s.q_off[de.x];
-  const WideRows rows = wide_rows(s, de.z, M);
-  u64* const weight = rows.weight + (size_t)(d - 1) * rows.pitch;
-  int* const tok = rows.tok + (size_t)(d - 1) * rows.pitch;
+  const WideItems rows = wide_items(s, de.z, M);
+  u64* const weight = rows.out + (size_t)(d - 1) * rows.pitch;
+  const int* const tok = rows.tok + (size_t)(d - 1) * rows.pitch;
   const bool counts = s.alpha != 1.0;
   const int cap = counts ? kWideSlots / 2 : kWideSlots;
   const WideTable t = wide_table(wide_smem, cap);
@@ -332,12 +369,18 @@ __device__ __forceinline__ void wide_sums(const Dev& s, const int4 de, int d, un
     for (int m0 = tid; m0 < M; m0 += N * kWideThreads) {
       int v[N];
       unsigned p[N];
-      wide_gather<N>(s, list, M, d, m0, v, p);
+      wide_row<N>(tok, M, m0, -1, v);
+#pragma unroll
+      for (int r = 0; r < N; ++r)
+        if ((wide_class(v[r]) & others) != mine) v[r] = -1;
+      // (from the store: other classes write their weights over the row of probabilities)
+#pragma unroll
+      for (int r = 0; r < N; ++r) p[r] = v[r] >= 0 ? (unsigned)__ldg(list + m0 + r * kWideThreads) : 0u;
+#pragma unroll
+      for (int r = 0; r < N; ++r) p[r] = v[r] >= 0 ? (unsigned)__ldg(s.pq + (int)p[r] + d) : 0u;
 #pragma unroll
       for (int r = 0; r < N; ++r) {
-        const int m = m0 + r * kWideThreads;
-        if (m < M) tok[m] = v[r];                      // (all classes write the same)
-        if (v[r] < 0 || (wide_class(v[r]) & others) != mine) continue;
+        if (v[r] < 0) continue;
         const int h = wide_claim(t, v[r]);
         if (h < 0) sh_over = 1;
         else wide_add(t, h, p[r], counts);
@@ -352,8 +395,7 @@ __device__ __forceinline__ void wide_sums(const Dev& s, const int4 de, int d, un
 #pragma unroll 1
     for (int m0 = tid; m0 < M; m0 += N * kWideThreads) {
       int v[N];
-#pragma unroll
-      for (int r = 0; r < N; ++r) v[r] = m0 + r * kWideThreads < M ? __ldcg(tok + m0 + r * kWideThreads) : -1;
+      wide_row<N>(tok, M, m0, -1, v);
 #pragma unroll
       for (int r = 0; r < N; ++r)
         if (v[r] >= 0 && (wide_class(v[r]) & others) == mine) weight[m0 + r * kWideThreads] = wide_weight(s, t, wide_claim(t, v[r]), counts);
@@ -388,7 +430,7 @@ __device__ __forceinline__ void wide_walk_rows(const Dev& s, const int4 de, cons
   constexpr int B = 8, kHits = kWideSmem / 4;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, D = s.D, i = de.x, M = de.y;
   const int32_t* const list = s.matches + s.q_off[i];
-  const WideRows rows = wide_rows(s, de.z, M);
+  const WideItems rows = wide_items(s, de.z, M);
   int* const hit = reinterpret_cast<int*>(wide_smem);
   if (tid < SDMS_MAX_DRAFT) { sh.e[tid][0] = 0u; sh.e[tid][1] = 0u; sh.e[tid][2] = 0u; }
   if (tid == 0) { sh.hits[0] = 0; sh.hits[1] = 0; }
@@ -398,7 +440,7 @@ __device__ __forceinline__ void wide_walk_rows(const Dev& s, const int4 de, cons
   for (int d = 1; d <= D; ++d) {
     const int* const row = rows.tok + (size_t)(d - 1) * rows.pitch;
     const int* const before = row - rows.pitch;
-    const u64* const row_w = rows.weight + (size_t)(d - 1) * rows.pitch;
+    const u64* const row_w = rows.out + (size_t)(d - 1) * rows.pitch;
     const bool all = d == 1 || s.mode == 1;            // successors of the root / of no node in particular
     if (!all) {
 #pragma unroll 1
@@ -511,7 +553,7 @@ __device__ __forceinline__ void wide_walk_known(const Dev& s, const int4 de, con
   if (s.mode == 1 && out.edge_w) {                     // the edges are known only now
     if (tid < 32) { sh_draft[tid] = -1; sh_e[tid][0] = 0u; sh_e[tid][1] = 0u; sh_e[tid][2] = 0u; }
     __syncthreads();
-    if (tid < D) { const int at = __ldcg(items.succ + (size_t)tid * M); if (at >= 0) sh_draft[tid] = wide_token(s, list, at, tid + 1); }
+    if (tid < D) { const int at = __ldcg(items.succ + (size_t)tid * items.pitch); if (at >= 0) sh_draft[tid] = __ldcg(items.tok + (size_t)tid * items.pitch + at); }
     __syncthreads();
     for (int m = tid; m < M; m += kWideThreads) {
       const int g = __ldg(list + m), j = path_of(s, g), n = min(D, __ldg(s.len + j) - 1 - (g - j * s.L));
@@ -533,12 +575,12 @@ __device__ __forceinline__ void wide_walk_known(const Dev& s, const int4 de, con
     for (int d = 1; d <= D && at >= 0; ++d) {
       if (tid == d - 1) mine = at;
       emitted = d;
-      at = d < D ? __ldcg(items.succ + (size_t)d * M + at) : -1;
+      at = d < D ? __ldcg(items.succ + (size_t)d * items.pitch + at) : -1;
     }
     if (tid < D) {
-      const size_t x = (size_t)i * D + tid, y = (size_t)tid * M + max(mine, 0);
+      const size_t x = (size_t)i * D + tid, y = (size_t)tid * items.pitch + max(mine, 0);
       const bool on = mine >= 0;
-      const int v = on ? wide_token(s, list, mine, tid + 1) : -1;
+      const int v = on ? __ldcg(items.tok + y) : -1;
       const u64 o = ld_u64(items.out + y);
       out.tok[x] = v;
       if (out.score) out.score[x] = on ? __uint_as_float((unsigned)o) : 0.0f;
@@ -564,7 +606,7 @@ __device__ __forceinline__ void wide_walk(const Dev& s, const int4 de, const Wid
 __global__ void __launch_bounds__(kWideThreads, 1)
 dag_wide_kernel(Dev s, int32_t* __restrict__ draft_tok, int32_t* __restrict__ draft_len,
                 float* __restrict__ draft_score, float* __restrict__ draft_edge_w) {
-  grid_wait();                                         // scheduled while dag_kernel drains; its list is complete from here on
+  grid_wait();
   const u64 registered = ld_u64(&s.w_ctl[0]);
   if (registered == 0) return;
   const int nq = (int)(registered < (u64)kMaxWide ? registered : (u64)kMaxWide);
@@ -675,6 +717,8 @@ cudaError_t launch_wait_timeout(const Dev& s, long long cycles, cudaStream_t str
 
 cudaError_t launch_dag_wide(const Dev& s, int32_t* draft_tok, int32_t* draft_len, float* draft_score,
                             float* draft_edge_w, cudaStream_t stream) {
+  const cudaError_t e = launch_overlapped(dag_rows_kernel, dim3(4 * s.w_grid), dim3(kRowThreads), 0, stream, s);
+  if (e != cudaSuccess) return e;
   return launch_overlapped(dag_wide_kernel, dim3(s.w_grid), dim3(kWideThreads), kWideSmem, stream, s, draft_tok, draft_len,
                            draft_score, draft_edge_w);
 }

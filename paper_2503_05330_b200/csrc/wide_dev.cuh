@@ -4,10 +4,13 @@
 
 namespace sdms {
 
-// Room (in table slots of 32 bytes) that a query with M matches takes: 12 bytes for every (match, layer).
+constexpr int kWideSlots = 16384;                    // most slots of a task's table (half of them where counts are kept too)
+// Most matches of a query whose layers are one task each: their table is at most 7/8 full.
+__device__ __forceinline__ int wide_alone(const Dev& s) { return (s.alpha != 1.0 ? kWideSlots / 2 : kWideSlots) / 8 * 7; }
+// Room (in table slots of 32 bytes) that a query with M matches takes: 16 bytes for every (match, layer), 12 above wide_alone().
 __device__ __forceinline__ int wide_pitch(int M) { return (M + 3) & ~3; }
 __device__ __forceinline__ unsigned long long wide_slots(const Dev& s, int M) {
-  return ((unsigned long long)wide_pitch(M) * s.D * 12 + sizeof(WideSlot) - 1) / sizeof(WideSlot);
+  return ((unsigned long long)wide_pitch(M) * s.D * (M <= wide_alone(s) ? 16 : 12) + sizeof(WideSlot) - 1) / sizeof(WideSlot);
 }
 
 // log2 of the slots of one layer's node table in the table area (beams): a power of two above 5/4 of the matches.
