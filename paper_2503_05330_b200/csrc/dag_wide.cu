@@ -613,8 +613,10 @@ dag_wide_kernel(Dev s, int32_t* __restrict__ draft_tok, int32_t* __restrict__ dr
   __shared__ int4 sh_desc[kMaxWide];
   __shared__ int sh_base[kMaxWide + 1];                // first task of each query
   __shared__ int sh_warp[kWideWarps];
-  __shared__ int sh_task, sh_last;
+  __shared__ int sh_task, sh_last, sh_large;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, D = s.D;
+  int spread;
+  if (tid == 0) sh_large = 0;
   static_assert(kMaxWide == 2 * kWideThreads, "two list entries per thread");
   // the list of queries, the largest first, and by a prefix sum the first task of each
   {
@@ -649,9 +651,23 @@ dag_wide_kernel(Dev s, int32_t* __restrict__ draft_tok, int32_t* __restrict__ dr
         if (2 * tid + r < nq) sh_desc[2 * tid + r].w = 2 * tid + r;
     }
     __syncthreads();
-    int c[2];
+    int c[2], large = 0;
 #pragma unroll
-    for (int r = 0; r < 2; ++r) c[r] = 2 * tid + r < nq ? D * wide_classes(s, sh_desc[2 * tid + r].y) : 0;
+    for (int r = 0; r < 2; ++r) {
+      const int M = 2 * tid + r < nq ? sh_desc[2 * tid + r].y : 0;
+      c[r] = M > 0 ? D * wide_classes(s, M) : 0;
+      if (M > wide_alone(s)) large += c[r];
+    }
+    if (large) atomicAdd(&sh_large, large);
+    __syncthreads();
+    // more and smaller classes while the large queries' tasks leave most of the CTAs without work (one query of 26 270 matches,
+    // D = 16: 333 us with 32 tasks, 250 with 128; where there are tasks for all CTAs four times the classes are 1.4 to 1.8 times the
+    // work: 16 prompts of 128 x 4096 tokens, k = 1, 1.39 against 2.44 ms)
+    spread = 1;
+    while (spread < 4 && sh_large > 0 && 2 * spread * sh_large <= (int)gridDim.x) spread *= 2;
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+      if (2 * tid + r < nq && sh_desc[2 * tid + r].y > wide_alone(s)) c[r] *= spread;
     int x = c[0] + c[1];
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) { const int y = __shfl_up_sync(FULL, x, o); if (lane >= o) x += y; }
@@ -677,7 +693,7 @@ dag_wide_kernel(Dev s, int32_t* __restrict__ draft_tok, int32_t* __restrict__ dr
     int a = 0, b = nq;                                 // sh_base[a] <= task < sh_base[b]
     while (b - a > 1) { const int mid = (a + b) >> 1; if (sh_base[mid] <= task) a = mid; else b = mid; }
     const int4 de = sh_desc[a];
-    const int classes = wide_classes(s, de.y), part = task - sh_base[a];
+    const int classes = wide_classes(s, de.y) * (de.y > wide_alone(s) ? spread : 1), part = task - sh_base[a];
     if (de.y <= wide_alone(s)) wide_task(s, de, part + 1);
     else wide_sums(s, de, part / classes + 1, (unsigned)(part % classes), (unsigned)classes);
     // done with it: its results are out before it is counted, and whoever counts the last one has seen all of them

@@ -136,6 +136,34 @@ def test_walk_at_the_edges_of_its_forms(M, alpha):
     pair.beams_and_compare(3, paths=[0])              # in shared memory up to 129 of these, lists in the table area for 600, all there for 1500
 
 
+@pytest.mark.parametrize("M,alpha,V", [(65, 1.0, 50), (2048, 0.5, 4000), (2049, 1.0, 4000), (7168, 0.5, 60000), (7169, 0.5, 60000),
+                                       (8193, 1.0, 60000), (14336, 1.0, 60000), (14337, 1.0, 60000), (30000, 1.0, 60000)])
+@pytest.mark.parametrize("mode", [0, 1])
+def test_layer_tasks_at_the_edges_of_their_forms(M, alpha, V, mode):
+    # a prompt too large for the single-launch build; one query with exactly M matches whose followers are half from a small
+    # alphabet with a heavy-tailed draw, half from all V tokens: candidates in registers to 2048, to 8192, to 14336 (7168 where
+    # weights need counts), by classes of tokens beyond
+    D, k, N = 6, 1, 16
+    step = D + 2
+    L = max((M // (N - 1) + 2) * step + 4, 9000)
+    rng = np.random.default_rng(7100 + M)
+    tokens = 1 + np.minimum((rng.random((N, L)) ** 3 * 48).astype(np.int32), 47)
+    tokens = np.where(rng.random((N, L)) < 0.5, rng.integers(1, V, (N, L)), tokens).astype(np.int32)
+    lps = -rng.exponential(0.5, (N, L)).astype(np.float32)
+    per = -(-M // (N - 1))
+    for m in range(M):
+        tokens[1 + m // per, 1 + (m % per) * step] = 0
+    tokens[0, L - 3] = 0
+    lens = np.full(N, L - 1)
+    lens[0] = L - 2
+    lens[1:] = np.minimum(lens[1:], 1 + per * step + np.arange(N - 1) % 3)             # some candidates end early
+    pair = Pair(1, N, L, V, k, D, alpha=alpha, mode=mode, B=2, Ke=2)
+    assert not pair.g.step_is_single_launch()
+    pair.append(tokens, lps, lens, expect_status=0)
+    tok, ln = pair.build_and_compare(k, check_dag=False)
+    assert len(pair.o.matches(0)) == M and ln[0] > 0
+
+
 @pytest.mark.parametrize("N,L", [(16, 1024), (64, 2048)])
 def test_reset_leaves_nothing_behind(N, L):
     # an index that is cleared and one whose buckets go out of date: more resets than there are epochs, other streams
