@@ -108,10 +108,12 @@ typedef struct {
   int32_t  max_beams;            /* largest number of drafts per path that sdms_get_beams will be asked for
                                     (0 = the call is not used; at most SDMS_MAX_BEAMS)               */
   int64_t  wide_table_bytes;     /* workspace set aside for node tables in global memory.  Two users: on
-                                    prompts too large for the single-launch build, queries with more than 32
-                                    matches are aggregated by all SMs together; and sdms_get_beams (max_beams
-                                    > 0) and search_mode 2.  A slot costs 40 + 16 * max(max_beams, 1) bytes and a path with M matches
-                                    needs between 2.5 and 5 * M * D slots (half of that for the beams).  0 = default (room for every position
+                                    prompts too large for the single-launch build, queries with more than 64
+                                    matches are aggregated by all SMs together, in 16 * M * D bytes for M
+                                    matches (12 * M * D above 14336 of them, 7168 with alpha < 1); and
+                                    sdms_get_beams (max_beams > 0) and search_mode 2 for paths whose tables
+                                    do not fit shared memory, in slots of 40 + 16 * max(max_beams, 1) bytes.
+                                    0 = default (room for every position
                                     matching every query of its prompt, but at most 320 MiB), -1 = none.  A build
                                     whose queries need more falls back to one thread block for those that
                                     did not fit, with the same results                                    */
@@ -309,7 +311,7 @@ int sdms_debug_read_history(sdms_ctx* ctx, int32_t* d_tok, int32_t* d_pq, int32_
  * 0 = no query or no index entry, 1 = from the index bucket, 2 = by scanning. */
 int sdms_debug_read_query_modes(sdms_ctx* ctx, int32_t* d_modes, void* stream);
 
-/* Every wait inside a kernel (grid barrier of the wide pass, copy barriers of the streaming scan) is bounded:
+/* Every wait inside a kernel (such as the copy barriers of the streaming scan) is bounded:
  * when it runs out, the kernel raises SDMS_STATUS_TIMEOUT and returns, and the context stays usable.  This call
  * shows what that looks like without anything going wrong: one thread waits, with the same bounded wait, about
  * half a millisecond for a count that nobody raises, sets the status bit and returns. */

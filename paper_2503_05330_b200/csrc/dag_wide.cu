@@ -2,21 +2,26 @@
 // single-launch build, spread over the whole device.
 //
 // One CTA that aggregates a query of thousands of matches by itself takes hundreds of microseconds while the other SMs idle,
-// so dag_kernel hands such queries over (wide_register).  Here every (query, layer) pair is a task of its own, done by one CTA
-// in its shared memory:
-//   sums    the layer's followers are gathered and summed up per token in a hash table
+// so dag_kernel hands such queries over (wide_register).  First all CTAs lay the followers of all candidates out layer by layer.
+// Then (query, layer) pairs are tasks that come from a counter, heavy queries first, each done by one CTA in its shared memory:
+//   sums    followers and probabilities of the layer, summed up per token in a hash table
 //   offers  a second table, by the token of the layer before: the heaviest node among its successors, found in three 32-bit
 //           maxima (upper and lower word of the weight, then the smaller token), and the sums of the edge to it
-// Every candidate gets its token, its node's weight and, as the best successor of the node it comes from, the index of one
-// candidate on it.  The CTA that completes the last layer of a query then walks it: one dependent load per layer.  Nobody
-// waits for anybody: tasks come from a counter, heavy queries first.  Sums are integers and every choice has a tie rule, so the
-// order in which things happen cannot show in a result.
+// so that every candidate has the best successor of the node it comes from, as the index of one candidate on it, and the CTA
+// that completes the last layer of a query walks it with one dependent load per layer.  Queries above wide_alone() matches: the
+// sums only, a task per class of tokens (a table holds at most 16 384), and a walk that picks the candidates on the current node
+// out of each layer's row.  Sums are integers and every choice has a tie rule, so the order in which things happen cannot show
+// in a result.
 //
-// What bounds a task: the gather (a 32-byte sector per follower) and the shared-memory atomics.  The forms before: all nodes
-// in tables in global memory and five passes over all items with grid barriers in between took 32 us for one query of 200
-// matches and D = 16, 165 us for 12 000 matches, and had room for a quarter of the 420 000 matches of 16 prompts of 128 x 4096
-// tokens, whose heaviest queries then kept one CTA each busy for 1.2 ms; sums by tasks as here but a walk that swept over the
-// candidates layer by layer left 1.0 us of one SM per thousand candidates and layer at the end.
+// What bounds a task: the latency of its chain of shared-memory steps up to a few hundred candidates (8 K cycles), the shared-
+// memory atomics beyond (a layer of 7300 candidates: 55 K cycles, of these 18 K claims and sums, 20 K offers).  The form before
+// (node tables in global memory, five passes with grid barriers between them) took 32 us for one query of 200 matches and
+// D = 16 against 17 + 5 here, 165 against 41 + 9 for one of 8000, and 10 to 25 KB of tables per match, so that 16 prompts of
+// 128 x 4096 tokens, 420 000 matches at k = 1, overran the area and kept one CTA each for their largest queries (1.2 ms).
+// Also measured: a task for all queries above wide_alone() by a cluster of 8 CTAs with the table in distributed shared memory
+// (26 270 matches: 187 us against 250, but 8 times slower than classes as soon as there are tasks for all CTAs, and 3 us for every
+// launch that has nothing to do); slots, tokens and weights of 64 candidates per thread (spills; 546 us); N table accesses of a
+// thread on their way together, predicated (no change: the atomics' throughput is what counts).
 #include <climits>
 #include "sdms_internal.h"
 #include "wide_dev.cuh"
@@ -27,6 +32,7 @@ namespace {
 
 constexpr int kWideSmem = kWideSlots * 12;
 constexpr int kWideWarps = kWideThreads / 32;
+constexpr long long kWideWait = 1ll << 32;            // cycles, about two seconds
 constexpr int kSortFrom = 256;                       // more queries than this balance without an order
 
 __device__ __forceinline__ u64 ld_u64(const u64* p) { return __ldcg(p); }
@@ -36,7 +42,7 @@ __device__ __forceinline__ bool wait_for_count(const u64* ctr, u64 target, long 
   const long long t0 = clock64();
   while (ld_u64(ctr) < target) {
     if (clock64() - t0 > cycles) return false;
-    __nanosleep(32);
+    __nanosleep(20);
   }
   return true;
 }
@@ -117,52 +123,38 @@ __device__ __forceinline__ void wide_row(const int* row, int M, int m0, int none
 // layer and each step on its own, they were 3 to 4 sectors of 32 bytes per (candidate, layer), and those were what a task
 // waited for (40 of the 90 K cycles of a layer of 7300 candidates).  Here a thread reads a candidate's followers and
 // probabilities, 16 aligned bytes at a time, and lays them out in rows.
-constexpr int kRowThreads = 256;
 __device__ __forceinline__ int4 shifted(int4 a, int4 b, int off) {      // words off .. off + 3 of a, b
   if (off & 2) { a.x = a.z; a.y = a.w; a.z = b.x; a.w = b.y; b.x = b.z; }
   if (off & 1) { a.x = a.y; a.y = a.z; a.z = a.w; a.w = b.x; }
   return a;
 }
-__global__ void __launch_bounds__(kRowThreads) dag_rows_kernel(Dev s) {
-  grid_wait();                                         // scheduled while dag_kernel drains; its list is complete from here on
-  const u64 registered = ld_u64(&s.w_ctl[0]);
-  const int nq = (int)(registered < (u64)kMaxWide ? registered : (u64)kMaxWide);
-  __shared__ int4 sh_desc[kMaxWide];
-  for (int q = threadIdx.x; q < nq; q += kRowThreads) sh_desc[q] = __ldcg(&s.w_desc[q]);
-  __syncthreads();
-  int skip = blockIdx.x;                               // chunks of kRowThreads candidates until this CTA's next one
-#pragma unroll 1
-  for (int q = 0; q < nq; ++q) {
-    const int4 de = sh_desc[q];
-    const int M = de.y, chunks = (M + kRowThreads - 1) / kRowThreads;
-    for (; skip < chunks; skip += gridDim.x) {
-      const int m = skip * kRowThreads + threadIdx.x;
-      if (m >= M) continue;
-      const WideItems items = wide_items(s, de.z, M);
-      const int g = __ldg(s.matches + s.q_off[de.x] + m), j = path_of(s, g);
-      const int n = min(s.D, __ldg(s.len + j) - 1 - (g - j * s.L));    // followers
-      const int off = (g + 1) & 3;
-      const int4* const st = reinterpret_cast<const int4*>(s.tok) + ((g + 1) >> 2);
-      const int4* const sp = reinterpret_cast<const int4*>(s.pq) + ((g + 1) >> 2);
-      int4 a = make_int4(0, 0, 0, 0), b = a, c = a, e = a;             // 16 bytes of tokens and the next 16, the same of probabilities
-      if (n > 0) { a = __ldg(st); c = __ldg(sp); }
-      int* tok = items.tok + m;
-      int* p = reinterpret_cast<int*>(items.out) + m;
-#pragma unroll 1
-      for (int l = 0, x = 1; l < s.D; l += 4, ++x) {
-        if (4 * x - off < n) { b = __ldg(st + x); e = __ldg(sp + x); } // (only what holds a follower)
-        const int4 v = shifted(a, b, off), q4 = shifted(c, e, off);
-        a = b; c = e;
-        const int vs[4] = {v.x, v.y, v.z, v.w}, ps[4] = {q4.x, q4.y, q4.z, q4.w};
+// Candidates c0 .. c0 + kWideThreads of a query.
+__device__ __forceinline__ void wide_lay_out(const Dev& s, const int4 de, int c0) {
+  const int M = de.y, m = c0 + threadIdx.x;
+  if (m >= M) return;
+  const WideItems items = wide_items(s, de.z, M);
+  const int g = __ldg(s.matches + s.q_off[de.x] + m), j = path_of(s, g);
+  const int n = min(s.D, __ldg(s.len + j) - 1 - (g - j * s.L));        // followers
+  const int off = (g + 1) & 3;
+  const int4* const st = reinterpret_cast<const int4*>(s.tok) + ((g + 1) >> 2);
+  const int4* const sp = reinterpret_cast<const int4*>(s.pq) + ((g + 1) >> 2);
+  int4 a = make_int4(0, 0, 0, 0), b = a, c = a, e = a;                 // 16 bytes of tokens and the next 16, the same of probabilities
+  if (n > 0) { a = __ldg(st); c = __ldg(sp); }
+  int* tok = items.tok + m;
+  int* p = reinterpret_cast<int*>(items.out) + m;
+#pragma unroll 4
+  for (int x = 1; 4 * x - 4 < s.D; ++x) {
+    const int l = 4 * x - 4;
+    if (4 * x - off < n) { b = __ldg(st + x); e = __ldg(sp + x); }     // (only what holds a follower)
+    const int4 v = shifted(a, b, off), q = shifted(c, e, off);
+    a = b; c = e;
+    const int vs[4] = {v.x, v.y, v.z, v.w}, ps[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
-        for (int y = 0; y < 4; ++y)
-          if (l + y < s.D) {
-            *tok = l + y < n ? vs[y] : -1; *p = ps[y];
-            tok += items.pitch; p += 2 * items.pitch;
-          }
+    for (int y = 0; y < 4; ++y)
+      if (l + y < s.D) {
+        *tok = l + y < n ? vs[y] : -1; *p = ps[y];
+        tok += items.pitch; p += 2 * items.pitch;
       }
-    }
-    skip -= chunks;
   }
 }
 
@@ -606,19 +598,20 @@ __device__ __forceinline__ void wide_walk(const Dev& s, const int4 de, const Wid
 __global__ void __launch_bounds__(kWideThreads, 1)
 dag_wide_kernel(Dev s, int32_t* __restrict__ draft_tok, int32_t* __restrict__ draft_len,
                 float* __restrict__ draft_score, float* __restrict__ draft_edge_w) {
-  grid_wait();
+  grid_wait();                                         // scheduled while dag_kernel drains; its list is complete from here on
   const u64 registered = ld_u64(&s.w_ctl[0]);
   if (registered == 0) return;
   const int nq = (int)(registered < (u64)kMaxWide ? registered : (u64)kMaxWide);
   __shared__ int4 sh_desc[kMaxWide];
   __shared__ int sh_base[kMaxWide + 1];                // first task of each query
+  __shared__ int sh_unit[kMaxWide + 1];                // first chunk of kWideThreads candidates of each query
   __shared__ int sh_warp[kWideWarps];
   __shared__ int sh_task, sh_last, sh_large;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, D = s.D;
   int spread;
   if (tid == 0) sh_large = 0;
   static_assert(kMaxWide == 2 * kWideThreads, "two list entries per thread");
-  // the list of queries, the largest first, and by a prefix sum the first task of each
+  // the list of queries, the largest first, and by prefix sums the first task and the first chunk of each
   {
     int4 de[2];
     int rank[2];
@@ -668,30 +661,68 @@ dag_wide_kernel(Dev s, int32_t* __restrict__ draft_tok, int32_t* __restrict__ dr
 #pragma unroll
     for (int r = 0; r < 2; ++r)
       if (2 * tid + r < nq && sh_desc[2 * tid + r].y > wide_alone(s)) c[r] *= spread;
-    int x = c[0] + c[1];
+    auto prefix = [&](int c0, int c1, int* first) {    // first[q] = sum of the counts before q, for two queries per thread
+      int x = c0 + c1;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) { const int y = __shfl_up_sync(FULL, x, o); if (lane >= o) x += y; }
-    if (lane == 31) sh_warp[warp] = x;
-    __syncthreads();
-    if (warp == 0) {
-      int w = lane < kWideWarps ? sh_warp[lane] : 0;
+      for (int o = 1; o < 32; o <<= 1) { const int y = __shfl_up_sync(FULL, x, o); if (lane >= o) x += y; }
+      if (lane == 31) sh_warp[warp] = x;
+      __syncthreads();
+      if (warp == 0) {
+        int w = lane < kWideWarps ? sh_warp[lane] : 0;
 #pragma unroll
-      for (int o = 1; o < 32; o <<= 1) { const int y = __shfl_up_sync(FULL, w, o); if (lane >= o) w += y; }
-      if (lane < kWideWarps) sh_warp[lane] = w;
-    }
-    __syncthreads();
-    const int ahead = (warp ? sh_warp[warp - 1] : 0) + x - c[0] - c[1];
-    sh_base[2 * tid] = ahead;
-    sh_base[2 * tid + 1] = ahead + c[0];
-    if (tid == kWideThreads - 1) sh_base[kMaxWide] = ahead + c[0] + c[1];
-    __syncthreads();
+        for (int o = 1; o < 32; o <<= 1) { const int y = __shfl_up_sync(FULL, w, o); if (lane >= o) w += y; }
+        if (lane < kWideWarps) sh_warp[lane] = w;
+      }
+      __syncthreads();
+      const int ahead = (warp ? sh_warp[warp - 1] : 0) + x - c0 - c1;
+      first[2 * tid] = ahead;
+      first[2 * tid + 1] = ahead + c0;
+      if (tid == kWideThreads - 1) first[kMaxWide] = ahead + c0 + c1;
+      __syncthreads();
+    };
+    prefix(c[0], c[1], sh_base);
+#pragma unroll
+    for (int r = 0; r < 2; ++r) c[r] = 2 * tid + r < nq ? (sh_desc[2 * tid + r].y + kWideThreads - 1) / kWideThreads : 0;
+    prefix(c[0], c[1], sh_unit);
   }
+  auto owner = [&](const int* first, int x) {          // first[owner] <= x < first[owner + 1], of those that are not empty
+    int a = 0, b = nq;
+    while (b - a > 1) { const int mid = (a + b) >> 1; if (first[mid] <= x) a = mid; else b = mid; }
+    return a;
+  };
+  // Everybody lays out rows, then waits until all rows are there.  Chunks come from a counter, so that the wait is for running
+  // CTAs only, whatever else is on the device; it is bounded all the same.
+  const int units = sh_unit[nq];
+  if (tid == 0) sh_task = (int)atomicAdd(&s.w_ctl[3], 1ull);
+  __syncthreads();
+#pragma unroll 1
+  for (int unit = sh_task; unit < units;) {
+    __syncthreads();
+    if (tid == 0) sh_task = (int)atomicAdd(&s.w_ctl[3], 1ull);         // (on its way during this one)
+    const int q = owner(sh_unit, unit);
+    wide_lay_out(s, sh_desc[q], (unit - sh_unit[q]) * kWideThreads);
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) atomicAdd(&s.w_ctl[4], 1ull);
+    unit = sh_task;
+  }
+  __syncthreads();
+  if (tid == 0) {
+    sh_last = wait_for_count(s.w_ctl + 4, (u64)units, kWideWait);
+    if (sh_last) sh_task = (int)atomicAdd(&s.w_ctl[2], 1ull);          // (whoever gives up here leaves no task undone)
+  }
+  __syncthreads();
+  if (!sh_last) {
+    if (tid == 0) atomicOr(s.status, SDMS_STATUS_TIMEOUT);
+    return;
+  }
+  __threadfence();
   const int tasks = sh_base[nq];
-  int task = blockIdx.x;                               // the first one without asking
+  int task = sh_task;
+  __syncthreads();
 #pragma unroll 1
   while (task < tasks) {
-    int a = 0, b = nq;                                 // sh_base[a] <= task < sh_base[b]
-    while (b - a > 1) { const int mid = (a + b) >> 1; if (sh_base[mid] <= task) a = mid; else b = mid; }
+    const int a = owner(sh_base, task);
     const int4 de = sh_desc[a];
     const int classes = wide_classes(s, de.y) * (de.y > wide_alone(s) ? spread : 1), part = task - sh_base[a];
     if (de.y <= wide_alone(s)) wide_task(s, de, part + 1);
@@ -700,7 +731,7 @@ dag_wide_kernel(Dev s, int32_t* __restrict__ draft_tok, int32_t* __restrict__ dr
     __threadfence();
     __syncthreads();
     if (tid == 0) {
-      sh_task = (int)gridDim.x + (int)atomicAdd(&s.w_ctl[2], 1ull);
+      sh_task = (int)atomicAdd(&s.w_ctl[2], 1ull);
       const int total = D * classes;
       sh_last = atomicAdd(&s.w_done[de.w], 1) == total - 1;
       if (sh_last) s.w_done[de.w] = 0;                 // the next build finds it at zero
@@ -733,8 +764,6 @@ cudaError_t launch_wait_timeout(const Dev& s, long long cycles, cudaStream_t str
 
 cudaError_t launch_dag_wide(const Dev& s, int32_t* draft_tok, int32_t* draft_len, float* draft_score,
                             float* draft_edge_w, cudaStream_t stream) {
-  const cudaError_t e = launch_overlapped(dag_rows_kernel, dim3(4 * s.w_grid), dim3(kRowThreads), 0, stream, s);
-  if (e != cudaSuccess) return e;
   return launch_overlapped(dag_wide_kernel, dim3(s.w_grid), dim3(kWideThreads), kWideSmem, stream, s, draft_tok, draft_len,
                            draft_score, draft_edge_w);
 }

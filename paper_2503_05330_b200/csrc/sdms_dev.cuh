@@ -22,7 +22,7 @@ constexpr int kFusedMaxTokens = 131072; // largest N*L a CTA scans on its own
 constexpr int kMaxWide = 1024;          // queries one build can hand to the device-wide aggregation pass
 constexpr int kWideSumShift = 47;       // packed node sums: count in the upper 17 bits, sum of probabilities below
 constexpr int kWideMaxMatches = (1 << 17) - 1;   // so that both parts of a packed sum fit
-constexpr int kWideCtlWords = 3;
+constexpr int kWideCtlWords = 5;
 
 // Q_DONE: a back-off build on a large prompt has found this path's matches at a longer suffix length
 enum QueryMode : int32_t { Q_NONE = 0, Q_INLINE = 1, Q_SCAN = 2, Q_DONE = 3 };
@@ -73,7 +73,7 @@ struct Dev {
   int32_t* g_trim;                     // [G] a path of the prompt was trimmed: its index is rebuilt
   int32_t* matches;                    // [match_cap] global positions j*L+e
   // device-wide aggregation of queries with many matches (dag_wide.cu); w_slots = 0: not in use
-  unsigned long long* w_ctl;           // [kWideCtlWords] queries registered, slots handed out, tasks handed out beyond the first of each CTA
+  unsigned long long* w_ctl;           // [kWideCtlWords] queries registered, slots handed out, tasks handed out, chunks handed out, chunks done
   int4* w_desc;                        // [kMaxWide] query path, matches, first slot, -
   int* w_done;                         // [kMaxWide] layers of the query that are done; zero between builds
   WideSlot* w_tab;                     // [w_slots]
