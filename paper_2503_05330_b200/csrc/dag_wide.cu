@@ -362,6 +362,11 @@ __device__ __forceinline__ void wide_sums(const Dev& s, const int4 de, int d, un
       int v[N];
       unsigned p[N];
       wide_row<N>(tok, M, m0, -1, v);
+      if (cls == 0u) {
+#pragma unroll
+        for (int r = 0; r < N; ++r)
+          if (v[r] < 0 && m0 + r * kWideThreads < M) weight[m0 + r * kWideThreads] = 0ull;   // (ended)
+      }
 #pragma unroll
       for (int r = 0; r < N; ++r)
         if ((wide_class(v[r]) & others) != mine) v[r] = -1;
@@ -405,8 +410,8 @@ __device__ __forceinline__ u64 warp_max64(u64 x) {
   return (u64)top << 32 | lo;
 }
 struct WideWalk {                        // what the walk over rows keeps in shared memory
-  u64 best[2][kWideWarps];
-  int tok[2][kWideWarps];
+  u64 best[kWideWarps];
+  int tok[kWideWarps];
   int draft[SDMS_MAX_DRAFT];
   u64 weight[SDMS_MAX_DRAFT];
   unsigned e[SDMS_MAX_DRAFT][3];         // edge sums: lower 15 bits, rest, count
@@ -463,57 +468,65 @@ __device__ __forceinline__ void wide_walk_rows(const Dev& s, const int4 de, cons
     const bool listed = !all && hits <= kHits;
     const int n = listed ? hits : M;
     if (tid == 0) sh.hits[(d + 1) & 1] = 0;
-    // the best successor
-    u64 best = 0ull;
-    int tok = INT_MAX;
-#pragma unroll 1
-    for (int x0 = tid; x0 < n; x0 += B * kWideThreads) {
-      int t[B];
-      u64 w[B];
-#pragma unroll
-      for (int r = 0; r < B; ++r) {
-        const int x = x0 + r * kWideThreads, m = x >= n ? 0 : listed ? hit[x] : x;
-        t[r] = x < n ? __ldcg(row + m) : -1;
-        w[r] = x < n ? ld_u64(row_w + m) : 0ull;
-        if (!all && !listed && x < n && __ldcg(before + m) != cur) t[r] = -1;
-      }
-#pragma unroll
-      for (int r = 0; r < B; ++r) {
-        // (a node of weight zero is still a node: what counts is whether there is a token)
-        const bool better = t[r] >= 0 && (tok == INT_MAX || w[r] > best || (w[r] == best && t[r] < tok));
-        best = better ? w[r] : best; tok = better ? t[r] : tok;
-      }
-    }
-    {
-      const u64 top = warp_max64(best);
-      tok = (int)__reduce_min_sync(FULL, best == top ? (unsigned)tok : (unsigned)INT_MAX);
-      if (lane == 0) { sh.best[d & 1][warp] = top; sh.tok[d & 1][warp] = tok; }
-      __syncthreads();
-      const u64 b = lane < kWideWarps ? sh.best[d & 1][lane] : 0ull;
-      const int bt = lane < kWideWarps ? sh.tok[d & 1][lane] : INT_MAX;
-      best = warp_max64(b);
-      tok = (int)__reduce_min_sync(FULL, b == best ? (unsigned)bt : (unsigned)INT_MAX);
-    }
-    if (tok == INT_MAX) break;                         // no successor: the draft ends here
-    // the candidates on the edge to it
-    unsigned lo = 0u, hi = 0u, count = 0u;
-#pragma unroll 1
-    for (int x0 = tid; x0 < n; x0 += B * kWideThreads) {
-      bool on[B];
-      int m[B];
-      unsigned p[B];
+    // The heaviest successor, the smallest token of those, the edge to it: weights of all hits, tokens only of the heaviest,
+    // probabilities only on the edge (what a CTA gathers from L2 takes 2 cycles per sector).  Read again for each step if there
+    // are more hits than are kept in registers.
+    const bool again = n > B * kWideThreads;
+    int m[B], t[B];
+    u64 w[B];
+    auto load_weights = [&](int x0) {
 #pragma unroll
       for (int r = 0; r < B; ++r) {
         const int x = x0 + r * kWideThreads;
-        m[r] = x >= n ? 0 : listed ? hit[x] : x;
-        on[r] = x < n && __ldcg(row + m[r]) == tok && (all ? d == 1 || __ldcg(before + m[r]) == cur : listed || __ldcg(before + m[r]) == cur);
+        m[r] = x >= n ? -1 : listed ? hit[x] : x;
+        if (!all && !listed && m[r] >= 0 && __ldcg(before + m[r]) != cur) m[r] = -1;
+        w[r] = m[r] >= 0 ? ld_u64(row_w + m[r]) : 0ull;
+      }
+    };
+    u64 best = 0ull;
+    auto load_tokens = [&]() {
+#pragma unroll
+      for (int r = 0; r < B; ++r) t[r] = m[r] >= 0 && w[r] == best ? __ldcg(row + m[r]) : -1;
+    };
+#pragma unroll 1
+    for (int x0 = tid; x0 - tid < n; x0 += B * kWideThreads) {
+      load_weights(x0);
+#pragma unroll
+      for (int r = 0; r < B; ++r) best = w[r] > best ? w[r] : best;
+    }
+    best = warp_max64(best);
+    if (lane == 0) sh.best[warp] = best;
+    __syncthreads();
+    best = warp_max64(lane < kWideWarps ? sh.best[lane] : 0ull);
+    int tok = INT_MAX;
+#pragma unroll 1
+    for (int x0 = tid; x0 - tid < n; x0 += B * kWideThreads) {
+      if (again) load_weights(x0);
+      load_tokens();
+#pragma unroll
+      for (int r = 0; r < B; ++r) tok = t[r] >= 0 && t[r] < tok ? t[r] : tok;        // (a candidate that has ended weighs nothing)
+    }
+    tok = (int)__reduce_min_sync(FULL, (unsigned)tok);
+    if (lane == 0) sh.tok[warp] = tok;
+    __syncthreads();
+    tok = (int)__reduce_min_sync(FULL, (unsigned)(lane < kWideWarps ? sh.tok[lane] : INT_MAX));
+    if (tok == INT_MAX) break;                         // no successor: the draft ends here
+    unsigned lo = 0u, hi = 0u, count = 0u;
+#pragma unroll 1
+    for (int x0 = tid; x0 - tid < n; x0 += B * kWideThreads) {
+      if (again) { load_weights(x0); load_tokens(); }
+      int g[B];
+      unsigned p[B];
+#pragma unroll
+      for (int r = 0; r < B; ++r) {
+        // (layer-wise search looks at all candidates, but the edge is from the node before)
+        const bool on = t[r] == tok && (!all || d == 1 || __ldcg(before + m[r]) == cur);
+        g[r] = on ? __ldg(list + m[r]) : -1;
       }
 #pragma unroll
-      for (int r = 0; r < B; ++r) m[r] = on[r] ? __ldg(list + m[r]) : 0;
+      for (int r = 0; r < B; ++r) p[r] = g[r] >= 0 ? (unsigned)__ldg(s.pq + g[r] + d) : 0u;
 #pragma unroll
-      for (int r = 0; r < B; ++r) p[r] = on[r] ? (unsigned)__ldg(s.pq + m[r] + d) : 0u;
-#pragma unroll
-      for (int r = 0; r < B; ++r) { lo += p[r] & 0x7fffu; hi += p[r] >> 15; count += on[r]; }
+      for (int r = 0; r < B; ++r) { lo += p[r] & 0x7fffu; hi += p[r] >> 15; count += g[r] >= 0; }
     }
     lo = __reduce_add_sync(FULL, lo); hi = __reduce_add_sync(FULL, hi); count = __reduce_add_sync(FULL, count);
     if (lane == 0 && count) { atomicAdd(&sh.e[d - 1][0], lo); atomicAdd(&sh.e[d - 1][1], hi); atomicAdd(&sh.e[d - 1][2], count); }
