@@ -269,7 +269,7 @@ int sdms_create(const sdms_config* cfg, void* d_workspace, size_t bytes, sdms_ct
   d.w_ctl = (unsigned long long*)(w + lay.w_ctl); d.w_desc = (int4*)(w + lay.w_desc);
   d.w_done = (int*)(w + lay.w_done);
   d.w_tab = (WideSlot*)(w + lay.w_tab); d.w_key = (uint32_t*)(w + lay.w_key); d.w_item = (int32_t*)(w + lay.w_item);
-  d.w_grid = lay.wide_on ? wide_kernel_grid() : 0;   // 0 (also without cooperative launch on this device): one thread block per query
+  d.w_grid = lay.wide_on ? wide_kernel_grid() : 0;   // 0: one thread block per query
   d.w_slots = lay.w_slots;
   d.b_ent = (BeamEnt*)(w + lay.b_ent); d.b_ctl = (unsigned long long*)(w + lay.b_ctl); d.bp_todo = (int32_t*)(w + lay.bp_todo); d.beam_stride = lay.w_slots ? (cfg->max_beams > 0 ? cfg->max_beams : (cfg->search_mode == 2 ? 1 : 0)) : 0;
   ctx->step_fits = step_kernel_fits(d);

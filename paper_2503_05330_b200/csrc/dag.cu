@@ -1084,7 +1084,7 @@ __device__ void dag_walk_warp(const Dev& s, int i, int M, const int32_t* mlist, 
 //          smaller token (PACKED: with alpha = 1 the weight is the sum itself; else weight and token stay apart)
 //   walk   per layer the largest key among the candidates on the current node, four candidates per lane: one warp, and no
 //          barrier, up to 128 candidates; a layer's rows do not depend on the walk and are fetched a layer ahead
-constexpr int kWideFrom = 64;            // matches from which a query of a large prompt goes to the wide pass: 64 here 20 us, there 29-35 us a launch that
+constexpr int kWideFrom = 64;            // matches from which a query of a large prompt goes to the wide pass: 64 here 20 us, there 17-22 us in a launch that
                                          // other queries need anyway; 1000 here 60 us
 constexpr int kWalkMaxCap = 8192;        // most slots of a layer's table
 

@@ -16,7 +16,7 @@
 // What bounds a task: the latency of its chain of shared-memory steps up to a few hundred candidates (8 K cycles), the shared-
 // memory atomics beyond (a layer of 7300 candidates: 55 K cycles, of these 18 K claims and sums, 20 K offers).  The form before
 // (node tables in global memory, five passes with grid barriers between them) took 32 us for one query of 200 matches and
-// D = 16 against 17 + 5 here, 165 against 41 + 9 for one of 8000, and 10 to 25 KB of tables per match, so that 16 prompts of
+// D = 16 against 22 here, 165 against 50 for one of 8000, and 1.3 to 2.6 KB of tables per match, so that 16 prompts of
 // 128 x 4096 tokens, 420 000 matches at k = 1, overran the area and kept one CTA each for their largest queries (1.2 ms).
 // Also measured: a task for all queries above wide_alone() by a cluster of 8 CTAs with the table in distributed shared memory
 // (26 270 matches: 187 us against 250, but 8 times slower than classes as soon as there are tasks for all CTAs, and 3 us for every

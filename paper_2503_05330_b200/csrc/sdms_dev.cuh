@@ -75,7 +75,7 @@ struct Dev {
   // device-wide aggregation of queries with many matches (dag_wide.cu); w_slots = 0: not in use
   unsigned long long* w_ctl;           // [kWideCtlWords] queries registered, slots handed out, tasks handed out, chunks handed out, chunks done
   int4* w_desc;                        // [kMaxWide] query path, matches, first slot, -
-  int* w_done;                         // [kMaxWide] layers of the query that are done; zero between builds
+  int* w_done;                         // [kMaxWide] tasks of the query that are done; zero between builds
   WideSlot* w_tab;                     // [w_slots]
   uint32_t* w_key;                     // [w_slots] token + 1 of the node in the slot, 0 = free
   int32_t* w_item;                     // [w_slots] per (layer, match): slot of the item's token in the layer's table
@@ -84,7 +84,7 @@ struct Dev {
   unsigned long long* b_ctl;           // [4] slots handed out by the beam kernel / by the best-path launch after a build; their CTAs that have reserved
   int32_t beam_stride;                 // continuations kept per node: the context's max_beams, 1 for search mode 2 alone
   int32_t* bp_todo;                    // [P] search mode 2: the path's best path is still to be searched over global tables
-  int32_t w_grid;                      // CTAs of the wide pass (all resident at once)
+  int32_t w_grid;                      // CTAs of the wide pass
   // DAG export of the last build
   int32_t* x_node_tok; int64_t* x_node_S; int32_t* x_node_cnt; int32_t* x_node_count;
   int32_t* x_edge_dst; int64_t* x_edge_S; int32_t* x_edge_cnt; int32_t* x_out_degree;
