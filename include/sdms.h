@@ -108,8 +108,8 @@ typedef struct {
   int32_t  max_beams;            /* largest number of drafts per path that sdms_get_beams will be asked for
                                     (0 = the call is not used; at most SDMS_MAX_BEAMS)               */
   int64_t  wide_table_bytes;     /* workspace set aside for node tables in global memory.  Two users: on
-                                    prompts too large for the single-launch build, queries with more than 64
-                                    matches are aggregated by all SMs together, in 16 * M * D bytes for M
+                                    prompts too large for the single-launch build, queries with more than 32
+                                    (many paths: 64) matches are aggregated by all SMs together, in 16 * M * D bytes for M
                                     matches (12 * M * D above 14336 of them, 7168 with alpha < 1); and
                                     sdms_get_beams (max_beams > 0) and search_mode 2 for paths whose tables
                                     do not fit shared memory, in slots of 40 + 16 * max(max_beams, 1) bytes.

@@ -1084,8 +1084,11 @@ __device__ void dag_walk_warp(const Dev& s, int i, int M, const int32_t* mlist, 
 //          smaller token (PACKED: with alpha = 1 the weight is the sum itself; else weight and token stay apart)
 //   walk   per layer the largest key among the candidates on the current node, four candidates per lane: one warp, and no
 //          barrier, up to 128 candidates; a layer's rows do not depend on the walk and are fetched a layer ahead
-constexpr int kWideFrom = 64;            // matches from which a query of a large prompt goes to the wide pass: 64 here 20 us, there 17-22 us in a launch that
-                                         // other queries need anyway; 1000 here 60 us
+// Matches above which a query of a large prompt goes to the wide pass (there 17-22 us in a launch that other queries need anyway;
+// 1000 here 60 us).  64 here are 20 us, 32 are 10: the length of the launch where all its CTAs run at once (256 x 8192 tokens:
+// 1487 us per session from 64, 1461 from 32; 96 x 3001 with tolerance 1: 585, 570), but out of the way of longer ones where they
+// take turns (16 prompts of 128 x 4096: 3251, 3322).
+__device__ __forceinline__ int wide_from(const Dev& s) { return (int)gridDim.x <= 2 * s.w_grid ? 32 : 64; }
 constexpr int kWalkMaxCap = 8192;        // most slots of a layer's table
 
 struct WalkPlan { int cap, stride, layers; bool packed; };    // slots per table, words per row of items, layers per round
@@ -1657,7 +1660,7 @@ __global__ void __launch_bounds__(kDagThreads, EXPORT ? 1 : 2) dag_kernel(Dev s,
     __syncthreads();
   }
   // more matches than a warp holds: all SMs share the work (the pass that follows this kernel)
-  if (!EXPORT && s.pool == 0 && s.mode != 2 && Mk > kWideFrom && wide_register(s, i, Mk)) return;
+  if (!EXPORT && s.pool == 0 && s.mode != 2 && Mk > wide_from(s) && wide_register(s, i, Mk)) return;
   dag_phase<EXPORT>(s, sm, i, Mk, mlist, sh_len, g * s.N, root, draft_tok, draft_len, draft_score, draft_edge_w);
 }
 

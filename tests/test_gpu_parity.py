@@ -136,7 +136,7 @@ def test_walk_at_the_edges_of_its_forms(M, alpha):
     pair.beams_and_compare(3, paths=[0])              # in shared memory up to 129 of these, lists in the table area for 600, all there for 1500
 
 
-@pytest.mark.parametrize("M,alpha,V", [(65, 1.0, 50), (2048, 0.5, 4000), (2049, 1.0, 4000), (7168, 0.5, 60000), (7169, 0.5, 60000),
+@pytest.mark.parametrize("M,alpha,V", [(32, 1.0, 50), (33, 1.0, 50), (65, 1.0, 50), (2048, 0.5, 4000), (2049, 1.0, 4000), (7168, 0.5, 60000), (7169, 0.5, 60000),
                                        (8193, 1.0, 60000), (14336, 1.0, 60000), (14337, 1.0, 60000), (30000, 1.0, 60000)])
 @pytest.mark.parametrize("mode", [0, 1])
 def test_layer_tasks_at_the_edges_of_their_forms(M, alpha, V, mode):
