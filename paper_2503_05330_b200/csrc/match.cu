@@ -432,7 +432,7 @@ scan_kernel(Dev s, int k, int ctas, int set_slots) {
       }
       const int4* const st4 = reinterpret_cast<const int4*>(sh_stage + stage * TILE);
       const int4 q = st4[threadIdx.x], q2 = st4[kScanThreads + threadIdx.x];   // tokens e0..e0+3 and e0+1024..e0+1027
-      cur.t[0] = q.x; cur.t[1] = q.y; cur.t[2] = q.z; cur.t[3] = q.w;  // beyond the copied bytes: stale, turned down in drain()
+      cur.t[0] = q.x; cur.t[1] = q.y; cur.t[2] = q.z; cur.t[3] = q.w;  // beyond the copied bytes: stale, turned down below (behind the row) and in drain()
       cur2.t[0] = q2.x; cur2.t[1] = q2.y; cur2.t[2] = q2.z; cur2.t[3] = q2.w;
       mbar_arrive(&sh_empty[stage]);                                   // this thread has its tokens; when all have, the stage is refilled
       if (++stage == kStreamStages) { stage = 0; phase ^= 1u; }
@@ -462,7 +462,8 @@ scan_kernel(Dev s, int k, int ctas, int set_slots) {
       any |= (wd[4] | wd[5]) | (wd[6] | wd[7]);
     }
     uint32_t hit = 0u;
-    if (any & 1u) {
+    // (behind the row's end a thread holds no token of it, whatever its words say: an entry from there would name the next row)
+    if ((any & 1u) && t0 + tid4 < s.L) {
 #pragma unroll
       for (int u = 0; u < (STREAM ? 8 : 4); ++u) hit |= (wd[u] & 1u) << u;
     }

@@ -811,6 +811,39 @@ def test_streaming_tile_scan_on_a_store_of_many_tiles():
         assert (pair.g.query_modes() == 2).sum() > G * N // 2
 
 
+@pytest.mark.parametrize("L,V", [(64, 300), (60, 40), (2100, 5000)])
+def test_streaming_tile_scan_with_rows_that_end_inside_a_tile(L, V):
+    # 2048 tokens to a tile, rows of 64, 60 and 2100: what a thread finds behind the end of a row is no token of any row
+    G, N, D = (128, 16, 8) if L < 100 else (4, 200, 8)
+    tokens, lps = synth.small_random(G * N, L, V, 9900 + L)
+    pair = Pair(G, N, L, V, 2, D, match_capacity=400000)
+    lens = (L - 1 - (np.arange(G * N) * 7) % 13).astype(np.int32)
+    pair.append(tokens[:, :L], lps[:, :L], lens, expect_status=0)
+    for k in (1, 2, 1):                                               # (the second build finds the first one's stages)
+        pair.build_and_compare(k, check_dag=False, paths=list(range(0, G * N, 3)))
+    assert (pair.g.query_modes() == 2).any()
+
+
+@pytest.mark.parametrize("L", [1500, 1501, 700])
+def test_tile_scan_of_tokens_that_look_like_no_token(L):
+    # a query whose last token shares its bit of the scan's reject table with "no token" (-1): the rest of a tile behind
+    # the end of a row must not be taken for the start of the next one
+    bit = lambda t: ((t * 2654435761) & 0xffffffff) >> 16  # noqa: E731
+    T = next(t for t in range(1, 200000) if bit(t) == bit(0xffffffff))
+    N, V, D = 5, 200000, 6
+    tokens, lps = synth.small_random(N, L, V, 9950 + L)
+    tokens[tokens == T] = 0
+    tokens[:, 3:600:9] = T                                             # many, at the front of every row
+    lens = (L - 1 - np.arange(N) * 3).astype(np.int32)
+    tokens[np.arange(N), lens - 1] = T                                 # and every query
+    pair = Pair(1, N, L, V, 2, D, match_capacity=N * N * L - 1)
+    pair.append(tokens, lps, lens, expect_status=0)
+    for k in (1, 2):
+        pair.build_and_compare(k, check_dag=False)
+    pair.build_and_compare(1, check_dag=False)
+    assert (pair.g.query_modes() == 2).all()
+
+
 @pytest.mark.parametrize("mode,pool", [(0, 0), (1, 0), (2, 0), (0, 1), (0, 2)])
 def test_search_modes_and_pools_through_the_probe_scan_dag_kernels(mode, pool):
     # match_capacity below P*N*L: the build takes the three-kernel path, where the searches and
