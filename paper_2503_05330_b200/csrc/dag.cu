@@ -1649,9 +1649,10 @@ __global__ void __launch_bounds__(kDagThreads, EXPORT ? 1 : 2) dag_kernel(Dev s,
     if (threadIdx.x == 0) { draft_len[i] = 0; if (used_k) used_k[i] = 0; }
     return;
   }
-  if ((round & kRoundBackoff) && threadIdx.x == 0) { s.q_mode[i] = Q_DONE; if (used_k) used_k[i] = k; }
   const int g = i / s.N;
   __syncthreads();
+  // (after the barrier: a warp that came to its own look at q_mode later would take the path for an earlier round's)
+  if ((round & kRoundBackoff) && threadIdx.x == 0) { s.q_mode[i] = Q_DONE; if (used_k) used_k[i] = k; }
   int32_t* const mlist = s.matches + q_off;
   int Mk = M;
   if (s.R > 0) {                                    // (a second pass over the same build finds nothing left to cut)

@@ -1218,3 +1218,35 @@ def test_a_wait_that_runs_out_sets_the_status_bit_and_leaves_the_context_usable(
     assert pair.g.status() == binding.STATUS_TIMEOUT
     assert pair.g.status() == 0                      # read and cleared
     pair.build_and_compare(1, check_dag=False)       # nothing else has changed
+
+
+def test_backoff_by_rounds_gives_every_path_the_draft_of_its_own_suffix_length():
+    # 2048 paths, one CTA each in every round: a path that finds its matches in a later round must be drafted by its
+    # whole CTA, however far apart its warps run (many builds, each compared with fixed-k builds composed per path)
+    from paper_2503_05330_b200 import binding
+    G, N, L, V, D, k_max = 16, 128, 2048, 90000, 16, 4
+    gen = torch.Generator(device="cuda:0")
+    gen.manual_seed(9820)
+    tokens = torch.randint(0, V, (G * N, L), generator=gen, device="cuda:0", dtype=torch.int32)
+    lps = -torch.rand((G * N, L), generator=gen, device="cuda:0")
+    g = binding.Sdms(G, N, L, V, k_max, D)
+    g.append(tokens, lps, torch.full((G * N,), L - 40, dtype=torch.int32, device="cuda:0"))
+    names = ("draft_tok", "draft_len", "draft_score", "draft_edge_w")
+    want = used = None
+    for k in range(1, k_max + 1):                                      # the longest k with a match decides
+        g.build_drafts(k)
+        off, _ = g.matches()
+        found = torch.from_numpy(np.diff(off.numpy()) > 0).to(g.device)
+        got = [getattr(g, n).clone() for n in names]
+        want = got if want is None else [torch.where(found[:, None] if x.dim() == 2 else found, x, y) for x, y in zip(got, want)]
+        used = torch.where(found, k, 0 if used is None else used)
+    assert g.status() == 0 and (used == 1).sum() > 1000
+    evict = torch.zeros(64 << 20, dtype=torch.int32, device="cuda:0")  # (histories out of the cache: loads take longer)
+    for _ in range(60):
+        evict += 1
+        g.build_drafts_backoff(k_max)
+        assert torch.equal(g.used_k, used)
+        for n, w in zip(names, want):
+            wrong = (getattr(g, n) != w).view(g.P, -1).any(1).nonzero().flatten()
+            assert len(wrong) == 0, (n, wrong[:8].tolist())
+    assert g.status() == 0
