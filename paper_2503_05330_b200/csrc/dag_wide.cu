@@ -111,6 +111,8 @@ __device__ __forceinline__ u64 wide_weight(const Dev& s, const WideTable& t, int
   const u64 S = ((u64)t.hi[h] << 15) + t.lo[h];
   return counts ? (u64)__double_as_longlong(eq5_weight(s.alpha, S, t.cnt[h])) : S;
 }
+// (The match list is read past L1 throughout: the kernel before this one still cuts it down in place, with a cap on the
+// matches per path, while CTAs of this one are resident.  Tokens, probabilities and lengths are older and go through __ldg.)
 // Entries m0, m0 + kWideThreads, ... of a row (`none` where there is no candidate).
 template <int N>
 __device__ __forceinline__ void wide_row(const int* row, int M, int m0, int none, int (&v)[N]) {
@@ -133,7 +135,7 @@ __device__ __forceinline__ void wide_lay_out(const Dev& s, const int4 de, int c0
   const int M = de.y, m = c0 + threadIdx.x;
   if (m >= M) return;
   const WideItems items = wide_items(s, de.z, M);
-  const int g = __ldg(s.matches + s.q_off[de.x] + m), j = path_of(s, g);
+  const int g = __ldcg(s.matches + s.q_off[de.x] + m), j = path_of(s, g);
   const int n = min(s.D, __ldg(s.len + j) - 1 - (g - j * s.L));        // followers
   const int off = (g + 1) & 3;
   const int4* const st = reinterpret_cast<const int4*>(s.tok) + ((g + 1) >> 2);
@@ -296,7 +298,7 @@ __device__ __forceinline__ void wide_layer(const Dev& s, const int4 de, int d) {
       for (int r = 0; r < N; ++r)
         if (best >> (c * N + r) & 1u) {
           const int m = (c * N + r) * kWideThreads + tid;
-          const unsigned q = (unsigned)(KEEP ? __ldcg(row_p + m) : __ldg(s.pq + __ldg(list + m) + d));
+          const unsigned q = (unsigned)(KEEP ? __ldcg(row_p + m) : __ldg(s.pq + __ldcg(list + m) + d));
           if (single) { lo += q & 0x7fffu; hi += q >> 15; }
           else {
             atomicAdd(&t.lo[slot[c][r]], q & 0x7fffu);
@@ -372,7 +374,7 @@ __device__ __forceinline__ void wide_sums(const Dev& s, const int4 de, int d, un
         if ((wide_class(v[r]) & others) != mine) v[r] = -1;
       // (from the store: other classes write their weights over the row of probabilities)
 #pragma unroll
-      for (int r = 0; r < N; ++r) p[r] = v[r] >= 0 ? (unsigned)__ldg(list + m0 + r * kWideThreads) : 0u;
+      for (int r = 0; r < N; ++r) p[r] = v[r] >= 0 ? (unsigned)__ldcg(list + m0 + r * kWideThreads) : 0u;
 #pragma unroll
       for (int r = 0; r < N; ++r) p[r] = v[r] >= 0 ? (unsigned)__ldg(s.pq + (int)p[r] + d) : 0u;
 #pragma unroll
@@ -521,7 +523,7 @@ __device__ __forceinline__ void wide_walk_rows(const Dev& s, const int4 de, cons
       for (int r = 0; r < B; ++r) {
         // (layer-wise search looks at all candidates, but the edge is from the node before)
         const bool on = t[r] == tok && (!all || d == 1 || __ldcg(before + m[r]) == cur);
-        g[r] = on ? __ldg(list + m[r]) : -1;
+        g[r] = on ? __ldcg(list + m[r]) : -1;
       }
 #pragma unroll
       for (int r = 0; r < B; ++r) p[r] = g[r] >= 0 ? (unsigned)__ldg(s.pq + g[r] + d) : 0u;
@@ -561,7 +563,7 @@ __device__ __forceinline__ void wide_walk_known(const Dev& s, const int4 de, con
     if (tid < D) { const int at = __ldcg(items.succ + (size_t)tid * items.pitch); if (at >= 0) sh_draft[tid] = __ldcg(items.tok + (size_t)tid * items.pitch + at); }
     __syncthreads();
     for (int m = tid; m < M; m += kWideThreads) {
-      const int g = __ldg(list + m), j = path_of(s, g), n = min(D, __ldg(s.len + j) - 1 - (g - j * s.L));
+      const int g = __ldcg(list + m), j = path_of(s, g), n = min(D, __ldg(s.len + j) - 1 - (g - j * s.L));
       bool on = true;                                  // this candidate is on the draft's node so far
       for (int l = 0; l < n && sh_draft[l] >= 0; ++l) {
         const bool here = __ldg(s.tok + g + l + 1) == sh_draft[l];

@@ -943,6 +943,19 @@ def test_match_cap_config5_heavy_queries(R):
         assert np.diff(off.numpy()).max() <= (w.N - 1) * R
 
 
+@pytest.mark.parametrize("R,alpha,mode", [(5, 1.0, 0), (9, 0.5, 0), (5, 1.0, 1)])
+def test_match_cap_leaves_hundreds_of_matches_to_the_wide_pass(R, alpha, mode):
+    # dag_kernel cuts every list down in place just before the wide pass reads it; neighbouring lists share cache lines
+    N, L, V, D = 40, 4096, 60, 8
+    tokens, lps = synth.small_random(N, L, V, 8890 + R)
+    pair = Pair(1, N, L, V, 2, D, alpha=alpha, mode=mode, max_matches=R)
+    pair.append(tokens[:, :4000], lps[:, :4000], (4000 - np.arange(N) * 7).astype(np.int32), expect_status=0)
+    for k in (1, 2, 1, 1):
+        pair.build_and_compare(k, check_dag=False)
+    off, _ = pair.g.matches()
+    assert (np.diff(off.numpy()) == (N - 1) * R).all()
+
+
 def test_match_cap_on_the_three_kernel_path_with_more_matches_than_the_cap_in_every_path():
     G, N, L, V, D = 1, 12, 1024, 2, 3
     tokens, lps = synth.small_random(G * N, L, V, 4243)
