@@ -76,7 +76,10 @@ __global__ void __launch_bounds__(kFzThreads) fuzzy_scan_kernel(Dev s, int k, in
   const int j = blockIdx.x / tiles, t0 = (blockIdx.x - j * tiles) * kFzTile;
   const int g = j / s.N, len_j = s.len[j];
   const int e_hi = min(t0 + kFzTile - 1, len_j - 2);        // last position of the tile with a follower
-  if (t0 > e_hi) return;
+  if (t0 > e_hi) {                                         // nothing to scan; but a launch none of whose CTAs waited would be over before
+    grid_wait();                                           // the kernel in front of it, and the one behind would not wait for that
+    return;
+  }
   const int32_t* row = s.tok + (size_t)j * s.L;
   for (int x = tid; x < kFzHalo + kFzTile; x += blockDim.x) {
     const int at = t0 - kFzHalo + x;

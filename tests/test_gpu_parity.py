@@ -369,6 +369,21 @@ def test_fuzzy_on_a_prompt_too_large_for_the_single_launch_build():
     assert np.diff(off.numpy()).max() > 32
 
 
+def test_fuzzy_on_a_large_prompt_of_short_paths():
+    # no path has a position with a follower, so no CTA of the two scans has anything to do: the launches still come one
+    # after the other, and what an earlier build left is gone
+    G, N, L, V, D = 1, 40, 4096, 60, 6
+    tokens, lps = synth.small_random(G * N, L, V, 9811)
+    pair = Pair(G, N, L, V, 3, D, eps=1)
+    lens = (300 - (np.arange(N) * 3)).astype(np.int32)
+    pair.append(tokens[:, :300], lps[:, :300], lens, expect_status=0)
+    pair.build_and_compare(2, check_dag=False)
+    for have in (0, 1):
+        pair.trim(np.full(N, have, np.int32))
+        for k in (1, 2):
+            pair.build_and_compare(k, check_dag=False)
+
+
 def test_fuzzy_config5():
     # the paper's experimental setting (tolerance 1) on the largest workload; the oracle's edit-distance search of
     # 2M positions per query is slow, so a handful of paths are compared
