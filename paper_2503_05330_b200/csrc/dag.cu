@@ -1628,11 +1628,12 @@ __global__ void __launch_bounds__(kDagThreads, EXPORT ? 1 : 2) dag_kernel(Dev s,
   const Smem sm = carve<EXPORT>(smem_raw);
   __shared__ int32_t sh_len[SDMS_MAX_PATHS_PER_GROUP];
   const int i = blockIdx.x;
-  // the path lengths are older than the kernels this one follows (probe, scan: their CTAs let it start only after
-  // their own wait): fetched while those drain
+  // in a build the path lengths are older than the kernels this one follows (probe, scan: their CTAs let it start only
+  // after their own wait): fetched while those drain.  The export follows any call, a step that still commits included
+  if (EXPORT) grid_wait();
   for (int n = threadIdx.x; n < s.N; n += blockDim.x) sh_len[n] = ldm(s.len + (i / s.N) * s.N + n);
   const int32_t root = ldm(s.rec + (size_t)i * kRecWords + 1);
-  grid_wait();
+  if (!EXPORT) grid_wait();
   grid_release();
   // what probe and scan left for this path, in one round trip
   const int32_t q_mode = s.q_mode[i];

@@ -598,6 +598,33 @@ def test_step_falls_back_to_separate_launches_for_wide_prompts():
 
 
 # ---- best-path search (search mode 2) --------------------------------------------------------
+def test_dag_export_right_behind_a_step_sees_what_the_step_committed():
+    # both calls are queued behind a busy device, so that the export is launched while the step still commits
+    from paper_2503_05330_b200 import binding
+    G, N, L, V, D = 1, 12, 96, 3, 6
+    tokens, lps = synth.small_random(G * N, L, V, 5150)
+    pair = Pair(G, N, L, V, 2, D, B=4, Ke=3)
+    pair.append(tokens[:, :20], lps[:, :20], np.full(N, 20, np.int32), expect_status=0)
+    pair.build_and_compare(1, check_dag=False)
+    assert pair.g.step_is_single_launch()
+    out = pair.g.dag_device()
+    order = ("node_tok", "node_S", "node_cnt", "node_count", "edge_dst", "edge_S", "edge_cnt", "out_degree")
+    for step in range(10):
+        lens = pair.o.lengths()
+        sampled, sampled_lp = synth.sampled_window(tokens, lps, lens, D + 1)
+        tok, ln, _, _ = pair.o.drafts()
+        pair.o.accept_commit(tok, ln, sampled, sampled_lp, pair.max_append)
+        pair.o.build_all(2)
+        sampled, sampled_lp = t32(sampled, pair.dev), t32(sampled_lp, pair.dev)
+        torch.cuda._sleep(2000000)
+        pair.g.step(2, sampled, sampled_lp)
+        binding.sdms_get_dag(pair.g.ctx, *(out[n] for n in order))
+        assert pair.g.status() == 0
+        for i in range(N):
+            for key, want in pair.o.export(i, 4, 3).items():
+                assert np.array_equal(out[key][i].cpu().numpy(), want), (step, i, key)
+
+
 @pytest.mark.parametrize("seed", range(4))
 @pytest.mark.parametrize("alpha,eps", [(1.0, 0), (0.5, 0), (0.0, 0), (1.0, 1)])
 def test_best_path_dense_small_vocab_every_step(seed, alpha, eps):
