@@ -97,7 +97,7 @@ Layout make_layout(const sdms_config* c) {
   }
   l.w_slots = (l.wide_on || (stride > 0 && wide > 0)) ? (uint64_t)wide / slot_bytes : 0;
   l.w_ctl = take((size_t)kWideCtlWords * 8);
-  l.b_ctl = take(32);
+  l.b_ctl = take(kBeamCtlWords * 8);
   l.bp_todo = take(P * 4);
   l.w_desc = take(l.wide_on ? (size_t)kMaxWide * 16 : 0);
   l.w_done = take(l.wide_on ? (size_t)kMaxWide * 4 : 0);
@@ -165,8 +165,8 @@ int drain_pending(sdms_ctx* ctx, size_t count) {
   return SDMS_OK;
 }
 
-// A best-path build marks the paths with more matches than its shared-memory search takes; this launch
-// searches them over node tables in the workspace's table area and replaces their (greedy) drafts.
+// A best-path build lists the paths with more matches than its shared-memory search takes; this launch
+// searches them, if need be over node tables in the workspace's table area, and replaces their (greedy) drafts.
 // Other contexts: nothing.
 int finish_best_paths(sdms_ctx* ctx, int32_t* draft_tok, int32_t* draft_len, float* draft_score, float* draft_edge_w,
                       cudaStream_t stream) {

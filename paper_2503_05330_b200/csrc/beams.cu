@@ -1,6 +1,6 @@
 // sdms_get_beams: several drafts per path.  One CTA per query path works out the B best paths of the
-// pool of the last build (beam_dev.cuh) over node tables that it reserves in the workspace's table
-// area and leaves empty again.
+// pool of the last build (beam_dev.cuh), in shared memory where its tables fit, else over node
+// tables that it reserves in the workspace's table area and leaves empty again.
 #include "sdms_internal.h"
 #include "beam_dev.cuh"
 
@@ -8,15 +8,42 @@ namespace sdms {
 
 namespace {
 
-constexpr int kBeamSmem = 200 * 1024;                 // shared memory of a CTA: one per SM
+// Shared memory of a CTA (one per SM).  Tables and lists want as much as there is, the form over the table area wants L1, and one
+// launch has both.  An SM splits its 256 KB at 164, 196 and 228 KB, so each size is what just fits below a step: 160 KB for one
+// beam, whose lists are short, 192 KB for more.  Pools of 944 and 26 236 matches, D = 16, one beam: 499 us and 12.6 ms with 200 KB
+// (28 KB of L1), 331 us and 8.7 ms with 160, 303 us and 8.7 ms with none; pools of up to 117, D = 8, four beams: 45 us with 192,
+// 59 with 160 (no room for the lists), 306 with none.  A launch for each form: side by side or not, the SMs keep the split of
+// the launch before (320 us for 203 on 32 prompts of 16 x 1024, k = 1).
+constexpr int kBeamSmem = 192 * 1024, kBeamSmemOne = 160 * 1024;
+inline int beam_smem(int B) { return B > 1 ? kBeamSmem : kBeamSmemOne; }
 
-// Called by one thread of every CTA once its slots are reserved: the last one leaves the count of reserved slots at zero.
-__device__ __forceinline__ void reserved(unsigned long long* slots, unsigned long long* done) {
-  __threadfence();
-  if (atomicAdd(done, 1ull) == gridDim.x - 1) { *slots = 0ull; *done = 0ull; }
+// First slot of the tables of a path with M matches in the table area, -1: no room.  By one thread.
+__device__ __forceinline__ long long reserve_tables(const Dev& s, int M) {
+  if (M <= 0 || M > kWideMaxMatches) return -1;
+  const unsigned long long need = (unsigned long long)s.D << beam_lcap(M);
+  const unsigned long long at = atomicAdd(&s.b_ctl[kBeamSlots], need);
+  return at + need <= s.w_slots ? (long long)at : -1;
 }
 
-__global__ void __launch_bounds__(kWideThreads, 1) beam_kernel(Dev s, int B, int32_t* __restrict__ beam_tok,
+// The beams of path i, in `bytes` of shared memory if they fit.  (The room in the table area decides who is served, also then.)
+__device__ __forceinline__ void beams_of_path(const Dev& s, unsigned bytes, int i, int M, long long first, int B, int32_t* tok, int32_t* len,
+                                              float* value, bool want0 = false, float* score0 = nullptr, float* edge0 = nullptr) {
+  const BeamPlan w = beam_plan(M, s.D, B, bytes);
+  BeamEnt* const ent = s.b_ent + (size_t)(unsigned)first * s.beam_stride;
+  const int32_t* const list = s.matches + s.q_off[i];
+  if (!w.cap) beams_of_query(s, i, M, list, (unsigned)first, beam_lcap(M), B, tok, len, value, want0, score0, edge0);
+  else if (w.lists) beams_in_shared<true>(s, w, M, list, B, ent, s.beam_stride, tok, len, value, want0, score0, edge0);
+  else beams_in_shared<false>(s, w, M, list, B, ent, s.beam_stride, tok, len, value, want0, score0, edge0);
+}
+
+// The launch's last CTA leaves all counts at zero.  By one thread of each, once it has its last slots and tickets.
+__device__ __forceinline__ void beam_counts_done(const Dev& s) {
+  __threadfence();
+  if (atomicAdd(&s.b_ctl[kBeamDone], 1ull) == gridDim.x - 1)
+    s.b_ctl[kBeamSlots] = s.b_ctl[kBeamTodo] = s.b_ctl[kBeamTicket] = s.b_ctl[kBeamDone] = 0ull;
+}
+
+__global__ void __launch_bounds__(kWideThreads, 1) beam_kernel(Dev s, int B, unsigned bytes, int32_t* __restrict__ beam_tok,
                                                                int32_t* __restrict__ beam_len,
                                                                float* __restrict__ beam_value) {
   grid_wait();
@@ -25,19 +52,10 @@ __global__ void __launch_bounds__(kWideThreads, 1) beam_kernel(Dev s, int B, int
   const int i = blockIdx.x, tid = threadIdx.x, D = s.D;
   int32_t* const my_tok = beam_tok + (size_t)i * B * D;
   const int M = s.q_mode[i] == Q_NONE ? 0 : min(s.q_cursor[i], s.q_reserved[i]);
-  const int lcap = beam_lcap(M);
   if (tid == 0) {
-    long long first = -1;
-    if (M > 0 && M <= kWideMaxMatches) {
-      const unsigned long long need = (unsigned long long)D << lcap;
-      const unsigned long long at = atomicAdd(s.b_ctl, need);
-      if (at + need <= s.w_slots) first = (long long)at;
-      else atomicOr(s.status, SDMS_STATUS_TABLES_FULL);
-    } else if (M > 0) {
-      atomicOr(s.status, SDMS_STATUS_TABLES_FULL);
-    }
-    sh_first = first;
-    reserved(s.b_ctl, s.b_ctl + 2);
+    sh_first = reserve_tables(s, M);
+    if (M > 0 && sh_first < 0) atomicOr(s.status, SDMS_STATUS_TABLES_FULL);
+    beam_counts_done(s);
   }
   __syncthreads();
   if (sh_first < 0) {                                  // no match, or no room: no beam
@@ -45,20 +63,13 @@ __global__ void __launch_bounds__(kWideThreads, 1) beam_kernel(Dev s, int B, int
     if (tid < B) { beam_len[(size_t)i * B + tid] = 0; beam_value[(size_t)i * B + tid] = 0.0f; }
     return;
   }
-  // (the room in the table area decides who is served, also where the work is done in shared memory)
-  const BeamPlan w = beam_plan(M, D, B, kBeamSmem);
-  if (w.cap) {
-    BeamEnt* const ent = s.b_ent + (size_t)(unsigned)sh_first * s.beam_stride;
-    if (w.lists) beams_in_shared<true>(s, w, M, s.matches + s.q_off[i], B, ent, s.beam_stride, my_tok, beam_len + (size_t)i * B, beam_value + (size_t)i * B);
-    else beams_in_shared<false>(s, w, M, s.matches + s.q_off[i], B, ent, s.beam_stride, my_tok, beam_len + (size_t)i * B, beam_value + (size_t)i * B);
-    return;
-  }
-  beams_of_query(s, i, M, s.matches + s.q_off[i], (unsigned)sh_first, lcap, B, my_tok, beam_len + (size_t)i * B,
-                 beam_value + (size_t)i * B);
+  beams_of_path(s, bytes, i, M, sh_first, B, my_tok, beam_len + (size_t)i * B, beam_value + (size_t)i * B);
 }
 
-// After a build with search mode 2: the paths that the build marked (more matches than its shared-memory
-// search takes) get their best path here, in place of the greedy draft the build left them.
+// Search mode 2: the paths that the build could not search in shared memory (dag_phase lists them in
+// bp_todo) get their best path: the first beam of their pool, with scores and edge weights, in place of
+// the greedy draft.  The CTAs take the listed paths in turn (one for each path of the context: 2048 of them, mostly with
+// nothing to do, took 20 us).
 __global__ void __launch_bounds__(kWideThreads, 1) best_path_fix_kernel(Dev s, int32_t* __restrict__ draft_tok,
                                                                         int32_t* __restrict__ draft_len,
                                                                         float* __restrict__ draft_score,
@@ -66,40 +77,28 @@ __global__ void __launch_bounds__(kWideThreads, 1) best_path_fix_kernel(Dev s, i
   grid_wait();
   grid_release();
   __shared__ long long sh_first;
+  __shared__ int sh_next;
   __shared__ float sh_value;
-  const int i = blockIdx.x, tid = threadIdx.x, D = s.D;
-  const bool mine = s.bp_todo[i] != 0;
-  __syncthreads();
-  const int M = min(s.q_cursor[i], s.q_reserved[i]);
-  const int lcap = beam_lcap(M);
-  if (tid == 0) {
-    long long first = -1;
-    if (mine) {
-      s.bp_todo[i] = 0;
-      if (M > 0 && M <= kWideMaxMatches) {
-        const unsigned long long need = (unsigned long long)D << lcap;
-        const unsigned long long at = atomicAdd(s.b_ctl + 1, need);
-        if (at + need <= s.w_slots) first = (long long)at;
-      }
-      if (first < 0) atomicOr(s.status, SDMS_STATUS_SEARCH_FALLBACK);     // the greedy draft stays
+  const int tid = threadIdx.x, D = s.D;
+  const int todo = (int)min(__ldcg(&s.b_ctl[kBeamTodo]), (unsigned long long)s.P);
+#pragma unroll 1
+  for (int x = blockIdx.x; x < todo;) {
+    const int i = s.bp_todo[x];
+    const int M = min(s.q_cursor[i], s.q_reserved[i]);
+    if (tid == 0) {
+      sh_first = reserve_tables(s, M);
+      if (sh_first < 0) atomicOr(s.status, SDMS_STATUS_SEARCH_FALLBACK);       // the greedy draft stays
+      sh_next = (int)(gridDim.x + atomicAdd(&s.b_ctl[kBeamTicket], 1ull));
     }
-    sh_first = first;
-    reserved(s.b_ctl + 1, s.b_ctl + 3);
+    __syncthreads();
+    const long long first = sh_first;
+    x = sh_next;
+    if (first >= 0)
+      beams_of_path(s, kBeamSmemOne, i, M, first, 1, draft_tok + (size_t)i * D, draft_len + i, &sh_value, true,
+                    draft_score ? draft_score + (size_t)i * D : nullptr, draft_edge_w ? draft_edge_w + (size_t)i * D : nullptr);
+    __syncthreads();                                   // before the next path's tables
   }
-  __syncthreads();
-  if (sh_first < 0) return;
-  const BeamPlan w = beam_plan(M, D, 1, kBeamSmem);
-  if (w.cap) {
-    BeamEnt* const ent = s.b_ent + (size_t)(unsigned)sh_first * s.beam_stride;
-    float* const score = draft_score ? draft_score + (size_t)i * D : nullptr;
-    float* const edge = draft_edge_w ? draft_edge_w + (size_t)i * D : nullptr;
-    if (w.lists) beams_in_shared<true>(s, w, M, s.matches + s.q_off[i], 1, ent, s.beam_stride, draft_tok + (size_t)i * D, draft_len + i, &sh_value, true, score, edge);
-    else beams_in_shared<false>(s, w, M, s.matches + s.q_off[i], 1, ent, s.beam_stride, draft_tok + (size_t)i * D, draft_len + i, &sh_value, true, score, edge);
-    return;
-  }
-  beams_of_query(s, i, M, s.matches + s.q_off[i], (unsigned)sh_first, lcap, 1, draft_tok + (size_t)i * D, draft_len + i,
-                 &sh_value, true, draft_score ? draft_score + (size_t)i * D : nullptr,
-                 draft_edge_w ? draft_edge_w + (size_t)i * D : nullptr);
+  if (tid == 0) beam_counts_done(s);
 }
 
 }  // namespace
@@ -107,18 +106,19 @@ __global__ void __launch_bounds__(kWideThreads, 1) best_path_fix_kernel(Dev s, i
 // Called when a context is created, with its device current.
 cudaError_t beam_kernel_setup() {
   const cudaError_t e = cudaFuncSetAttribute(beam_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kBeamSmem);
-  return e != cudaSuccess ? e : cudaFuncSetAttribute(best_path_fix_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kBeamSmem);
+  return e != cudaSuccess ? e : cudaFuncSetAttribute(best_path_fix_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kBeamSmemOne);
 }
 
 cudaError_t launch_best_path_fix(const Dev& s, int32_t* draft_tok, int32_t* draft_len, float* draft_score,
                                  float* draft_edge_w, cudaStream_t stream) {
-  return launch_overlapped(best_path_fix_kernel, dim3(s.P), dim3(kWideThreads), kBeamSmem, stream, s, draft_tok, draft_len,
-                           draft_score, draft_edge_w);
+  return launch_overlapped(best_path_fix_kernel, dim3((unsigned)(s.P < 148 ? s.P : 148)), dim3(kWideThreads), kBeamSmemOne, stream, s,
+                           draft_tok, draft_len, draft_score, draft_edge_w);
 }
 
 cudaError_t launch_beams(const Dev& s, int B, int32_t* beam_tok, int32_t* beam_len, float* beam_value,
                          cudaStream_t stream) {
-  return launch_overlapped(beam_kernel, dim3(s.P), dim3(kWideThreads), kBeamSmem, stream, s, B, beam_tok, beam_len, beam_value);
+  return launch_overlapped(beam_kernel, dim3(s.P), dim3(kWideThreads), beam_smem(B), stream, s, B, (unsigned)beam_smem(B), beam_tok,
+                           beam_len, beam_value);
 }
 
 }  // namespace sdms

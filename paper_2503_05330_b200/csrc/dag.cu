@@ -1590,11 +1590,14 @@ __device__ __forceinline__ void dag_phase(const Dev& s, const Smem& sm, int i, i
       dag_best_path(s, sm, i, M, cap, mlist, plen, poff, draft_tok, draft_len, draft_score, draft_edge_w);
       return;
     }
-    // too many matches for tables in shared memory: the path gets the greedy draft for now and is marked; the
-    // launch that follows a best-path build (beams.cu) searches the marked paths over node tables in the
-    // workspace's table area and replaces their drafts.  Without a table area the greedy draft stays, and says so.
+    // too many matches for tables in shared memory: the path gets the greedy draft for now and is listed; the
+    // launch that follows a best-path build (beams.cu) searches the listed paths, if need be over node tables in the
+    // workspace's table area, and replaces their drafts.  Without a table area the greedy draft stays, and says so.
     if (s.beam_stride > 0) {
-      if (threadIdx.x == 0) s.bp_todo[i] = 1;
+      if (threadIdx.x == 0) {
+        const unsigned long long at = atomicAdd(&s.b_ctl[kBeamTodo], 1ull);
+        if (at < (unsigned long long)s.P) s.bp_todo[at] = i;           // (a count left by a launch that failed)
+      }
     } else if (threadIdx.x == 0) {
       atomicOr(s.status, SDMS_STATUS_SEARCH_FALLBACK);
     }

@@ -49,7 +49,7 @@ __device__ __forceinline__ bool wait_for_count(const u64* ctr, u64 target, long 
 
 // sdms_debug_wait_timeout: a bounded wait on a count that nobody raises.
 __global__ void wait_timeout_kernel(Dev s, long long cycles) {
-  if (threadIdx.x == 0 && !wait_for_count(s.b_ctl + 1, ~0ull, cycles)) atomicOr(s.status, SDMS_STATUS_TIMEOUT);
+  if (threadIdx.x == 0 && !wait_for_count(s.b_ctl + kBeamNever, ~0ull, cycles)) atomicOr(s.status, SDMS_STATUS_TIMEOUT);
 }
 
 // What is kept for a query, in rows of `pitch` entries, one for every layer:

@@ -23,6 +23,8 @@ constexpr int kMaxWide = 1024;          // queries one build can hand to the dev
 constexpr int kWideSumShift = 47;       // packed node sums: count in the upper 17 bits, sum of probabilities below
 constexpr int kWideMaxMatches = (1 << 17) - 1;   // so that both parts of a packed sum fit
 constexpr int kWideCtlWords = 5;
+// b_ctl: table slots handed out, a count that stays zero (sdms_debug_wait_timeout waits for it), paths in bp_todo, paths dealt out, CTAs done
+enum BeamCtl : int { kBeamSlots = 0, kBeamNever = 1, kBeamTodo = 2, kBeamTicket = 3, kBeamDone = 4, kBeamCtlWords = 8 };
 
 // Q_DONE: a back-off build on a large prompt has found this path's matches at a longer suffix length
 enum QueryMode : int32_t { Q_NONE = 0, Q_INLINE = 1, Q_SCAN = 2, Q_DONE = 3 };
@@ -81,9 +83,9 @@ struct Dev {
   int32_t* w_item;                     // [w_slots] per (layer, match): slot of the item's token in the layer's table
   unsigned long long w_slots;
   BeamEnt* b_ent;                      // [w_slots][beam_stride] continuations kept per node (sdms_get_beams)
-  unsigned long long* b_ctl;           // [4] slots handed out by the beam kernel / by the best-path launch after a build; their CTAs that have reserved
+  unsigned long long* b_ctl;           // [kBeamCtlWords] counts of the beam kernels, all zero between calls
   int32_t beam_stride;                 // continuations kept per node: the context's max_beams, 1 for search mode 2 alone
-  int32_t* bp_todo;                    // [P] search mode 2: the path's best path is still to be searched over global tables
+  int32_t* bp_todo;                    // [P] search mode 2: paths whose best path is still to be searched, in no particular order
   int32_t w_grid;                      // CTAs of the wide pass
   // DAG export of the last build
   int32_t* x_node_tok; int64_t* x_node_S; int32_t* x_node_cnt; int32_t* x_node_count;

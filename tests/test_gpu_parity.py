@@ -1125,6 +1125,25 @@ def test_beams_on_benchmark_workloads(wid, k):
     pair.beams_and_compare(1, paths=sample)
 
 
+@pytest.mark.parametrize("alpha", [1.0, 0.5])
+def test_beams_of_pools_on_both_sides_of_what_shared_memory_holds(alpha):
+    # D = 8: a node table of a layer has 1024 slots up to 818 matches (fits), 2048 above (does not); both kinds in one call,
+    # calls one after the other, and the same pools by best-path search
+    G, N, L, V, D = 1, 12, 1024, 12, 8
+    tokens, lps = synth.small_random(G * N, L, V, 6500)
+    pair = Pair(G, N, L, V, 2, D, alpha=alpha, mode=2, max_beams=4)
+    lens = (1000 - (np.arange(N) * 41) % 300).astype(np.int32)
+    pair.append(tokens[:, :1000], lps[:, :1000], lens, expect_status=0)
+    for k in (1, 2, 1):
+        pair.build_and_compare(k, check_dag=False)
+        off, _ = pair.g.matches()
+        if k == 1:
+            m = np.diff(off.numpy())
+            assert (m > 818).any() and (m <= 818).any(), m
+        for B in (1, 4, 1):
+            pair.beams_and_compare(B)
+
+
 def test_beams_need_room_and_a_build():
     from paper_2503_05330_b200 import binding
     G, N, L, V, D = 1, 6, 64, 3, 4
