@@ -130,33 +130,39 @@ __device__ __forceinline__ int4 shifted(int4 a, int4 b, int off) {      // words
   if (off & 1) { a.x = a.y; a.y = a.z; a.z = a.w; a.w = b.x; }
   return a;
 }
-// Candidates c0 .. c0 + kWideThreads of a query.
-__device__ __forceinline__ void wide_lay_out(const Dev& s, const int4 de, int c0) {
+// Candidates c0 .. c0 + kWideThreads of a query, their followers l0 .. l1 (a multiple of 4 each, or D).  The loads of 16 layers go out
+// together: one after the other they were 32 K cycles out of a cold cache, for 13 chunks of a few hundred candidates.
+__device__ __forceinline__ void wide_lay_out(const Dev& s, const int4 de, int c0, int l0, int l1) {
   const int M = de.y, m = c0 + threadIdx.x;
   if (m >= M) return;
   const WideItems items = wide_items(s, de.z, M);
   const int g = __ldcg(s.matches + s.q_off[de.x] + m), j = path_of(s, g);
-  const int n = min(s.D, __ldg(s.len + j) - 1 - (g - j * s.L));        // followers
+  const int n = min(l1, __ldg(s.len + j) - 1 - (g - j * s.L));         // followers
   const int off = (g + 1) & 3;
   const int4* const st = reinterpret_cast<const int4*>(s.tok) + ((g + 1) >> 2);
   const int4* const sp = reinterpret_cast<const int4*>(s.pq) + ((g + 1) >> 2);
-  int4 a = make_int4(0, 0, 0, 0), b = a, c = a, e = a;                 // 16 bytes of tokens and the next 16, the same of probabilities
-  if (n > 0) { a = __ldg(st); c = __ldg(sp); }
-  int* tok = items.tok + m;
-  int* p = reinterpret_cast<int*>(items.out) + m;
-#pragma unroll 4
-  for (int x = 1; 4 * x - 4 < s.D; ++x) {
-    const int l = 4 * x - 4;
-    if (4 * x - off < n) { b = __ldg(st + x); e = __ldg(sp + x); }     // (only what holds a follower)
-    const int4 v = shifted(a, b, off), q = shifted(c, e, off);
-    a = b; c = e;
-    const int vs[4] = {v.x, v.y, v.z, v.w}, ps[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll 1
+  for (int lb = l0; lb < l1; lb += 16) {
+    int4 a[5], c[5];                                                   // 16 bytes each of tokens and probabilities
 #pragma unroll
-    for (int y = 0; y < 4; ++y)
-      if (l + y < s.D) {
-        *tok = l + y < n ? vs[y] : -1; *p = ps[y];
+    for (int x = 0; x < 5; ++x) {
+      a[x] = make_int4(0, 0, 0, 0); c[x] = a[x];
+      const int at = lb + 4 * x - off;                                 // the first follower in them
+      if (at < n && at < lb + 16) { a[x] = __ldg(st + (lb >> 2) + x); c[x] = __ldg(sp + (lb >> 2) + x); }   // (only what holds a follower)
+    }
+    int* tok = items.tok + (size_t)lb * items.pitch + m;
+    int* p = reinterpret_cast<int*>(items.out + (size_t)lb * items.pitch) + m;
+#pragma unroll
+    for (int x = 0; x < 4; ++x) {
+      const int4 v = shifted(a[x], a[x + 1], off), q = shifted(c[x], c[x + 1], off);
+      const int vs[4] = {v.x, v.y, v.z, v.w}, ps[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+      for (int y = 0; y < 4; ++y) {
+        const int l = lb + 4 * x + y;
+        if (l < l1) { *tok = l < n ? vs[y] : -1; *p = ps[y]; }
         tok += items.pitch; p += 2 * items.pitch;
       }
+    }
   }
 }
 
@@ -173,8 +179,11 @@ __device__ __forceinline__ void wide_layer(const Dev& s, const int4 de, int d) {
   const int* const row = items.tok + (size_t)(d - 1) * items.pitch;
   const int* const row_p = reinterpret_cast<const int*>(weight);
   const bool counts = s.alpha != 1.0;                  // with alpha = 1 a weight does not depend on the count
+  // At most half full where there is room for that, in any case 7/8: a CTA waits for its unluckiest lane's probe sequence (a layer
+  // of 862 candidates: 47 to 58 K cycles in 1024 slots, 16 K in 2048).
+  const int most = counts ? kWideSlots / 2 : kWideSlots;
   int cap = 64;
-  while (7 * cap < 8 * M) cap *= 2;
+  while (cap < 2 * M && cap < most) cap *= 2;
   const WideTable t = wide_table(wide_smem, cap);
   int v[N], p[N];
   wide_row<N>(row, M, tid, -1, v);                     // on its way while the table is emptied
@@ -707,15 +716,19 @@ dag_wide_kernel(Dev s, int32_t* __restrict__ draft_tok, int32_t* __restrict__ dr
   };
   // Everybody lays out rows, then waits until all rows are there.  Chunks come from a counter, so that the wait is for running
   // CTAs only, whatever else is on the device; it is bounded all the same.
-  const int units = sh_unit[nq];
+  const int whole = sh_unit[nq], quads = (D + 3) >> 2;
+  int parts = 1;                                       // a chunk is split by layers while that gives more CTAs something to do
+  while (parts < quads && 2 * parts * whole <= (int)gridDim.x) parts *= 2;
+  const int units = whole * parts, span = 4 * ((quads + parts - 1) / parts);
   if (tid == 0) sh_task = (int)atomicAdd(&s.w_ctl[3], 1ull);
   __syncthreads();
 #pragma unroll 1
   for (int unit = sh_task; unit < units;) {
     __syncthreads();
     if (tid == 0) sh_task = (int)atomicAdd(&s.w_ctl[3], 1ull);         // (on its way during this one)
-    const int q = owner(sh_unit, unit);
-    wide_lay_out(s, sh_desc[q], (unit - sh_unit[q]) * kWideThreads);
+    const int chunk = unit / parts, l0 = (unit - chunk * parts) * span;
+    const int q = owner(sh_unit, chunk);
+    if (l0 < D) wide_lay_out(s, sh_desc[q], (chunk - sh_unit[q]) * kWideThreads, l0, min(D, l0 + span));
     __threadfence();
     __syncthreads();
     if (tid == 0) atomicAdd(&s.w_ctl[4], 1ull);
