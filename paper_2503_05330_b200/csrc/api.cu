@@ -100,7 +100,7 @@ Layout make_layout(const sdms_config* c) {
   l.b_ctl = take(kBeamCtlWords * 8);
   l.bp_todo = take(P * 4);
   l.w_desc = take(l.wide_on ? (size_t)kMaxWide * 16 : 0);
-  l.w_done = take(l.wide_on ? (size_t)kMaxWide * 4 : 0);
+  l.w_done = take(l.wide_on ? (size_t)kMaxWide * 8 : 0);
   l.w_tab = take((size_t)l.w_slots * sizeof(WideSlot));
   l.w_key = take(stride > 0 ? (size_t)l.w_slots * 4 : 0);
   l.w_item = take(stride > 0 ? (size_t)l.w_slots * 4 : 0);

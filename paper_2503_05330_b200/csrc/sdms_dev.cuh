@@ -77,7 +77,7 @@ struct Dev {
   // device-wide aggregation of queries with many matches (dag_wide.cu); w_slots = 0: not in use
   unsigned long long* w_ctl;           // [kWideCtlWords] queries registered, slots handed out, tasks handed out, chunks handed out, chunks done
   int4* w_desc;                        // [kMaxWide] query path, matches, first slot, -
-  int* w_done;                         // [kMaxWide] tasks of the query that are done; zero between builds
+  int* w_done;                         // [kMaxWide][2] tasks of the query that are done, of these sums; zero between builds
   WideSlot* w_tab;                     // [w_slots]
   uint32_t* w_key;                     // [w_slots] token + 1 of the node in the slot, 0 = free
   int32_t* w_item;                     // [w_slots] per (layer, match): slot of the item's token in the layer's table

@@ -164,6 +164,50 @@ def test_layer_tasks_at_the_edges_of_their_forms(M, alpha, V, mode):
     assert len(pair.o.matches(0)) == M and ln[0] > 0
 
 
+@pytest.mark.parametrize("M,alpha,mode", [(16000, 1.0, 0), (20000, 1.0, 0), (20000, 0.5, 0), (16000, 0.5, 1), (40000, 1.0, 0)])
+def test_class_tasks_whose_tables_and_lists_overrun(M, alpha, mode):
+    # queries whose layers are split by classes of tokens (the low bits of a hash), with followers that are nearly all distinct and
+    # nearly all of one class, whatever the number of classes: more nodes than a table holds (the class is halved, again and again),
+    # more candidates than the list of a class holds; some tokens are common, some candidates end early
+    D, N = 4, 16
+    step = D + 1
+    L = (M // (N - 1) + 2) * step + 4
+    V = 1 << 22
+    rng = np.random.default_rng(7300 + M)
+    every = np.arange(1, V, dtype=np.uint64)
+    one_class = every[(((every * 0x85ebca6b) & 0xffffffff) >> 8) % 64 == 5].astype(np.int32)
+    tokens = rng.choice(one_class, (N, L)).astype(np.int32)
+    tokens = np.where(rng.random((N, L)) < 0.1, rng.choice(one_class[:40], (N, L)), tokens).astype(np.int32)
+    lps = -rng.exponential(0.5, (N, L)).astype(np.float32)
+    per = -(-M // (N - 1))
+    for m in range(M):
+        tokens[1 + m // per, 1 + (m % per) * step] = 0
+    tokens[0, L - 3] = 0
+    lens = np.full(N, L - 1)
+    lens[0] = L - 2
+    lens[1:] = np.minimum(lens[1:], 1 + per * step + np.arange(N - 1) % 3)
+    pair = Pair(1, N, L, V, 1, D, alpha=alpha, mode=mode, match_capacity=N * N * L - 1)
+    pair.append(tokens, lps, lens, expect_status=0)
+    for _ in range(2):
+        _, ln = pair.build_and_compare(1, check_dag=False)
+        assert len(pair.o.matches(0)) == M and ln[0] > 0
+
+
+@pytest.mark.parametrize("G,N,L,mode", [(6, 60, 60, 0), (10, 110, 40, 0), (10, 110, 40, 1)])
+def test_more_wide_queries_than_are_ordered_and_than_the_list_holds(G, N, L, mode):
+    # 360 paths: more queries than the pass puts in order (256); 1100: more than its list holds (1024), the rest keep their CTA
+    V, D = 20, 5
+    tokens, lps = synth.small_random(G * N, L, V, 7400 + N)
+    pair = Pair(G, N, L, V, 2, D, alpha=0.5, mode=mode, match_capacity=1000000)
+    lens = (L - 2 - (np.arange(G * N) * 7) % 5).astype(np.int32)
+    pair.append(tokens, lps, lens, expect_status=0)
+    for k in (1, 2, 1):
+        pair.build_and_compare(k, check_dag=False, paths=list(range(0, G * N, 11)))
+        if k == 1:
+            off, _ = pair.g.matches()
+            assert (np.diff(off.numpy()) > 64).sum() > (1024 if G * N > 1024 else 256)
+
+
 @pytest.mark.parametrize("N,L", [(16, 1024), (64, 2048)])
 def test_reset_leaves_nothing_behind(N, L):
     # an index that is cleared and one whose buckets go out of date: more resets than there are epochs, other streams
