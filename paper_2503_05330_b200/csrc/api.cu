@@ -92,7 +92,9 @@ Layout make_layout(const sdms_config* c) {
   l.wide_on = !fused && c->wide_table_bytes >= 0;
   int64_t wide = c->wide_table_bytes;
   if (wide == 0) {
-    wide = slot_bytes * 5 * (int64_t)D * (int64_t)c->paths_per_group * (int64_t)(P * L);   // room for every position matching every query
+    // room for every position matching every query: up to 5 slots of a beam table per (match, layer), 16 bytes in the wide pass
+    const int64_t items = (int64_t)D * (int64_t)c->paths_per_group * (int64_t)(P * L);
+    wide = stride > 0 ? slot_bytes * 5 * items : 16 * (items + 4 * (int64_t)(D * P));
     if (wide > (320LL << 20)) wide = 320LL << 20;
   }
   l.w_slots = (l.wide_on || (stride > 0 && wide > 0)) ? (uint64_t)wide / slot_bytes : 0;

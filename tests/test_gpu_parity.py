@@ -136,6 +136,21 @@ def test_walk_at_the_edges_of_its_forms(M, alpha):
     pair.beams_and_compare(3, paths=[0])              # in shared memory up to 129 of these, lists in the table area for 600, all there for 1500
 
 
+def test_default_table_area_holds_every_position_matching_every_query():
+    # one token only: every query matches every position of the other paths, and all of them go to the wide pass
+    from paper_2503_05330_b200 import binding
+    N, L, V, D = 6, 200, 1, 7
+    pair = Pair(1, N, L, V, 1, D, match_capacity=N * N * L - 1)
+    tokens, lps = synth.small_random(N, L, V, 4300)
+    pair.append(tokens, lps, np.full(N, L - 9, np.int32), expect_status=0)
+    binding.sdms_profile_enable(pair.g.ctx, True)
+    pair.build_and_compare(1, check_dag=False)
+    area = N * D * ((N - 1) * (L - 2) + 3) // 4 * 4 * 16
+    with_it, without = (binding.sdms_workspace_bytes(binding.make_config(1, N, L, V, 1, D, match_capacity=N * N * L - 1,
+                                                                         wide_table_bytes=w)) for w in (0, -1))
+    assert area <= with_it - without <= 2 * area + 65536
+
+
 @pytest.mark.parametrize("M,alpha,V", [(32, 1.0, 50), (33, 1.0, 50), (65, 1.0, 50), (2048, 0.5, 4000), (2049, 1.0, 4000), (7168, 0.5, 60000), (7169, 0.5, 60000),
                                        (8193, 1.0, 60000), (14336, 1.0, 60000), (14337, 1.0, 60000), (30000, 1.0, 60000)])
 @pytest.mark.parametrize("mode", [0, 1])
@@ -1093,9 +1108,8 @@ def test_wide_pass_with_many_distinct_followers_and_ragged_ends():
 @pytest.mark.parametrize("N,L,V,D,match_capacity", [(4, 400, 3, 32, 5000), (4, 400, 3, 10, 5000), (5, 300, 2, 3, 7000),
                                                      (24, 900, 50, 32, 400000)])
 def test_wide_pass_units_split_by_layers_and_drafts_longer_than_a_batch(N, L, V, D, match_capacity):
-    # few heavy queries: their chunks of 128 matches are split by layers into 2, 4 or 8 units (D = 32: eight rounds of
-    # layers per thread; D = 10: three, so the last unit is short; D = 3: one, no split); many heavy queries: no split,
-    # several units per CTA, and with D = 32 a thread's layers take two batches of four
+    # few heavy queries: their chunks of 512 matches are laid out in units of a few layers (D = 32: eight of four layers; D = 10: three,
+    # the last one short; D = 3: no split); many heavy queries: no split, and with D = 32 two batches of sixteen layers
     G = 1
     tokens, lps = synth.small_random(G * N, L, V, 4260 + D)
     pair = Pair(G, N, L, V, 2, D, match_capacity=match_capacity, alpha=0.5)
