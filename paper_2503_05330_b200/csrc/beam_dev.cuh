@@ -190,12 +190,6 @@ __device__ __forceinline__ BeamPlan beam_plan(int M, int D, int B, unsigned byte
   return w;
 }
 
-__device__ __forceinline__ u64 beam_warp_max(u64 x) {
-  const unsigned hi = (unsigned)(x >> 32), top = __reduce_max_sync(FULL, hi);
-  const unsigned lo = __reduce_max_sync(FULL, hi == top ? (unsigned)x : 0u);
-  return (u64)top << 32 | lo;
-}
-
 // ent0: the path's lists in the table area, ent_stride entries per slot (used if !SHARED_LISTS; left zero).  want0, score0,
 // edge0: as for beams_of_query.
 template <bool SHARED_LISTS>
@@ -279,8 +273,8 @@ __device__ __forceinline__ void beams_in_shared(const Dev& s, const BeamPlan w, 
           const bool after = o.val < prev.val || (o.val == prev.val && o.nx < prev.nx);
           if (o.nx != 0ull && after && (o.val > best.val || (o.val == best.val && o.nx > best.nx))) best = o;
         }
-        prev.val = beam_warp_max(best.val);
-        prev.nx = beam_warp_max(best.val == prev.val ? best.nx : 0ull);
+        prev.val = warp_max64(best.val);
+        prev.nx = warp_max64(best.val == prev.val ? best.nx : 0ull);
         if (prev.nx == 0ull) break;
         if (lane == r) sn = (int)(prev.nx & 0xffffffu);
       }
@@ -288,7 +282,7 @@ __device__ __forceinline__ void beams_in_shared(const Dev& s, const BeamPlan w, 
     int j = 0;
     Offer mine = offer_of(l, sn, 0, add, w_u);
     for (int r = 0; r < B; ++r) {
-      const u64 val = beam_warp_max(mine.val), nx = beam_warp_max(mine.val == val ? mine.nx : 0ull);
+      const u64 val = warp_max64(mine.val), nx = warp_max64(mine.val == val ? mine.nx : 0ull);
       if (nx == 0ull) {
         if (r == 0) return false;
         if (lane == 0) for (int x = r; x < B; ++x) to[x] = BeamEnt{0ull, 0ull};

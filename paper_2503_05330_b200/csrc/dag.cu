@@ -34,8 +34,6 @@ namespace sdms {
 
 namespace {
 
-typedef unsigned long long u64;
-constexpr unsigned FULL = 0xffffffffu;
 constexpr int CAP = kDagCap;
 constexpr int MAXB = SDMS_MAX_DAG_NODES;
 constexpr int MAXKE = SDMS_MAX_DAG_EDGES;
@@ -236,8 +234,8 @@ __device__ void write_defaults(const Dev& s, int i, int32_t* draft_tok, float* d
 }
 
 // ---------------------------------------------------------------------------
-// M <= 32: one warp per layer, then one warp walks.  The export rows must hold
-// their defaults already (write_defaults followed by a barrier).
+// M <= 32, tree pool, layer-wise search and export: one warp per layer, then (not for the export) one
+// warp walks.  The export rows must hold their defaults already (write_defaults followed by a barrier).
 // ---------------------------------------------------------------------------
 template <bool EXPORT>
 __device__ void dag_small(const Dev& s, const Smem& sm, int i, int M, const int32_t* mlist,
@@ -250,7 +248,7 @@ __device__ void dag_small(const Dev& s, const Smem& sm, int i, int M, const int3
   int* L_u = sm.st_tok + 32 * SDMS_MAX_DRAFT;
   unsigned* L_lead = reinterpret_cast<unsigned*>(sm.st_tok + 2 * 32 * SDMS_MAX_DRAFT);
   unsigned* L_elead = L_lead + SDMS_MAX_DRAFT;
-  unsigned* L_best = L_elead + SDMS_MAX_DRAFT;      // per layer: the best edge out of each source / the best node
+  unsigned* L_best = L_elead + SDMS_MAX_DRAFT;      // per layer: the best node
   int* L_p = sm.st_tok + 3 * 32 * SDMS_MAX_DRAFT;   // fixed-point probability of the follower (tree pool)
   double* L_W = reinterpret_cast<double*>(sm.st_pq);
   double* L_we = L_W + 32 * SDMS_MAX_DRAFT;
@@ -279,22 +277,12 @@ __device__ void dag_small(const Dev& s, const Smem& sm, int i, int M, const int3
     const double W = eq5_weight(s.alpha, S_all, c_all);
     const double w_uv = eq5_weight(s.alpha, S_uv, c_uv);
     const unsigned leaders = __ballot_sync(FULL, leader), eleaders = __ballot_sync(FULL, eleader);
-    // is this edge the best way out of its source, judged by the score of its destination?
-    bool beaten = false;
-    for (unsigned rem = eleaders; rem; rem &= rem - 1) {
-      const int src = __ffs(rem) - 1;
-      const int ou = __shfl_sync(FULL, u, src);
-      const int ot = __shfl_sync(FULL, v, src);
-      const double oW = __shfl_sync(FULL, W, src);
-      if (ou == u && ranks_before(oW, ot, W, v)) beaten = true;
-    }
-    const unsigned best_out = __ballot_sync(FULL, eleader && !beaten);
-    const int top = s.mode == 1 ? warp_arg_first(leader, W, v) : -1;   // best node of the layer
+    const int top = !EXPORT && s.mode == 1 ? warp_arg_first(leader, W, v) : -1;   // best node of the layer
     L_v[(d - 1) * 32 + lane] = v; L_u[(d - 1) * 32 + lane] = u; L_p[(d - 1) * 32 + lane] = (int)p;
     L_W[(d - 1) * 32 + lane] = W; L_we[(d - 1) * 32 + lane] = w_uv;
     if (lane == 0) {
       L_lead[d - 1] = leaders; L_elead[d - 1] = eleaders;
-      L_best[d - 1] = s.mode == 1 ? (top >= 0 ? 1u << top : 0u) : best_out;
+      L_best[d - 1] = top >= 0 ? 1u << top : 0u;
     }
     if (EXPORT && live) {
       int rank = 0;
@@ -345,9 +333,10 @@ __device__ void dag_small(const Dev& s, const Smem& sm, int i, int M, const int3
       }
     }
   }
+  if (EXPORT) return;
   __syncthreads();
   if (warp != 0) return;
-  if (!EXPORT && s.pool == 1) {
+  if (s.pool == 1) {
     // tree pool: only the candidates that spell the draft so far stay in play
     bool in_play = lane < M;
     int emitted = 0;
@@ -378,12 +367,12 @@ __device__ void dag_small(const Dev& s, const Smem& sm, int i, int M, const int3
   for (int d = 1; d <= D; ++d) {
     const int v = L_v[(d - 1) * 32 + lane], u = L_u[(d - 1) * 32 + lane];
     const unsigned from_cur = __ballot_sync(FULL, u == cur);
-    const unsigned pick = s.mode == 1 ? L_best[d - 1] : (L_best[d - 1] & from_cur);
+    const unsigned pick = L_best[d - 1];
     if (pick == 0) break;
     const int src = __ffs(pick) - 1;
     const int tok = __shfl_sync(FULL, v, src);
     const double W = __shfl_sync(FULL, L_W[(d - 1) * 32 + lane], src);
-    // the edge taken: in mode 0 the picked lane leads it; in mode 1 it may not exist
+    // the edge taken may not exist
     const unsigned emask = L_elead[d - 1] & from_cur & __ballot_sync(FULL, v == tok);
     const double we = __shfl_sync(FULL, L_we[(d - 1) * 32 + lane], emask ? __ffs(emask) - 1 : 0);
     if (lane == 0) {
@@ -775,28 +764,20 @@ __device__ void list_pool(const Dev& s, int i, int M, const int32_t* mlist, cons
   if (lane == 0) draft_len[i] = n_m;
 }
 
-// ---- all layers at once (DAG pool, no export, a few hundred matches) ------------------------------
+// ---- all layers at once (layer-wise search, a few hundred matches) --------------------------------
 // dag_block takes the layers one after the other because the walk decides which node's successors
 // count; each layer then costs a few barriers and a chain of shared-memory atomics whatever M is.
-// Here every layer is aggregated at the same time into tables of its own:
-//   node table of layer d : follower token v -> sum of probabilities, count          (Eq. 5 inputs)
-//   pred table of layer d : token u of layer d - 1 -> its best successor v at layer d
-// and the walk is D table look-ups.  The pool of shared words (staging area and dag_block's tables,
-// kPoolWords in a row) holds the staged followers and as many layers' tables as fit; more layers
-// take more rounds.
+// Here every layer is aggregated at the same time into a table of its own (follower token -> sum of
+// probabilities, count) and its heaviest node found.  The pool of shared words (staging area and
+// dag_block's tables, kPoolWords in a row) holds the staged followers and as many layers' tables as
+// fit; more layers take more rounds.
 constexpr int kPoolWords = 2 * kStageWords + 8 * CAP;
-constexpr int kLayerWords = 8;                    // per table slot: pred weight (2), node key/Slo/Shi/cnt, pred key/token
+constexpr int kLayerWords = 4;                    // per table slot: key, low and high part of the sum, count
 
-struct LayerTables {
-  unsigned* p_whi; unsigned* p_wlo; int* n_key; unsigned* n_Slo; unsigned* n_Shi; unsigned* n_cnt; int* p_key; int* p_tok;
-};
-__device__ __forceinline__ LayerTables layer_tables(int* pool, int cap, int l) {
+struct LayerTable { int* key; unsigned* lo; unsigned* hi; unsigned* cnt; };
+__device__ __forceinline__ LayerTable layer_table(int* pool, int cap, int l) {
   int* b = pool + (size_t)l * kLayerWords * cap;
-  LayerTables t;
-  t.p_whi = reinterpret_cast<unsigned*>(b); t.p_wlo = reinterpret_cast<unsigned*>(b + cap);
-  t.n_key = b + 2 * cap; t.n_Slo = reinterpret_cast<unsigned*>(b + 3 * cap); t.n_Shi = reinterpret_cast<unsigned*>(b + 4 * cap);
-  t.n_cnt = reinterpret_cast<unsigned*>(b + 5 * cap); t.p_key = b + 6 * cap; t.p_tok = b + 7 * cap;
-  return t;
+  return LayerTable{b, reinterpret_cast<unsigned*>(b + cap), reinterpret_cast<unsigned*>(b + 2 * cap), reinterpret_cast<unsigned*>(b + 3 * cap)};
 }
 // slot of `key` in an open-addressing table of `cap` (power of two) slots; claims one if INSERT
 template <bool INSERT>
@@ -842,26 +823,25 @@ __device__ __forceinline__ bool layers_in_round_ok(int M, int D) {
 }
 
 __device__ void dag_layers(const Dev& s, const Smem& sm, int i, int M, const int32_t* mlist, const int32_t* plen,
-                           int poff, int root, int32_t* draft_tok, int32_t* draft_len, float* draft_score,
-                           float* draft_edge_w) {
+                           int poff, int32_t* draft_tok, int32_t* draft_len, float* draft_score, float* draft_edge_w) {
   __shared__ int sh_draft[SDMS_MAX_DRAFT];
-  __shared__ unsigned sh_lwhi[SDMS_MAX_DRAFT], sh_lwlo[SDMS_MAX_DRAFT];   // mode 1: heaviest node of the layer
+  __shared__ unsigned sh_lwhi[SDMS_MAX_DRAFT], sh_lwlo[SDMS_MAX_DRAFT];   // heaviest node of the layer
   __shared__ int sh_lt[SDMS_MAX_DRAFT];
   __shared__ unsigned sh_eSlo[SDMS_MAX_DRAFT], sh_eShi[SDMS_MAX_DRAFT], sh_ec[SDMS_MAX_DRAFT];
-  __shared__ int sh_cur, sh_emitted, sh_walking;
+  __shared__ int sh_emitted, sh_walking;
   const int tid = threadIdx.x, D = s.D;
   int cap;
   const int per_round = min(D, layers_per_round(M, D, &cap));
   const int lcap = 31 - __clz(cap), shift = 32 - lcap;
   int* st_tok = sm.st_tok;                         // [m * D + d - 1], -1 past the end of the path
   int* st_pq = sm.st_tok + M * D;
-  int* st_slot = sm.st_tok + 2 * M * D;            // node slot | pred slot << 16 of each staged follower
+  int* st_slot = sm.st_tok + 2 * M * D;            // slot of each staged follower
   int* pool = sm.st_tok + ((3 * M * D + 1) & ~1);
   const int lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
   const int nchunk = (M + 31) >> 5;                // a warp takes 32 matches of one layer at a time
 
   if (tid < D) { sh_lwhi[tid] = 0; sh_lwlo[tid] = 0; sh_lt[tid] = INT_MAX; sh_eSlo[tid] = 0; sh_eShi[tid] = 0; sh_ec[tid] = 0; }
-  if (tid == 0) { sh_cur = root; sh_emitted = 0; sh_walking = 1; }
+  if (tid == 0) { sh_emitted = 0; sh_walking = 1; }
   // stage the followers: a thread asks for four entries before it stores the first
   {
     int lD = 0;
@@ -892,17 +872,13 @@ __device__ void dag_layers(const Dev& s, const Smem& sm, int i, int M, const int
 #pragma unroll 1
   for (int d0 = 1; d0 <= D; d0 += per_round) {
     const int nl = min(per_round, D - d0 + 1);
-    // empty tables: keys -1, sums 0, best weight 0, best token "none"
+    // empty tables: keys -1, sums 0
 #pragma unroll 1
-    for (int x = tid; x < ((nl * kLayerWords) << lcap); x += blockDim.x) {
-      const int w = (x >> lcap) & (kLayerWords - 1);
-      pool[x] = (w == 2 || w == 6) ? -1 : (w == 7 ? INT_MAX : 0);
-    }
+    for (int x = tid; x < ((nl * kLayerWords) << lcap); x += blockDim.x) pool[x] = ((x >> lcap) & (kLayerWords - 1)) == 0 ? -1 : 0;
     __syncthreads();
     if (!sh_walking) break;
-    // pass 0: node sums; passes 1, 2: heaviest successor weight of every predecessor, the upper half of
-    // the weight's bit pattern first, then the lower half among those (weights are >= 0, so the
-    // patterns order like the values); pass 3: the smallest token that has this weight
+    // pass 0: node sums; passes 1, 2: the layer's heaviest weight, the upper half of the weight's bit pattern first, then the
+    // lower half among those (weights are >= 0, so the patterns order like the values); pass 3: the smallest token that has it
 #pragma unroll 1
     for (int pass = 0; pass < 4; ++pass) {
 #pragma unroll 1
@@ -911,56 +887,35 @@ __device__ void dag_layers(const Dev& s, const Smem& sm, int i, int M, const int
         const int d = d0 + l, at = m * D + d - 1;
         const int v = m < M ? st_tok[at] : -1;
         if (v < 0) continue;
-        const LayerTables t = layer_tables(pool, cap, l);
+        const LayerTable t = layer_table(pool, cap, l);
         if (pass == 0) {
-          const int sl = table_slot<true>(t.n_key, cap, shift, v);
+          const int sl = table_slot<true>(t.key, cap, shift, v);
           st_slot[at] = sl;
-          add_split(&t.n_Slo[sl], &t.n_Shi[sl], &t.n_cnt[sl], (unsigned)st_pq[at]);
+          add_split(&t.lo[sl], &t.hi[sl], &t.cnt[sl], (unsigned)st_pq[at]);
           continue;
         }
-        const u64 w = weight_bits(s.alpha, t.n_Slo, t.n_Shi, t.n_cnt, st_slot[at] & 0xffff);
+        const u64 w = weight_bits(s.alpha, t.lo, t.hi, t.cnt, st_slot[at]);
         const unsigned whi = (unsigned)(w >> 32), wlo = (unsigned)w;
-        if (pass == 1) {
-          const int claimed = table_slot<true>(t.p_key, cap, shift, d == 1 ? root : st_tok[at - 1]);
-          st_slot[at] |= claimed << 16;
-          atomicMax(&t.p_whi[claimed], whi);
-          if (s.mode == 1) atomicMax(&sh_lwhi[d - 1], whi);
-          continue;
-        }
-        const int ps = (unsigned)st_slot[at] >> 16;
-        if (pass == 2) {
-          if (t.p_whi[ps] == whi) atomicMax(&t.p_wlo[ps], wlo);
-          if (s.mode == 1 && sh_lwhi[d - 1] == whi) atomicMax(&sh_lwlo[d - 1], wlo);
-        } else {
-          if (t.p_whi[ps] == whi && t.p_wlo[ps] == wlo) atomicMin(&t.p_tok[ps], v);
-          if (s.mode == 1 && sh_lwhi[d - 1] == whi && sh_lwlo[d - 1] == wlo) atomicMin(&sh_lt[d - 1], v);
-        }
+        if (pass == 1) atomicMax(&sh_lwhi[d - 1], whi);
+        else if (pass == 2) { if (sh_lwhi[d - 1] == whi) atomicMax(&sh_lwlo[d - 1], wlo); }
+        else if (sh_lwhi[d - 1] == whi && sh_lwlo[d - 1] == wlo) atomicMin(&sh_lt[d - 1], v);
       }
       __syncthreads();
     }
-    // the walk through this round's layers
+    // the draft through this round's layers
     if (tid == 0) {
-      int cur = sh_cur, emitted = sh_emitted;
+      int emitted = sh_emitted;
 #pragma unroll 1
-      for (int l = 0; l < nl; ++l) {
-        const int d = d0 + l;
-        const LayerTables t = layer_tables(pool, cap, l);
-        int next;
-        u64 w;
-        if (s.mode == 1) {
-          next = sh_lt[d - 1]; w = ((u64)sh_lwhi[d - 1] << 32) | sh_lwlo[d - 1];
-          if (next == INT_MAX) { sh_walking = 0; break; }
-        } else {
-          const int ps = table_slot<false>(t.p_key, cap, shift, cur);
-          if (ps < 0) { sh_walking = 0; break; }
-          next = t.p_tok[ps]; w = ((u64)t.p_whi[ps] << 32) | t.p_wlo[ps];
-        }
+      for (int d = d0; d < d0 + nl; ++d) {
+        const int next = sh_lt[d - 1];
+        if (next == INT_MAX) { sh_walking = 0; break; }
         draft_tok[(size_t)i * D + d - 1] = next;
-        if (draft_score) draft_score[(size_t)i * D + d - 1] = (float)__longlong_as_double((long long)w);
+        if (draft_score)
+          draft_score[(size_t)i * D + d - 1] = (float)__longlong_as_double((long long)((u64)sh_lwhi[d - 1] << 32 | sh_lwlo[d - 1]));
         sh_draft[d - 1] = next;
-        cur = next; ++emitted;
+        ++emitted;
       }
-      sh_cur = cur; sh_emitted = emitted;
+      sh_emitted = emitted;
     }
     __syncthreads();
   }
@@ -984,12 +939,6 @@ __device__ void dag_layers(const Dev& s, const Smem& sm, int i, int M, const int
 // One CTA is bound here by how many dependent instructions follow one another (4.3 cycles each, 33 for a shared load, 50 to
 // 70 for a taken or divergent branch): so items are handled in fixed batches of registers, without branches in between.
 
-// Largest value of the warp (values are >= 0), in every lane: 57 cycles.
-__device__ __forceinline__ u64 warp_max64(u64 x) {
-  const unsigned hi = (unsigned)(x >> 32), top = __reduce_max_sync(FULL, hi);
-  const unsigned lo = __reduce_max_sync(FULL, hi == top ? (unsigned)x : 0u);
-  return (u64)top << 32 | lo;
-}
 __device__ __forceinline__ u64 max64(u64 a, u64 b) { return a > b ? a : b; }
 
 // M <= 32: lane m of a warp holds candidate m.  A warp per layer fetches the followers and forms every candidate's node
@@ -1084,11 +1033,6 @@ __device__ void dag_walk_warp(const Dev& s, int i, int M, const int32_t* mlist, 
 //          smaller token (PACKED: with alpha = 1 the weight is the sum itself; else weight and token stay apart)
 //   walk   per layer the largest key among the candidates on the current node, four candidates per lane: one warp, and no
 //          barrier, up to 128 candidates; a layer's rows do not depend on the walk and are fetched a layer ahead
-// Matches above which a query of a large prompt goes to the wide pass (there 17-22 us in a launch that other queries need anyway;
-// 1000 here 60 us).  64 here are 20 us, 32 are 10: the length of the launch where all its CTAs run at once (256 x 8192 tokens:
-// 1487 us per session from 64, 1461 from 32; 96 x 3001 with tolerance 1: 585, 570), but out of the way of longer ones where they
-// take turns (16 prompts of 128 x 4096: 3251, 3322).
-__device__ __forceinline__ int wide_from(const Dev& s) { return (int)gridDim.x <= 2 * s.w_grid ? 32 : 64; }
 constexpr int kWalkMaxCap = 8192;        // most slots of a layer's table
 
 struct WalkPlan { int cap, stride, layers; bool packed; };    // slots per table, words per row of items, layers per round
@@ -1616,10 +1560,16 @@ __device__ __forceinline__ void dag_phase(const Dev& s, const Smem& sm, int i, i
   }
   if (!EXPORT && s.pool == 2) list_pool(s, i, M, mlist, plen, poff, draft_tok, draft_len, draft_score, draft_edge_w);
   else if (M <= 32) dag_small<EXPORT>(s, sm, i, M, mlist, plen, poff, root, draft_tok, draft_len, draft_score, draft_edge_w);
-  else if (!EXPORT && s.pool == 0 && M * s.D <= kStageWords && layers_in_round_ok(M, s.D))
-    dag_layers(s, sm, i, M, mlist, plen, poff, root, draft_tok, draft_len, draft_score, draft_edge_w);
+  else if (!EXPORT && s.pool == 0 && s.mode == 1 && M * s.D <= kStageWords && layers_in_round_ok(M, s.D))
+    dag_layers(s, sm, i, M, mlist, plen, poff, draft_tok, draft_len, draft_score, draft_edge_w);
   else dag_block<EXPORT>(s, sm, i, M, mlist, plen, poff, root, draft_tok, draft_len, draft_score, draft_edge_w);
 }
+
+// Matches above which a query of a large prompt goes to the wide pass (there 17-22 us in a launch that other queries need anyway;
+// 1000 here 60 us).  64 here are 20 us, 32 are 10: the length of the launch where all its CTAs run at once (256 x 8192 tokens:
+// 1487 us per session from 64, 1461 from 32; 96 x 3001 with tolerance 1: 585, 570), but out of the way of longer ones where they
+// take turns (16 prompts of 128 x 4096: 3251, 3322).
+__device__ __forceinline__ int wide_from(const Dev& s) { return (int)gridDim.x <= 2 * s.w_grid ? 32 : 64; }
 
 template <bool EXPORT>
 __global__ void __launch_bounds__(kDagThreads, EXPORT ? 1 : 2) dag_kernel(Dev s, int32_t* __restrict__ draft_tok,
@@ -1664,7 +1614,7 @@ __global__ void __launch_bounds__(kDagThreads, EXPORT ? 1 : 2) dag_kernel(Dev s,
     if (threadIdx.x == 0) s.q_cursor[i] = Mk;
     __syncthreads();
   }
-  // more matches than a warp holds: all SMs share the work (the pass that follows this kernel)
+  // many matches: all SMs share the work (the pass that follows this kernel)
   if (!EXPORT && s.pool == 0 && s.mode != 2 && Mk > wide_from(s) && wide_register(s, i, Mk)) return;
   dag_phase<EXPORT>(s, sm, i, Mk, mlist, sh_len, g * s.N, root, draft_tok, draft_len, draft_score, draft_edge_w);
 }

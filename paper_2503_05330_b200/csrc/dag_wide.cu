@@ -67,13 +67,6 @@ __global__ void wait_timeout_kernel(Dev s, long long cycles) {
   if (threadIdx.x == 0 && !wait_for_count(s.b_ctl + kBeamNever, ~0ull, cycles)) atomicOr(s.status, SDMS_STATUS_TIMEOUT);
 }
 
-// Largest value of the warp, in every lane.
-__device__ __forceinline__ u64 warp_max64(u64 x) {
-  const unsigned hi = (unsigned)(x >> 32), top = __reduce_max_sync(FULL, hi);
-  const unsigned lo = __reduce_max_sync(FULL, hi == top ? (unsigned)x : 0u);
-  return (u64)top << 32 | lo;
-}
-
 // What is kept for a query, in rows of `pitch` entries, one for every layer:
 //   tok    the candidates' followers (-1: ended), from wide_lay_out
 //   out    first their probabilities (32 bits each, the first half of the row), then node weights, in the end for those

@@ -36,8 +36,7 @@ struct WideSlot {
   uint32_t tok1;                 // token + 1, written by whoever claimed the slot
   uint32_t unused;
   unsigned long long sum;        // count << kWideSumShift | sum of fixed-point probabilities of the node
-  unsigned long long succ_w;     // bit pattern of the largest Eq. 5 weight among the node's successors
-  unsigned long long succ;       // ~token << 32 | slot of the successor with that weight and the smallest token; 0 = none
+  unsigned long long pad[2];
 };
 struct BeamEnt;
 

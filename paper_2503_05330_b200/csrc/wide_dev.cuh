@@ -47,6 +47,14 @@ __device__ __forceinline__ bool wide_register(const Dev& s, int i, int M) {
 typedef unsigned long long u64;
 constexpr unsigned FULL = 0xffffffffu;
 constexpr int kWideThreads = 512;
+
+// Largest value of the warp, in every lane: 57 cycles.
+__device__ __forceinline__ u64 warp_max64(u64 x) {
+  const unsigned hi = (unsigned)(x >> 32), top = __reduce_max_sync(FULL, hi);
+  const unsigned lo = __reduce_max_sync(FULL, hi == top ? (unsigned)x : 0u);
+  return (u64)top << 32 | lo;
+}
+
 constexpr int kWideChunk = 128;                      // matches per unit of work: thread t owns match t % 128 ...
 constexpr int kLayerWays = kWideThreads / kWideChunk;  // ... and the layers d = t / 128 + 1, + 5, + 9, ...
 constexpr int kMaxRounds = 4;                          // layers of a thread that are in flight together (16 layers of the query)
@@ -65,15 +73,12 @@ __device__ __forceinline__ u64 group_sum(unsigned group, unsigned shared, unsign
   return sum;
 }
 
-// Node sums of one unit: the matches list[m0 .. m0 + 128) of a query with M matches, all layers, into the
+// Node sums (beams) of one unit: the matches list[m0 .. m0 + 128) of a query with M matches, all layers, into the
 // query's tables (first slot `base`, 2^lcap slots per layer).  Called by all kWideThreads threads of a
 // CTA.  The lanes of a warp hold 32 matches at the same layer; lanes whose followers are the same token
 // form a group and the group's leader claims the node's slot and sends one add for all of them.
 // Every item's slot (-1: the candidate has ended) is noted in w_item[base + (d - 1) * M + m].
-// A thread's layers are d_first + 4 r; with r_lo / r_hi the call takes only the rounds r_lo <= r < r_hi of them (a unit
-// split by layers: more, shorter units when there are fewer units than CTAs).
-__device__ __forceinline__ void wide_insert_unit(const Dev& s, const int32_t* list, unsigned base, int lcap, int M, int m0,
-                                                 int r_lo = 0, int r_hi = SDMS_MAX_DRAFT) {
+__device__ __forceinline__ void wide_insert_unit(const Dev& s, const int32_t* list, unsigned base, int lcap, int M, int m0) {
   const int tid = threadIdx.x, lane = tid & 31;
   const int D = s.D;
   const int ml = tid & (kWideChunk - 1), d_first = tid / kWideChunk + 1;   // d_first is the same in all lanes of a warp
@@ -86,16 +91,15 @@ __device__ __forceinline__ void wide_insert_unit(const Dev& s, const int32_t* li
       const int j = path_of(s, gpos);
       n_m = min(D, __ldg(s.len + j) - 1 - (gpos - j * s.L));
     }
-  for (int r0 = r_lo; r0 < r_hi && d_first + r0 * kLayerWays <= D; r0 += kMaxRounds) {     // the same trip count for the whole warp
+  for (int r0 = 0; d_first + r0 * kLayerWays <= D; r0 += kMaxRounds) {     // the same trip count for the whole warp
     const int d_base = d_first + r0 * kLayerWays;
-    const int d_end = min(D, d_first + (r_hi - 1) * kLayerWays);    // the last layer of this thread that belongs to the unit
     int v[kMaxRounds];
     unsigned p[kMaxRounds];
 #pragma unroll
     for (int r = 0; r < kMaxRounds; ++r) {            // every follower this thread needs is asked for before the first is used
       const int d = d_base + r * kLayerWays;
       v[r] = -1; p[r] = 0u;
-      if (d <= n_m && d <= d_end) { v[r] = __ldg(s.tok + gpos + d); p[r] = (unsigned)__ldg(s.pq + gpos + d); }
+      if (d <= n_m && d <= D) { v[r] = __ldg(s.tok + gpos + d); p[r] = (unsigned)__ldg(s.pq + gpos + d); }
     }
     // the key sector and the slot every follower hashes to are asked for now: when the rounds below get to
     // them (one after the other, the lanes of a warp in step) they are on their way from memory
@@ -117,7 +121,7 @@ __device__ __forceinline__ void wide_insert_unit(const Dev& s, const int32_t* li
     for (int r = 0; r < kMaxRounds; ++r) {
       const int d = d_base + r * kLayerWays;
       leader[r] = 0; sv[r] = -1; add[r] = 0ull;
-      if (d > d_end) continue;                          // the same for the whole warp
+      if (d > D) continue;                          // the same for the whole warp
       const unsigned group = __match_any_sync(FULL, v[r]);          // lanes whose items are the same node
       leader[r] = __ffs(group) - 1;
       const unsigned shared = __ballot_sync(FULL, v[r] >= 0 && (group & (group - 1)) != 0u);
@@ -134,7 +138,7 @@ __device__ __forceinline__ void wide_insert_unit(const Dev& s, const int32_t* li
     for (int r = 0; r < kMaxRounds; ++r) {
       const int d = d_base + r * kLayerWays;
       h[r] = ((unsigned)v[r] * 2654435761u) >> (32 - lcap);
-      if (d <= d_end && v[r] >= 0 && lane == leader[r]) todo |= 1u << r;
+      if (d <= D && v[r] >= 0 && lane == leader[r]) todo |= 1u << r;
     }
     uint4 ka[kMaxRounds], kb[kMaxRounds];                // the sector of keys each sequence is looking at
     unsigned fresh = 0;                                 // layers whose sector is in ka / kb
@@ -201,7 +205,7 @@ __device__ __forceinline__ void wide_insert_unit(const Dev& s, const int32_t* li
 #pragma unroll
     for (int r = 0; r < kMaxRounds; ++r) {
       const int d = d_base + r * kLayerWays;
-      if (d > d_end) continue;
+      if (d > D) continue;
       if (sv[r] >= 0) atomicAdd(&s.w_tab[base + ((size_t)(d - 1) << lcap) + sv[r]].sum, add[r]);
       const int mine = __shfl_sync(FULL, sv[r], leader[r]);
       if (ml < nm) item[(size_t)(d - 1) * M] = v[r] >= 0 ? mine : -1;

@@ -136,6 +136,27 @@ def test_walk_at_the_edges_of_its_forms(M, alpha):
     pair.beams_and_compare(3, paths=[0])              # in shared memory up to 129 of these, lists in the table area for 600, all there for 1500
 
 
+@pytest.mark.parametrize("M", [32, 33, 255, 256, 600, 910, 911, 1500])
+@pytest.mark.parametrize("alpha", [1.0, 0.5])
+@pytest.mark.parametrize("D", [9, 1])
+def test_layer_wise_search_at_the_edges_of_its_forms(M, alpha, D):
+    # a warp per layer to 32 matches, a table per layer to 8192 staged followers (910 matches at D = 9), layer by layer beyond
+    V, k = 50, 1
+    step = D + 2
+    L = 2 + ((M + 1) // 2 + 1) * step
+    rng = np.random.default_rng(7050 + M)
+    tokens = 1 + np.minimum((rng.random((3, L)) ** 3 * (V - 1)).astype(np.int32), V - 2)
+    lps = -rng.exponential(0.5, (3, L)).astype(np.float32)
+    at = [(p, 1 + m * step) for m in range((M + 1) // 2) for p in (1, 2)][:M]
+    for p, x in at:
+        tokens[p, x] = 0
+    tokens[0, L - 3] = 0
+    pair = Pair(1, 3, L, V, k, D, alpha=alpha, mode=1, B=2, Ke=2)
+    pair.append(tokens, lps, np.array([L - 2, L - 1, L - 1]), expect_status=0)
+    _, ln = pair.build_and_compare(k, paths=[0])
+    assert len(pair.o.matches(0)) == M and ln[0] > 0
+
+
 def test_default_table_area_holds_every_position_matching_every_query():
     # one token only: every query matches every position of the other paths, and all of them go to the wide pass
     from paper_2503_05330_b200 import binding
