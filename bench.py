@@ -534,6 +534,41 @@ def gather_at_scale(device, G=64, N=256, L=8192, V=16384, D=16):
     return out
 
 
+def rounded(x):
+    """Floats of a nested value to six significant digits."""
+    if isinstance(x, float):
+        return float(f"{x:.6g}")
+    if isinstance(x, dict):
+        return {k: rounded(v) for k, v in x.items()}
+    return [rounded(v) for v in x] if isinstance(x, (list, tuple)) else x
+
+
+def printed(line):
+    """The line that is printed: whoever records it keeps a few KB, so builds by workload are their median times, and figures that
+    explain others (per launch, per leg, percentiles, what was counted) are left to --detail."""
+    by_k = lambda r: None if r is None else {  # noqa: E731
+        "us_by_k": {k: v["us"] for k, v in r["build_by_k"].items()},
+        **({"get_beams_us_by_k": {k: v["get_beams_us"] for k, v in r["build_by_k"].items()}}
+           if any("get_beams_us" in v for v in r["build_by_k"].values()) else {})}
+    scale = lambda r: None if r is None else {k: r[k] for k in ("store_bytes", "gbs", "frac")}  # noqa: E731
+    out = dict(line)
+    roof = dict(line["roofline"])
+    roof["steady_state_full_history"] = by_k(roof["steady_state_full_history"])
+    roof["by_config"] = None if roof["by_config"] is None else {n: by_k(r) for n, r in roof["by_config"].items()}
+    roof["match_at_scale"], roof["gather_at_scale"] = scale(roof["match_at_scale"]), scale(roof["gather_at_scale"])
+    for name in ("bytes_model", "note"):
+        roof.pop(name)
+    out["roofline"] = roof
+    out["e2e"] = {k: v for k, v in line["e2e"].items() if k not in ("clock", "device_us_from", "how")}
+    out["kernels"] = {n: v["us_per_launch"] for n, v in line["kernels"].items()}
+    out["dag_export"] = line["dag_export"]["us_per_sdms_get_dag_call"]
+    for name in ("fuzzy_epsilon_1", "backoff_from_k_max"):
+        out[name] = None if line[name] is None else line[name]["us_per_step"]
+    if "cpu_baseline" in line:
+        out["cpu_baseline"] = {k: v for k, v in line["cpu_baseline"].items() if k not in ("by_threads", "sample")}
+    return rounded(out)
+
+
 def rank_seed(w, rank):
     """Every rank owns its own prompts: same recipe, different seed."""
     return synth.BASE_SEED + w.index + 7919 * rank
@@ -770,7 +805,10 @@ def ours_main(args, w):
                                 "by_threads": {str(t): legs[t] for t in legs},
                                 "sample": f"{legs[best]['steps']} decode steps of {w.name} ({legs[best]['runs']} whole run(s) from "
                                           f"the warm start, every step timed); the faster of 1 thread and {cores} threads"}
-    print(json.dumps(line), flush=True)
+    if args.detail:
+        with open(args.detail, "w") as f:
+            json.dump(line, f, indent=1)
+    print(json.dumps(printed(line)), flush=True)
     if world > 1:
         dist.destroy_process_group()
 
@@ -787,6 +825,7 @@ def main():
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--no-fuzzy", action="store_true", help="skip the extra pass with tolerance 1")
     ap.add_argument("--no-others", action="store_true", help="skip the build-only figures of the other workloads")
+    ap.add_argument("--detail", default="", help="also write every figure to this file (JSON)")
     ap.add_argument("--steady", type=int, default=0,
                     help="only print the build-only figures of this workload at 97 %% full histories (for profiling)")
     ap.add_argument("--gather-scale", type=int, default=0,

@@ -44,3 +44,25 @@ def test_two_ranks_draw_different_prompts_and_reduce_max_time_sum_units():
 def test_single_process_passthrough():
     import bench
     assert bench.whole_job([3.0], [4.0], "cpu") == ([3.0], [4.0])
+
+
+def test_the_printed_line_stays_short_and_keeps_what_the_contract_names():
+    import json
+    import bench
+    k = {"us": 1.23456789, "p10_us": 1.0, "p90_us": 2.0, "kernel_us": {"dag": 1.0}, "get_beams_us": 3.0}
+    builds = {"workspace_bytes": 1, "build_by_k": {str(n): dict(k) for n in range(1, 9)}}
+    scale = {"store_bytes": 1, "gbs": 2.0, "frac": 0.5, "groups": 64}
+    line = {"metric": bench.METRIC, "value": 1234567.891, "unit": bench.UNIT, "n_gpus": 1, "steps": 2, "warmup": 3, "ms_per_step": 0.1,
+            "e2e": {"value": 1.0, "unit": bench.UNIT, "h2d_bytes_per_step": 5, "d2h_bytes_per_step": 6, "how": "x" * 500},
+            "gpu_launches": 9, "clocks": {"sm_mhz": 1965.0, "reasons": []}, "kernels": {"step": {"us_per_launch": 15.0, "gbs": 1.0}},
+            "roofline": {"steady_state_full_history": builds, "by_config": {f"config {n}": builds for n in range(10)},
+                         "match_at_scale": scale, "gather_at_scale": scale, "bytes_model": "x" * 300, "note": "x" * 300},
+            "dag_export": {"us_per_sdms_get_dag_call": 60.0}, "fuzzy_epsilon_1": {"us_per_step": 1.0}, "backoff_from_k_max": None,
+            "cpu_baseline": {"value": 1.0, "by_threads": {}, "sample": "x" * 300}}
+    text = json.dumps(bench.printed(line))
+    assert len(text) < 6000
+    out = json.loads(text)
+    assert out["value"] == 1234570.0 and out["e2e"]["h2d_bytes_per_step"] == 5 and out["gpu_launches"] == 9
+    assert out["roofline"]["by_config"]["config 3"]["us_by_k"]["8"] == 1.23457
+    line["roofline"].update(steady_state_full_history=None, by_config=None, match_at_scale=None, gather_at_scale=None)
+    assert json.loads(json.dumps(bench.printed(line)))["roofline"]["by_config"] is None       # several ranks: those passes are left out
