@@ -52,7 +52,7 @@ extern "C" {
 #define SDMS_STATUS_MATCH_OVERFLOW 0x20u /* match workspace exhausted: the affected paths get draft_len 0 */
 #define SDMS_STATUS_SEARCH_FALLBACK 0x40u /* search_mode 2: a path had too many matches for shared memory (more than about
                                             24576 / (11 * max_draft_len)) and the table area had no room: greedy draft */
-#define SDMS_STATUS_TIMEOUT        0x80u /* a bounded wait inside a kernel ran out (never expected): the build's matches are incomplete */
+#define SDMS_STATUS_TIMEOUT        0x80u /* a bounded wait inside a kernel ran out (never expected): the build's matches or drafts are incomplete */
 #define SDMS_STATUS_TABLES_FULL    0x100u /* sdms_get_beams: the table area of the workspace (wide_table_bytes) did not hold
                                              every path's node tables; the paths left out have no beam */
 
@@ -312,7 +312,7 @@ int sdms_debug_read_history(sdms_ctx* ctx, int32_t* d_tok, int32_t* d_pq, int32_
 int sdms_debug_read_query_modes(sdms_ctx* ctx, int32_t* d_modes, void* stream);
 
 /* Every wait inside a kernel (such as the copy barriers of the streaming scan) is bounded:
- * when it runs out, the kernel raises SDMS_STATUS_TIMEOUT and returns, and the context stays usable.  This call
+ * when it runs out, the kernel raises SDMS_STATUS_TIMEOUT and comes to its end all the same, and the context stays usable.  This call
  * shows what that looks like without anything going wrong: one thread waits, with the same bounded wait, about
  * half a millisecond for a count that nobody raises, sets the status bit and returns. */
 int sdms_debug_wait_timeout(sdms_ctx* ctx, void* stream);
