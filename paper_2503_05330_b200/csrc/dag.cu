@@ -1957,8 +1957,9 @@ __global__ void __launch_bounds__(kFusedThreads, 1) step_kernel(Dev s, int k, in
 // keep the cache.  An SM splits its 256 KB at 164, 196 and 228 KB: with 200 KB 28 KB of L1 are left, with 184 (and 10 KB
 // of arrays) 60.  k = 1 builds of 64 x 2048 and 32 x 16 x 4096 tokens, queries of up to 4139 matches: 117 and 193 us with 200 KB, 98 and
 // 172 with 184, 124 and 206 with 106; alpha = 0.5, whose tables are a third larger, 144 and 222 / 127 and 206 / 125 and 205;
-// tree pools 126 and 197 with 200 KB, 101 and 175 with 106.  (Pools of 5350 to 6370 matches, whose tables only fit the 200: 64 x 2048 tokens
-// of a small alphabet 197 us for 179; larger ones 212 for 239, smaller ones 127 for 150.)
+// tree pools 126 and 197 with 200 KB, 101 and 175 with 106.  What loses: with alpha = 1, pools
+// of 5089 to 6112 matches, whose walk_plan only fits the 200 (64 x 2048 tokens, V = 21 and 23, at most 6035 and 5497 matches: 198 and 185 us
+// for 179 and 171).  On either side 184 is the faster: at most 6304 matches (V = 20) 212 for 239, at most 4228 (V = 30) 127 for 151.
 constexpr size_t kBigPool = 184 * 1024;
 constexpr long long kBigPoolFrom = 32768;             // tokens of a prompt
 static size_t fused_smem_bytes(const Dev& s) {
