@@ -179,17 +179,6 @@ __device__ __forceinline__ void beams_of_query(const Dev& s, int i, int M, const
 // over the lanes.  With more candidates than lanes the B best next nodes are found first, by the heads of their lists: no
 // other one can contribute.  Bound by dependent accesses; with everything in the table area (two rounds of L2 atomics and a
 // barrier per layer and rank) 139 us for 30 matches, 570 us for 760, D = 8, B = 4.
-struct BeamPlan { int cap, stride; bool lists; };    // slots per layer's table (0: does not fit), items per row, lists in shared memory
-__device__ __forceinline__ BeamPlan beam_plan(int M, int D, int B, unsigned bytes) {
-  BeamPlan w;
-  w.cap = 1 << beam_lcap(min(M, 1 << 20));
-  w.stride = (M + 31) & ~31;
-  const long long tables = (long long)D * (w.cap * 16ll + w.stride * 2ll) + w.cap * 6ll + w.stride * 2ll;
-  w.lists = tables + (long long)D * w.cap * B * 16 <= (long long)bytes;
-  if (tables > (long long)bytes || M >= 0xffff) w.cap = 0;
-  return w;
-}
-
 // ent0: the path's lists in the table area, ent_stride entries per slot (used if !SHARED_LISTS; left zero).  want0, score0,
 // edge0: as for beams_of_query.
 template <bool SHARED_LISTS>

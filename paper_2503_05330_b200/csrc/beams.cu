@@ -8,15 +8,6 @@ namespace sdms {
 
 namespace {
 
-// Shared memory of a CTA (one per SM).  Tables and lists want as much as there is, the form over the table area wants L1, and one
-// launch has both.  An SM splits its 256 KB at 164, 196 and 228 KB, so each size is what just fits below a step: 160 KB for one
-// beam, whose lists are short, 192 KB for more.  Pools of 944 and 26 236 matches, D = 16, one beam: 499 us and 12.6 ms with 200 KB
-// (28 KB of L1), 331 us and 8.7 ms with 160, 303 us and 8.7 ms with none; pools of up to 117, D = 8, four beams: 45 us with 192,
-// 59 with 160 (no room for the lists), 306 with none.  A launch for each form: side by side or not, the SMs keep the split of
-// the launch before (320 us for 203 on 32 prompts of 16 x 1024, k = 1).
-constexpr int kBeamSmem = 192 * 1024, kBeamSmemOne = 160 * 1024;
-inline int beam_smem(int B) { return B > 1 ? kBeamSmem : kBeamSmemOne; }
-
 // First slot of the tables of a path with M matches in the table area, -1: no room.  By one thread.
 __device__ __forceinline__ long long reserve_tables(const Dev& s, int M) {
   if (M <= 0 || M > kWideMaxMatches) return -1;
@@ -70,7 +61,7 @@ __global__ void __launch_bounds__(kWideThreads, 1) beam_kernel(Dev s, int B, uns
 // bp_todo) get their best path: the first beam of their pool, with scores and edge weights, in place of
 // the greedy draft.  The CTAs take the listed paths in turn (one for each path of the context: 2048 of them, mostly with
 // nothing to do, took 20 us).
-__global__ void __launch_bounds__(kWideThreads, 1) best_path_fix_kernel(Dev s, int32_t* __restrict__ draft_tok,
+__global__ void __launch_bounds__(kWideThreads, 1) best_path_fix_kernel(Dev s, unsigned bytes, int32_t* __restrict__ draft_tok,
                                                                         int32_t* __restrict__ draft_len,
                                                                         float* __restrict__ draft_score,
                                                                         float* __restrict__ draft_edge_w) {
@@ -94,7 +85,7 @@ __global__ void __launch_bounds__(kWideThreads, 1) best_path_fix_kernel(Dev s, i
     const long long first = sh_first;
     x = sh_next;
     if (first >= 0)
-      beams_of_path(s, kBeamSmemOne, i, M, first, 1, draft_tok + (size_t)i * D, draft_len + i, &sh_value, true,
+      beams_of_path(s, bytes, i, M, first, 1, draft_tok + (size_t)i * D, draft_len + i, &sh_value, true,
                     draft_score ? draft_score + (size_t)i * D : nullptr, draft_edge_w ? draft_edge_w + (size_t)i * D : nullptr);
     __syncthreads();                                   // before the next path's tables
   }
@@ -105,20 +96,25 @@ __global__ void __launch_bounds__(kWideThreads, 1) best_path_fix_kernel(Dev s, i
 
 // Called when a context is created, with its device current.
 cudaError_t beam_kernel_setup() {
-  const cudaError_t e = cudaFuncSetAttribute(beam_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kBeamSmem);
-  return e != cudaSuccess ? e : cudaFuncSetAttribute(best_path_fix_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kBeamSmemOne);
+  int bytes = 0;
+  for (int d = 1; d <= SDMS_MAX_DRAFT; ++d)
+    for (int b = 1; b <= SDMS_MAX_BEAMS; ++b) bytes = max(bytes, beam_bytes(d, b));
+  const cudaError_t e = cudaFuncSetAttribute(beam_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  return e != cudaSuccess ? e : cudaFuncSetAttribute(best_path_fix_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
 }
 
 cudaError_t launch_best_path_fix(const Dev& s, int32_t* draft_tok, int32_t* draft_len, float* draft_score,
                                  float* draft_edge_w, cudaStream_t stream) {
-  return launch_overlapped(best_path_fix_kernel, dim3((unsigned)(s.P < 148 ? s.P : 148)), dim3(kWideThreads), kBeamSmemOne, stream, s,
-                           draft_tok, draft_len, draft_score, draft_edge_w);
+  const int bytes = beam_bytes(s.D, 1);
+  return launch_overlapped(best_path_fix_kernel, dim3((unsigned)(s.P < 148 ? s.P : 148)), dim3(kWideThreads), bytes, stream, s,
+                           (unsigned)bytes, draft_tok, draft_len, draft_score, draft_edge_w);
 }
 
 cudaError_t launch_beams(const Dev& s, int B, int32_t* beam_tok, int32_t* beam_len, float* beam_value,
                          cudaStream_t stream) {
-  return launch_overlapped(beam_kernel, dim3(s.P), dim3(kWideThreads), beam_smem(B), stream, s, B, (unsigned)beam_smem(B), beam_tok,
-                           beam_len, beam_value);
+  const int bytes = beam_bytes(s.D, B);
+  return launch_overlapped(beam_kernel, dim3(s.P), dim3(kWideThreads), bytes, stream, s, B, (unsigned)bytes, beam_tok, beam_len,
+                           beam_value);
 }
 
 }  // namespace sdms

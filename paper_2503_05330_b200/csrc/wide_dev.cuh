@@ -1,6 +1,7 @@
 // Hand-over of a query with many matches to the device-wide aggregation pass (dag_wide.cu).
 #pragma once
 #include "sdms_dev.cuh"
+#include "beam_plan.h"
 
 namespace sdms {
 
@@ -11,13 +12,6 @@ __device__ __forceinline__ int wide_alone(const Dev& s) { return (s.alpha != 1.0
 __device__ __forceinline__ int wide_pitch(int M) { return (M + 3) & ~3; }
 __device__ __forceinline__ unsigned long long wide_slots(const Dev& s, int M) {
   return ((unsigned long long)wide_pitch(M) * s.D * (M <= wide_alone(s) ? 16 : 12) + sizeof(WideSlot) - 1) / sizeof(WideSlot);
-}
-
-// log2 of the slots of one layer's node table in the table area (beams): a power of two above 5/4 of the matches.
-__device__ __forceinline__ int beam_lcap(int M) {
-  int l = 6;
-  while ((1ll << l) < (long long)M + (M >> 2) + 1) ++l;
-  return l;
 }
 
 // Called by every thread of the query's CTA.  Reserves room for all D layers and enters the

@@ -1223,6 +1223,21 @@ def test_beams_of_pools_on_both_sides_of_what_shared_memory_holds(alpha):
             pair.beams_and_compare(B)
 
 
+@pytest.mark.parametrize("D,V,lo,hi", [(5, 8, 820, 1638), (10, 16, 410, 819), (11, 16, 410, 768), (20, 30, 205, 409)])
+def test_beams_of_pools_that_fit_at_the_larger_sizes_only(D, V, lo, hi):
+    # pools of lo..hi matches: their tables take 160 to 200 KB; by beams and by best-path search
+    G, N, L = 1, 10, 1024
+    tokens, lps = synth.small_random(G * N, L, V, 6600 + D)
+    pair = Pair(G, N, L, V, 2, D, mode=2, max_beams=4)
+    lens = (1000 - (np.arange(N) * 67) % 400).astype(np.int32)
+    pair.append(tokens[:, :1000], lps[:, :1000], lens, expect_status=0)
+    pair.build_and_compare(1, check_dag=False)
+    m = np.diff(pair.g.matches()[0].numpy())
+    assert ((m >= lo) & (m <= hi)).any(), m
+    for B in (1, 2, 4):
+        pair.beams_and_compare(B)
+
+
 def test_beams_need_room_and_a_build():
     from paper_2503_05330_b200 import binding
     G, N, L, V, D = 1, 6, 64, 3, 4
