@@ -48,6 +48,9 @@ int check_config(const sdms_config* c) {
   return SDMS_OK;
 }
 
+// n-gram lengths the index has tables for
+int index_lengths(const sdms_config* c) { return c->index_max_n ? c->index_max_n : c->k_max; }
+
 Layout make_layout(const sdms_config* c) {
   Layout l;
   const size_t P = (size_t)c->num_groups * c->paths_per_group;
@@ -69,7 +72,7 @@ Layout make_layout(const sdms_config* c) {
   l.len = take(P * 4);
   l.rec = take(P * kRecWords * 4);
   l.status = take(4);
-  l.index = take((size_t)c->num_groups * (c->index_max_n ? c->index_max_n : c->k_max) * cap * kBucketWords * 4);
+  l.index = take((size_t)c->num_groups * index_lengths(c) * cap * kBucketWords * 4);
   l.q_fp = take(P * 4); l.q_mode = take(P * 4); l.q_reserved = take(P * 4);
   l.q_off = take(P * 4); l.q_cursor = take(P * 4);
   l.match_cursor = take(8);
@@ -236,7 +239,7 @@ int sdms_create(const sdms_config* cfg, void* d_workspace, size_t bytes, sdms_ct
   std::memset(ctx->prof_n, 0, sizeof(ctx->prof_n));
   Dev& d = ctx->dev;
   d.G = cfg->num_groups; d.N = cfg->paths_per_group; d.L = cfg->capacity; d.V = cfg->vocab;
-  d.k_max = cfg->k_max; d.idx_n = cfg->index_max_n ? cfg->index_max_n : cfg->k_max; d.D = cfg->max_draft_len; d.max_append = cfg->max_append;
+  d.k_max = cfg->k_max; d.idx_n = index_lengths(cfg); d.D = cfg->max_draft_len; d.max_append = cfg->max_append;
   d.B = cfg->dag_nodes_per_layer; d.Ke = cfg->dag_nodes_per_layer ? cfg->dag_edges_per_node : 0;
   d.mode = cfg->search_mode; d.P = d.G * d.N;
   d.alpha = (double)cfg->alpha;

@@ -15,6 +15,7 @@ namespace sdms {
 
 namespace {
 
+template <bool CHAINED>
 __global__ void __launch_bounds__(128) append_kernel(Dev s, const int32_t* __restrict__ tokens,
                                                      const float* __restrict__ logprobs,
                                                      const int32_t* __restrict__ counts, int row_width) {
@@ -45,23 +46,24 @@ __global__ void __launch_bounds__(128) append_kernel(Dev s, const int32_t* __res
   uint32_t st = 0;
   const int n = sh_bad;
   if (threadIdx.x == 0 && n < sh_n) st |= SDMS_STATUS_BAD_TOKEN;
-  append_tokens(s, p, sh_len0, n, in_tok, in_lp, sh_rec, &st);
+  append_tokens<CHAINED>(s, p, sh_len0, n, in_tok, in_lp, sh_rec, &st);
   if (st) atomicOr(&sh_st, st);
   __syncthreads();
   if (threadIdx.x == 0 && sh_st) atomicOr(s.status, sh_st);
 }
 
 // ---- wide rows ---------------------------------------------------------------------------------------
-// Prefill: thousands of tokens per row.  What bounds it is the random read-modify-write of the index, one 32-byte
-// sector per token and n-gram length in tables far larger than L2 (a B200 does 24 G/s of them in a 1 GiB region,
-// 110 G/s in 32 MiB).  So a row is cut into chunks with CTAs of their own, at 2048 threads per SM and one insert
-// per thread at a time (four inserts per thread with their atomics in flight together, at half the threads, were no
-// faster); and the n-gram lengths go one after the other over the grid, so that what is being written at a time is
-// one table per prompt and not all k_max of them: 256 paths x 7800 tokens x 8 lengths 530 us, with all lengths in one
-// CTA 750 us, with one CTA of 128 threads per path (append_kernel) 2270 us.
+// Prefill: thousands of tokens per row.  What bounds it is the read-modify-write of the index at random, one or two 32-byte sectors
+// per token (chained index), and how long each takes: 26 G positions/s with 1536 threads per SM and one bucket per thread at a time,
+// DRAM at 19 % and L2 at 29 % of their rates.  So a row is cut into chunks with CTAs of their own (append of 32 x 16 x 3700 tokens, lengths
+// up to 5: 118 us; 256 x 7800, up to 8: 140; with an entry per length 269 and 497, and the same in one CTA of 128 threads per path, append_kernel,
+// 2270).  Also measured: four positions of a thread with their reads and claims on their way together, at 1024 threads per SM (32 x 16: 220 us,
+// the lanes' ways through the lengths part), single tokens in a table of their own without hashing (256 x 7800: 155), prompts taken in turn (16 x 128 x 3900
+// without a common token 351 for 302, with many 433 for 417).
+// Indexes that are cleared have an entry per length, and a CTA each for it: 16 x 1024 17 us.
 constexpr int kPlanThreads = 256;
 constexpr int kBulkThreads = 256;
-constexpr int kBulkChunk = 512;          // positions per CTA; half of it when that leaves SMs without a full load
+constexpr int kBulkChunk = 512;          // most positions per CTA
 
 // What every path takes of its row: tokens held so far, tokens to append.
 __global__ void __launch_bounds__(kPlanThreads) append_plan_kernel(Dev s, const int32_t* __restrict__ tokens,
@@ -94,23 +96,80 @@ __global__ void __launch_bounds__(kPlanThreads) append_plan_kernel(Dev s, const 
   }
 }
 
-// The n-grams of length n that end at positions [x0, x1) of path p into the prompt's table.  win[kHalo - 1 + t] = token
-// at x0 + t (shared memory).
+// Buckets that are known to be full, and what this CTA has to add to their counts.  The commonest token of a text is a few percent of
+// it: counted one by one, its tens of thousands of occurrences queue up at one address (16 x 128 x 3900 tokens, a quarter of them
+// Zipf(1.1): 568 us counted one by one, 417 with this; 2 x 256 x 3900, 60 % of them, 32000 different: 529 and 234).  Lengths 1 and 2 of a chained index; the whole hash is compared, and what
+// hashes to the same is in the same bucket.
+constexpr int kFullSlots = 128;
+struct FullBuckets { unsigned long long key[2][kFullSlots]; uint32_t bucket[2][kFullSlots]; unsigned count[2][kFullSlots]; };
+__device__ __forceinline__ void full_empty(FullBuckets& f) {
+  for (int x = threadIdx.x; x < 2 * kFullSlots; x += kBulkThreads) { (&f.key[0][0])[x] = 0ull; (&f.count[0][0])[x] = 0u; }
+}
+__device__ __forceinline__ void full_count(const Dev& s, int g, const FullBuckets& f) {
+  for (int x = threadIdx.x; x < 2 * kFullSlots; x += kBulkThreads) {
+    const unsigned c = (&f.count[0][0])[x];
+    if (c == 0u) continue;
+    uint32_t* const bucket = index_table(s, g, x / kFullSlots + 1) + (size_t)(&f.bucket[0][0])[x] * kBucketWords;
+    atomicAdd(reinterpret_cast<unsigned long long*>(bucket), (unsigned long long)c << 32);
+  }
+}
+
+// The n-grams of length n that end at positions [x0, x1) of path p into the prompt's tables.  win[kHalo - 1 + t] = token at x0 + t
+// (shared memory).
+__device__ __forceinline__ uint64_t window_hash(const int32_t* win, int t, int n) {
+  uint64_t h = gram_init(n);
+  const int32_t* q = win + kHalo - n + t;
+  for (int u = 0; u < n; ++u) h = gram_step(h, q[u]);
+  return gram_final(h);
+}
 __device__ __forceinline__ void insert_positions(const Dev& s, int p, int n, int x0, int x1, const int32_t* win, uint32_t* st) {
   const int g = p / s.N;
   const uint32_t epoch = epoch_of(s.rec[(size_t)p * kRecWords + kRecEpoch]);
   const uint32_t lbase = (uint32_t)(p - g * s.N) * (uint32_t)s.L;
+  for (int x = x0 + (int)threadIdx.x; x < x1; x += kBulkThreads)
+    if (x + 1 >= n) index_insert<true, false>(s, g, n, window_hash(win, x - x0, n), lbase + (uint32_t)x, epoch, st);
+}
+
+// The same for a chained index, one length after the other.  FULL: with FullBuckets.  Every thread of the CTA, after a barrier.
+template <bool FULL>
+__device__ __forceinline__ void chain_positions(const Dev& s, int p, int x0, int x1, const int32_t* win, uint32_t* st) {
+  __shared__ FullBuckets f;
+  const int g = p / s.N;
+  const uint32_t epoch = epoch_of(s.rec[(size_t)p * kRecWords + kRecEpoch]);
+  const uint32_t lbase = (uint32_t)(p - g * s.N) * (uint32_t)s.L;
+  if (FULL) {
+    full_empty(f);
+    __syncthreads();
+  }
   for (int x = x0 + (int)threadIdx.x; x < x1; x += kBulkThreads) {
-    if (x + 1 < n) continue;
-    uint64_t h = gram_init(n);
-    const int32_t* q = win + kHalo - n + (x - x0);
-    for (int t = 0; t < n; ++t) h = gram_step(h, q[t]);
-    index_insert<true>(s, g, n, gram_final(h), lbase + (uint32_t)x, epoch, st);
+    const int last = min(s.idx_n, x + 1);
+#pragma unroll 1
+    for (int n = 1; n <= last; ++n) {
+      const uint64_t h = window_hash(win, x - x0, n);
+      const int at = (int)(h >> 40) & (kFullSlots - 1), l = n - 1;
+      if (FULL && l < 2 && *(volatile unsigned long long*)&f.key[l][at] == h && h != 0ull) { atomicAdd(&f.count[l][at], 1u); continue; }
+      auto full = [&](uint32_t b) {
+        if (!FULL || l >= 2 || h == 0ull) return false;
+        const unsigned long long k = atomicCAS(&f.key[l][at], 0ull, (unsigned long long)h);
+        if (k != 0ull && k != h) return false;
+        f.bucket[l][at] = b;
+        atomicAdd(&f.count[l][at], 1u);
+        return true;
+      };
+      if (index_insert<true, true>(s, g, n, h, lbase + (uint32_t)x, epoch, st, full)) break;
+    }
+  }
+  if (FULL) {
+    __syncthreads();
+    full_count(s, g, f);
   }
 }
 
-// Grid: (path, chunk of its row) x n, n slowest.
-__global__ void __launch_bounds__(kBulkThreads, 8) append_bulk_kernel(Dev s, const int32_t* __restrict__ tokens,
+// Grid: (path, chunk of its row) x n, n slowest; chained index, or none: x 1.
+enum BulkForm { kPerLength, kChain, kChainFull };
+constexpr int bulk_ctas(int form) { return form == kPerLength ? 8 : 6; }
+template <int FORM>
+__global__ void __launch_bounds__(kBulkThreads, bulk_ctas(FORM)) append_bulk_kernel(Dev s, const int32_t* __restrict__ tokens,
                                                                       const float* __restrict__ logprobs, int row_width,
                                                                       int chunk, int chunks) {
   __shared__ int32_t sh_win[kHalo - 1 + kBulkChunk];
@@ -144,10 +203,12 @@ __global__ void __launch_bounds__(kBulkThreads, 8) append_bulk_kernel(Dev s, con
       s.pq[(size_t)p * s.L + len0 + c0 + t] = prob_to_fixed(in_lp[c0 + t], &st);
     }
   }
-  insert_positions(s, p, (int)blockIdx.y + 1, len0 + c0, len0 + c0 + m, sh_win, &st);
+  if (FORM != kPerLength) chain_positions<FORM == kChainFull>(s, p, len0 + c0, len0 + c0 + m, sh_win, &st);
+  else if (s.idx_n > 0) insert_positions(s, p, (int)blockIdx.y + 1, len0 + c0, len0 + c0 + m, sh_win, &st);
   if (st) atomicOr(s.status, st);
 }
 
+template <bool CHAINED>
 __global__ void __launch_bounds__(128) accept_kernel(Dev s, const int32_t* __restrict__ draft_tok,
                                                      const int32_t* __restrict__ draft_len,
                                                      const int32_t* __restrict__ sampled,
@@ -155,7 +216,7 @@ __global__ void __launch_bounds__(128) accept_kernel(Dev s, const int32_t* __res
                                                      int32_t* __restrict__ accept_len) {
   grid_wait();
   grid_release();
-  accept_commit_phase(s, blockIdx.x, draft_tok, draft_len, sampled, sampled_lp, accept_len);
+  accept_commit_phase<CHAINED>(s, blockIdx.x, draft_tok, draft_len, sampled, sampled_lp, accept_len);
 }
 
 // sdms_reset of a large index: lengths, records and the small state between `a` / `b` and their ends become zero, the
@@ -220,7 +281,8 @@ __global__ void __launch_bounds__(256) trim_clear_kernel(Dev s) {
 }
 
 // Third launch: every n-gram (n = 1..k_max) of every path of those prompts goes into the tables again.
-__global__ void __launch_bounds__(kBulkThreads, 8) trim_reindex_kernel(Dev s, int chunk, int chunks) {
+template <int FORM>
+__global__ void __launch_bounds__(kBulkThreads, bulk_ctas(FORM)) trim_reindex_kernel(Dev s, int chunk, int chunks) {
   __shared__ int32_t sh_win[kHalo - 1 + kBulkChunk];
   grid_wait();
   grid_release();
@@ -235,7 +297,8 @@ __global__ void __launch_bounds__(kBulkThreads, 8) trim_reindex_kernel(Dev s, in
   }
   __syncthreads();
   uint32_t st = 0;
-  insert_positions(s, p, (int)blockIdx.y + 1, x0, x1, sh_win, &st);
+  if (FORM != kPerLength) chain_positions<FORM == kChainFull>(s, p, x0, x1, sh_win, &st);
+  else if (s.idx_n > 0) insert_positions(s, p, (int)blockIdx.y + 1, x0, x1, sh_win, &st);
   if (st) atomicOr(s.status, st);
 }
 
@@ -249,37 +312,45 @@ cudaError_t launch_reset(const Dev& s, void* a, size_t a_bytes, void* b, size_t 
 }
 
 namespace {
-// Positions per CTA of the kernels that index rows of `width` positions of every path: few, short CTAs where the device
-// has room for all of them at once (16 x 700: 26 us, with 512 30 us).
-int bulk_chunk(const Dev& s, int width) {
-  const long long ctas = (long long)s.P * s.idx_n * ((width + kBulkChunk - 1) / kBulkChunk);
-  return ctas > 148LL * 8 ? kBulkChunk : kBulkChunk / 2;
+// The kernels that index rows of `width` positions of every path.  Few, short CTAs where the device has room for all of them at once
+// (16 x 700: 26 us, with 512 30 us).
+struct BulkPlan { int chunk, chunks, lengths; BulkForm form; };
+BulkPlan bulk_plan(const Dev& s, int width) {
+  BulkPlan b;
+  b.lengths = s.epochs || s.idx_n == 0 ? 1 : s.idx_n;
+  const bool many = (long long)s.P * b.lengths * ((width + kBulkChunk - 1) / kBulkChunk) > 148LL * 8;
+  b.chunk = many ? kBulkChunk : kBulkChunk / 2;
+  b.chunks = (width + b.chunk - 1) / b.chunk;
+  b.form = !s.epochs ? kPerLength : many ? kChainFull : kChain;
+  return b;
 }
 }  // namespace
 
 cudaError_t launch_trim(const Dev& s, int phase, const int32_t* keep, cudaStream_t stream) {
   if (phase == 0) return launch_overlapped(trim_shift_kernel, dim3(s.P), dim3(128), 0, stream, s, keep);
   if (phase == 1) return launch_overlapped(trim_clear_kernel, dim3(148 * 8), dim3(256), 0, stream, s);
-  const int chunk = bulk_chunk(s, s.L), chunks = (s.L + chunk - 1) / chunk;
-  return launch_overlapped(trim_reindex_kernel, dim3((unsigned)(s.P * chunks), s.idx_n), dim3(kBulkThreads), 0, stream, s, chunk, chunks);
+  const BulkPlan b = bulk_plan(s, s.L);
+  const auto kernel = b.form == kPerLength ? trim_reindex_kernel<kPerLength> : b.form == kChain ? trim_reindex_kernel<kChain> : trim_reindex_kernel<kChainFull>;
+  return launch_overlapped(kernel, dim3((unsigned)(s.P * b.chunks), b.lengths), dim3(kBulkThreads), 0, stream, s, b.chunk, b.chunks);
 }
 
 cudaError_t launch_append(const Dev& s, const int32_t* tokens, const float* logprobs, const int32_t* counts,
                           int row_width, cudaStream_t stream) {
   if (row_width < kBulkAppendFrom)
-    return launch_overlapped(append_kernel, dim3(s.P), dim3(128), 0, stream, s, tokens, logprobs, counts, row_width);
+    return launch_overlapped(s.epochs ? append_kernel<true> : append_kernel<false>, dim3(s.P), dim3(128), 0, stream, s, tokens, logprobs, counts, row_width);
   const cudaError_t e = launch_overlapped(append_plan_kernel, dim3(s.P), dim3(kPlanThreads), 0, stream, s, tokens, counts, row_width);
   if (e != cudaSuccess) return e;
   const int width = row_width < s.L ? row_width : s.L;                // no path takes more
-  const int chunk = bulk_chunk(s, width), chunks = (width + chunk - 1) / chunk;
-  return launch_overlapped(append_bulk_kernel, dim3((unsigned)(s.P * chunks), s.idx_n), dim3(kBulkThreads), 0, stream, s, tokens,
-                           logprobs, row_width, chunk, chunks);
+  const BulkPlan b = bulk_plan(s, width);
+  const auto kernel = b.form == kPerLength ? append_bulk_kernel<kPerLength> : b.form == kChain ? append_bulk_kernel<kChain> : append_bulk_kernel<kChainFull>;
+  return launch_overlapped(kernel, dim3((unsigned)(s.P * b.chunks), b.lengths), dim3(kBulkThreads), 0, stream, s, tokens, logprobs,
+                           row_width, b.chunk, b.chunks);
 }
 
 cudaError_t launch_accept(const Dev& s, const int32_t* draft_tok, const int32_t* draft_len,
                           const int32_t* sampled, const float* sampled_lp, int32_t* accept_len,
                           cudaStream_t stream) {
-  return launch_overlapped(accept_kernel, dim3(s.P), dim3(128), 0, stream, s, draft_tok, draft_len, sampled, sampled_lp,
+  return launch_overlapped(s.epochs ? accept_kernel<true> : accept_kernel<false>, dim3(s.P), dim3(128), 0, stream, s, draft_tok, draft_len, sampled, sampled_lp,
                            accept_len);
 }
 

@@ -106,8 +106,11 @@ __device__ __forceinline__ BucketHead bucket_cas(uint32_t* bucket, BucketHead ex
 // was never claimed (step of 16 x 1024: 13.1 us, with the look below 13.3).  On an index with epochs the bucket is looked at
 // first, together with the one behind it: one round trip decides between claim, count and moving on (commit of 256 x 8192:
 // 12.7 us by guessing on a cleared index, 14.7 by guessing with epochs, 9.3 by looking).
-template <bool BULK>
-__device__ __forceinline__ void index_insert(const Dev& s, int g, int n, uint64_t h, uint32_t lpos, uint32_t epoch, uint32_t* st) {
+// Returns whether the position got one of the bucket's places.
+// full(bucket number): BULK, whether the count of a bucket whose places are taken is kept elsewhere.
+struct CountNow { __device__ bool operator()(uint32_t) const { return false; } };
+template <bool BULK, bool CHAINED, class Full = CountNow>
+__device__ __forceinline__ bool index_insert(const Dev& s, int g, int n, uint64_t h, uint32_t lpos, uint32_t epoch, uint32_t* st, Full full = Full()) {
   uint32_t* table = index_table(s, g, n);
   const uint32_t tag = index_tag(h, epoch);
   uint32_t b = gram_bucket(h, s.table_cap);
@@ -122,36 +125,95 @@ __device__ __forceinline__ void index_insert(const Dev& s, int g, int n, uint64_
       old = v.x;
       if (bucket_empty((uint32_t)old, epoch)) {
         const BucketHead now = bucket_cas(bucket, BucketHead{v.x, v.y}, BucketHead{(1ull << 32) | tag, lpos});
-        if (now.head == v.x && now.pos == v.y) return;
+        if (now.head == v.x && now.pos == v.y) return true;
         old = now.head;
       }
-    } else if (!s.epochs) {
+    } else if (!CHAINED) {
       old = atomicCAS(head, 0ull, (1ull << 32) | tag);
-      if (old == 0ull) { bucket[2] = lpos; return; }
+      if (old == 0ull) { bucket[2] = lpos; return true; }
     } else {
       old = probe & 1u ? next : __ldcg(head);
       if (!(probe & 1u)) next = __ldcg(reinterpret_cast<const unsigned long long*>(table + (size_t)((b + 1) & (s.table_cap - 1)) * kBucketWords));
       if (bucket_empty((uint32_t)old, epoch)) {
         const unsigned long long seen = old;
         old = atomicCAS(head, seen, (1ull << 32) | tag);
-        if (old == seen) { bucket[2] = lpos; return; }
+        if (old == seen) { bucket[2] = lpos; return true; }
       }
     }
     if ((uint32_t)old == tag) {
-      if (BULK && (uint32_t)(old >> 32) >= (uint32_t)kInlineSlots) { atomicAdd(head, 1ull << 32); return; }
+      if (BULK && (uint32_t)(old >> 32) >= (uint32_t)kInlineSlots) {
+        if (!full(b)) atomicAdd(head, 1ull << 32);
+        return false;
+      }
       const uint32_t slot = (uint32_t)(atomicAdd(head, 1ull << 32) >> 32);
       if (slot < (uint32_t)kInlineSlots) bucket[2 + slot] = lpos;
-      return;
+      return slot < (uint32_t)kInlineSlots;
     }
     b = (b + 1) & (s.table_cap - 1);
   }
   *st |= SDMS_STATUS_INDEX_FULL;
+  return true;
+}
+
+// ---- chained index (s.epochs; CHAINED) --------------------------------------------------------------------------------
+// A position is listed once: in the bucket of the shortest n-gram ending at it that still had a place when it came.  It is
+// counted in the buckets it passes, and an n-gram has a bucket only if the one a token shorter has more than kInlineSlots
+// occurrences.  What a query of k tokens looks for is then in the buckets of its last 1, 2, .. k tokens (whoever ends in the same k
+// tokens passed the same buckets); only if the last one has more occurrences than places are there others.  Most n-grams of a
+// text are rare, so that a token costs one or two random sectors and not one per length (append of 32 x 16 x 3700 tokens, lengths up
+// to 5: 269 us with an entry per length, 118 now; 256 x 7800, up to 8: 497, 140; 16 x 128 x 3900, up to 4: 1017, 417; commit of 256 paths,
+// up to 8: 9.3, 5.9).
+// The commit of a step: all lengths of a position are looked at side by side, by a group of lanes of one warp, so that a
+// position costs one look and one claim however many buckets it passes.  active: the lane's n-gram exists (length n, at most n_max;
+// gram(n): its hash; it ends at lpos); lanes: those with the same position.  Whole warps.
+template <class Gram>
+__device__ __forceinline__ void chain_insert(const Dev& s, int g, bool active, int n, int n_max, Gram gram, uint32_t lpos, uint32_t epoch,
+                                             unsigned lanes, uint32_t* st) {
+  const uint64_t h = active ? gram(n) : 0ull;
+  const uint32_t tag = index_tag(h, epoch);
+  uint32_t* bucket = nullptr;
+  unsigned long long old = 0ull;
+  if (active) {
+    uint32_t* const table = index_table(s, g, n);
+    uint32_t b = gram_bucket(h, s.table_cap);
+    for (uint32_t probe = 0; probe < s.table_cap; probe += 2) {         // two buckets per round trip
+      uint32_t* const b0 = table + (size_t)b * kBucketWords;
+      uint32_t* const b1 = table + (size_t)((b + 1) & (s.table_cap - 1)) * kBucketWords;
+      const unsigned long long h0 = __ldcg(reinterpret_cast<const unsigned long long*>(b0));
+      const unsigned long long h1 = __ldcg(reinterpret_cast<const unsigned long long*>(b1));
+      bucket = b0; old = h0;
+      if ((uint32_t)old == tag || bucket_empty((uint32_t)old, epoch)) break;
+      bucket = b1; old = h1;
+      if ((uint32_t)old == tag || bucket_empty((uint32_t)old, epoch)) break;
+      b = (b + 2) & (s.table_cap - 1);
+    }
+  }
+  const bool mine = (uint32_t)old == tag;
+  const bool passes = active && mine && (uint32_t)(old >> 32) >= (uint32_t)kInlineSlots;
+  const unsigned stops = __ballot_sync(0xffffffffu, active && !passes) & lanes;
+  if (!active) return;
+  unsigned long long* const head = reinterpret_cast<unsigned long long*>(bucket);
+  const int first = stops ? __ffs(stops) - 1 : 32, lane = threadIdx.x & 31;
+  if (lane < first) { atomicAdd(head, 1ull << 32); return; }
+  if (lane > first) return;
+  if (mine) {
+    const uint32_t slot = (uint32_t)(atomicAdd(head, 1ull << 32) >> 32);
+    if (slot < (uint32_t)kInlineSlots) { bucket[2 + slot] = lpos; return; }
+    ++n;
+  } else if (bucket_empty((uint32_t)old, epoch) && atomicCAS(head, old, (1ull << 32) | tag) == old) {
+    bucket[2] = lpos;
+    return;
+  }
+  // others of this launch were faster: on from here, one length after the other
+  for (; n <= n_max; ++n)
+    if (index_insert<false, true>(s, g, n, gram(n), lpos, epoch, st)) return;
 }
 
 // Block-cooperative append of n validated tokens to path p whose length is len0.  rec is the
 // path's record as it was before the call (shared memory): rec[1 + t] = token at len0 - 1 - t.
 // Also writes the path's new record and length (and a copy of the record to rec_out, shared
 // memory, if given); no barrier inside.
+template <bool CHAINED>
 __device__ void append_tokens(const Dev& s, int p, int len0, int n, const int32_t* in_tok,
                               const float* in_lp, const int32_t* rec, uint32_t* st, int32_t* rec_out = nullptr) {
   int32_t* tok = s.tok + (size_t)p * s.L;
@@ -165,14 +227,26 @@ __device__ void append_tokens(const Dev& s, int p, int len0, int n, const int32_
   }
   const int g = p / s.N;
   const uint32_t lbase = (uint32_t)(p - g * s.N) * (uint32_t)s.L;
-  for (int w = threadIdx.x; w < n * s.idx_n; w += blockDim.x) {
-    const int a = w / s.idx_n, nn = w % s.idx_n + 1;
-    const int pos = len0 + a;
-    if (pos + 1 < nn) continue;
+  // old tokens from the record, new from the input
+  auto gram = [&](int pos, int nn) {
     uint64_t h = gram_init(nn);
-    for (int t = pos - nn + 1; t <= pos; ++t)
-      h = gram_step(h, t < len0 ? rec[len0 - t] : in_tok[t - len0]);   // old tokens from the record, new from the input
-    index_insert<false>(s, g, nn, gram_final(h), lbase + (uint32_t)pos, epoch_of(rec[kRecEpoch]), st);
+    for (int t = pos - nn + 1; t <= pos; ++t) h = gram_step(h, t < len0 ? rec[len0 - t] : in_tok[t - len0]);
+    return gram_final(h);
+  };
+  const uint32_t epoch = epoch_of(rec[kRecEpoch]);
+  if (CHAINED) {
+    const int lg = s.idx_n > 1 ? 32 - __clz(s.idx_n - 1) : 0, group = 1 << lg;      // lanes per position: at most 16
+    const unsigned lanes = ((1u << group) - 1u) << (threadIdx.x & 31 & ~(group - 1));
+    for (int w = threadIdx.x; (w & ~31) < n << lg; w += blockDim.x) {   // whole warps
+      const int a = w >> lg, nn = (w & (group - 1)) + 1, pos = len0 + a;
+      chain_insert(s, g, a < n && nn <= s.idx_n && pos + 1 >= nn, nn, min(s.idx_n, pos + 1), [&](int x) { return gram(pos, x); },
+                   lbase + (uint32_t)pos, epoch, lanes, st);
+    }
+  } else {
+    for (int w = threadIdx.x; w < n * s.idx_n; w += blockDim.x) {
+      const int a = w / s.idx_n, nn = w % s.idx_n + 1, pos = len0 + a;
+      if (pos + 1 >= nn) index_insert<false, false>(s, g, nn, gram(pos, nn), lbase + (uint32_t)pos, epoch, st);
+    }
   }
   // the record after the append: new length, then the newest k_max tokens
   int32_t* out = s.rec + (size_t)p * kRecWords;
@@ -193,10 +267,11 @@ __device__ void append_tokens(const Dev& s, int p, int len0, int n, const int32_
 // sampled[0 .. min(tau + 1, max_append)).  Block-cooperative, any block size >= 64; every thread of
 // the CTA must call it.  draft_tok / draft_len are only read.  If rec_out is given (shared memory,
 // kRecWords words) it receives the path's record as it is after the call.  next_k > 0 announces
-// the suffix length of the query the path makes next: its index bucket is prefetched into L2.
+// the suffix length of the query the path makes next (next_lo: the shortest it may back off to): its buckets are prefetched into L2.
+template <bool CHAINED>
 __device__ void accept_commit_phase(const Dev& s, int p, const int32_t* draft_tok, const int32_t* draft_len,
                                     const int32_t* sampled, const float* sampled_lp, int32_t* accept_len,
-                                    int32_t* rec_out = nullptr, int next_k = 0) {
+                                    int32_t* rec_out = nullptr, int next_k = 0, int next_lo = 0) {
   __shared__ int sh_len0, sh_n;
   __shared__ uint32_t sh_st;
   __shared__ int32_t sh_rec[kRecWords];
@@ -243,10 +318,9 @@ __device__ void accept_commit_phase(const Dev& s, int p, const int32_t* draft_to
   if (!sampled_lp) return;                            // uniform: check only
   __syncthreads();
   uint32_t st = 0;
-  if (next_k > 0 && s.eps == 0 && threadIdx.x == blockDim.x - 64) {
-    const int len0 = sh_len0, len1 = len0 + sh_n;
-    if (len1 >= next_k && len1 < s.L) {
-      const int nx = min(next_k, s.idx_n);               // the query's last nx tokens are what the index is asked for
+  if (next_k > 0 && s.eps == 0 && (threadIdx.x >> 5) == (blockDim.x >> 5) - 2) {     // a lane per n-gram length that will be looked up
+    const int len0 = sh_len0, len1 = len0 + sh_n, nx = (int)(threadIdx.x & 31) + 1;
+    if (nx <= min(next_k, s.idx_n) && nx >= (CHAINED ? 1 : min(next_lo, s.idx_n)) && len1 >= nx && len1 < s.L) {
       uint64_t h = gram_init(nx);
       for (int x = len1 - nx; x < len1; ++x) h = gram_step(h, x >= len0 ? sh_smp[x - len0] : sh_rec[len0 - x]);
       const uint32_t* bucket =
@@ -254,7 +328,7 @@ __device__ void accept_commit_phase(const Dev& s, int p, const int32_t* draft_to
       asm volatile("prefetch.global.L2 [%0];" ::"l"(bucket));
     }
   }
-  append_tokens(s, p, sh_len0, sh_n, sh_smp, sh_lp, sh_rec, &st, rec_out);
+  append_tokens<CHAINED>(s, p, sh_len0, sh_n, sh_smp, sh_lp, sh_rec, &st, rec_out);
   if (st) atomicOr(&sh_st, st);
   __syncthreads();
   if (threadIdx.x == 0 && sh_st) atomicOr(s.status, sh_st);

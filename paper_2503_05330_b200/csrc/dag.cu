@@ -1777,15 +1777,16 @@ __device__ void shared_scan(const Dev& s, int g, int k, int nq, const int32_t (*
 
 // SHARE: the code of the cluster-shared scan is compiled in (kernels for prompts below kShareMinTokens leave it
 // out: after a cold start the step fetches every instruction it may run past)
-template <bool EXPORT, bool SHARE>
+template <bool EXPORT, bool SHARE, bool CHAINED>
 __device__ void build_phase(const Dev& s, const Smem& sm, int k_hi, int k_lo, int32_t* draft_tok, int32_t* draft_len,
                             float* draft_score, float* draft_edge_w, int32_t* used_k,
                             const int32_t* own_rec = nullptr, int csize = 0) {
-  __shared__ int sh_mode, sh_M;
+  __shared__ int sh_M;
   __shared__ int32_t sh_pub[kPubWords];                     // this CTA's query as its cluster sees it: path, mode, tokens
   __shared__ int32_t sh_cq[kMaxClusterPaths][kPubWords];    // the scan queries of the cluster
   __shared__ int sh_nq;
-  __shared__ uint32_t sh_count, sh_pos[kInlineSlots];
+  __shared__ uint32_t sh_have[SDMS_MAX_K], sh_pos[SDMS_MAX_K][kInlineSlots];   // buckets of the path's last 1, 2, .. tokens: occurrences, positions
+  __shared__ int32_t sh_rec[kRecWords];
   __shared__ int32_t sh_q[SDMS_MAX_K];
   __shared__ int32_t sh_len[SDMS_MAX_PATHS_PER_GROUP];
   const int i = blockIdx.x, tid = threadIdx.x;
@@ -1795,71 +1796,76 @@ __device__ void build_phase(const Dev& s, const Smem& sm, int k_hi, int k_lo, in
   int32_t* my_matches = s.matches + (size_t)i * slice;
 
   write_defaults<EXPORT>(s, i, draft_tok, draft_score, draft_edge_w);
+  // The path's record: length and last tokens (newest first) in one 128-byte line (or the copy the caller already holds in
+  // shared memory).  Lane n - 1 looks up the path's last n tokens: the lengths that will be asked for, and, where the lengths are
+  // chained, all shorter ones.
+  if (tid >= (int)blockDim.x - 32) {                        // (the last warp: the first ones fetch lengths and write defaults)
+    const int lane = tid & 31;
+    const int32_t word = ldm((own_rec ? own_rec : s.rec + (size_t)i * kRecWords) + lane);
+    sh_rec[lane] = word;
+    __syncwarp();
+    const int n = lane + 1, len_i = sh_rec[0];
+    uint32_t have = 0u;
+    if (s.eps == 0 && len_i < s.L && n <= min(min(k_hi, s.idx_n), len_i) && (CHAINED || n >= min(k_lo, s.idx_n))) {
+      uint64_t h = gram_init(n);
+      for (int t = n; t >= 1; --t) h = gram_step(h, sh_rec[t]);
+      uint4 lo, hi;
+      if (find_bucket(s, g, n, gram_final(h), epoch_of(sh_rec[kRecEpoch]), &lo, &hi)) {
+        have = lo.y;
+        uint32_t* const pos = sh_pos[n - 1];
+        pos[0] = lo.z; pos[1] = lo.w; pos[2] = hi.x; pos[3] = hi.y; pos[4] = hi.z; pos[5] = hi.w;
+      }
+    }
+    if (n <= SDMS_MAX_K) sh_have[n - 1] = have;
+  }
   // the cluster shares its scans (same decision in every CTA of the launch)
   const bool share = SHARE && csize > 1 && k_lo == k_hi && s.eps == 0 && (s.L & 3) == 0 && slice >= kShareMinTokens;
+  if (tid == 0) sh_M = 0;
+  __syncthreads();
+  const int len_i = sh_rec[0];
   // With k_lo < k_hi the suffix length backs off: the longest k in [k_lo, k_hi] that has a match wins.
   int k = k_hi;
   for (;; --k) {
+  // the index is asked for the query's last nx tokens: all k of them unless the context keeps fewer tables
+  const int nx = min(k, s.idx_n);
+  int mode = Q_NONE;
+  if (len_i >= k && len_i < s.L) {
+    if (s.eps > 0) mode = Q_SCAN;                           // fuzzy matches are found by scanning only
+    else if (sh_have[CHAINED ? 0 : nx - 1] > 0u) mode = sh_have[nx - 1] <= (uint32_t)kInlineSlots ? Q_INLINE : Q_SCAN;
+  }
+  if (tid < k) sh_q[tid] = sh_rec[k - tid];
   if (tid == 0) {
-    // the path's record: length and last tokens (newest first) in one 128-byte line (or the copy
-    // the caller already holds in shared memory)
-    const int32_t* rec = own_rec ? own_rec : s.rec + (size_t)i * kRecWords;
-    const int len_i = ldm(rec);
-    int mode = Q_NONE;
-    uint32_t fp = 0, count = 0;
-    if (len_i >= k && len_i < s.L && s.eps > 0) {      // fuzzy matches are found by scanning only
-      for (int t = 0; t < k; ++t) sh_q[t] = ldm(rec + k - t);
-      mode = Q_SCAN;
-    } else if (len_i >= k && len_i < s.L) {
-      // the index is asked for the query's last nx tokens: all k of them unless the context keeps fewer tables
-      const int nx = min(k, s.idx_n);
-      uint64_t h = gram_init(nx);
-      for (int t = 0; t < k; ++t) { const int32_t x = ldm(rec + k - t); sh_q[t] = x; if (t >= k - nx) h = gram_step(h, x); }
-      h = gram_final(h);
-      const uint32_t epoch = epoch_of(ldm(rec + kRecEpoch));
-      fp = index_tag(h, epoch);
-      const uint32_t* table = index_table(s, g, nx);
-      uint32_t b = gram_bucket(h, s.table_cap);
-      for (uint32_t probe = 0; probe < s.table_cap; ++probe) {
-        const uint4* cand = reinterpret_cast<const uint4*>(table + (size_t)b * kBucketWords);
-        const uint4 lo = ldm(cand), hi = ldm(cand + 1);      // both halves in flight together
-        if (lo.x == fp) {
-          count = lo.y;
-          sh_pos[0] = lo.z; sh_pos[1] = lo.w; sh_pos[2] = hi.x; sh_pos[3] = hi.y; sh_pos[4] = hi.z; sh_pos[5] = hi.w;
-          mode = count <= (uint32_t)kInlineSlots ? Q_INLINE : Q_SCAN;
-          break;
-        }
-        if (bucket_empty(lo.x, epoch)) break;
-        b = (b + 1) & (s.table_cap - 1);
-      }
-    }
-    sh_mode = mode; sh_count = count; sh_M = 0;
-    s.q_fp[i] = fp; s.q_mode[i] = mode; s.q_reserved[i] = mode == Q_NONE ? 0 : slice; s.q_off[i] = i * slice;
+    s.q_mode[i] = mode; s.q_reserved[i] = mode == Q_NONE ? 0 : slice; s.q_off[i] = i * slice;
     if (share) {
       sh_pub[0] = i; sh_pub[1] = mode;
-      for (int t = 0; t < k; ++t) sh_pub[2 + t] = sh_q[t];
+      for (int t = 0; t < k; ++t) sh_pub[2 + t] = sh_rec[k - t];
       if (mode == Q_SCAN) s.q_cursor[i] = 0;              // the cluster's scanners count this query's matches here
     }
   }
-  __syncthreads();
-  const int mode = sh_mode;
   if (mode == Q_INLINE) {
-    if (tid < (int)sh_count) {
-      const uint32_t lpos = sh_pos[tid];
-      const int jn = (int)(lpos / (uint32_t)s.L);
-      const int j = g * s.N + jn;
-      const int e = (int)(lpos % (uint32_t)s.L);
-      if (j != i && e >= k - 1 && e <= sh_len[jn] - 2) {
-        const int32_t* c = s.tok + (size_t)j * s.L + (e - k + 1);
-        bool same = true;
-        for (int t = 0; t < k; ++t) same = same && (ldm(c + t) == sh_q[t]);
-        if (same) {
-          const int at = atomicAdd(&sh_M, 1);
-          sm.list[at] = j * s.L + e;
-          my_matches[at] = j * s.L + e;
+    // all occurrences of the n-gram stand in its bucket, or in that and those of the shorter ones
+    const int n0 = CHAINED ? 1 : nx;
+    if (tid < (nx - n0 + 1) * kInlineSlots) {
+      const int n = n0 + tid / kInlineSlots, slot = tid % kInlineSlots;
+      if (slot < (int)min(sh_have[n - 1], (uint32_t)kInlineSlots)) {
+        const uint32_t lpos = sh_pos[n - 1][slot];
+        const int jn = (int)(lpos / (uint32_t)s.L);
+        const int j = g * s.N + jn;
+        const int e = (int)(lpos % (uint32_t)s.L);
+        if (j != i && e >= k - 1 && e <= sh_len[jn] - 2) {
+          const int32_t* c = s.tok + (size_t)j * s.L + (e - k + 1);
+          bool same = true;
+          for (int t = 0; t < k; ++t) same = same && (ldm(c + t) == sh_rec[k - t]);
+          if (same) {
+            const int at = atomicAdd(&sh_M, 1);
+            sm.list[at] = j * s.L + e;
+            my_matches[at] = j * s.L + e;
+          }
         }
       }
     }
+  } else if (mode == Q_SCAN && !share) {
+    __syncthreads();                                        // the query's tokens
   }
   if (share) {
     cluster_sync_all();                                     // every query of the cluster is published
@@ -1897,7 +1903,7 @@ __device__ void build_phase(const Dev& s, const Smem& sm, int k_hi, int k_lo, in
   }
   __syncthreads();
   if (sh_M > 0 || k <= k_lo) break;
-  __syncthreads();                                   // everybody has read sh_M before the next probe resets it
+  __syncthreads();                                   // everybody has read sh_M before the next length adds to it
   }
   int M = sh_M;
   if (s.R > 0 && M > s.R) {                          // (uniform) the cap can only bite with more than R matches
@@ -1916,7 +1922,7 @@ __device__ void build_phase(const Dev& s, const Smem& sm, int k_hi, int k_lo, in
                     draft_len, draft_score, draft_edge_w);
 }
 
-template <bool EXPORT, bool SHARE>
+template <bool EXPORT, bool SHARE, bool CHAINED>
 __global__ void __launch_bounds__(kFusedThreads, 1) build_fused_kernel(Dev s, int k_hi, int k_lo, int32_t* draft_tok,
                                                                   int32_t* draft_len, float* draft_score,
                                                                   float* draft_edge_w, int32_t* used_k, int csize) {
@@ -1924,7 +1930,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) build_fused_kernel(Dev s, in
   grid_release();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const Smem sm = carve<EXPORT>(smem_raw);
-  build_phase<EXPORT, SHARE>(s, sm, k_hi, k_lo, draft_tok, draft_len, draft_score, draft_edge_w, used_k, nullptr, csize);
+  build_phase<EXPORT, SHARE, CHAINED>(s, sm, k_hi, k_lo, draft_tok, draft_len, draft_score, draft_edge_w, used_k, nullptr, csize);
 }
 
 // One launch per decode step.  The CTAs of a prompt form a thread-block cluster.  Each CTA first
@@ -1933,7 +1939,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) build_fused_kernel(Dev s, in
 // path of the prompt is up to date and each CTA builds its path's next draft.  draft_tok / draft_len
 // hold the previous drafts on entry and the new ones on exit.
 // k_lo < k: the suffix length backs off from k to k_lo (used_k, if given, receives each path's choice).
-template <bool SHARE>
+template <bool SHARE, bool CHAINED>
 __global__ void __launch_bounds__(kFusedThreads, 1) step_kernel(Dev s, int k, int k_lo, const int32_t* sampled,
                                                            const float* sampled_lp, int32_t* accept_len,
                                                            int32_t* draft_tok, int32_t* draft_len,
@@ -1944,10 +1950,10 @@ __global__ void __launch_bounds__(kFusedThreads, 1) step_kernel(Dev s, int k, in
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const Smem sm = carve<false>(smem_raw);
   __shared__ int32_t sh_own_rec[kRecWords];
-  accept_commit_phase(s, blockIdx.x, draft_tok, draft_len, sampled, sampled_lp, accept_len, sh_own_rec, k);
+  accept_commit_phase<CHAINED>(s, blockIdx.x, draft_tok, draft_len, sampled, sampled_lp, accept_len, sh_own_rec, k, k_lo);
   // every thread of every CTA of the cluster gets here exactly once (no early exit above)
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-  build_phase<false, SHARE>(s, sm, k, k_lo, draft_tok, draft_len, draft_score, draft_edge_w, used_k, sh_own_rec, s.N);
+  build_phase<false, SHARE, CHAINED>(s, sm, k, k_lo, draft_tok, draft_len, draft_score, draft_edge_w, used_k, sh_own_rec, s.N);
 }
 
 }  // namespace
@@ -1966,22 +1972,29 @@ static size_t fused_smem_bytes(const Dev& s) {
   return (long long)s.N * s.L >= kBigPoolFrom && s.pool == 0 && s.mode != 1 ? kBigPool : dag_smem_bytes<false>();
 }
 
+namespace {
+// Their instances: a context runs the one that has the code it needs (after a cold start a step fetches every instruction it may
+// run past: 0.15 us of 9.7 with the chained index's code in the step of an index that is not).
+auto build_variant(bool share, bool chained) {
+  return share ? (chained ? build_fused_kernel<false, true, true> : build_fused_kernel<false, true, false>)
+               : (chained ? build_fused_kernel<false, false, true> : build_fused_kernel<false, false, false>);
+}
+auto step_variant(bool share, bool chained) {
+  return share ? (chained ? step_kernel<true, true> : step_kernel<true, false>) : (chained ? step_kernel<false, true> : step_kernel<false, false>);
+}
+}  // namespace
+
 cudaError_t dag_kernel_setup() {
   cudaError_t e = cudaFuncSetAttribute(dag_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)dag_smem_bytes<false>());
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(dag_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)dag_smem_bytes<true>());
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(build_fused_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBigPool);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(build_fused_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBigPool);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(step_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBigPool);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(step_kernel<false>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(step_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBigPool);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(step_kernel<true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  for (int v = 0; v < 4 && e == cudaSuccess; ++v) {
+    e = cudaFuncSetAttribute(build_variant(v & 1, v & 2), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBigPool);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(step_variant(v & 1, v & 2), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBigPool);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(step_variant(v & 1, v & 2), cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  }
   return e;
 }
 
@@ -2005,7 +2018,7 @@ bool step_kernel_fits(const Dev& s) {
   step_launch_config(s, 0, &cfg, attr);
   cfg.numAttrs = 1;                                   // occupancy only looks at the cluster shape
   int clusters = 0;
-  if (cudaOccupancyMaxActiveClusters(&clusters, step_kernel<true>, &cfg) != cudaSuccess) { cudaGetLastError(); return false; }
+  if (cudaOccupancyMaxActiveClusters(&clusters, step_variant(true, s.epochs), &cfg) != cudaSuccess) { cudaGetLastError(); return false; }
   // every prompt's cluster resident at once: large clusters leave SMs of a GPC idle, and a launch whose
   // clusters queue up for the device is slower than the separate accept and build launches
   return (long long)clusters * s.N >= s.P;
@@ -2016,8 +2029,8 @@ cudaError_t launch_step(const Dev& s, int k, int k_lo, const int32_t* sampled, c
                         float* draft_edge_w, int32_t* used_k, cudaStream_t stream) {
   cudaLaunchConfig_t cfg; cudaLaunchAttribute attr[2];
   step_launch_config(s, stream, &cfg, attr);
-  const bool share = (s.L & 3) == 0 && (long long)s.N * s.L >= kShareMinTokens;       // the prompt is worth sharing its scan
-  return cudaLaunchKernelEx(&cfg, share ? step_kernel<true> : step_kernel<false>, s, k, k_lo, sampled, sampled_lp, accept_len,
+  const bool share = s.eps == 0 && (s.L & 3) == 0 && (long long)s.N * s.L >= kShareMinTokens;       // the prompt is worth sharing its scan
+  return cudaLaunchKernelEx(&cfg, step_variant(share, s.epochs), s, k, k_lo, sampled, sampled_lp, accept_len,
                             draft_tok, draft_len, draft_score, draft_edge_w, used_k);
 }
 
@@ -2046,7 +2059,7 @@ int build_cluster_size(const Dev& s) {
     attr[0].val.clusterDim.x = c; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr; cfg.numAttrs = 1;
     int clusters = 0;
-    if (cudaOccupancyMaxActiveClusters(&clusters, build_fused_kernel<false, true>, &cfg) != cudaSuccess) { cudaGetLastError(); continue; }
+    if (cudaOccupancyMaxActiveClusters(&clusters, build_variant(true, s.epochs), &cfg) != cudaSuccess) { cudaGetLastError(); continue; }
     if ((long long)clusters * c >= s.P) return c;
   }
   return 1;
@@ -2054,8 +2067,8 @@ int build_cluster_size(const Dev& s) {
 
 cudaError_t launch_build_fused(const Dev& s, int k_hi, int k_lo, int32_t* draft_tok, int32_t* draft_len,
                                float* draft_score, float* draft_edge_w, int32_t* used_k, cudaStream_t stream) {
-  if (s.build_cluster <= 1 || k_lo != k_hi)
-    return launch_overlapped(build_fused_kernel<false, false>, dim3(s.P), dim3(kFusedThreads), fused_smem_bytes(s), stream,
+  if (s.build_cluster <= 1 || k_lo != k_hi || s.eps > 0)
+    return launch_overlapped(build_variant(false, s.epochs), dim3(s.P), dim3(kFusedThreads), fused_smem_bytes(s), stream,
                              s, k_hi, k_lo, draft_tok, draft_len, draft_score, draft_edge_w, used_k, 0);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(s.P); cfg.blockDim = dim3(kFusedThreads);
@@ -2066,7 +2079,7 @@ cudaError_t launch_build_fused(const Dev& s, int k_hi, int k_lo, int32_t* draft_
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr; cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, build_fused_kernel<false, true>, s, k_hi, k_lo, draft_tok, draft_len, draft_score, draft_edge_w,
+  return cudaLaunchKernelEx(&cfg, build_variant(true, s.epochs), s, k_hi, k_lo, draft_tok, draft_len, draft_score, draft_edge_w,
                             used_k, (int)s.build_cluster);
 }
 

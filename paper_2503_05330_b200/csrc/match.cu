@@ -1,12 +1,12 @@
 // Cross-path suffix match (Eq. 3).
 //
-// probe_kernel : one thread per query path.  Hashes the path's last k tokens,
-//                finds the bucket of that k-gram in the prompt's table and reads
-//                its occurrence count.  The count is an upper bound on the number
-//                of matches, so it sizes the query's slice of the match list.
-//                Up to kInlineSlots occurrences are stored in the bucket itself:
-//                such queries are answered here, from one 32-byte sector.  The
-//                others are handed to the scan.
+// probe_kernel : one warp per query path.  Hashes the path's last k tokens (and, in
+//                a chained index, its last 1 .. k - 1), finds the buckets of those
+//                n-grams in the prompt's tables and reads their occurrence counts.
+//                Up to kInlineSlots occurrences are stored in a bucket itself: queries
+//                whose k-gram has no more are answered here, from a 32-byte sector per
+//                length.  For the others the counts size the query's slice of the match
+//                list, and they are handed to the scan.
 // scan_kernel  : the histories of a prompt are read once, in tiles, for all of
 //                its scan queries together.  A token is first tested against a
 //                bit table of the queries' last tokens; the few positions that
@@ -51,96 +51,113 @@ __device__ __forceinline__ long long block_exclusive_scan(long long v, long long
   return before + x - v;
 }
 
-// One warp per query path.  The path's record (length and newest tokens, one 128-byte line) gives the
-// query; the warp looks at four neighbouring buckets of the k-gram's table at a time (eight lanes per
-// bucket, one round trip).  A k-gram with at most kInlineSlots occurrences is answered here: lane sl
-// checks occurrence sl (other path, a follower exists, tokens equal) and the matches go to the
-// query's own kInlineArea slots at the front of the match list.  Any other query reserves as many slots
-// as the k-gram has occurrences behind that area (one atomic on a cursor that the build's last kernel
-// leaves at zero) and is handed to the scan.  Slices therefore lie in no particular order.
+// One warp per query path.  The path's record (length and newest tokens, one 128-byte line) gives the query; lane n - 1 looks
+// up the bucket of its last n tokens: only the longest length there are tables for, or all up to it where the lengths are
+// chained.  If that longest n-gram has at most kInlineSlots occurrences, all there are stand in the buckets: a lane each checks them
+// (other path, a follower exists, tokens equal) and the matches go to the query's own kInlineArea slots at the front of the
+// match list, or, if there are more, behind all those.  Any other query reserves as many slots there as the n-gram has occurrences
+// (one atomic on a cursor that the build's last kernel leaves at zero) and is handed to the scan.  Slices therefore lie in no
+// particular order.
 constexpr int kProbeWarps = 8;
 constexpr int kInlineArea = 8;
-static_assert(kInlineArea >= kInlineSlots && kRecWords == 32 && kBucketWords == 8, "lane layout of the probe");
+static_assert(kInlineArea >= kInlineSlots && kRecWords == 32 && kBucketWords == 8 && SDMS_MAX_K < 32, "lane layout of the probe");
 
 __global__ void __launch_bounds__(kProbeWarps * 32) probe_kernel(Dev s, int k, int skip_done) {
+  __shared__ uint32_t sh_pos[kProbeWarps][SDMS_MAX_K * kInlineSlots];
   grid_wait();
   grid_release();
-  const int lane = threadIdx.x & 31;
-  const int i = blockIdx.x * kProbeWarps + (threadIdx.x >> 5);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int i = blockIdx.x * kProbeWarps + warp;
   if (i >= s.P) return;                                          // whole warps
   if (skip_done && s.q_mode[i] == Q_DONE) return;                // back-off: this path has its matches from a longer suffix
   const int g = i / s.N;
   const int32_t mine = s.rec[(size_t)i * kRecWords + lane];
   const int len_i = __shfl_sync(FULL_MASK, mine, 0);
-  int mode = Q_NONE, written = 0, off = i * kInlineArea;
-  uint32_t fp = 0, count = 0;
+  int mode = Q_NONE, written = 0, reserved = 0, off = i * kInlineArea;
+  uint32_t fp = 0;
   if (len_i >= k && len_i < s.L) {
-    // the query, oldest token first: token x of it sits in lane k - x of the record
-    // fp names the whole k-gram (the scan looks queries up by it); the index is asked for the last nx tokens
-    const int nx = min(k, s.idx_n);
-    uint64_t h = gram_init(k), hx = gram_init(nx);
+    // token x of the query (oldest first) sits in lane k - x of the record.  fp names the whole k-gram (the scan looks queries up by it)
+    const int nx = min(k, s.idx_n), shortest = s.epochs ? 1 : nx, n = lane + 1;
+    uint64_t h = gram_init(k), hx = gram_init(n);
     for (int x = 0; x < k; ++x) {
       const int32_t t = __shfl_sync(FULL_MASK, mine, k - x);
       h = gram_step(h, t);
-      if (x >= k - nx) hx = gram_step(hx, t);
+      if (x >= k - n) hx = gram_step(hx, t);
     }
     fp = gram_fp(gram_final(h));
-    hx = gram_final(hx);
-    const uint32_t epoch = epoch_of(__shfl_sync(FULL_MASK, mine, kRecEpoch)), want = index_tag(hx, epoch);
-    const uint32_t* table = index_table(s, g, nx);
-    uint32_t b = gram_bucket(hx, s.table_cap);
-    int found = -1;                                              // lane that holds the bucket's first word
-    uint32_t word = 0;
-    for (uint32_t probe = 0; probe < s.table_cap && found < 0; probe += 4) {
-      const uint32_t bb = (b + (lane >> 3)) & (s.table_cap - 1);
-      word = table[(size_t)bb * kBucketWords + (lane & 7)];
-      bool end = false;
-      for (int r = 0; r < 4 && found < 0 && !end; ++r) {
-        const uint32_t w0 = __shfl_sync(FULL_MASK, word, 8 * r);
-        if (w0 == want) found = 8 * r;
-        else if (bucket_empty(w0, epoch)) end = true;
-      }
-      if (end) break;
-      b = (b + 4) & (s.table_cap - 1);
+    const uint32_t epoch = epoch_of(__shfl_sync(FULL_MASK, mine, kRecEpoch));
+    uint32_t have = 0u;
+    if (n >= shortest && n <= nx) {
+      uint4 lo, hi;
+      if (find_bucket(s, g, n, gram_final(hx), epoch, &lo, &hi)) have = lo.y;
+      uint32_t* const pos = sh_pos[warp] + (n - shortest) * kInlineSlots;
+      pos[0] = have > 0u ? lo.z : ~0u; pos[1] = have > 1u ? lo.w : ~0u; pos[2] = have > 2u ? hi.x : ~0u;
+      pos[3] = have > 3u ? hi.y : ~0u; pos[4] = have > 4u ? hi.z : ~0u; pos[5] = have > 5u ? hi.w : ~0u;
     }
-    if (found >= 0) {
-      count = __shfl_sync(FULL_MASK, word, found + 1);
-      mode = count <= (uint32_t)kInlineSlots ? Q_INLINE : Q_SCAN;
-      if (mode == Q_INLINE) {
-        const uint32_t lpos = __shfl_sync(FULL_MASK, word, found + 2 + (lane < kInlineSlots ? lane : 0));
-        bool same = false;
-        int gpos = 0;
-        if (lane < (int)count) {
-          const int jn = (int)(lpos / (uint32_t)s.L);
-          const int j = g * s.N + jn, e = (int)(lpos - (uint32_t)jn * (uint32_t)s.L);
-          gpos = j * s.L + e;
-          if (j != i && e >= k - 1) {
-            const int len_j = s.len[j];
-            const int32_t* c = s.tok + (size_t)j * s.L + (e - k + 1);
-            const int32_t* q = s.tok + (size_t)i * s.L + (len_i - k);
-            same = true;
-            for (int t = 0; t < k; ++t) same = same && (c[t] == q[t]);          // no early exit: the loads go out together
-            same = same && e <= len_j - 2;
-          }
-        }
-        const unsigned ok = __ballot_sync(FULL_MASK, same);
-        written = __popc(ok);
-        if ((long long)off + kInlineArea > s.match_cap) {
-          if (lane == 0) atomicOr(s.status, SDMS_STATUS_MATCH_OVERFLOW);
-          mode = Q_NONE; written = 0;
-        } else if (same) {
-          s.matches[off + __popc(ok & ((1u << lane) - 1u))] = gpos;
-        }
+    static_assert(kInlineSlots == 6, "the positions of a bucket");
+    __syncwarp();
+    const uint32_t count = __shfl_sync(FULL_MASK, have, nx - 1);
+    const int listed = __any_sync(FULL_MASK, have != 0u) ? (nx - shortest + 1) * kInlineSlots : 0;
+    if (listed) mode = count <= (uint32_t)kInlineSlots ? Q_INLINE : Q_SCAN;
+    // the listed positions: whether they match, or (for a query that will be scanned) end in the n-gram that was looked up at all
+    auto check = [&](int c, int* gpos) {
+      const uint32_t lpos = c < listed ? sh_pos[warp][c] : ~0u;
+      if (lpos == ~0u) return false;
+      const int jn = (int)(lpos / (uint32_t)s.L);
+      const int j = g * s.N + jn, e = (int)(lpos - (uint32_t)jn * (uint32_t)s.L);
+      *gpos = j * s.L + e;
+      if (j == i || e < k - 1) return false;
+      const int len_j = s.len[j];
+      const int32_t* t_j = s.tok + (size_t)j * s.L + (e - k + 1);
+      const int32_t* q = s.tok + (size_t)i * s.L + (len_i - k);
+      bool same = true;
+      for (int t = 0; t < k; ++t) same = same && (t_j[t] == q[t]);          // no early exit: the loads go out together
+      return same && e <= len_j - 2;
+    };
+    auto reserve = [&](int slots) {                               // behind the kInlineArea slots of all queries
+      long long at = 0;
+      if (lane == 0) at = (long long)atomicAdd(s.match_cursor, (unsigned long long)slots) + (long long)s.P * kInlineArea;
+      at = __shfl_sync(FULL_MASK, at, 0);
+      if (at + slots > s.match_cap) {
+        if (lane == 0) atomicOr(s.status, SDMS_STATUS_MATCH_OVERFLOW);
+        mode = Q_NONE;
+        return;
+      }
+      off = (int)at; reserved = slots;
+    };
+    if (mode != Q_NONE) {
+      // a query that will be scanned: the occurrences that stand in the buckets of shorter n-grams count for its slice too
+      const int to = mode == Q_SCAN ? listed - kInlineSlots : listed;
+      int gpos[3], found = 0;
+      bool same[3];
+      constexpr int kRounds = 3;
+      static_assert(kRounds * 32 >= SDMS_MAX_K * kInlineSlots, "every listed position has a lane");
+#pragma unroll
+      for (int r = 0; r < kRounds; ++r) {
+        const int c = r * 32 + lane;
+        gpos[r] = 0;
+        same[r] = r * 32 < to && c < to && check(c, &gpos[r]);
+        found += __popc(__ballot_sync(FULL_MASK, same[r]));
+      }
+      if (mode == Q_SCAN) {
+        reserve((int)count + found);
+        if (mode == Q_SCAN && lane == 0) atomicAdd(&s.g_nscan[g], 1);
       } else {
-        long long at = 0;
-        if (lane == 0) at = (long long)atomicAdd(s.match_cursor, (unsigned long long)count) + (long long)s.P * kInlineArea;
-        at = __shfl_sync(FULL_MASK, at, 0);
-        if (at + (long long)count > s.match_cap) {
+        if (found > kInlineArea) {
+          reserve(found);
+        } else if ((long long)off + kInlineArea > s.match_cap) {
           if (lane == 0) atomicOr(s.status, SDMS_STATUS_MATCH_OVERFLOW);
           mode = Q_NONE;
         } else {
-          off = (int)at;
-          if (lane == 0) atomicAdd(&s.g_nscan[g], 1);
+          reserved = kInlineArea;
+        }
+        if (mode == Q_INLINE) {
+#pragma unroll
+          for (int r = 0; r < kRounds; ++r) {
+            const unsigned ok = __ballot_sync(FULL_MASK, same[r]);
+            if (same[r]) s.matches[off + written + __popc(ok & ((1u << lane) - 1u))] = gpos[r];
+            written += __popc(ok);
+          }
         }
       }
     }
@@ -148,7 +165,7 @@ __global__ void __launch_bounds__(kProbeWarps * 32) probe_kernel(Dev s, int k, i
   if (lane == 0) {
     s.q_fp[i] = fp;
     s.q_mode[i] = mode;
-    s.q_reserved[i] = mode == Q_NONE ? 0 : (mode == Q_INLINE ? kInlineArea : (int32_t)count);
+    s.q_reserved[i] = reserved;
     s.q_off[i] = off;
     s.q_cursor[i] = written;
   }

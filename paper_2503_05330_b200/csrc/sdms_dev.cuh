@@ -48,7 +48,8 @@ struct Dev {
   int32_t eps;                         // edit-distance tolerance of the suffix match (0 or 1)
   int32_t fused;                       // one kernel per build (small prompts) instead of probe + scan + dag
   int32_t build_cluster;               // CTAs per cluster of the single-launch build (they share their prompt's scan); 1 = none
-  int32_t epochs;                      // a reset does not clear the index but moves on to the next epoch (1: large indexes)
+  int32_t epochs;                      // a large index: a reset does not clear it but moves on to the next epoch, and its n-gram lengths are
+                                       // chained (append_dev.cuh)
   int32_t R;                           // matches kept per (query path, source path): the R most recent; 0 = all
   double alpha;
   uint32_t table_cap;                  // buckets per (prompt, n) table, power of two
@@ -116,6 +117,22 @@ __device__ __forceinline__ uint32_t gram_bucket(uint64_t h, uint32_t cap) { retu
 
 __device__ __forceinline__ uint32_t* index_table(const Dev& s, int g, int n) {
   return s.index + ((size_t)(g * s.idx_n + (n - 1)) * s.table_cap) * kBucketWords;
+}
+
+// The bucket of the n-gram with hash h in the prompt's table, as two 16-byte words: false if there is none.  Ordinary loads: in the
+// one-launch step other CTAs write the index earlier in the same launch.
+__device__ __forceinline__ bool find_bucket(const Dev& s, int g, int n, uint64_t h, uint32_t epoch, uint4* lo, uint4* hi) {
+  const uint4* const table = reinterpret_cast<const uint4*>(index_table(s, g, n));
+  const uint32_t want = index_tag(h, epoch);
+  uint32_t b = gram_bucket(h, s.table_cap);
+#pragma unroll 1
+  for (uint32_t probe = 0; probe < s.table_cap; ++probe) {
+    *lo = table[2 * (size_t)b]; *hi = table[2 * (size_t)b + 1];        // both halves in flight together
+    if (lo->x == want) return true;
+    if (bucket_empty(lo->x, epoch)) return false;
+    b = (b + 1) & (s.table_cap - 1);
+  }
+  return false;
 }
 
 // Path (row of the store) a global position x = j * L + e lies in, without a division: L_magic =
