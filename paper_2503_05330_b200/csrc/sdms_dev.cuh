@@ -43,7 +43,7 @@ struct BeamEnt;
 // Everything a kernel needs, passed by value.
 struct Dev {
   int32_t G, N, L, V, k_max, D, max_append, B, Ke, mode, P;
-  int32_t idx_n;                       // n-gram lengths 1..idx_n have index tables (<= k_max)
+  int32_t idx_n;                       // n-gram lengths 1..idx_n have index tables (<= k_max; 0 with tolerance 1: nothing would look them up)
   int32_t pool;                        // 0 DAG, 1 tree, 2 list
   int32_t eps;                         // edit-distance tolerance of the suffix match (0 or 1)
   int32_t fused;                       // one kernel per build (small prompts) instead of probe + scan + dag
