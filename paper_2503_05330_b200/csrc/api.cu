@@ -13,7 +13,7 @@ constexpr size_t kEpochIndexBytes = 16 << 20;   // index from which a reset coun
 inline size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
 struct Layout {
-  size_t tok, pq, len, rec, status, index, q_fp, q_mode, q_reserved, q_off, q_cursor, match_cursor, g_nscan, g_trim, a_plan, matches, e_ctl;
+  size_t tok, pq, len, rec, status, index, q_fp, q_mode, q_reserved, q_off, q_cursor, match_cursor, f_notes, g_nscan, g_trim, a_plan, matches, e_ctl;
   size_t w_ctl, w_desc, w_done, w_tab, w_key, w_item, b_ent, b_ctl, bp_todo;
   bool wide_on;
   uint64_t w_slots;
@@ -77,6 +77,7 @@ Layout make_layout(const sdms_config* c) {
   l.q_fp = take(P * 4); l.q_mode = take(P * 4); l.q_reserved = take(P * 4);
   l.q_off = take(P * 4); l.q_cursor = take(P * 4);
   l.match_cursor = take(8);
+  l.f_notes = take(8);
   l.g_nscan = take((size_t)c->num_groups * 4);
   l.g_trim = take((size_t)c->num_groups * 4);
   l.a_plan = take(P * 8);
@@ -264,6 +265,7 @@ int sdms_create(const sdms_config* cfg, void* d_workspace, size_t bytes, sdms_ct
   d.q_fp = (uint32_t*)(w + lay.q_fp); d.q_mode = (int32_t*)(w + lay.q_mode);
   d.q_reserved = (int32_t*)(w + lay.q_reserved); d.q_off = (int32_t*)(w + lay.q_off);
   d.match_cursor = (unsigned long long*)(w + lay.match_cursor);
+  d.f_notes = (unsigned long long*)(w + lay.f_notes);
   d.q_cursor = (int32_t*)(w + lay.q_cursor); d.g_nscan = (int32_t*)(w + lay.g_nscan); d.g_trim = (int32_t*)(w + lay.g_trim);
   d.a_plan = (int2*)(w + lay.a_plan); d.e_ctl = (uint32_t*)(w + lay.e_ctl);
   d.matches = (int32_t*)(w + lay.matches);

@@ -5,9 +5,12 @@
 // many such positions there are, so the match slices are sized by counting first:
 //   fuzzy_prepare  every path with a query (k tokens, not full) is marked for scanning, counters zeroed
 //   fuzzy_scan     (count) one CTA per 512-token tile of one path j: positions that can end a match of
-//                  ANY query of the prompt are picked out by a bit table, then tested against every query
+//                  ANY query of the prompt are picked out by a bit table, then tested against every query;
+//                  what matches is counted, and noted as (query, position) in the last two thirds of the match list
 //   fuzzy_alloc    slices handed out from the match list by the counts
-//   fuzzy_scan     (fill) the same scan writes the positions
+//   fuzzy_fill     the positions go from the notes to the slices; only if the notes did not have room for all
+//                  matches, or slices would overlap them, does the same scan once more write the positions
+// (96 x 2500 tokens, sessions of seven builds: 511 us with a second scan in every build, 397 with the notes)
 // after which dag_kernel (and the wide pass) aggregate as for exact matching.
 //
 // The filter.  Let q be the query, |q| = k >= 2.  A window within one edit of q that ends at e either ends
@@ -32,11 +35,17 @@ constexpr int kFzHalo = SDMS_MAX_K + 1;            // tokens in front of a tile 
 constexpr int kFzBits = 65536;
 constexpr int kFzQueries = 128;                    // queries whose tokens are staged at a time
 
+// The notes of a build: pairs behind the first third of the match list.
+__device__ __forceinline__ int64_t fz_notes_from(const Dev& s) { return (s.match_cap / 3 + 1) & ~1ll; }
+__device__ __forceinline__ int64_t fz_notes_cap(const Dev& s) { return (s.match_cap - fz_notes_from(s)) / 2; }
+__device__ __forceinline__ int2* fz_notes(const Dev& s) { return reinterpret_cast<int2*>(s.matches + fz_notes_from(s)); }
+
 __device__ __forceinline__ uint32_t fz_bit(int32_t tok) { return ((uint32_t)tok * 2654435761u) >> 16; }
 
 __global__ void __launch_bounds__(256) fuzzy_prepare_kernel(Dev s, int k, int skip_done) {
   grid_wait();
   grid_release();
+  if (blockIdx.x == 0 && threadIdx.x == 0) *s.f_notes = 0ull;
   if (blockIdx.x == 0 && threadIdx.x < kWideCtlWords && s.w_grid) s.w_ctl[threadIdx.x] = 0ull;   // the wide pass of this build starts with an empty list
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= s.P) return;
@@ -62,6 +71,7 @@ __global__ void __launch_bounds__(256) fuzzy_alloc_kernel(Dev s) {
   }
 }
 
+// FILL: behind fuzzy_alloc; fills the slices from the notes if they are complete.
 template <bool FILL>
 __global__ void __launch_bounds__(kFzThreads) fuzzy_scan_kernel(Dev s, int k, int tiles) {
   __shared__ int32_t sh_tok[kFzHalo + kFzTile];            // sh_tok[kFzHalo + x] = token at t0 + x
@@ -76,7 +86,20 @@ __global__ void __launch_bounds__(kFzThreads) fuzzy_scan_kernel(Dev s, int k, in
   const int j = blockIdx.x / tiles, t0 = (blockIdx.x - j * tiles) * kFzTile;
   const int g = j / s.N, len_j = s.len[j];
   const int e_hi = min(t0 + kFzTile - 1, len_j - 2);        // last position of the tile with a follower
-  if (t0 > e_hi) {                                         // nothing to scan; but a launch none of whose CTAs waited would be over before
+  if (FILL) {
+    grid_wait();
+    grid_release();
+    const int64_t notes = (int64_t)*s.f_notes;
+    if (notes <= fz_notes_cap(s) && (int64_t)*s.match_cursor <= fz_notes_from(s)) {
+      for (int64_t x = (int64_t)blockIdx.x * kFzThreads + tid; x < notes; x += (int64_t)gridDim.x * kFzThreads) {
+        const int2 note = fz_notes(s)[x];
+        const int n = atomicAdd(&s.q_cursor[note.x], 1);
+        if (n < s.q_reserved[note.x]) s.matches[(size_t)s.q_off[note.x] + n] = note.y;
+      }
+      return;
+    }
+    if (t0 > e_hi) return;
+  } else if (t0 > e_hi) {                                         // nothing to scan; but a launch none of whose CTAs waited would be over before
     grid_wait();                                           // the kernel in front of it, and the one behind would not wait for that
     return;
   }
@@ -89,8 +112,12 @@ __global__ void __launch_bounds__(kFzThreads) fuzzy_scan_kernel(Dev s, int k, in
   if (tid == 0) sh_ncand = 0;
   // tokens and path lengths are older than the kernels this one follows (their CTAs let it start only after their own
   // wait): the tile was staged while those drained; the queries' state is read from here on
-  grid_wait();
-  grid_release();
+  if (!FILL) {
+    grid_wait();
+    grid_release();
+  }
+  // (earlier rounds of a back-off build have their slices at the front: they may reach into the notes)
+  const int64_t room = !FILL && (int64_t)*s.match_cursor <= fz_notes_from(s) ? fz_notes_cap(s) : 0;
   __syncthreads();
   // the tokens that can sit at the end of a match: the last two of every query of the prompt
   if (k >= 2)
@@ -140,15 +167,27 @@ __global__ void __launch_bounds__(kFzThreads) fuzzy_scan_kernel(Dev s, int k, in
     auto test = [&](int take) {
       __syncwarp();
       waiting -= take;
+      int hit = -1, at = 0;
       if (lane < take) {
         const int pair = sh_pair[warp][waiting + lane], pos = pair >> 8, q = pair & 255;
         if (k < 2 || one_edit_end(sh_tok + kFzHalo + pos, t0 + pos, sh_q[q], k)) {
+          hit = sh_qi[q];
           if (FILL) {
-            const int i = sh_qi[q], n = atomicAdd(&s.q_cursor[i], 1);
-            if (n < s.q_reserved[i]) s.matches[(size_t)s.q_off[i] + n] = j * s.L + t0 + pos;
+            const int n = atomicAdd(&s.q_cursor[hit], 1);
+            if (n < s.q_reserved[hit]) s.matches[(size_t)s.q_off[hit] + n] = j * s.L + t0 + pos;
           } else {
             atomicAdd(&sh_count[q], 1);
+            at = j * s.L + t0 + pos;
           }
+        }
+      }
+      if (!FILL) {
+        const unsigned hits = __ballot_sync(0xffffffffu, hit >= 0);
+        if (hits) {                                            // the warp's matches side by side
+          unsigned long long first = 0ull;
+          if (lane == 0) first = atomicAdd(s.f_notes, (unsigned long long)__popc(hits));
+          const int64_t note = (int64_t)__shfl_sync(0xffffffffu, first, 0) + __popc(hits & ((1u << lane) - 1u));
+          if (hit >= 0 && note < room) fz_notes(s)[note] = make_int2(hit, at);
         }
       }
       __syncwarp();

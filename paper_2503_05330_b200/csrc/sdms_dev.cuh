@@ -69,6 +69,7 @@ struct Dev {
   int32_t* q_off;                      // [P] start in `matches`
   int32_t* q_cursor;                   // [P] matches written
   unsigned long long* match_cursor;    // match slots handed to scan queries by the probe; zero between builds
+  unsigned long long* f_notes;         // tolerance 1 on large prompts: matches noted by the counting scan
   int32_t* g_nscan;                    // [G] queries of the prompt that need the scan; zero between builds
   uint32_t* e_ctl;                     // [2] the word kRecEpoch of every record; CTAs of a reset that are done
   int2* a_plan;                        // [P] an append of wide rows: tokens the path held before, tokens it takes
