@@ -110,11 +110,16 @@ typedef struct {
   int64_t  wide_table_bytes;     /* workspace set aside for node tables in global memory.  Two users: on
                                     prompts too large for the single-launch build, queries with more than 32
                                     (many paths: 64) matches are aggregated by all SMs together, in 16 * M * D bytes for M
-                                    matches (12 * M * D above 14336 of them, 7168 with alpha < 1); and
+                                    matches (12 * M * D above 14336 of them, 7168 with alpha < 1); on prompts of
+                                    the single-launch build from 65536 tokens (16384 with epsilon 1), up to 592
+                                    (296) paths in all, queries with more than 128 matches at k = 1 (epsilon 1:
+                                    k <= 2), if the pool is the DAG and neither beams nor search_mode 2 are asked
+                                    for; and
                                     sdms_get_beams (max_beams > 0) and search_mode 2 for paths whose tables
                                     do not fit shared memory, in slots of 40 + 16 * max(max_beams, 1) bytes.
                                     0 = default (room for every position
-                                    matching every query of its prompt, but at most 320 MiB), -1 = none.  A build
+                                    matching every query of its prompt, but at most 320 MiB, 64 MiB with the
+                                    single-launch build), -1 = none.  A build
                                     whose queries need more falls back to one thread block for those that
                                     did not fit, with the same results                                    */
   int32_t  index_max_n;          /* n-gram lengths the index keeps tables for: 1..index_max_n (0 = k_max, every
@@ -220,7 +225,7 @@ int sdms_accept(sdms_ctx* ctx, const int32_t* d_draft_tok, const int32_t* d_draf
  * single-launch build applies and the device can hold the clusters of all prompts
  * at once) the step is ONE kernel launch: the paths of a prompt commit, meet at a cluster
  * barrier, and build (search_mode 2 adds the launch that searches the paths with many
- * matches).  Otherwise the call issues the separate launches.
+ * matches, k = 1 on large prompts the one that aggregates them: wide_table_bytes).  Otherwise the call issues the separate launches.
  * sdms_step_is_single_launch reports which (1 / 0).
  */
 int sdms_step(sdms_ctx* ctx, int32_t k, const int32_t* d_sampled, const float* d_sampled_logprobs,

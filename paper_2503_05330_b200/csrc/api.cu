@@ -94,13 +94,16 @@ Layout make_layout(const sdms_config* c) {
   const bool fused = group_tokens <= kFusedMaxTokens && (int64_t)P * group_tokens <= mc;
   const int64_t stride = c->max_beams > 0 ? c->max_beams : (c->search_mode == 2 ? 1 : 0);   // continuations kept per node
   const int64_t slot_bytes = stride > 0 ? 40 + 16 * stride : 32;
-  l.wide_on = !fused && c->wide_table_bytes >= 0;
+  const bool hands_over = fused && stride == 0 && c->pool_mode == 0 && group_tokens >= (c->epsilon > 0 ? kHandOverTokensFuzzy : kHandOverTokens) &&
+                          (int64_t)P <= (c->epsilon > 0 ? kHandOverPathsFuzzy : kHandOverPaths);
+  l.wide_on = (!fused || hands_over) && c->wide_table_bytes >= 0;
   int64_t wide = c->wide_table_bytes;
   if (wide == 0) {
     // room for every position matching every query: up to 5 slots of a beam table per (match, layer), 16 bytes in the wide pass
     const int64_t items = (int64_t)D * (int64_t)c->paths_per_group * (int64_t)(P * L);
     wide = stride > 0 ? slot_bytes * 5 * items : 16 * (items + 4 * (int64_t)(D * P));
-    if (wide > (320LL << 20)) wide = 320LL << 20;
+    const int64_t most = hands_over ? kHandOverTable : 320LL << 20;
+    if (wide > most) wide = most;
   }
   l.w_slots = (l.wide_on || (stride > 0 && wide > 0)) ? (uint64_t)wide / slot_bytes : 0;
   l.w_ctl = take((size_t)kWideCtlWords * 8);
@@ -203,6 +206,17 @@ int timed(sdms_ctx* ctx, int kernel, cudaStream_t stream, F launch) {
     if (ctx->pending.size() >= kMaxPendingEvents) drain_pending(ctx, kMaxPendingEvents / 2);   // a long loop that never reads
   }
   return e == cudaSuccess ? SDMS_OK : SDMS_ERR_CUDA;
+}
+
+// The wide pass behind a single-launch build or step that hands queries over.
+int finish_handed_over(sdms_ctx* ctx, int32_t k, int32_t* draft_tok, int32_t* draft_len, float* draft_score, float* draft_edge_w,
+                       cudaStream_t stream) {
+  if (hand_over_from(ctx->dev, k, k) == 0) return SDMS_OK;
+  const int rc = timed(ctx, SDMS_KERNEL_DAG_WIDE, stream, [&] {
+    return launch_dag_wide(ctx->dev, draft_tok, draft_len, draft_score, draft_edge_w, stream); });
+  // (a list that was not worked off would be taken for the next build's)
+  if (rc != SDMS_OK) cudaMemsetAsync(ctx->dev.w_ctl, 0, (size_t)kWideCtlWords * 8, stream);
+  return rc;
 }
 
 }  // namespace
@@ -325,8 +339,9 @@ int sdms_build_drafts(sdms_ctx* ctx, int32_t k, int32_t* d_draft_tok, int32_t* d
   if (k < 1 || k > ctx->cfg.k_max) return SDMS_ERR_INVALID_ARG;
   cudaStream_t st = (cudaStream_t)stream;
   if (ctx->dev.fused) {
-    const int rc = timed(ctx, SDMS_KERNEL_BUILD_FUSED, st, [&] {
+    int rc = timed(ctx, SDMS_KERNEL_BUILD_FUSED, st, [&] {
       return launch_build_fused(ctx->dev, k, k, d_draft_tok, d_draft_len, d_draft_score, d_draft_edge_w, nullptr, st); });
+    if (rc == SDMS_OK) rc = finish_handed_over(ctx, k, d_draft_tok, d_draft_len, d_draft_score, d_draft_edge_w, st);
     if (rc != SDMS_OK) return rc;
     ctx->built = true;
     return finish_best_paths(ctx, d_draft_tok, d_draft_len, d_draft_score, d_draft_edge_w, st);
@@ -423,9 +438,10 @@ int sdms_step(sdms_ctx* ctx, int32_t k, const int32_t* d_sampled, const float* d
   }
   cudaStream_t st = (cudaStream_t)stream;
   ctx->built = false;
-  const int rc = timed(ctx, SDMS_KERNEL_STEP, st, [&] {
+  int rc = timed(ctx, SDMS_KERNEL_STEP, st, [&] {
     return launch_step(ctx->dev, k, k, d_sampled, d_sampled_logprobs, d_accept_len, d_draft_tok, d_draft_len,
                        d_draft_score, d_draft_edge_w, nullptr, st); });
+  if (rc == SDMS_OK) rc = finish_handed_over(ctx, k, d_draft_tok, d_draft_len, d_draft_score, d_draft_edge_w, st);
   if (rc != SDMS_OK) return rc;
   ctx->built = true;
   return finish_best_paths(ctx, d_draft_tok, d_draft_len, d_draft_score, d_draft_edge_w, st);

@@ -1780,7 +1780,7 @@ __device__ void shared_scan(const Dev& s, int g, int k, int nq, const int32_t (*
 template <bool EXPORT, bool SHARE, bool CHAINED>
 __device__ void build_phase(const Dev& s, const Smem& sm, int k_hi, int k_lo, int32_t* draft_tok, int32_t* draft_len,
                             float* draft_score, float* draft_edge_w, int32_t* used_k,
-                            const int32_t* own_rec = nullptr, int csize = 0) {
+                            const int32_t* own_rec, int csize, int hand) {
   __shared__ int sh_M;
   __shared__ int32_t sh_pub[kPubWords];                     // this CTA's query as its cluster sees it: path, mode, tokens
   __shared__ int32_t sh_cq[kMaxClusterPaths][kPubWords];    // the scan queries of the cluster
@@ -1918,6 +1918,8 @@ __device__ void build_phase(const Dev& s, const Smem& sm, int k_hi, int k_lo, in
     if (tid == 0) draft_len[i] = 0;
     return;
   }
+  if (hand > 0 && M > ((int)(blockIdx.x + s.w_grid) >= (int)gridDim.x ? hand : kHandOverEarly) && M <= wide_alone(s) && wide_register(s, i, M))
+    return;                                          // all SMs share the work (the launch that follows)
   dag_phase<EXPORT>(s, sm, i, M, M <= kListCap ? sm.list : my_matches, sh_len, g * s.N, sh_q[k - 1], draft_tok,
                     draft_len, draft_score, draft_edge_w);
 }
@@ -1925,12 +1927,12 @@ __device__ void build_phase(const Dev& s, const Smem& sm, int k_hi, int k_lo, in
 template <bool EXPORT, bool SHARE, bool CHAINED>
 __global__ void __launch_bounds__(kFusedThreads, 1) build_fused_kernel(Dev s, int k_hi, int k_lo, int32_t* draft_tok,
                                                                   int32_t* draft_len, float* draft_score,
-                                                                  float* draft_edge_w, int32_t* used_k, int csize) {
+                                                                  float* draft_edge_w, int32_t* used_k, int csize, int hand) {
   grid_wait();
   grid_release();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const Smem sm = carve<EXPORT>(smem_raw);
-  build_phase<EXPORT, SHARE, CHAINED>(s, sm, k_hi, k_lo, draft_tok, draft_len, draft_score, draft_edge_w, used_k, nullptr, csize);
+  build_phase<EXPORT, SHARE, CHAINED>(s, sm, k_hi, k_lo, draft_tok, draft_len, draft_score, draft_edge_w, used_k, nullptr, csize, hand);
 }
 
 // One launch per decode step.  The CTAs of a prompt form a thread-block cluster.  Each CTA first
@@ -1944,7 +1946,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) step_kernel(Dev s, int k, in
                                                            const float* sampled_lp, int32_t* accept_len,
                                                            int32_t* draft_tok, int32_t* draft_len,
                                                            float* draft_score, float* draft_edge_w,
-                                                           int32_t* used_k) {
+                                                           int32_t* used_k, int hand) {
   grid_wait();
   grid_release();
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1953,7 +1955,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) step_kernel(Dev s, int k, in
   accept_commit_phase<CHAINED>(s, blockIdx.x, draft_tok, draft_len, sampled, sampled_lp, accept_len, sh_own_rec, k, k_lo);
   // every thread of every CTA of the cluster gets here exactly once (no early exit above)
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-  build_phase<false, SHARE, CHAINED>(s, sm, k, k_lo, draft_tok, draft_len, draft_score, draft_edge_w, used_k, sh_own_rec, s.N);
+  build_phase<false, SHARE, CHAINED>(s, sm, k, k_lo, draft_tok, draft_len, draft_score, draft_edge_w, used_k, sh_own_rec, s.N, hand);
 }
 
 }  // namespace
@@ -1998,6 +2000,21 @@ cudaError_t dag_kernel_setup() {
   return e;
 }
 
+// Matches from which the single-launch build of suffix lengths k_lo .. k hands a query over to the wide pass; 0: it hands none over, and
+// is not followed by that pass.  A CTA walks a thousand matches in about 20 us, and the launch waits for the heaviest query; the pass
+// costs 1.3 us where there is nothing to do and 17 to 25 where there is.  Only the shortest suffixes have such queries: k = 1, with
+// tolerance 1 also k = 2.  Builds without / with it (us):
+//   k = 1, at most 4 rounds of CTAs, from 65536 tokens per prompt: 64 x 2048 83 / 51, 8 prompts of 16 x 4096 118 / 62, 16 x 4096 112 / 53,
+//     128 x 1024 212 / 71, 2 of 256 x 512 237 / 154, 8 of 16 x 8000 377 / 107, 32 of 16 x 4096 138 / 123; 4 of 128 x 512 100 / 101;
+//     32 of 32 x 2048 (1024 paths) 80 / 101: there the SMs are busy either way
+//     below: 16 of 32 x 1024 65 / 73, 16 of 16 x 2048 47 / 50, 16 x 1024 16 / 23
+//   tolerance 1, at most 2 rounds, from 16384 tokens, k = 2: 16 x 1024 48 / 35 (600 of 1024 tokens held: 33 / 34), 32 x 2048 110 / 64,
+//     8 of 32 x 1024 104 / 85; 32 of 16 x 1024 (512 paths) 72 / 94; 8 x 1024 17 / 19.  k = 3, with 284 matches at most, 46 / 52
+// Queries split by classes of tokens (above wide_alone() matches) stay: with tolerance 1 and k = 1 every query is one (32 x 2048: 5.8 / 6.3 ms).
+int hand_over_from(const Dev& s, int k, int k_lo) {
+  return s.fused && s.w_grid > 0 && k_lo == k && k <= (s.eps > 0 ? 2 : 1) ? kHandOverFrom : 0;
+}
+
 namespace {
 void step_launch_config(const Dev& s, cudaStream_t stream, cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr) {
   *cfg = cudaLaunchConfig_t{};
@@ -2031,7 +2048,7 @@ cudaError_t launch_step(const Dev& s, int k, int k_lo, const int32_t* sampled, c
   step_launch_config(s, stream, &cfg, attr);
   const bool share = s.eps == 0 && (s.L & 3) == 0 && (long long)s.N * s.L >= kShareMinTokens;       // the prompt is worth sharing its scan
   return cudaLaunchKernelEx(&cfg, step_variant(share, s.epochs), s, k, k_lo, sampled, sampled_lp, accept_len,
-                            draft_tok, draft_len, draft_score, draft_edge_w, used_k);
+                            draft_tok, draft_len, draft_score, draft_edge_w, used_k, hand_over_from(s, k, k_lo));
 }
 
 cudaError_t launch_dag(const Dev& s, bool with_export, int32_t* draft_tok, int32_t* draft_len, float* draft_score,
@@ -2069,7 +2086,7 @@ cudaError_t launch_build_fused(const Dev& s, int k_hi, int k_lo, int32_t* draft_
                                float* draft_score, float* draft_edge_w, int32_t* used_k, cudaStream_t stream) {
   if (s.build_cluster <= 1 || k_lo != k_hi || s.eps > 0)
     return launch_overlapped(build_variant(false, s.epochs), dim3(s.P), dim3(kFusedThreads), fused_smem_bytes(s), stream,
-                             s, k_hi, k_lo, draft_tok, draft_len, draft_score, draft_edge_w, used_k, 0);
+                             s, k_hi, k_lo, draft_tok, draft_len, draft_score, draft_edge_w, used_k, 0, hand_over_from(s, k_hi, k_lo));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(s.P); cfg.blockDim = dim3(kFusedThreads);
   cfg.dynamicSmemBytes = fused_smem_bytes(s); cfg.stream = stream;
@@ -2080,7 +2097,7 @@ cudaError_t launch_build_fused(const Dev& s, int k_hi, int k_lo, int32_t* draft_
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr; cfg.numAttrs = 2;
   return cudaLaunchKernelEx(&cfg, build_variant(true, s.epochs), s, k_hi, k_lo, draft_tok, draft_len, draft_score, draft_edge_w,
-                            used_k, (int)s.build_cluster);
+                            used_k, (int)s.build_cluster, hand_over_from(s, k_hi, k_lo));
 }
 
 }  // namespace sdms

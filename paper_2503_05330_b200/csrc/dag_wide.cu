@@ -974,12 +974,23 @@ __device__ __forceinline__ void wide_walk(const Dev& s, const int4 de, int class
   }
 }
 
+// The launch's last CTA leaves all counts at zero: the single-launch build that registers queries next has no kernel in front of
+// it that would.  By one thread of each CTA, once it has its last tickets.
+__device__ __forceinline__ void wide_counts_done(const Dev& s) {
+  __threadfence();
+  if (atomicAdd(&s.w_ctl[kWideCtlWords - 1], 1ull) == gridDim.x - 1)
+    for (int x = 0; x < kWideCtlWords; ++x) s.w_ctl[x] = 0ull;
+}
+
 __global__ void __launch_bounds__(kWideThreads, 1)
 dag_wide_kernel(Dev s, int32_t* __restrict__ draft_tok, int32_t* __restrict__ draft_len,
                 float* __restrict__ draft_score, float* __restrict__ draft_edge_w) {
   grid_wait();                                         // scheduled while dag_kernel drains; its list is complete from here on
   const u64 registered = ld_u64(&s.w_ctl[0]);
-  if (registered == 0) return;
+  if (registered == 0) {                               // (room may have been asked for in vain)
+    if (blockIdx.x == 0 && threadIdx.x == 0) s.w_ctl[1] = 0ull;
+    return;
+  }
   const int nq = (int)(registered < (u64)kMaxWide ? registered : (u64)kMaxWide);
   __shared__ int4 sh_desc[kMaxWide];
   __shared__ int sh_base[kMaxWide + 1];                // first task of each query: layers, or sums by classes
@@ -1103,7 +1114,7 @@ dag_wide_kernel(Dev s, int32_t* __restrict__ draft_tok, int32_t* __restrict__ dr
   }
   __syncthreads();
   if (!sh_last) {
-    if (tid == 0) atomicOr(s.status, SDMS_STATUS_TIMEOUT);
+    if (tid == 0) { atomicOr(s.status, SDMS_STATUS_TIMEOUT); wide_counts_done(s); }
     return;
   }
   __threadfence();
@@ -1146,6 +1157,7 @@ dag_wide_kernel(Dev s, int32_t* __restrict__ draft_tok, int32_t* __restrict__ dr
     task = sh_task;
     __syncthreads();
   }
+  if (tid == 0) wide_counts_done(s);
 }
 
 }  // namespace

@@ -19,10 +19,19 @@ constexpr int kMaxClusterPaths = 16;    // largest thread-block cluster (one CTA
 constexpr int kFusedThreads = 512;     // the single-launch build: more loads in flight while it scans
 constexpr int kDagCap = 1024;          // entries of the shared-memory node / edge tables
 constexpr int kFusedMaxTokens = 131072; // largest N*L a CTA scans on its own
+// The single-launch build's hand-over to the wide pass (hand_over_from, dag.cu): tokens N*L of a prompt from which, and paths up to which,
+// there is one (exact, tolerance 1).
+constexpr int kHandOverTokens = 65536, kHandOverPaths = 4 * 148;
+constexpr int kHandOverTokensFuzzy = 16384, kHandOverPathsFuzzy = 2 * 148;
+constexpr int64_t kHandOverTable = 64ll << 20;   // most bytes of table area taken for it by default: the queries that do not fit keep their CTA
+// Matches above which a query is handed over: 128 (256: 64 x 2048 53 us for 51, tolerance 1 36 to 46 for 34 to 41; 64: 46, but 113 for 108 with
+// 4 x 128 x 512); for a CTA that others wait for an SM behind, whose time is not the launch's, 512 (k = 1, 32 x 16 x 4096: 125 us from 256, 122
+// from 512, 126 from 1024, 144 from 2048; 4 x 64 x 2048: 65, 65, 73, 84).
+constexpr int kHandOverFrom = 128, kHandOverEarly = 512;
 constexpr int kMaxWide = 1024;          // queries one build can hand to the device-wide aggregation pass
 constexpr int kWideSumShift = 47;       // packed node sums: count in the upper 17 bits, sum of probabilities below
 constexpr int kWideMaxMatches = (1 << 17) - 1;   // so that both parts of a packed sum fit
-constexpr int kWideCtlWords = 5;
+constexpr int kWideCtlWords = 6;
 // b_ctl: table slots handed out, a count that stays zero (sdms_debug_wait_timeout waits for it), paths in bp_todo, paths dealt out, CTAs done
 enum BeamCtl : int { kBeamSlots = 0, kBeamNever = 1, kBeamTodo = 2, kBeamTicket = 3, kBeamDone = 4, kBeamCtlWords = 8 };
 
@@ -76,7 +85,8 @@ struct Dev {
   int32_t* g_trim;                     // [G] a path of the prompt was trimmed: its index is rebuilt
   int32_t* matches;                    // [match_cap] global positions j*L+e
   // device-wide aggregation of queries with many matches (dag_wide.cu); w_slots = 0: not in use
-  unsigned long long* w_ctl;           // [kWideCtlWords] queries registered, slots handed out, tasks handed out, chunks handed out, chunks done
+  unsigned long long* w_ctl;           // [kWideCtlWords] queries registered, slots handed out, tasks handed out, chunks handed out, chunks done, CTAs done;
+                                       // zero between builds
   int4* w_desc;                        // [kMaxWide] query path, matches, first slot, -
   int* w_done;                         // [kMaxWide][2] tasks of the query that are done, of these sums; zero between builds
   WideSlot* w_tab;                     // [w_slots]

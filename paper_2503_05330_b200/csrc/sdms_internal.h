@@ -37,6 +37,7 @@ cudaError_t launch_build_fused(const Dev& s, int k_hi, int k_lo, int32_t* draft_
                                float* draft_score, float* draft_edge_w, int32_t* used_k, cudaStream_t stream);
 // phase 0: shift the histories; 1: empty the index tables of the prompts that changed; 2: index them again
 cudaError_t launch_trim(const Dev& s, int phase, const int32_t* keep, cudaStream_t stream);
+int hand_over_from(const Dev& s, int k, int k_lo);
 bool step_kernel_fits(const Dev& s);
 int build_cluster_size(const Dev& s);
 cudaError_t launch_step(const Dev& s, int k, int k_lo, const int32_t* sampled, const float* sampled_lp,
