@@ -118,7 +118,7 @@ typedef struct {
                                     sdms_get_beams (max_beams > 0) and search_mode 2 for paths whose tables
                                     do not fit shared memory, in slots of 40 + 16 * max(max_beams, 1) bytes.
                                     0 = default (room for every position
-                                    matching every query of its prompt, but at most 320 MiB, 64 MiB with the
+                                    matching every query of its prompt, but at most 320 MiB, 32 MiB with the
                                     single-launch build), -1 = none.  A build
                                     whose queries need more falls back to one thread block for those that
                                     did not fit, with the same results                                    */
@@ -136,7 +136,7 @@ typedef struct {
 int sdms_workspace_bytes(const sdms_config* cfg, size_t* bytes);
 
 /* Create a context over caller-owned device memory.  Zero-fills the workspace on
- * the default stream and waits for it.  Starts with all paths empty. */
+ * the default stream and waits for it (its table area only where beams or search_mode 2 use it).  Starts with all paths empty. */
 int sdms_create(const sdms_config* cfg, void* d_workspace, size_t bytes, sdms_ctx** out);
 
 /* Forget every token (same effect as destroying and re-creating the context). */

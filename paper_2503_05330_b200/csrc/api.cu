@@ -241,7 +241,9 @@ int sdms_create(const sdms_config* cfg, void* d_workspace, size_t bytes, sdms_ct
   if (!d_workspace || ((uintptr_t)d_workspace & (kAlign - 1))) return SDMS_ERR_INVALID_ARG;
   if (bytes < lay.total) return SDMS_ERR_WORKSPACE_TOO_SMALL;
   if (dag_kernel_setup() != cudaSuccess || scan_kernel_setup() != cudaSuccess || beam_kernel_setup() != cudaSuccess) return SDMS_ERR_CUDA;
-  if (cudaMemsetAsync(d_workspace, 0, lay.total, 0) != cudaSuccess) return SDMS_ERR_CUDA;
+  // (the wide pass writes its table area before it reads it; beams want theirs empty)
+  const size_t clear = cfg->max_beams > 0 || cfg->search_mode == 2 ? lay.total : lay.w_tab;
+  if (cudaMemsetAsync(d_workspace, 0, clear, 0) != cudaSuccess) return SDMS_ERR_CUDA;
   if (cudaStreamSynchronize(0) != cudaSuccess) return SDMS_ERR_CUDA;
   sdms_ctx* ctx = new (std::nothrow) sdms_ctx();
   if (!ctx) return SDMS_ERR_BAD_STATE;

@@ -23,7 +23,7 @@ constexpr int kFusedMaxTokens = 131072; // largest N*L a CTA scans on its own
 // there is one (exact, tolerance 1).
 constexpr int kHandOverTokens = 65536, kHandOverPaths = 4 * 148;
 constexpr int kHandOverTokensFuzzy = 16384, kHandOverPathsFuzzy = 2 * 148;
-constexpr int64_t kHandOverTable = 64ll << 20;   // most bytes of table area taken for it by default: the queries that do not fit keep their CTA
+constexpr int64_t kHandOverTable = 32ll << 20;   // most bytes of table area taken for it by default: the queries that do not fit keep their CTA
 // Matches above which a query is handed over: 128 (256: 64 x 2048 53 us for 51, tolerance 1 36 to 46 for 34 to 41; 64: 46, but 113 for 108 with
 // 4 x 128 x 512); for a CTA that others wait for an SM behind, whose time is not the launch's, 512 (k = 1, 32 x 16 x 4096: 125 us from 256, 122
 // from 512, 126 from 1024, 144 from 2048; 4 x 64 x 2048: 65, 65, 73, 84).

@@ -32,7 +32,9 @@ def test_workspace_bytes_and_config_validation(lib):
     assert n >= 2 * 16 * 1024 * 4 + 4 * 2 * 16 * 1024 * 32
     assert n % 256 == 0
     assert binding.sdms_workspace_bytes(binding.make_config(1, 16, 1024, 128256, 4, 8, index_max_n=2)) < n - 2 * 2 * 16 * 1024 * 32 + 4096
-    assert binding.sdms_workspace_bytes(binding.make_config(1, 16, 1024, 128256, 4, 8, epsilon=1)) <= n - 4 * 2 * 16 * 1024 * 32   # no tables
+    assert binding.sdms_workspace_bytes(binding.make_config(1, 16, 1024, 128256, 4, 8, epsilon=1, wide_table_bytes=-1)) <= n - 4 * 2 * 16 * 1024 * 32   # no index
+    # (with a table area: at most the 32 MiB of the hand-over to the wide pass)
+    assert 0 < binding.sdms_workspace_bytes(binding.make_config(1, 16, 1024, 128256, 4, 8, epsilon=1)) <= n + (32 << 20)
     bigger = binding.make_config(1, 16, 1024, 128256, 4, 8, B=8, Ke=4)
     assert binding.sdms_workspace_bytes(bigger) > n
     bad = [dict(G=0), dict(N=0), dict(N=2000), dict(L=1), dict(V=0), dict(k_max=0), dict(k_max=17), dict(D=0),
