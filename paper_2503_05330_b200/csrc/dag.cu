@@ -1962,7 +1962,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) step_kernel(Dev s, int k, in
 
 // Dynamic shared memory of the single-launch kernels.  A CTA has its SM to itself (registers), so prompts with room for
 // thousands of matches take more for the walk over them (dag_walk; trees, lists and layer-wise search do not walk), small prompts
-// keep the cache.  An SM splits its 256 KB at 164, 196 and 228 KB: with 200 KB 28 KB of L1 are left, with 184 (and 10 KB
+// keep the cache.  (Figures of builds that hand nothing over, see hand_over_from.)  An SM splits its 256 KB at 164, 196 and 228 KB: with 200 KB 28 KB of L1 are left, with 184 (and 10 KB
 // of arrays) 60.  k = 1 builds of 64 x 2048 and 32 x 16 x 4096 tokens, queries of up to 4139 matches: 117 and 193 us with 200 KB, 98 and
 // 172 with 184, 124 and 206 with 106; alpha = 0.5, whose tables are a third larger, 144 and 222 / 127 and 206 / 125 and 205;
 // tree pools 126 and 197 with 200 KB, 101 and 175 with 106.  What loses: with alpha = 1, pools
