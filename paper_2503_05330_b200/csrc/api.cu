@@ -81,6 +81,7 @@ Layout make_layout(const sdms_config* c) {
   l.g_nscan = take((size_t)c->num_groups * 4);
   l.g_trim = take((size_t)c->num_groups * 4);
   l.a_plan = take(P * 8);
+  l.w_ctl = take((size_t)kWideCtlWords * 8);                           // (in front of the match list: a reset clears it)
   l.matches = take((size_t)mc * 4);
   l.e_ctl = take(8);
   l.x_draft_tok = take(P * D * 4); l.x_draft_len = take(P * 4);
@@ -106,7 +107,6 @@ Layout make_layout(const sdms_config* c) {
     if (wide > most) wide = most;
   }
   l.w_slots = (l.wide_on || (stride > 0 && wide > 0)) ? (uint64_t)wide / slot_bytes : 0;
-  l.w_ctl = take((size_t)kWideCtlWords * 8);
   l.b_ctl = take(kBeamCtlWords * 8);
   l.bp_todo = take(P * 4);
   l.w_desc = take(l.wide_on ? (size_t)kMaxWide * 16 : 0);
@@ -208,15 +208,18 @@ int timed(sdms_ctx* ctx, int kernel, cudaStream_t stream, F launch) {
   return e == cudaSuccess ? SDMS_OK : SDMS_ERR_CUDA;
 }
 
-// The wide pass behind a single-launch build or step that hands queries over.
-int finish_handed_over(sdms_ctx* ctx, int32_t k, int32_t* draft_tok, int32_t* draft_len, float* draft_score, float* draft_edge_w,
-                       cudaStream_t stream) {
-  if (hand_over_from(ctx->dev, k, k) == 0) return SDMS_OK;
-  const int rc = timed(ctx, SDMS_KERNEL_DAG_WIDE, stream, [&] {
-    return launch_dag_wide(ctx->dev, draft_tok, draft_len, draft_score, draft_edge_w, stream); });
-  // (a list that was not worked off would be taken for the next build's)
-  if (rc != SDMS_OK) cudaMemsetAsync(ctx->dev.w_ctl, 0, (size_t)kWideCtlWords * 8, stream);
-  return rc;
+// What follows a single-launch build or step of suffix lengths k_lo .. k.  The rule that told its kernel to hand heavy queries over
+// (hand_over_from) launches the wide pass here: one without the other would leave them without a draft.
+int finish_single_launch(sdms_ctx* ctx, int32_t k, int32_t k_lo, int32_t* draft_tok, int32_t* draft_len, float* draft_score,
+                         float* draft_edge_w, cudaStream_t stream) {
+  if (hand_over_from(ctx->dev, k, k_lo) > 0) {
+    const int rc = timed(ctx, SDMS_KERNEL_DAG_WIDE, stream, [&] {
+      return launch_dag_wide(ctx->dev, draft_tok, draft_len, draft_score, draft_edge_w, stream); });
+    // (a list that was not worked off would be taken for the next build's)
+    if (rc != SDMS_OK) { cudaMemsetAsync(ctx->dev.w_ctl, 0, (size_t)kWideCtlWords * 8, stream); return rc; }
+  }
+  ctx->built = true;
+  return finish_best_paths(ctx, draft_tok, draft_len, draft_score, draft_edge_w, stream);
 }
 
 }  // namespace
@@ -341,12 +344,10 @@ int sdms_build_drafts(sdms_ctx* ctx, int32_t k, int32_t* d_draft_tok, int32_t* d
   if (k < 1 || k > ctx->cfg.k_max) return SDMS_ERR_INVALID_ARG;
   cudaStream_t st = (cudaStream_t)stream;
   if (ctx->dev.fused) {
-    int rc = timed(ctx, SDMS_KERNEL_BUILD_FUSED, st, [&] {
+    const int rc = timed(ctx, SDMS_KERNEL_BUILD_FUSED, st, [&] {
       return launch_build_fused(ctx->dev, k, k, d_draft_tok, d_draft_len, d_draft_score, d_draft_edge_w, nullptr, st); });
-    if (rc == SDMS_OK) rc = finish_handed_over(ctx, k, d_draft_tok, d_draft_len, d_draft_score, d_draft_edge_w, st);
     if (rc != SDMS_OK) return rc;
-    ctx->built = true;
-    return finish_best_paths(ctx, d_draft_tok, d_draft_len, d_draft_score, d_draft_edge_w, st);
+    return finish_single_launch(ctx, k, k, d_draft_tok, d_draft_len, d_draft_score, d_draft_edge_w, st);
   }
   int rc;
   if (ctx->dev.eps > 0) {                            // matches with tolerance: sized by counting, four launches
@@ -402,8 +403,7 @@ int sdms_build_drafts_backoff(sdms_ctx* ctx, int32_t k_hi, int32_t* d_draft_tok,
   const int rc = timed(ctx, SDMS_KERNEL_BUILD_FUSED, st, [&] {
     return launch_build_fused(ctx->dev, k_hi, 1, d_draft_tok, d_draft_len, d_draft_score, d_draft_edge_w, d_used_k, st); });
   if (rc != SDMS_OK) return rc;
-  ctx->built = true;
-  return finish_best_paths(ctx, d_draft_tok, d_draft_len, d_draft_score, d_draft_edge_w, st);
+  return finish_single_launch(ctx, k_hi, 1, d_draft_tok, d_draft_len, d_draft_score, d_draft_edge_w, st);
 }
 
 int sdms_accept(sdms_ctx* ctx, const int32_t* d_draft_tok, const int32_t* d_draft_len, const int32_t* d_sampled,
@@ -440,13 +440,11 @@ int sdms_step(sdms_ctx* ctx, int32_t k, const int32_t* d_sampled, const float* d
   }
   cudaStream_t st = (cudaStream_t)stream;
   ctx->built = false;
-  int rc = timed(ctx, SDMS_KERNEL_STEP, st, [&] {
+  const int rc = timed(ctx, SDMS_KERNEL_STEP, st, [&] {
     return launch_step(ctx->dev, k, k, d_sampled, d_sampled_logprobs, d_accept_len, d_draft_tok, d_draft_len,
                        d_draft_score, d_draft_edge_w, nullptr, st); });
-  if (rc == SDMS_OK) rc = finish_handed_over(ctx, k, d_draft_tok, d_draft_len, d_draft_score, d_draft_edge_w, st);
   if (rc != SDMS_OK) return rc;
-  ctx->built = true;
-  return finish_best_paths(ctx, d_draft_tok, d_draft_len, d_draft_score, d_draft_edge_w, st);
+  return finish_single_launch(ctx, k, k, d_draft_tok, d_draft_len, d_draft_score, d_draft_edge_w, st);
 }
 
 int sdms_step_backoff(sdms_ctx* ctx, int32_t k_hi, const int32_t* d_sampled, const float* d_sampled_logprobs,
@@ -467,8 +465,7 @@ int sdms_step_backoff(sdms_ctx* ctx, int32_t k_hi, const int32_t* d_sampled, con
     return launch_step(ctx->dev, k_hi, 1, d_sampled, d_sampled_logprobs, d_accept_len, d_draft_tok, d_draft_len,
                        d_draft_score, d_draft_edge_w, d_used_k, st); });
   if (rc != SDMS_OK) return rc;
-  ctx->built = true;
-  return finish_best_paths(ctx, d_draft_tok, d_draft_len, d_draft_score, d_draft_edge_w, st);
+  return finish_single_launch(ctx, k_hi, 1, d_draft_tok, d_draft_len, d_draft_score, d_draft_edge_w, st);
 }
 
 int sdms_step_is_single_launch(sdms_ctx* ctx, int32_t* yes) {

@@ -3,7 +3,9 @@ more, k <= 2 with tolerance 1 from 16384): match counts around its limits, its f
 import numpy as np
 import pytest
 
-from harness import Pair, run_step_protocol
+from harness import Pair, run_step_protocol, t32
+from oracle import Oracle
+from paper_2503_05330_b200 import synth
 
 pytestmark = pytest.mark.gpu
 
@@ -76,3 +78,47 @@ def test_tolerance_one_at_its_shortest_suffixes():
     pair.append(tokens, lps, (L - 3 - (np.arange(G * N) * 3) % 29).astype(np.int32), expect_status=0)
     for k in (2, 1, 3, 2, 1):
         pair.build_and_compare(k)
+
+
+def backoff_step_and_compare(pair, sampled, sampled_lp):
+    """sdms_step_backoff with k_hi = 1 on both sides."""
+    tok, ln, _, _ = pair.o.drafts()
+    tau_o, st_o = pair.o.accept_commit(tok, ln, sampled, sampled_lp, pair.max_append)
+    pair.o.build_all(1)
+    pair.g.draft_score.fill_(7.0)
+    tau, gt, gl, gk = pair.g.step_backoff(1, t32(sampled, pair.dev), t32(sampled_lp, pair.dev))
+    assert pair.g.status() == st_o
+    tok, ln, sc, ew = pair.o.drafts()
+    assert np.array_equal(tau.cpu().numpy(), tau_o)
+    assert np.array_equal(gl.cpu().numpy(), ln) and np.array_equal(gt.cpu().numpy(), tok)
+    assert np.array_equal(gk.cpu().numpy(), [int(len(pair.o.matches(i)) > 0) for i in range(pair.P)])
+    np.testing.assert_allclose(pair.g.draft_score.cpu().numpy(), sc, rtol=1e-5, atol=0)
+    np.testing.assert_allclose(pair.g.draft_edge_w.cpu().numpy(), ew, rtol=1e-5, atol=0)
+
+
+@pytest.mark.parametrize("G,N,L,eps", [(1, 32, 2048, 0), (9, 40, 1640, 0), (1, 16, 4100, 0), (1, 16, 1026, 1)])
+def test_back_off_that_starts_at_one_token(G, N, L, eps):
+    # k_hi = 1 is a build of one suffix length: what its launch hands over is worked off behind it, and nothing of it is left for later builds
+    tokens, lps, lens, V = planted(G, N, L, 9100 + L)
+    if eps:                                                            # (every position matches: few enough for the wide pass)
+        lens = lens - L // 3
+    pair = Pair(G, N, L, V, 3, 6, eps=eps, max_append=6)
+    for again in range(2):
+        if again:
+            pair.g.reset()
+            pair.o = Oracle(G, N, L, V, 6, eps=eps)
+        pair.append(tokens, lps, lens - 40 * again, expect_status=0)
+        pair.g.draft_len.fill_(77)
+        pair.backoff_and_compare(1)
+        heavy = sum(len(pair.o.matches(i)) > 128 for i in range(G * N))
+        assert heavy > 0 if again == 0 else True
+        pair.build_and_compare(1)
+        pair.g.draft_len.fill_(77)
+        pair.backoff_and_compare(1)
+        pair.backoff_and_compare(3)
+        pair.build_and_compare(1)
+        for _ in range(3):
+            backoff_step_and_compare(pair, *synth.sampled_window(tokens, lps, pair.o.lengths(), 7))
+        pair.build_and_compare(2)
+        pair.g.draft_len.fill_(77)
+        pair.backoff_and_compare(1)                                    # (its list is what the reset finds)
