@@ -151,7 +151,7 @@ __device__ __forceinline__ void beams_of_query(const Dev& s, int i, int M, const
                           (d == 1 || __ldcg(item + (size_t)(d - 2) * M + m) == sh_bslot[d - 2]);
           const unsigned group = __ballot_sync(FULL, on);
           if (group == 0u) continue;
-          const u64 sum = group_sum(group, group, on ? (unsigned)__ldg(s.pq + list[m] + d) : 0u);
+          const u64 sum = group_sum(group, group, on ? (unsigned)ldm(s.pq + list[m] + d) : 0u);
           if ((tid & 31) == __ffs(group) - 1) atomicAdd(&sh_bedge[d - 1], ((u64)__popc(group) << kWideSumShift) | sum);
         }
       }
@@ -214,7 +214,7 @@ __device__ __forceinline__ void beams_in_shared(const Dev& s, const BeamPlan w, 
     unsigned p = 0u;
     if (m < M) {
       const int gpos = list[m], j = path_of(s, gpos);
-      if (l + 1 <= __ldg(s.len + j) - 1 - (gpos - j * s.L)) { v = __ldg(s.tok + gpos + l + 1); p = (unsigned)__ldg(s.pq + gpos + l + 1); }
+      if (l + 1 <= ldm(s.len + j) - 1 - (gpos - j * s.L)) { v = ldm(s.tok + gpos + l + 1); p = (unsigned)ldm(s.pq + gpos + l + 1); }
     }
     if (v >= 0) {
       unsigned h = ((unsigned)v * 2654435761u) >> shift;
@@ -353,7 +353,7 @@ __device__ __forceinline__ void beams_in_shared(const Dev& s, const BeamPlan w, 
         unsigned e0 = 0u, e1 = 0u, e2 = 0u;
         for (int m = lane; m < M; m += 32) {
           if (slot[l * stride + m] != sh_bslot[l] || (l > 0 && slot[(l - 1) * stride + m] != sh_bslot[l - 1])) continue;
-          const unsigned p = (unsigned)__ldg(s.pq + list[m] + l + 1);
+          const unsigned p = (unsigned)ldm(s.pq + list[m] + l + 1);
           e0 += p & 0xffffu; e1 += p >> 16; ++e2;
         }
         e0 = __reduce_add_sync(FULL, e0); e1 = __reduce_add_sync(FULL, e1); e2 = __reduce_add_sync(FULL, e2);

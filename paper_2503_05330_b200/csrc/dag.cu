@@ -43,12 +43,6 @@ constexpr int kLoadBatch = 4;          // candidates a thread loads before it to
 constexpr int kListCap = 2048;         // matches a fused CTA keeps in shared memory besides its global slice
 static_assert(kStageWords >= 4 * 32 * SDMS_MAX_DRAFT, "dag_small keeps its per-layer lanes in the staging area");
 
-// Loads of path state (tokens, probabilities, lengths, records, index buckets).  In the one-launch
-// step other CTAs write this state earlier in the same launch, so it is read with ordinary loads,
-// which a cluster-scope acquire keeps coherent, never through the read-only (non-coherent) path.
-template <class T>
-__device__ __forceinline__ T ldm(const T* p) { return *p; }
-
 struct Cand {            // a node or an edge competing in a selection
   double w; u64 S; unsigned cnt; int tok; int valid;
 };

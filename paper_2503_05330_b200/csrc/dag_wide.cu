@@ -127,8 +127,8 @@ __device__ __forceinline__ u64 wide_weight(const Dev& s, const WideTable& t, int
   const u64 S = ((u64)t.hi[h] << 15) + t.lo[h];
   return counts ? (u64)__double_as_longlong(eq5_weight(s.alpha, S, t.cnt[h])) : S;
 }
-// (The match list is read past L1 throughout: the kernel before this one still cuts it down in place, with a cap on the
-// matches per path, while CTAs of this one are resident.  Tokens, probabilities and lengths are older and go through __ldg.)
+// (The match list is read past L1 throughout: the kernel before this one still cuts it down in place, with a cap on the matches per
+// path, while CTAs of this one are resident.  So it does, if it is a step, with tokens, probabilities and lengths: ldm.)
 // Entries m0, m0 + kWideThreads, ... of a row (`none` where there is no candidate).
 template <int N>
 __device__ __forceinline__ void wide_row(const int* row, int M, int m0, int none, int (&v)[N]) {
@@ -153,7 +153,7 @@ __device__ __forceinline__ void wide_lay_out(const Dev& s, const int4 de, int c0
   if (m >= M) return;
   const WideItems items = wide_items(s, de.z, M);
   const int g = __ldcg(s.matches + s.q_off[de.x] + m), j = path_of(s, g);
-  const int n = min(l1, __ldg(s.len + j) - 1 - (g - j * s.L));         // followers
+  const int n = min(l1, ldm(s.len + j) - 1 - (g - j * s.L));         // followers
   const bool probs = M <= wide_alone(s);
   const int off = (g + 1) & 3;
   const int4* const st = reinterpret_cast<const int4*>(s.tok) + ((g + 1) >> 2);
@@ -165,7 +165,7 @@ __device__ __forceinline__ void wide_lay_out(const Dev& s, const int4 de, int c0
     for (int x = 0; x < 5; ++x) {
       a[x] = make_int4(0, 0, 0, 0); c[x] = a[x];
       const int at = lb + 4 * x - off;                                 // the first follower in them
-      if (at < n && at < lb + 16) { a[x] = __ldg(st + (lb >> 2) + x); c[x] = __ldg(sp + (lb >> 2) + x); }   // (only what holds a follower)
+      if (at < n && at < lb + 16) { a[x] = ldm(st + (lb >> 2) + x); c[x] = ldm(sp + (lb >> 2) + x); }   // (only what holds a follower)
     }
     int* tok = items.tok + (size_t)lb * items.pitch + m;
     int* p = reinterpret_cast<int*>(items.out + (size_t)lb * items.pitch) + m;
@@ -325,7 +325,7 @@ __device__ __forceinline__ void wide_layer(const Dev& s, const int4 de, int d) {
       for (int r = 0; r < N; ++r)
         if (best >> (c * N + r) & 1u) {
           const int m = (c * N + r) * kWideThreads + tid;
-          const unsigned q = (unsigned)(KEEP ? __ldcg(row_p + m) : __ldg(s.pq + __ldcg(list + m) + d));
+          const unsigned q = (unsigned)(KEEP ? __ldcg(row_p + m) : ldm(s.pq + __ldcg(list + m) + d));
           if (single) { lo += q & 0x7fffu; hi += q >> 15; }
           else {
             atomicAdd(&t.lo[slot[c][r]], q & 0x7fffu);
@@ -477,7 +477,7 @@ __device__ __forceinline__ void wide_sums(const Dev& s, const int4 de, int d, un
 #pragma unroll
       for (int r = 0; r < N; ++r) { v[r] = m[r] >= 0 ? __ldcg(row + m[r]) : -1; p[r] = m[r] >= 0 ? (unsigned)__ldcg(list + m[r]) : 0u; }
 #pragma unroll
-      for (int r = 0; r < N; ++r) p[r] = m[r] >= 0 ? (unsigned)__ldg(s.pq + (int)p[r] + d) : 0u;
+      for (int r = 0; r < N; ++r) p[r] = m[r] >= 0 ? (unsigned)ldm(s.pq + (int)p[r] + d) : 0u;
 #pragma unroll
       for (int r = 0; r < N; ++r) {
         if (x0 - tid + r * kWideThreads >= total) break;               // (the same for everybody)
@@ -645,7 +645,7 @@ __device__ __forceinline__ void wide_offers(const Dev& s, const int4 de, int d, 
     each([&](int r) {
       if (!top(r) || best_tok[h[r]] != ~(unsigned)v[r]) return false;
       named[h[r]] = m[r] + 1;                          // any one of them
-      const unsigned q = (unsigned)__ldg(s.pq + __ldcg(list + m[r]) + d);
+      const unsigned q = (unsigned)ldm(s.pq + __ldcg(list + m[r]) + d);
       atomicAdd(&e_lo[h[r]], q & 0x7fffu);
       atomicAdd(&e_hi[h[r]], q >> 15);
       atomicAdd(&e_cnt[h[r]], 1u);
@@ -702,7 +702,7 @@ __device__ __forceinline__ void wide_edges(const Dev& s, const WideItems& rows, 
         }
         unsigned p[4 * B];
 #pragma unroll
-        for (int y = 0; y < 4 * B; ++y) p[y] = g[y] >= 0 ? (unsigned)__ldg(s.pq + g[y] + l + 1) : 0u;
+        for (int y = 0; y < 4 * B; ++y) p[y] = g[y] >= 0 ? (unsigned)ldm(s.pq + g[y] + l + 1) : 0u;
 #pragma unroll
         for (int y = 0; y < 4 * B; ++y) { lo += p[y] & 0x7fffu; hi += p[y] >> 15; cnt += g[y] >= 0; }
       }
@@ -905,7 +905,7 @@ __device__ __forceinline__ void wide_walk_rows(const Dev& s, const int4 de, int 
 #pragma unroll
       for (int r = 0; r < B; ++r) g[r] = t[r] == tok ? __ldcg(list + m[r]) : -1;
 #pragma unroll
-      for (int r = 0; r < B; ++r) p[r] = g[r] >= 0 ? (unsigned)__ldg(s.pq + g[r] + d) : 0u;
+      for (int r = 0; r < B; ++r) p[r] = g[r] >= 0 ? (unsigned)ldm(s.pq + g[r] + d) : 0u;
 #pragma unroll
       for (int r = 0; r < B; ++r) { lo += p[r] & 0x7fffu; hi += p[r] >> 15; count += g[r] >= 0; }
     }

@@ -191,6 +191,12 @@ __device__ __forceinline__ bool one_edit_end(const int32_t* at, int e, const int
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// Loads of path state (tokens, probabilities, lengths, records, index buckets).  In the one-launch step other CTAs write this
+// state earlier in the same launch, and kernels that are launched over the step's end are resident while it still does: it is read
+// with ordinary loads, which a cluster-scope acquire or grid_wait() keeps coherent, never through the read-only (non-coherent) path.
+template <class T>
+__device__ __forceinline__ T ldm(const T* p) { return *p; }
+
 // Total order of the export and of the search: larger weight first, then smaller token.
 __device__ __forceinline__ bool ranks_before(double wa, int ta, double wb, int tb) {
   return wa > wb || (wa == wb && ta < tb);

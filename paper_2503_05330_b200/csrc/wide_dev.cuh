@@ -83,7 +83,7 @@ __device__ __forceinline__ void wide_insert_unit(const Dev& s, const int32_t* li
     if (ml < nm) {
       gpos = list[m0 + ml];
       const int j = path_of(s, gpos);
-      n_m = min(D, __ldg(s.len + j) - 1 - (gpos - j * s.L));
+      n_m = min(D, ldm(s.len + j) - 1 - (gpos - j * s.L));
     }
   for (int r0 = 0; d_first + r0 * kLayerWays <= D; r0 += kMaxRounds) {     // the same trip count for the whole warp
     const int d_base = d_first + r0 * kLayerWays;
@@ -93,7 +93,7 @@ __device__ __forceinline__ void wide_insert_unit(const Dev& s, const int32_t* li
     for (int r = 0; r < kMaxRounds; ++r) {            // every follower this thread needs is asked for before the first is used
       const int d = d_base + r * kLayerWays;
       v[r] = -1; p[r] = 0u;
-      if (d <= n_m && d <= D) { v[r] = __ldg(s.tok + gpos + d); p[r] = (unsigned)__ldg(s.pq + gpos + d); }
+      if (d <= n_m && d <= D) { v[r] = ldm(s.tok + gpos + d); p[r] = (unsigned)ldm(s.pq + gpos + d); }
     }
     // the key sector and the slot every follower hashes to are asked for now: when the rounds below get to
     // them (one after the other, the lanes of a warp in step) they are on their way from memory

@@ -122,3 +122,16 @@ def test_back_off_that_starts_at_one_token(G, N, L, eps):
         pair.build_and_compare(2)
         pair.g.draft_len.fill_(77)
         pair.backoff_and_compare(1)                                    # (its list is what the reset finds)
+
+
+def test_steps_of_prompts_whose_lengths_share_a_sector():
+    # the launch for the heavy queries is resident while the step in front of it commits lengths, tokens and probabilities
+    G, N, L = 2, 12, 5500
+    rng = np.random.default_rng(90)
+    tokens = np.minimum((rng.random((G * N, L)) ** 3 * 150).astype(np.int32), 149)
+    lps = (-rng.exponential(0.5, tokens.shape)).astype(np.float32)
+    pair = Pair(G, N, L, 150, 3, 7, max_append=7)
+    assert pair.g.step_is_single_launch()
+    start = (L - 80 - (np.arange(G * N) * 5) % 31).astype(np.int32)
+    st = run_step_protocol(pair, tokens, lps, [1, 1, 2], steps=20, warm=0, start_lens=start, check_every=5)
+    assert st["steps"] > 10

@@ -71,3 +71,12 @@ def test_create_rejects_bad_arguments_without_touching_the_device(lib):
     assert lib.sdms_append(None, None, None, None, 1, None) == binding.ERR_INVALID_ARG
     assert lib.sdms_strerror(binding.ERR_WORKSPACE_TOO_SMALL) == b"workspace too small"
     assert lib.sdms_kernel_name(2) == b"scan"
+
+
+def test_kernels_that_follow_a_step_do_not_read_path_state_as_read_only():
+    # they are resident while it commits (launch_overlapped): no load through the non-coherent path
+    csrc = os.path.join(ROOT, "paper_2503_05330_b200", "csrc")
+    for name in ("dag.cu", "dag_wide.cu", "beams.cu", "wide_dev.cuh", "beam_dev.cuh"):
+        with open(os.path.join(csrc, name)) as f:
+            text = f.read()
+        assert "__ldg" not in text and "ld.global.nc" not in text, name
