@@ -15,10 +15,11 @@ namespace sdms {
 
 namespace {
 
+// (What a call is given may be what the call before it wrote, drafts or accept lengths, and this kernel is resident while that still
+// does: no __restrict__ on inputs that are read behind grid_wait(), which would let them be read as read-only data.)
 template <bool CHAINED>
-__global__ void __launch_bounds__(128) append_kernel(Dev s, const int32_t* __restrict__ tokens,
-                                                     const float* __restrict__ logprobs,
-                                                     const int32_t* __restrict__ counts, int row_width) {
+__global__ void __launch_bounds__(128) append_kernel(Dev s, const int32_t* tokens, const float* logprobs, const int32_t* counts,
+                                                     int row_width) {
   grid_wait();
   grid_release();
   const int p = blockIdx.x;
@@ -66,8 +67,7 @@ constexpr int kBulkThreads = 256;
 constexpr int kBulkChunk = 512;          // most positions per CTA
 
 // What every path takes of its row: tokens held so far, tokens to append.
-__global__ void __launch_bounds__(kPlanThreads) append_plan_kernel(Dev s, const int32_t* __restrict__ tokens,
-                                                                   const int32_t* __restrict__ counts, int row_width) {
+__global__ void __launch_bounds__(kPlanThreads) append_plan_kernel(Dev s, const int32_t* tokens, const int32_t* counts, int row_width) {
   grid_wait();
   grid_release();
   __shared__ int sh_bad;
@@ -209,11 +209,8 @@ __global__ void __launch_bounds__(kBulkThreads, bulk_ctas(FORM)) append_bulk_ker
 }
 
 template <bool CHAINED>
-__global__ void __launch_bounds__(128) accept_kernel(Dev s, const int32_t* __restrict__ draft_tok,
-                                                     const int32_t* __restrict__ draft_len,
-                                                     const int32_t* __restrict__ sampled,
-                                                     const float* __restrict__ sampled_lp,
-                                                     int32_t* __restrict__ accept_len) {
+__global__ void __launch_bounds__(128) accept_kernel(Dev s, const int32_t* draft_tok, const int32_t* draft_len, const int32_t* sampled,
+                                                     const float* sampled_lp, int32_t* accept_len) {
   grid_wait();
   grid_release();
   accept_commit_phase<CHAINED>(s, blockIdx.x, draft_tok, draft_len, sampled, sampled_lp, accept_len);
@@ -242,7 +239,7 @@ __global__ void __launch_bounds__(256) reset_kernel(Dev s, uint4* a, size_t a_wo
 }
 
 // sdms_trim, first launch: path p keeps its newest keep[p] tokens, moved to the front of its store.
-__global__ void __launch_bounds__(128) trim_shift_kernel(Dev s, const int32_t* __restrict__ keep) {
+__global__ void __launch_bounds__(128) trim_shift_kernel(Dev s, const int32_t* keep) {
   grid_wait();
   grid_release();
   const int p = blockIdx.x;

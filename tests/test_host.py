@@ -80,3 +80,11 @@ def test_kernels_that_follow_a_step_do_not_read_path_state_as_read_only():
         with open(os.path.join(csrc, name)) as f:
             text = f.read()
         assert "__ldg" not in text and "ld.global.nc" not in text, name
+
+
+def test_inputs_that_another_call_may_still_write_are_not_declared_read_only():
+    with open(os.path.join(ROOT, "paper_2503_05330_b200", "csrc", "append.cu")) as f:
+        text = f.read()
+    for kernel in ("append_kernel", "append_plan_kernel", "accept_kernel", "trim_shift_kernel"):
+        params = re.search(kernel + r"\(Dev s,([^)]*)\) \{", text).group(1)
+        assert "__restrict__" not in params, kernel
