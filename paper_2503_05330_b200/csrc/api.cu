@@ -103,8 +103,15 @@ Layout make_layout(const sdms_config* c) {
     // room for every position matching every query: up to 5 slots of a beam table per (match, layer), 16 bytes in the wide pass
     const int64_t items = (int64_t)D * (int64_t)c->paths_per_group * (int64_t)(P * L);
     wide = stride > 0 ? slot_bytes * 5 * items : 16 * (items + 4 * (int64_t)(D * P));
-    const int64_t most = hands_over ? kHandOverTable : 320LL << 20;
-    if (wide > most) wide = most;
+    if (hands_over) {
+      // Matches of all queries handed over: at k = 1 paths * tokens of a prompt * the sum of the tokens' squared frequencies, which is 1/110
+      // and less in streams with much in common (tolerance 1, k = 2: 1/60).  Room for 1/64 (1/16), and for a few of the largest.
+      const int64_t largest = 14336, few = (int64_t)(P < 8 ? P : 8) * (group_tokens < largest ? group_tokens : largest);
+      const int64_t matches = (int64_t)P * group_tokens / (c->epsilon > 0 ? 16 : 64);
+      const int64_t most = 16 * (int64_t)D * (matches > few ? matches : few);
+      if (wide > most) wide = most;
+    }
+    if (wide > (320LL << 20)) wide = 320LL << 20;
   }
   l.w_slots = (l.wide_on || (stride > 0 && wide > 0)) ? (uint64_t)wide / slot_bytes : 0;
   l.b_ctl = take(kBeamCtlWords * 8);
@@ -208,11 +215,14 @@ int timed(sdms_ctx* ctx, int kernel, cudaStream_t stream, F launch) {
   return e == cudaSuccess ? SDMS_OK : SDMS_ERR_CUDA;
 }
 
-// What follows a single-launch build or step of suffix lengths k_lo .. k.  The rule that told its kernel to hand heavy queries over
-// (hand_over_from) launches the wide pass here: one without the other would leave them without a draft.
-int finish_single_launch(sdms_ctx* ctx, int32_t k, int32_t k_lo, int32_t* draft_tok, int32_t* draft_len, float* draft_score,
-                         float* draft_edge_w, cudaStream_t stream) {
-  if (hand_over_from(ctx->dev, k, k_lo) > 0) {
+// Every path may have grown by n tokens.
+void grows(sdms_ctx* ctx, int32_t n) { ctx->dev.held = n < ctx->dev.L - ctx->dev.held ? ctx->dev.held + n : ctx->dev.L; }
+
+// What follows a single-launch build or step.  hand: what its kernel was told (hand_over_from); whom that hands over to the wide pass
+// would be without a draft if it were not launched here.
+int finish_single_launch(sdms_ctx* ctx, int hand, int32_t* draft_tok, int32_t* draft_len, float* draft_score, float* draft_edge_w,
+                         cudaStream_t stream) {
+  if (hand > 0) {
     const int rc = timed(ctx, SDMS_KERNEL_DAG_WIDE, stream, [&] {
       return launch_dag_wide(ctx->dev, draft_tok, draft_len, draft_score, draft_edge_w, stream); });
     // (a list that was not worked off would be taken for the next build's)
@@ -276,6 +286,7 @@ int sdms_create(const sdms_config* cfg, void* d_workspace, size_t bytes, sdms_ct
   d.eps = cfg->epsilon;
   d.pool = cfg->pool_mode;
   d.R = cfg->max_matches_per_path;
+  d.held = 0;
   d.epochs = lay.q_fp - lay.index >= kEpochIndexBytes;
   ctx->step_fits = false;                        // decided below, once the kernels' attributes are set
   unsigned char* w = ctx->ws;
@@ -311,6 +322,7 @@ int sdms_reset(sdms_ctx* ctx, void* stream) {
   // the path store need not be cleared: lengths say what is valid
   const Layout& l = ctx->lay;
   ctx->built = false;
+  ctx->dev.held = 0;
   // a large index is not cleared: its buckets go out of date with the epoch
   if (ctx->dev.epochs) {
     ++ctx->launches;
@@ -333,6 +345,7 @@ int sdms_append(sdms_ctx* ctx, const int32_t* d_tokens, const float* d_logprobs,
   if (!ctx || !d_tokens || !d_logprobs || !d_counts || row_width < 1) return SDMS_ERR_INVALID_ARG;
   cudaStream_t st = (cudaStream_t)stream;
   ctx->built = false;
+  grows(ctx, row_width);
   if (row_width >= kBulkAppendFrom) ++ctx->launches;   // two launches
   return timed(ctx, SDMS_KERNEL_APPEND, st,
                [&] { return launch_append(ctx->dev, d_tokens, d_logprobs, d_counts, row_width, st); });
@@ -344,10 +357,11 @@ int sdms_build_drafts(sdms_ctx* ctx, int32_t k, int32_t* d_draft_tok, int32_t* d
   if (k < 1 || k > ctx->cfg.k_max) return SDMS_ERR_INVALID_ARG;
   cudaStream_t st = (cudaStream_t)stream;
   if (ctx->dev.fused) {
+    const int hand = hand_over_from(ctx->dev, k, k, st);
     const int rc = timed(ctx, SDMS_KERNEL_BUILD_FUSED, st, [&] {
-      return launch_build_fused(ctx->dev, k, k, d_draft_tok, d_draft_len, d_draft_score, d_draft_edge_w, nullptr, st); });
+      return launch_build_fused(ctx->dev, k, k, d_draft_tok, d_draft_len, d_draft_score, d_draft_edge_w, nullptr, hand, st); });
     if (rc != SDMS_OK) return rc;
-    return finish_single_launch(ctx, k, k, d_draft_tok, d_draft_len, d_draft_score, d_draft_edge_w, st);
+    return finish_single_launch(ctx, hand, d_draft_tok, d_draft_len, d_draft_score, d_draft_edge_w, st);
   }
   int rc;
   if (ctx->dev.eps > 0) {                            // matches with tolerance: sized by counting, four launches
@@ -400,17 +414,18 @@ int sdms_build_drafts_backoff(sdms_ctx* ctx, int32_t k_hi, int32_t* d_draft_tok,
     ctx->built = true;
     return SDMS_OK;
   }
+  const int hand = hand_over_from(ctx->dev, k_hi, 1, st);
   const int rc = timed(ctx, SDMS_KERNEL_BUILD_FUSED, st, [&] {
-    return launch_build_fused(ctx->dev, k_hi, 1, d_draft_tok, d_draft_len, d_draft_score, d_draft_edge_w, d_used_k, st); });
+    return launch_build_fused(ctx->dev, k_hi, 1, d_draft_tok, d_draft_len, d_draft_score, d_draft_edge_w, d_used_k, hand, st); });
   if (rc != SDMS_OK) return rc;
-  return finish_single_launch(ctx, k_hi, 1, d_draft_tok, d_draft_len, d_draft_score, d_draft_edge_w, st);
+  return finish_single_launch(ctx, hand, d_draft_tok, d_draft_len, d_draft_score, d_draft_edge_w, st);
 }
 
 int sdms_accept(sdms_ctx* ctx, const int32_t* d_draft_tok, const int32_t* d_draft_len, const int32_t* d_sampled,
                 const float* d_sampled_logprobs, int32_t* d_accept_len, void* stream) {
   if (!ctx || !d_draft_tok || !d_draft_len || !d_sampled || !d_accept_len) return SDMS_ERR_INVALID_ARG;
   cudaStream_t st = (cudaStream_t)stream;
-  if (d_sampled_logprobs) ctx->built = false;          // the commit changes the histories
+  if (d_sampled_logprobs) { ctx->built = false; grows(ctx, ctx->dev.max_append); }          // the commit changes the histories
   return timed(ctx, SDMS_KERNEL_ACCEPT, st, [&] {
     return launch_accept(ctx->dev, d_draft_tok, d_draft_len, d_sampled, d_sampled_logprobs, d_accept_len, st); });
 }
@@ -440,11 +455,13 @@ int sdms_step(sdms_ctx* ctx, int32_t k, const int32_t* d_sampled, const float* d
   }
   cudaStream_t st = (cudaStream_t)stream;
   ctx->built = false;
+  grows(ctx, ctx->dev.max_append);
+  const int hand = hand_over_from(ctx->dev, k, k, st);
   const int rc = timed(ctx, SDMS_KERNEL_STEP, st, [&] {
     return launch_step(ctx->dev, k, k, d_sampled, d_sampled_logprobs, d_accept_len, d_draft_tok, d_draft_len,
-                       d_draft_score, d_draft_edge_w, nullptr, st); });
+                       d_draft_score, d_draft_edge_w, nullptr, hand, st); });
   if (rc != SDMS_OK) return rc;
-  return finish_single_launch(ctx, k, k, d_draft_tok, d_draft_len, d_draft_score, d_draft_edge_w, st);
+  return finish_single_launch(ctx, hand, d_draft_tok, d_draft_len, d_draft_score, d_draft_edge_w, st);
 }
 
 int sdms_step_backoff(sdms_ctx* ctx, int32_t k_hi, const int32_t* d_sampled, const float* d_sampled_logprobs,
@@ -461,11 +478,13 @@ int sdms_step_backoff(sdms_ctx* ctx, int32_t k_hi, const int32_t* d_sampled, con
   }
   cudaStream_t st = (cudaStream_t)stream;
   ctx->built = false;
+  grows(ctx, ctx->dev.max_append);
+  const int hand = hand_over_from(ctx->dev, k_hi, 1, st);
   const int rc = timed(ctx, SDMS_KERNEL_STEP, st, [&] {
     return launch_step(ctx->dev, k_hi, 1, d_sampled, d_sampled_logprobs, d_accept_len, d_draft_tok, d_draft_len,
-                       d_draft_score, d_draft_edge_w, d_used_k, st); });
+                       d_draft_score, d_draft_edge_w, d_used_k, hand, st); });
   if (rc != SDMS_OK) return rc;
-  return finish_single_launch(ctx, k_hi, 1, d_draft_tok, d_draft_len, d_draft_score, d_draft_edge_w, st);
+  return finish_single_launch(ctx, hand, d_draft_tok, d_draft_len, d_draft_score, d_draft_edge_w, st);
 }
 
 int sdms_step_is_single_launch(sdms_ctx* ctx, int32_t* yes) {

@@ -1769,6 +1769,41 @@ __device__ void shared_scan(const Dev& s, int g, int k, int nq, const int32_t (*
   }
 }
 
+// ---- hand-over of heavy queries to the wide pass (hand_over_from) ----------------------------------------
+// Is the pass worth its while for this build (exact matches, k = 1)?  Without it the launch waits for the walk of the heaviest query, `most` matches;
+// the pass has its fixed cost and takes `sum`, those of all queries handed over, by all SMs, which is more work than walks are.  The time gained (us), fitted
+// to 156 builds with and without it (1 to 36 prompts of 16 to 256 paths, 20 to 97 % full, D = 6 to 16): of those this line takes 99, none slower with
+// warm caches, nine up to 10 % slower with cold ones, and misses gains of up to 13 us.  All or none: with the heavier ones handed over and the others
+// walked the launch waits for those first and then for the pass (32 x 16 x 4096, 97 % full: none 165, all 155, those above 1536 matches 208).
+__device__ __forceinline__ bool hand_over_pays(const Dev& s, int most, int sum) {
+  if ((unsigned long long)sum * s.D * 16 > s.w_slots * sizeof(WideSlot)) return false;
+  const float x = 1e-3f * (float)s.D * (float)most, y = 1e-5f * (float)s.D * (float)sum;
+  return 0.4f * x + 0.023f * x * x - 3.0f * y > 10.0f;
+}
+// Occurrences of the last tokens of paths p0 .. p1: the most, and the sum, of those that would be handed over; for the paths that this
+// warp looks at.  Every thread of the CTA.
+struct Heavy { int most[kFusedThreads / 32], sum[kFusedThreads / 32], said; };
+__device__ __forceinline__ void occurrences(const Dev& s, int p0, int p1, Heavy& heavy) {
+  const uint32_t epoch = epoch_of(ldm(s.rec + (size_t)p0 * kRecWords + kRecEpoch));
+  unsigned most = 0u, sum = 0u;
+  for (int p = p0 + (int)threadIdx.x; p < p1; p += kFusedThreads) {
+    const int len = ldm(s.rec + (size_t)p * kRecWords), last = ldm(s.rec + (size_t)p * kRecWords + 1);
+    if (len < 1 || len >= s.L) continue;
+    uint4 lo, hi;
+    if (!find_bucket(s, p / s.N, 1, gram_final(gram_step(gram_init(1), last)), epoch, &lo, &hi)) continue;
+    const unsigned n = s.R > 0 ? min(lo.y, (unsigned)s.R * (unsigned)(s.N - 1)) : lo.y;
+    if (n <= (unsigned)kHandOverFrom || n > (unsigned)wide_alone(s)) continue;
+    most = max(most, n); sum += n;
+  }
+  most = __reduce_max_sync(FULL, most); sum = __reduce_add_sync(FULL, sum);
+  if ((threadIdx.x & 31) == 0) { heavy.most[threadIdx.x >> 5] = (int)most; heavy.sum[threadIdx.x >> 5] = (int)sum; }
+}
+__device__ __forceinline__ bool hand_over_pays(const Dev& s, const Heavy& heavy) {
+  int most = 0, sum = 0;
+  for (int w = 0; w < kFusedThreads / 32; ++w) { most = max(most, heavy.most[w]); sum += heavy.sum[w]; }
+  return hand_over_pays(s, most, sum);
+}
+
 // SHARE: the code of the cluster-shared scan is compiled in (kernels for prompts below kShareMinTokens leave it
 // out: after a cold start the step fetches every instruction it may run past)
 template <bool EXPORT, bool SHARE, bool CHAINED>
@@ -1781,6 +1816,7 @@ __device__ void build_phase(const Dev& s, const Smem& sm, int k_hi, int k_lo, in
   __shared__ int sh_nq;
   __shared__ uint32_t sh_have[SDMS_MAX_K], sh_pos[SDMS_MAX_K][kInlineSlots];   // buckets of the path's last 1, 2, .. tokens: occurrences, positions
   __shared__ int32_t sh_rec[kRecWords];
+  __shared__ Heavy sh_heavy;
   __shared__ int32_t sh_q[SDMS_MAX_K];
   __shared__ int32_t sh_len[SDMS_MAX_PATHS_PER_GROUP];
   const int i = blockIdx.x, tid = threadIdx.x;
@@ -1812,6 +1848,11 @@ __device__ void build_phase(const Dev& s, const Smem& sm, int k_hi, int k_lo, in
     }
     if (n <= SDMS_MAX_K) sh_have[n - 1] = have;
   }
+  // Launches whose CTAs all run at once look at all queries here, beside their own; the others only when one of them has found a heavy query and
+  // nobody has before (32 x 16 x 4096: 8 us for 2).  A step knows only its own prompt's paths as they will be.
+  const bool weigh = hand > 0 && s.eps == 0, at_once = (int)gridDim.x <= s.w_grid;
+  const int w0 = own_rec ? g * s.N : 0, w1 = own_rec ? w0 + s.N : s.P;
+  if (weigh && at_once) occurrences(s, w0, w1, sh_heavy);
   // the cluster shares its scans (same decision in every CTA of the launch)
   const bool share = SHARE && csize > 1 && k_lo == k_hi && s.eps == 0 && (s.L & 3) == 0 && slice >= kShareMinTokens;
   if (tid == 0) sh_M = 0;
@@ -1912,8 +1953,31 @@ __device__ void build_phase(const Dev& s, const Smem& sm, int k_hi, int k_lo, in
     if (tid == 0) draft_len[i] = 0;
     return;
   }
-  if (hand > 0 && M > ((int)(blockIdx.x + s.w_grid) >= (int)gridDim.x ? hand : kHandOverEarly) && M <= wide_alone(s) && wide_register(s, i, M))
-    return;                                          // all SMs share the work (the launch that follows)
+  if (hand > 0 && M > hand && M <= wide_alone(s)) {
+    bool pays = true;
+    if (weigh) {
+      volatile unsigned long long* const known = &s.w_ctl[kWideHeavy];                   // 1: it pays, 2: it does not
+      if (at_once) {
+        pays = hand_over_pays(s, sh_heavy);
+        if (own_rec) {                                       // what one prompt has reason enough for, the others' queries go along with
+          if (pays && tid == 0) *known = 1ull;
+          pays = __syncthreads_or(pays || (tid == 0 && *known == 1ull));
+        }
+      } else {
+        if (tid == 0) sh_heavy.said = (int)*known;
+        __syncthreads();
+        pays = sh_heavy.said == 1;
+        if (sh_heavy.said == 0) {
+          occurrences(s, w0, w1, sh_heavy);
+          __syncthreads();
+          pays = hand_over_pays(s, sh_heavy);
+          if (tid == 0) *known = pays ? 1ull : 2ull;
+        }
+      }
+    }
+    const bool last = (int)blockIdx.x + s.w_grid >= (int)gridDim.x;
+    if (pays && M > (last ? hand : kHandOverEarly) && wide_register(s, i, M)) return;    // all SMs share the work (the launch that follows)
+  }
   dag_phase<EXPORT>(s, sm, i, M, M <= kListCap ? sm.list : my_matches, sh_len, g * s.N, sh_q[k - 1], draft_tok,
                     draft_len, draft_score, draft_edge_w);
 }
@@ -2005,8 +2069,13 @@ cudaError_t dag_kernel_setup() {
 //   tolerance 1, at most 2 rounds, from 16384 tokens, k = 2: 16 x 1024 48 / 35 (600 of 1024 tokens held: 33 / 34), 32 x 2048 110 / 64,
 //     8 of 32 x 1024 104 / 85; 32 of 16 x 1024 (512 paths) 72 / 94; 8 x 1024 17 / 19.  k = 3, with 284 matches at most, 46 / 52
 // Queries split by classes of tokens (above wide_alone() matches) stay: with tolerance 1 and k = 1 every query is one (32 x 2048: 5.8 / 6.3 ms).
-int hand_over_from(const Dev& s, int k, int k_lo) {
-  return s.fused && s.w_grid > 0 && k_lo == k && k <= (s.eps > 0 ? 2 : 1) ? kHandOverFrom : 0;
+int hand_over_from(const Dev& s, int k, int k_lo, cudaStream_t stream) {
+  if (!s.fused || s.w_grid == 0 || k_lo != k || k > (s.eps > 0 ? 2 : 1)) return 0;
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  cudaStreamIsCapturing(stream, &capture);             // (a graph is there for histories that have grown since)
+  const int held = s.N * (capture == cudaStreamCaptureStatusNone ? s.held : s.L);
+  if (s.eps == 0) return held * s.D >= kHandOverHeld ? kHandOverFrom : 0;
+  return held >= (s.P <= s.w_grid ? kHandOverHeldFuzzy : kHandOverHeldFuzzyRounds) ? kHandOverFrom : 0;
 }
 
 namespace {
@@ -2037,12 +2106,12 @@ bool step_kernel_fits(const Dev& s) {
 
 cudaError_t launch_step(const Dev& s, int k, int k_lo, const int32_t* sampled, const float* sampled_lp,
                         int32_t* accept_len, int32_t* draft_tok, int32_t* draft_len, float* draft_score,
-                        float* draft_edge_w, int32_t* used_k, cudaStream_t stream) {
+                        float* draft_edge_w, int32_t* used_k, int hand, cudaStream_t stream) {
   cudaLaunchConfig_t cfg; cudaLaunchAttribute attr[2];
   step_launch_config(s, stream, &cfg, attr);
   const bool share = s.eps == 0 && (s.L & 3) == 0 && (long long)s.N * s.L >= kShareMinTokens;       // the prompt is worth sharing its scan
   return cudaLaunchKernelEx(&cfg, step_variant(share, s.epochs), s, k, k_lo, sampled, sampled_lp, accept_len,
-                            draft_tok, draft_len, draft_score, draft_edge_w, used_k, hand_over_from(s, k, k_lo));
+                            draft_tok, draft_len, draft_score, draft_edge_w, used_k, hand);
 }
 
 cudaError_t launch_dag(const Dev& s, bool with_export, int32_t* draft_tok, int32_t* draft_len, float* draft_score,
@@ -2077,10 +2146,10 @@ int build_cluster_size(const Dev& s) {
 }
 
 cudaError_t launch_build_fused(const Dev& s, int k_hi, int k_lo, int32_t* draft_tok, int32_t* draft_len,
-                               float* draft_score, float* draft_edge_w, int32_t* used_k, cudaStream_t stream) {
+                               float* draft_score, float* draft_edge_w, int32_t* used_k, int hand, cudaStream_t stream) {
   if (s.build_cluster <= 1 || k_lo != k_hi || s.eps > 0)
     return launch_overlapped(build_variant(false, s.epochs), dim3(s.P), dim3(kFusedThreads), fused_smem_bytes(s), stream,
-                             s, k_hi, k_lo, draft_tok, draft_len, draft_score, draft_edge_w, used_k, 0, hand_over_from(s, k_hi, k_lo));
+                             s, k_hi, k_lo, draft_tok, draft_len, draft_score, draft_edge_w, used_k, 0, hand);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(s.P); cfg.blockDim = dim3(kFusedThreads);
   cfg.dynamicSmemBytes = fused_smem_bytes(s); cfg.stream = stream;
@@ -2091,7 +2160,7 @@ cudaError_t launch_build_fused(const Dev& s, int k_hi, int k_lo, int32_t* draft_
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr; cfg.numAttrs = 2;
   return cudaLaunchKernelEx(&cfg, build_variant(true, s.epochs), s, k_hi, k_lo, draft_tok, draft_len, draft_score, draft_edge_w,
-                            used_k, (int)s.build_cluster, hand_over_from(s, k_hi, k_lo));
+                            used_k, (int)s.build_cluster, hand);
 }
 
 }  // namespace sdms

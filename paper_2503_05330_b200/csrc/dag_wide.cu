@@ -978,7 +978,7 @@ __device__ __forceinline__ void wide_walk(const Dev& s, const int4 de, int class
 // it that would.  By one thread of each CTA, once it has its last tickets.
 __device__ __forceinline__ void wide_counts_done(const Dev& s) {
   __threadfence();
-  if (atomicAdd(&s.w_ctl[kWideCtlWords - 1], 1ull) == gridDim.x - 1)
+  if (atomicAdd(&s.w_ctl[kWideLeft], 1ull) == gridDim.x - 1)
     for (int x = 0; x < kWideCtlWords; ++x) s.w_ctl[x] = 0ull;
 }
 
@@ -986,9 +986,9 @@ __global__ void __launch_bounds__(kWideThreads, 1)
 dag_wide_kernel(Dev s, int32_t* __restrict__ draft_tok, int32_t* __restrict__ draft_len,
                 float* __restrict__ draft_score, float* __restrict__ draft_edge_w) {
   grid_wait();                                         // scheduled while dag_kernel drains; its list is complete from here on
-  const u64 registered = ld_u64(&s.w_ctl[0]);
+  const u64 registered = ld_u64(&s.w_ctl[kWideListed]);
   if (registered == 0) {                               // (room may have been asked for in vain)
-    if (blockIdx.x == 0 && threadIdx.x == 0) s.w_ctl[1] = 0ull;
+    if (blockIdx.x == 0 && threadIdx.x == 0) s.w_ctl[kWideTaken] = s.w_ctl[kWideHeavy] = 0ull;
     return;
   }
   const int nq = (int)(registered < (u64)kMaxWide ? registered : (u64)kMaxWide);
@@ -1093,24 +1093,24 @@ dag_wide_kernel(Dev s, int32_t* __restrict__ draft_tok, int32_t* __restrict__ dr
   int parts = 1;                                       // a chunk is split by layers while that gives more CTAs something to do
   while (parts < quads && 2 * parts * whole <= (int)gridDim.x) parts *= 2;
   const int units = whole * parts, span = 4 * ((quads + parts - 1) / parts);
-  if (tid == 0) sh_task = (int)atomicAdd(&s.w_ctl[3], 1ull);
+  if (tid == 0) sh_task = (int)atomicAdd(&s.w_ctl[kWideChunkNext], 1ull);
   __syncthreads();
 #pragma unroll 1
   for (int unit = sh_task; unit < units;) {
     __syncthreads();
-    if (tid == 0) sh_task = (int)atomicAdd(&s.w_ctl[3], 1ull);         // (on its way during this one)
+    if (tid == 0) sh_task = (int)atomicAdd(&s.w_ctl[kWideChunkNext], 1ull);         // (on its way during this one)
     const int chunk = unit / parts, l0 = (unit - chunk * parts) * span;
     const int q = owner(sh_unit, chunk);
     if (l0 < D) wide_lay_out(s, sh_desc[q], (chunk - sh_unit[q]) * kWideThreads, l0, min(D, l0 + span));
     __threadfence();
     __syncthreads();
-    if (tid == 0) atomicAdd(&s.w_ctl[4], 1ull);
+    if (tid == 0) atomicAdd(&s.w_ctl[kWideChunksDone], 1ull);
     unit = sh_task;
   }
   __syncthreads();
   if (tid == 0) {
-    sh_last = wait_for_count(s.w_ctl + 4, (u64)units, kWideWait);
-    if (sh_last) sh_task = (int)atomicAdd(&s.w_ctl[2], 1ull);          // (whoever gives up here leaves no task undone)
+    sh_last = wait_for_count(s.w_ctl + kWideChunksDone, (u64)units, kWideWait);
+    if (sh_last) sh_task = (int)atomicAdd(&s.w_ctl[kWideTask], 1ull);          // (whoever gives up here leaves no task undone)
   }
   __syncthreads();
   if (!sh_last) {
@@ -1145,7 +1145,7 @@ dag_wide_kernel(Dev s, int32_t* __restrict__ draft_tok, int32_t* __restrict__ dr
     __threadfence();
     __syncthreads();
     if (tid == 0) {
-      sh_task = (int)atomicAdd(&s.w_ctl[2], 1ull);
+      sh_task = (int)atomicAdd(&s.w_ctl[kWideTask], 1ull);
       const int total = (large && few && s.mode != 1 ? 2 * D - 1 : D) * classes;
       if (large && !offers) atomicAdd(done + 1, 1);
       sh_last = atomicAdd(done, 1) == total - 1;

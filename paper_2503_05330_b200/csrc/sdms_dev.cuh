@@ -23,15 +23,20 @@ constexpr int kFusedMaxTokens = 131072; // largest N*L a CTA scans on its own
 // there is one (exact, tolerance 1).
 constexpr int kHandOverTokens = 65536, kHandOverPaths = 4 * 148;
 constexpr int kHandOverTokensFuzzy = 16384, kHandOverPathsFuzzy = 2 * 148;
-constexpr int64_t kHandOverTable = 32ll << 20;   // most bytes of table area taken for it by default: the queries that do not fit keep their CTA
-// Matches above which a query is handed over: 128 (256: 64 x 2048 53 us for 51, tolerance 1 36 to 46 for 34 to 41; 64: 46, but 113 for 108 with
+// Tokens held by a prompt (as far as the calls made tell) below which it is left out: the pass is 2 us (out of a cold cache 4 to 9) where there is nothing
+// to do for it.  Exact, tokens times layers, which is what a walk costs: 64 x 409, D = 8, 33 / 36; 16 x 1230, D = 12, 47 / 33, 48 / 33, 54 / 43.  Tolerance 1 (where nothing is known of the queries before they are scanned), k = 2, without / with it: 16 x 614 29 and 34 / 33 and 31, 16 x 768
+// 31 and 38 / 31 and 34; more CTAs than SMs: 8 x 32 x 614 75 and 76 / 81 and 73, x 768 86 and 86 / 86 and 84, x 1000 106 / 97; 9 x 32 x 900 108 and 92 / 103 and 94.
+constexpr int kHandOverHeld = 229376, kHandOverHeldFuzzy = 11000, kHandOverHeldFuzzyRounds = 30000;
+// Matches above which a query is handed over: 128 (256: 64 x 2048 47 to 58 us for 40 to 55, tolerance 1 36 to 46 for 34 to 41; 64: 46, but 113 for 108 with
 // 4 x 128 x 512); for a CTA that others wait for an SM behind, whose time is not the launch's, 512 (k = 1, 32 x 16 x 4096: 125 us from 256, 122
 // from 512, 126 from 1024, 144 from 2048; 4 x 64 x 2048: 65, 65, 73, 84).
 constexpr int kHandOverFrom = 128, kHandOverEarly = 512;
 constexpr int kMaxWide = 1024;          // queries one build can hand to the device-wide aggregation pass
 constexpr int kWideSumShift = 47;       // packed node sums: count in the upper 17 bits, sum of probabilities below
 constexpr int kWideMaxMatches = (1 << 17) - 1;   // so that both parts of a packed sum fit
-constexpr int kWideCtlWords = 6;
+// w_ctl: queries registered, slots handed out, tasks handed out, chunks handed out, chunks done, CTAs done, whether the pass
+// is worth its while for this single-launch build.  Zero between builds
+enum WideCtl : int { kWideListed = 0, kWideTaken = 1, kWideTask = 2, kWideChunkNext = 3, kWideChunksDone = 4, kWideLeft = 5, kWideHeavy = 6, kWideCtlWords = 7 };
 // b_ctl: table slots handed out, a count that stays zero (sdms_debug_wait_timeout waits for it), paths in bp_todo, paths dealt out, CTAs done
 enum BeamCtl : int { kBeamSlots = 0, kBeamNever = 1, kBeamTodo = 2, kBeamTicket = 3, kBeamDone = 4, kBeamCtlWords = 8 };
 
@@ -59,6 +64,7 @@ struct Dev {
   int32_t build_cluster;               // CTAs per cluster of the single-launch build (they share their prompt's scan); 1 = none
   int32_t epochs;                      // a large index: a reset does not clear it but moves on to the next epoch, and its n-gram lengths are
                                        // chained (append_dev.cuh)
+  int32_t held;                        // most tokens a path can hold, by the calls made so far
   int32_t R;                           // matches kept per (query path, source path): the R most recent; 0 = all
   double alpha;
   uint32_t table_cap;                  // buckets per (prompt, n) table, power of two
@@ -85,8 +91,7 @@ struct Dev {
   int32_t* g_trim;                     // [G] a path of the prompt was trimmed: its index is rebuilt
   int32_t* matches;                    // [match_cap] global positions j*L+e
   // device-wide aggregation of queries with many matches (dag_wide.cu); w_slots = 0: not in use
-  unsigned long long* w_ctl;           // [kWideCtlWords] queries registered, slots handed out, tasks handed out, chunks handed out, chunks done, CTAs done;
-                                       // zero between builds
+  unsigned long long* w_ctl;           // [kWideCtlWords]
   int4* w_desc;                        // [kMaxWide] query path, matches, first slot, -
   int* w_done;                         // [kMaxWide][2] tasks of the query that are done, of these sums; zero between builds
   WideSlot* w_tab;                     // [w_slots]

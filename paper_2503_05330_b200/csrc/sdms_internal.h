@@ -33,16 +33,17 @@ cudaError_t launch_fuzzy_match(const Dev& s, int k, int skip_done, cudaStream_t 
 // round: 0 for an ordinary build; kRound* flags, k and used_k for one round of a back-off build on a large prompt
 cudaError_t launch_dag(const Dev& s, bool with_export, int32_t* draft_tok, int32_t* draft_len, float* draft_score,
                        float* draft_edge_w, cudaStream_t stream, int round = 0, int k = 0, int32_t* used_k = nullptr);
+// (hand: hand_over_from)
 cudaError_t launch_build_fused(const Dev& s, int k_hi, int k_lo, int32_t* draft_tok, int32_t* draft_len,
-                               float* draft_score, float* draft_edge_w, int32_t* used_k, cudaStream_t stream);
+                               float* draft_score, float* draft_edge_w, int32_t* used_k, int hand, cudaStream_t stream);
 // phase 0: shift the histories; 1: empty the index tables of the prompts that changed; 2: index them again
 cudaError_t launch_trim(const Dev& s, int phase, const int32_t* keep, cudaStream_t stream);
-int hand_over_from(const Dev& s, int k, int k_lo);
+int hand_over_from(const Dev& s, int k, int k_lo, cudaStream_t stream);
 bool step_kernel_fits(const Dev& s);
 int build_cluster_size(const Dev& s);
 cudaError_t launch_step(const Dev& s, int k, int k_lo, const int32_t* sampled, const float* sampled_lp,
                         int32_t* accept_len, int32_t* draft_tok, int32_t* draft_len, float* draft_score,
-                        float* draft_edge_w, int32_t* used_k, cudaStream_t stream);
+                        float* draft_edge_w, int32_t* used_k, int hand, cudaStream_t stream);
 cudaError_t launch_compact_matches(const Dev& s, int32_t* offsets, int32_t* gpos, size_t cap, cudaStream_t stream);
 // queries with many matches, aggregated by all SMs (dag_wide.cu)
 int wide_kernel_grid();

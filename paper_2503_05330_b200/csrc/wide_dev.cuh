@@ -23,20 +23,21 @@ __device__ __forceinline__ bool wide_register(const Dev& s, int i, int M) {
   if (threadIdx.x == 0) {
     int q = -1;
     const unsigned long long need = wide_slots(s, M);
-    const unsigned long long first = atomicAdd(&s.w_ctl[1], need);
+    const unsigned long long first = atomicAdd(&s.w_ctl[kWideTaken], need);
     if (first + need <= s.w_slots) {
-      const unsigned long long n = atomicAdd(&s.w_ctl[0], 1ull);
+      const unsigned long long n = atomicAdd(&s.w_ctl[kWideListed], 1ull);
       if (n < (unsigned long long)kMaxWide) {
         q = (int)n;
         s.w_desc[q] = make_int4(i, M, (int)(unsigned)first, 0);
       }
+    } else {
+      atomicCAS(&s.w_ctl[kWideTaken], first + need, first);            // smaller ones may still fit (if nobody has come since)
     }
     sh_wide_q = q;
   }
   __syncthreads();
   return sh_wide_q >= 0;
 }
-
 
 typedef unsigned long long u64;
 constexpr unsigned FULL = 0xffffffffu;
