@@ -113,13 +113,14 @@ typedef struct {
                                     matches (12 * M * D above 14336 of them, 7168 with alpha < 1); on prompts of
                                     the single-launch build from 65536 tokens (16384 with epsilon 1), up to 592
                                     (296) paths in all, queries with more than 128 matches at k = 1 (epsilon 1:
-                                    k <= 2), if the pool is the DAG and neither beams nor search_mode 2 are asked
-                                    for; and
+                                    k <= 2), if the pool is the DAG, neither beams nor search_mode 2 are asked
+                                    for, and the heaviest is worth a launch (epsilon 1: if the tokens held are
+                                    many); and
                                     sdms_get_beams (max_beams > 0) and search_mode 2 for paths whose tables
                                     do not fit shared memory, in slots of 40 + 16 * max(max_beams, 1) bytes.
                                     0 = default (room for every position
-                                    matching every query of its prompt, but at most 320 MiB, 32 MiB with the
-                                    single-launch build), -1 = none.  A build
+                                    matching every query of its prompt, with the single-launch build every 64th
+                                    (epsilon 1: 16th), but at most 320 MiB), -1 = none.  A build
                                     whose queries need more falls back to one thread block for those that
                                     did not fit, with the same results                                    */
   int32_t  index_max_n;          /* n-gram lengths the index keeps tables for: 1..index_max_n (0 = k_max, every

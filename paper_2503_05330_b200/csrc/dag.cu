@@ -2059,15 +2059,15 @@ cudaError_t dag_kernel_setup() {
 }
 
 // Matches from which the single-launch build of suffix lengths k_lo .. k hands a query over to the wide pass; 0: it hands none over, and
-// is not followed by that pass.  A CTA walks a thousand matches in about 20 us, and the launch waits for the heaviest query; the pass
-// costs 1.3 us where there is nothing to do and 17 to 25 where there is.  Only the shortest suffixes have such queries: k = 1, with
-// tolerance 1 also k = 2.  Builds without / with it (us):
-//   k = 1, at most 4 rounds of CTAs, from 65536 tokens per prompt: 64 x 2048 83 / 51, 8 prompts of 16 x 4096 118 / 62, 16 x 4096 112 / 53,
-//     128 x 1024 212 / 71, 2 of 256 x 512 237 / 154, 8 of 16 x 8000 377 / 107, 32 of 16 x 4096 138 / 123; 4 of 128 x 512 100 / 101;
-//     32 of 32 x 2048 (1024 paths) 80 / 101: there the SMs are busy either way
-//     below: 16 of 32 x 1024 65 / 73, 16 of 16 x 2048 47 / 50, 16 x 1024 16 / 23
-//   tolerance 1, at most 2 rounds, from 16384 tokens, k = 2: 16 x 1024 48 / 35 (600 of 1024 tokens held: 33 / 34), 32 x 2048 110 / 64,
-//     8 of 32 x 1024 104 / 85; 32 of 16 x 1024 (512 paths) 72 / 94; 8 x 1024 17 / 19.  k = 3, with 284 matches at most, 46 / 52
+// is not followed by that pass.  A CTA walks a thousand matches in 15 to 60 us (D = 8 to 16), and the launch waits for the heaviest query; the pass
+// costs 2 us where there is nothing to do and 17 to 25 and more where there is.  Only the shortest suffixes have such queries: k = 1, with
+// tolerance 1 also k = 2.  The kernel decides whether they are worth it (hand_over_pays).  Builds without / with that rule, and handing over in any case (us):
+//   k = 1, at most 4 rounds of CTAs, from 65536 tokens per prompt: 64 x 2048, 97 % full, 87 / 52 / 52, half full 68 / 53 / 53 and 45 / 48 / 40; 16 x 4096
+//     119 / 56 / 55; 8 prompts of 16 x 4096 124 / 71 / 69; 4 of 128 x 1024 446 / 231 / 229; 36 of 16 x 8000 508 / 299 / 302; 32 of 16 x 4096, 97 % full, 165 / 152 / 150,
+//     half full 94 / 97 / 111, a fifth full 66 / 66 / 82; 32 of 32 x 2048 (1024 paths) 80 / - / 101: there the SMs are busy either way
+//     below: 16 of 32 x 1024 65 / - / 73, 16 of 16 x 2048 47 / - / 50, 16 x 1024 16 / - / 23
+//   tolerance 1, at most 2 rounds, from 16384 tokens, k = 2: 16 x 1024 44 / 35 / 35, 32 x 2048 117 / 69 / 69, 8 of 32 x 1024 105 / 85 / 85, 18 of 16 x 1024 56 / 56 / 65;
+//     32 of 16 x 1024 (512 paths) 72 / - / 94; 8 x 1024 17 / - / 19.  k = 3, with 284 matches at most, 46 / - / 52
 // Queries split by classes of tokens (above wide_alone() matches) stay: with tolerance 1 and k = 1 every query is one (32 x 2048: 5.8 / 6.3 ms).
 int hand_over_from(const Dev& s, int k, int k_lo, cudaStream_t stream) {
   if (!s.fused || s.w_grid == 0 || k_lo != k || k > (s.eps > 0 ? 2 : 1)) return 0;
