@@ -275,6 +275,12 @@ int sdms_create(const sdms_config* cfg, void* d_workspace, size_t bytes, sdms_ct
   d.mode = cfg->search_mode; d.P = d.G * d.N;
   d.alpha = (double)cfg->alpha;
   d.table_cap = lay.table_cap; d.match_cap = lay.match_cap;
+  d.epochs = lay.q_fp - lay.index >= kEpochIndexBytes;
+  d.pos_mask = ~0u;
+  if (d.epochs) {
+    d.pos_mask = 1u;
+    while (d.pos_mask < (uint32_t)(d.N * d.L - 1)) d.pos_mask = 2u * d.pos_mask + 1u;
+  }
   {
     int l = 0;
     while ((1ll << l) < (long long)d.L) ++l;                          // l = ceil(log2 L)
@@ -287,7 +293,6 @@ int sdms_create(const sdms_config* cfg, void* d_workspace, size_t bytes, sdms_ct
   d.pool = cfg->pool_mode;
   d.R = cfg->max_matches_per_path;
   d.held = 0;
-  d.epochs = lay.q_fp - lay.index >= kEpochIndexBytes;
   ctx->step_fits = false;                        // decided below, once the kernels' attributes are set
   unsigned char* w = ctx->ws;
   d.tok = (int32_t*)(w + lay.tok); d.pq = (int32_t*)(w + lay.pq); d.len = (int32_t*)(w + lay.len); d.rec = (int32_t*)(w + lay.rec);

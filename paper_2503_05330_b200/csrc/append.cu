@@ -156,7 +156,8 @@ __device__ __forceinline__ void chain_positions(const Dev& s, int p, int x0, int
         atomicAdd(&f.count[l][at], 1u);
         return true;
       };
-      if (index_insert<true, true>(s, g, n, h, lbase + (uint32_t)x, epoch, st, full)) break;
+      const int32_t before = n < kHalo ? win[kHalo - 1 - n + x - x0] : 0;        // (no query is longer than kHalo)
+      if (index_insert<true, true>(s, g, n, h, entry_of(s, lbase + (uint32_t)x, before), epoch, st, full)) break;
     }
   }
   if (FULL) {

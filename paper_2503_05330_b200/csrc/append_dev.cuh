@@ -98,7 +98,7 @@ __device__ __forceinline__ BucketHead bucket_cas(uint32_t* bucket, BucketHead ex
   return old;
 }
 
-// Adds one occurrence of an n-gram (hash h) ending at prompt-local position lpos.
+// Adds one occurrence of an n-gram (hash h), listed as entry (entry_of).
 // BULK: one of thousands of inserts, where throughput counts and not the latency of one: the bucket is read before any
 // atomic, so that an occurrence of a known n-gram costs one atomic (none whose result is waited for once the bucket's places
 // are taken: the buckets of popular n-grams take thousands, one after the other) and a bucket of another n-gram costs none.
@@ -110,7 +110,7 @@ __device__ __forceinline__ BucketHead bucket_cas(uint32_t* bucket, BucketHead ex
 // full(bucket number): BULK, whether the count of a bucket whose places are taken is kept elsewhere.
 struct CountNow { __device__ bool operator()(uint32_t) const { return false; } };
 template <bool BULK, bool CHAINED, class Full = CountNow>
-__device__ __forceinline__ bool index_insert(const Dev& s, int g, int n, uint64_t h, uint32_t lpos, uint32_t epoch, uint32_t* st, Full full = Full()) {
+__device__ __forceinline__ bool index_insert(const Dev& s, int g, int n, uint64_t h, uint32_t entry, uint32_t epoch, uint32_t* st, Full full = Full()) {
   uint32_t* table = index_table(s, g, n);
   const uint32_t tag = index_tag(h, epoch);
   uint32_t b = gram_bucket(h, s.table_cap);
@@ -124,20 +124,20 @@ __device__ __forceinline__ bool index_insert(const Dev& s, int g, int n, uint64_
       const ulonglong2 v = __ldcg(reinterpret_cast<const ulonglong2*>(bucket));
       old = v.x;
       if (bucket_empty((uint32_t)old, epoch)) {
-        const BucketHead now = bucket_cas(bucket, BucketHead{v.x, v.y}, BucketHead{(1ull << 32) | tag, lpos});
+        const BucketHead now = bucket_cas(bucket, BucketHead{v.x, v.y}, BucketHead{(1ull << 32) | tag, entry});
         if (now.head == v.x && now.pos == v.y) return true;
         old = now.head;
       }
     } else if (!CHAINED) {
       old = atomicCAS(head, 0ull, (1ull << 32) | tag);
-      if (old == 0ull) { bucket[2] = lpos; return true; }
+      if (old == 0ull) { bucket[2] = entry; return true; }
     } else {
       old = probe & 1u ? next : __ldcg(head);
       if (!(probe & 1u)) next = __ldcg(reinterpret_cast<const unsigned long long*>(table + (size_t)((b + 1) & (s.table_cap - 1)) * kBucketWords));
       if (bucket_empty((uint32_t)old, epoch)) {
         const unsigned long long seen = old;
         old = atomicCAS(head, seen, (1ull << 32) | tag);
-        if (old == seen) { bucket[2] = lpos; return true; }
+        if (old == seen) { bucket[2] = entry; return true; }
       }
     }
     if ((uint32_t)old == tag) {
@@ -146,7 +146,7 @@ __device__ __forceinline__ bool index_insert(const Dev& s, int g, int n, uint64_
         return false;
       }
       const uint32_t slot = (uint32_t)(atomicAdd(head, 1ull << 32) >> 32);
-      if (slot < (uint32_t)kInlineSlots) bucket[2 + slot] = lpos;
+      if (slot < (uint32_t)kInlineSlots) bucket[2 + slot] = entry;
       return slot < (uint32_t)kInlineSlots;
     }
     b = (b + 1) & (s.table_cap - 1);
@@ -165,9 +165,9 @@ __device__ __forceinline__ bool index_insert(const Dev& s, int g, int n, uint64_
 // up to 8: 9.3, 5.9).
 // The commit of a step: all lengths of a position are looked at side by side, by a group of lanes of one warp, so that a
 // position costs one look and one claim however many buckets it passes.  active: the lane's n-gram exists (length n, at most n_max;
-// gram(n): its hash; it ends at lpos); lanes: those with the same position.  Whole warps.
-template <class Gram>
-__device__ __forceinline__ void chain_insert(const Dev& s, int g, bool active, int n, int n_max, Gram gram, uint32_t lpos, uint32_t epoch,
+// gram(n): its hash; entry(n): what is listed); lanes: those with the same position.  Whole warps.
+template <class Gram, class Entry>
+__device__ __forceinline__ void chain_insert(const Dev& s, int g, bool active, int n, int n_max, Gram gram, Entry entry, uint32_t epoch,
                                              unsigned lanes, uint32_t* st) {
   const uint64_t h = active ? gram(n) : 0ull;
   const uint32_t tag = index_tag(h, epoch);
@@ -198,15 +198,15 @@ __device__ __forceinline__ void chain_insert(const Dev& s, int g, bool active, i
   if (lane > first) return;
   if (mine) {
     const uint32_t slot = (uint32_t)(atomicAdd(head, 1ull << 32) >> 32);
-    if (slot < (uint32_t)kInlineSlots) { bucket[2 + slot] = lpos; return; }
+    if (slot < (uint32_t)kInlineSlots) { bucket[2 + slot] = entry(n); return; }
     ++n;
   } else if (bucket_empty((uint32_t)old, epoch) && atomicCAS(head, old, (1ull << 32) | tag) == old) {
-    bucket[2] = lpos;
+    bucket[2] = entry(n);
     return;
   }
   // others of this launch were faster: on from here, one length after the other
   for (; n <= n_max; ++n)
-    if (index_insert<false, true>(s, g, n, gram(n), lpos, epoch, st)) return;
+    if (index_insert<false, true>(s, g, n, gram(n), entry(n), epoch, st)) return;
 }
 
 // Block-cooperative append of n validated tokens to path p whose length is len0.  rec is the
@@ -228,9 +228,10 @@ __device__ void append_tokens(const Dev& s, int p, int len0, int n, const int32_
   const int g = p / s.N;
   const uint32_t lbase = (uint32_t)(p - g * s.N) * (uint32_t)s.L;
   // old tokens from the record, new from the input
+  auto token = [&](int t) { return t < len0 ? rec[len0 - t] : in_tok[t - len0]; };
   auto gram = [&](int pos, int nn) {
     uint64_t h = gram_init(nn);
-    for (int t = pos - nn + 1; t <= pos; ++t) h = gram_step(h, t < len0 ? rec[len0 - t] : in_tok[t - len0]);
+    for (int t = pos - nn + 1; t <= pos; ++t) h = gram_step(h, token(t));
     return gram_final(h);
   };
   const uint32_t epoch = epoch_of(rec[kRecEpoch]);
@@ -240,7 +241,7 @@ __device__ void append_tokens(const Dev& s, int p, int len0, int n, const int32_
     for (int w = threadIdx.x; (w & ~31) < n << lg; w += blockDim.x) {   // whole warps
       const int a = w >> lg, nn = (w & (group - 1)) + 1, pos = len0 + a;
       chain_insert(s, g, a < n && nn <= s.idx_n && pos + 1 >= nn, nn, min(s.idx_n, pos + 1), [&](int x) { return gram(pos, x); },
-                   lbase + (uint32_t)pos, epoch, lanes, st);
+                   [&](int x) { return entry_of(s, lbase + (uint32_t)pos, pos >= x ? token(pos - x) : 0); }, epoch, lanes, st);
     }
   } else {
     for (int w = threadIdx.x; w < n * s.idx_n; w += blockDim.x) {

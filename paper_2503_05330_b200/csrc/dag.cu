@@ -1883,11 +1883,11 @@ __device__ void build_phase(const Dev& s, const Smem& sm, int k_hi, int k_lo, in
     if (tid < (nx - n0 + 1) * kInlineSlots) {
       const int n = n0 + tid / kInlineSlots, slot = tid % kInlineSlots;
       if (slot < (int)min(sh_have[n - 1], (uint32_t)kInlineSlots)) {
-        const uint32_t lpos = sh_pos[n - 1][slot];
+        const uint32_t entry = sh_pos[n - 1][slot], lpos = CHAINED ? entry & s.pos_mask : entry;
         const int jn = (int)(lpos / (uint32_t)s.L);
         const int j = g * s.N + jn;
         const int e = (int)(lpos % (uint32_t)s.L);
-        if (j != i && e >= k - 1 && e <= sh_len[jn] - 2) {
+        if (j != i && e >= k - 1 && e <= sh_len[jn] - 2 && (!CHAINED || n == k || entry_may_follow(s, entry, sh_rec[n + 1]))) {
           const int32_t* c = s.tok + (size_t)j * s.L + (e - k + 1);
           bool same = true;
           for (int t = 0; t < k; ++t) same = same && (ldm(c + t) == sh_rec[k - t]);

@@ -86,33 +86,53 @@ __global__ void __launch_bounds__(kProbeWarps * 32) probe_kernel(Dev s, int k, i
     }
     fp = gram_fp(gram_final(h));
     const uint32_t epoch = epoch_of(__shfl_sync(FULL_MASK, mine, kRecEpoch));
+    const int32_t before = __shfl_sync(FULL_MASK, mine, min(n + 1, 31));               // the token in front of the last n
     uint32_t have = 0u;
-    if (n >= shortest && n <= nx) {
-      uint4 lo, hi;
-      if (find_bucket(s, g, n, gram_final(hx), epoch, &lo, &hi)) have = lo.y;
-      uint32_t* const pos = sh_pos[warp] + (n - shortest) * kInlineSlots;
-      pos[0] = have > 0u ? lo.z : ~0u; pos[1] = have > 1u ? lo.w : ~0u; pos[2] = have > 2u ? hi.x : ~0u;
-      pos[3] = have > 3u ? hi.y : ~0u; pos[4] = have > 4u ? hi.z : ~0u; pos[5] = have > 5u ? hi.w : ~0u;
-    }
-    static_assert(kInlineSlots == 6, "the positions of a bucket");
-    __syncwarp();
+    uint4 lo = make_uint4(0u, 0u, 0u, 0u), hi = lo;
+    if (n >= shortest && n <= nx && find_bucket(s, g, n, gram_final(hx), epoch, &lo, &hi)) have = lo.y;
     const uint32_t count = __shfl_sync(FULL_MASK, have, nx - 1);
-    const int listed = __any_sync(FULL_MASK, have != 0u) ? (nx - shortest + 1) * kInlineSlots : 0;
-    if (listed) mode = count <= (uint32_t)kInlineSlots ? Q_INLINE : Q_SCAN;
-    // the listed positions: whether they match, or (for a query that will be scanned) end in the n-gram that was looked up at all
+    if (__any_sync(FULL_MASK, have != 0u)) mode = count <= (uint32_t)kInlineSlots ? Q_INLINE : Q_SCAN;
+    // The listed positions that the query may mean, side by side (of a query that will be scanned: those in the buckets of shorter
+    // n-grams).  Builds of 256 x 8192 tokens, k = 8, out of a cold cache: 62 us; every listed position checked, in up to three rounds, 67.
+    int total = 0;
+    {
+      static_assert(kInlineSlots == 6, "the positions of a bucket");
+      const uint32_t entry[kInlineSlots] = {lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+      const uint32_t places = mode == Q_SCAN && n == nx ? 0u : min(have, (uint32_t)kInlineSlots);
+      unsigned means = 0u;
+#pragma unroll
+      for (int x = 0; x < kInlineSlots; ++x)
+        means |= (unsigned)((uint32_t)x < places && (n >= k || entry_may_follow(s, entry[x], before))) << x;
+      int end = __popc(means);
+#pragma unroll
+      for (int o = 1; o < SDMS_MAX_K; o <<= 1) { const int y = __shfl_up_sync(FULL_MASK, end, o); if (lane >= o) end += y; }
+      total = __shfl_sync(FULL_MASK, end, SDMS_MAX_K - 1);
+      int at = end - __popc(means);
+#pragma unroll
+      for (int x = 0; x < kInlineSlots; ++x)
+        if (means >> x & 1u) sh_pos[warp][at++] = entry[x] & s.pos_mask;
+    }
+    __syncwarp();
+    // Do they match?  The query's tokens come from the record, the position's all at once.
     auto check = [&](int c, int* gpos) {
-      const uint32_t lpos = c < listed ? sh_pos[warp][c] : ~0u;
-      if (lpos == ~0u) return false;
+      bool on = c < total;
+      const uint32_t lpos = on ? sh_pos[warp][c] : 0u;
       const int jn = (int)(lpos / (uint32_t)s.L);
       const int j = g * s.N + jn, e = (int)(lpos - (uint32_t)jn * (uint32_t)s.L);
       *gpos = j * s.L + e;
-      if (j == i || e < k - 1) return false;
-      const int len_j = s.len[j];
-      const int32_t* t_j = s.tok + (size_t)j * s.L + (e - k + 1);
-      const int32_t* q = s.tok + (size_t)i * s.L + (len_i - k);
-      bool same = true;
-      for (int t = 0; t < k; ++t) same = same && (t_j[t] == q[t]);          // no early exit: the loads go out together
-      return same && e <= len_j - 2;
+      on = on && j != i && e >= k - 1;
+      const int len_j = on ? s.len[j] : 0;
+      int32_t x[SDMS_MAX_K];
+#pragma unroll
+      for (int t = 0; t < SDMS_MAX_K; ++t) x[t] = on && t < k ? s.tok[(size_t)*gpos - t] : -1;
+      bool same = on && e <= len_j - 2;
+#pragma unroll
+      for (int t = 0; t < SDMS_MAX_K; ++t) {
+        if (t >= k) break;                                         // (the same for all lanes)
+        const int32_t q = __shfl_sync(FULL_MASK, mine, 1 + t);
+        same = same && x[t] == q;
+      }
+      return same;
     };
     auto reserve = [&](int slots) {                               // behind the kInlineArea slots of all queries
       long long at = 0;
@@ -126,9 +146,7 @@ __global__ void __launch_bounds__(kProbeWarps * 32) probe_kernel(Dev s, int k, i
       off = (int)at; reserved = slots;
     };
     if (mode != Q_NONE) {
-      // a query that will be scanned: the occurrences that stand in the buckets of shorter n-grams count for its slice too
-      const int to = mode == Q_SCAN ? listed - kInlineSlots : listed;
-      int gpos[3], found = 0;
+      int gpos[3], found = 0;             // (a query that will be scanned: its slice has room for them too)
       bool same[3];
       constexpr int kRounds = 3;
       static_assert(kRounds * 32 >= SDMS_MAX_K * kInlineSlots, "every listed position has a lane");
@@ -136,7 +154,7 @@ __global__ void __launch_bounds__(kProbeWarps * 32) probe_kernel(Dev s, int k, i
       for (int r = 0; r < kRounds; ++r) {
         const int c = r * 32 + lane;
         gpos[r] = 0;
-        same[r] = r * 32 < to && c < to && check(c, &gpos[r]);
+        same[r] = r * 32 < total && check(c, &gpos[r]);
         found += __popc(__ballot_sync(FULL_MASK, same[r]));
       }
       if (mode == Q_SCAN) {

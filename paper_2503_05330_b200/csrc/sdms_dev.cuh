@@ -68,6 +68,7 @@ struct Dev {
   int32_t R;                           // matches kept per (query path, source path): the R most recent; 0 = all
   double alpha;
   uint32_t table_cap;                  // buckets per (prompt, n) table, power of two
+  uint32_t pos_mask;                   // bits of a bucket's entry that hold the position (entry_of)
   uint32_t L_magic; int32_t L_shift;   // x / L for 0 <= x < 2^31 as (x * L_magic) >> L_shift (path_of)
   int64_t match_cap;
   // path store
@@ -133,6 +134,15 @@ __device__ __forceinline__ uint32_t gram_bucket(uint64_t h, uint32_t cap) { retu
 
 __device__ __forceinline__ uint32_t* index_table(const Dev& s, int g, int n) {
   return s.index + ((size_t)(g * s.idx_n + (n - 1)) * s.table_cap) * kBucketWords;
+}
+
+// An entry of a bucket: the position (path within the prompt * L + position), and in a chained index, in the bits that leaves free, a hash of
+// the token in front of the n-gram: a look-up for more tokens than the bucket's need not read the histories of those it cannot mean.
+__device__ __forceinline__ uint32_t entry_of(const Dev& s, uint32_t lpos, int32_t before) {
+  return lpos | ((uint32_t)before * 2654435761u & ~s.pos_mask);
+}
+__device__ __forceinline__ bool entry_may_follow(const Dev& s, uint32_t entry, int32_t before) {
+  return ((entry ^ (uint32_t)before * 2654435761u) & ~s.pos_mask) == 0u;
 }
 
 // The bucket of the n-gram with hash h in the prompt's table, as two 16-byte words: false if there is none.  Ordinary loads: in the
