@@ -69,3 +69,20 @@ def test_steps_that_commit_into_full_and_half_full_buckets(G, N, L, match_capaci
     pair = Pair(G, N, L, vocab + 150, 5, 6, match_capacity=match_capacity, max_append=6)
     st = run_step_protocol(pair, tokens, lps, [5, 2, 3, 4, 1], steps=20, warm=0, start_lens=lens, check_every=2)
     assert st["steps"] == 20 and st["accepted"] > 0
+
+
+def test_rows_whose_chunks_count_full_buckets_for_themselves():
+    # more chunks than run at once, by the append and by the trim: common 1- and 2-grams are added up per chunk
+    G, N, L, V, k_max = 8, 64, 1600, 3000, 5
+    tokens, lps, start, vocab = phrases(G, N, L, V, 78)
+    rng = np.random.default_rng(79)
+    common = (tokens < V) & (rng.random(tokens.shape) < 0.3)
+    tokens[common] = rng.integers(0, 3, common.sum())
+    pair = Pair(G, N, L, vocab, k_max, 6)
+    pair.append(tokens, lps, start, expect_status=0)
+    some = range(0, G * N, 7)
+    for k in (2, 3, k_max):
+        pair.build_and_compare(k, paths=some)
+    pair.trim(np.where(np.arange(G * N) % 3 == 0, start - 200, L))
+    for k in (2, 4):
+        pair.build_and_compare(k, paths=some)
