@@ -1805,8 +1805,8 @@ __device__ __forceinline__ bool hand_over_pays(const Dev& s, const Heavy& heavy)
 }
 
 // SHARE: the code of the cluster-shared scan is compiled in (kernels for prompts below kShareMinTokens leave it
-// out: after a cold start the step fetches every instruction it may run past)
-template <bool EXPORT, bool SHARE, bool CHAINED>
+// out: after a cold start the step fetches every instruction it may run past).  WEIGH: that of the exact hand-over.
+template <bool EXPORT, bool SHARE, bool CHAINED, bool WEIGH>
 __device__ void build_phase(const Dev& s, const Smem& sm, int k_hi, int k_lo, int32_t* draft_tok, int32_t* draft_len,
                             float* draft_score, float* draft_edge_w, int32_t* used_k,
                             const int32_t* own_rec, int csize, int hand) {
@@ -1850,9 +1850,9 @@ __device__ void build_phase(const Dev& s, const Smem& sm, int k_hi, int k_lo, in
   }
   // Launches whose CTAs all run at once look at all queries here, beside their own; the others only when one of them has found a heavy query and
   // nobody has before (32 x 16 x 4096: 8 us for 2).  A step knows only its own prompt's paths as they will be.
-  const bool weigh = hand > 0 && s.eps == 0, at_once = (int)gridDim.x <= s.w_grid;
+  const bool at_once = (int)gridDim.x <= s.w_grid;
   const int w0 = own_rec ? g * s.N : 0, w1 = own_rec ? w0 + s.N : s.P;
-  if (weigh && at_once) occurrences(s, w0, w1, sh_heavy);
+  if (WEIGH && at_once) occurrences(s, w0, w1, sh_heavy);
   // the cluster shares its scans (same decision in every CTA of the launch)
   const bool share = SHARE && csize > 1 && k_lo == k_hi && s.eps == 0 && (s.L & 3) == 0 && slice >= kShareMinTokens;
   if (tid == 0) sh_M = 0;
@@ -1955,7 +1955,7 @@ __device__ void build_phase(const Dev& s, const Smem& sm, int k_hi, int k_lo, in
   }
   if (hand > 0 && M > hand && M <= wide_alone(s)) {
     bool pays = true;
-    if (weigh) {
+    if (WEIGH) {
       volatile unsigned long long* const known = &s.w_ctl[kWideHeavy];                   // 1: it pays, 2: it does not
       if (at_once) {
         pays = hand_over_pays(s, sh_heavy);
@@ -1982,7 +1982,7 @@ __device__ void build_phase(const Dev& s, const Smem& sm, int k_hi, int k_lo, in
                     draft_len, draft_score, draft_edge_w);
 }
 
-template <bool EXPORT, bool SHARE, bool CHAINED>
+template <bool EXPORT, bool SHARE, bool CHAINED, bool WEIGH>
 __global__ void __launch_bounds__(kFusedThreads, 1) build_fused_kernel(Dev s, int k_hi, int k_lo, int32_t* draft_tok,
                                                                   int32_t* draft_len, float* draft_score,
                                                                   float* draft_edge_w, int32_t* used_k, int csize, int hand) {
@@ -1990,7 +1990,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) build_fused_kernel(Dev s, in
   grid_release();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const Smem sm = carve<EXPORT>(smem_raw);
-  build_phase<EXPORT, SHARE, CHAINED>(s, sm, k_hi, k_lo, draft_tok, draft_len, draft_score, draft_edge_w, used_k, nullptr, csize, hand);
+  build_phase<EXPORT, SHARE, CHAINED, WEIGH>(s, sm, k_hi, k_lo, draft_tok, draft_len, draft_score, draft_edge_w, used_k, nullptr, csize, hand);
 }
 
 // One launch per decode step.  The CTAs of a prompt form a thread-block cluster.  Each CTA first
@@ -1999,7 +1999,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) build_fused_kernel(Dev s, in
 // path of the prompt is up to date and each CTA builds its path's next draft.  draft_tok / draft_len
 // hold the previous drafts on entry and the new ones on exit.
 // k_lo < k: the suffix length backs off from k to k_lo (used_k, if given, receives each path's choice).
-template <bool SHARE, bool CHAINED>
+template <bool SHARE, bool CHAINED, bool WEIGH>
 __global__ void __launch_bounds__(kFusedThreads, 1) step_kernel(Dev s, int k, int k_lo, const int32_t* sampled,
                                                            const float* sampled_lp, int32_t* accept_len,
                                                            int32_t* draft_tok, int32_t* draft_len,
@@ -2013,7 +2013,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) step_kernel(Dev s, int k, in
   accept_commit_phase<CHAINED>(s, blockIdx.x, draft_tok, draft_len, sampled, sampled_lp, accept_len, sh_own_rec, k, k_lo);
   // every thread of every CTA of the cluster gets here exactly once (no early exit above)
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-  build_phase<false, SHARE, CHAINED>(s, sm, k, k_lo, draft_tok, draft_len, draft_score, draft_edge_w, used_k, sh_own_rec, s.N, hand);
+  build_phase<false, SHARE, CHAINED, WEIGH>(s, sm, k, k_lo, draft_tok, draft_len, draft_score, draft_edge_w, used_k, sh_own_rec, s.N, hand);
 }
 
 }  // namespace
@@ -2033,15 +2033,21 @@ static size_t fused_smem_bytes(const Dev& s) {
 }
 
 namespace {
-// Their instances: a context runs the one that has the code it needs (after a cold start a step fetches every instruction it may
-// run past: 0.15 us of 9.7 with the chained index's code in the step of an index that is not).
-auto build_variant(bool share, bool chained) {
-  return share ? (chained ? build_fused_kernel<false, true, true> : build_fused_kernel<false, true, false>)
-               : (chained ? build_fused_kernel<false, false, true> : build_fused_kernel<false, false, false>);
+// Their instances: a launch runs the one that has the code it needs (after a cold start a step fetches every instruction it may
+// run past: 0.15 us of 9.7 with the chained index's code in the step of an index that is not; 0.2 of 15 with that of the exact hand-over in a step
+// that has none; and 32 x 16 x 4096, k = 1, where every CTA scans for itself, 127 to 148 us, with the cluster-shared scan's code 142 to 170).
+template <bool WEIGH>
+auto build_variant_of(bool share, bool chained) {
+  return share ? (chained ? build_fused_kernel<false, true, true, WEIGH> : build_fused_kernel<false, true, false, WEIGH>)
+               : (chained ? build_fused_kernel<false, false, true, WEIGH> : build_fused_kernel<false, false, false, WEIGH>);
 }
-auto step_variant(bool share, bool chained) {
-  return share ? (chained ? step_kernel<true, true> : step_kernel<true, false>) : (chained ? step_kernel<false, true> : step_kernel<false, false>);
+template <bool WEIGH>
+auto step_variant_of(bool share, bool chained) {
+  return share ? (chained ? step_kernel<true, true, WEIGH> : step_kernel<true, false, WEIGH>)
+               : (chained ? step_kernel<false, true, WEIGH> : step_kernel<false, false, WEIGH>);
 }
+auto build_variant(bool share, bool chained, bool weigh) { return weigh ? build_variant_of<true>(share, chained) : build_variant_of<false>(share, chained); }
+auto step_variant(bool share, bool chained, bool weigh) { return weigh ? step_variant_of<true>(share, chained) : step_variant_of<false>(share, chained); }
 }  // namespace
 
 cudaError_t dag_kernel_setup() {
@@ -2050,10 +2056,12 @@ cudaError_t dag_kernel_setup() {
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(dag_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)dag_smem_bytes<true>());
-  for (int v = 0; v < 4 && e == cudaSuccess; ++v) {
-    e = cudaFuncSetAttribute(build_variant(v & 1, v & 2), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBigPool);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(step_variant(v & 1, v & 2), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBigPool);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(step_variant(v & 1, v & 2), cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  for (int v = 0; v < 8 && e == cudaSuccess; ++v) {
+    const auto build = build_variant(v & 1, v & 2, v & 4);
+    const auto step = step_variant(v & 1, v & 2, v & 4);
+    e = cudaFuncSetAttribute(build, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBigPool);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(step, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBigPool);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(step, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   }
   return e;
 }
@@ -2098,7 +2106,7 @@ bool step_kernel_fits(const Dev& s) {
   step_launch_config(s, 0, &cfg, attr);
   cfg.numAttrs = 1;                                   // occupancy only looks at the cluster shape
   int clusters = 0;
-  if (cudaOccupancyMaxActiveClusters(&clusters, step_variant(true, s.epochs), &cfg) != cudaSuccess) { cudaGetLastError(); return false; }
+  if (cudaOccupancyMaxActiveClusters(&clusters, step_variant(true, s.epochs, false), &cfg) != cudaSuccess) { cudaGetLastError(); return false; }
   // every prompt's cluster resident at once: large clusters leave SMs of a GPC idle, and a launch whose
   // clusters queue up for the device is slower than the separate accept and build launches
   return (long long)clusters * s.N >= s.P;
@@ -2110,7 +2118,7 @@ cudaError_t launch_step(const Dev& s, int k, int k_lo, const int32_t* sampled, c
   cudaLaunchConfig_t cfg; cudaLaunchAttribute attr[2];
   step_launch_config(s, stream, &cfg, attr);
   const bool share = s.eps == 0 && (s.L & 3) == 0 && (long long)s.N * s.L >= kShareMinTokens;       // the prompt is worth sharing its scan
-  return cudaLaunchKernelEx(&cfg, step_variant(share, s.epochs), s, k, k_lo, sampled, sampled_lp, accept_len,
+  return cudaLaunchKernelEx(&cfg, step_variant(share, s.epochs, hand > 0 && s.eps == 0), s, k, k_lo, sampled, sampled_lp, accept_len,
                             draft_tok, draft_len, draft_score, draft_edge_w, used_k, hand);
 }
 
@@ -2139,7 +2147,7 @@ int build_cluster_size(const Dev& s) {
     attr[0].val.clusterDim.x = c; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr; cfg.numAttrs = 1;
     int clusters = 0;
-    if (cudaOccupancyMaxActiveClusters(&clusters, build_variant(true, s.epochs), &cfg) != cudaSuccess) { cudaGetLastError(); continue; }
+    if (cudaOccupancyMaxActiveClusters(&clusters, build_variant(true, s.epochs, false), &cfg) != cudaSuccess) { cudaGetLastError(); continue; }
     if ((long long)clusters * c >= s.P) return c;
   }
   return 1;
@@ -2148,7 +2156,7 @@ int build_cluster_size(const Dev& s) {
 cudaError_t launch_build_fused(const Dev& s, int k_hi, int k_lo, int32_t* draft_tok, int32_t* draft_len,
                                float* draft_score, float* draft_edge_w, int32_t* used_k, int hand, cudaStream_t stream) {
   if (s.build_cluster <= 1 || k_lo != k_hi || s.eps > 0)
-    return launch_overlapped(build_variant(false, s.epochs), dim3(s.P), dim3(kFusedThreads), fused_smem_bytes(s), stream,
+    return launch_overlapped(build_variant(false, s.epochs, hand > 0 && s.eps == 0), dim3(s.P), dim3(kFusedThreads), fused_smem_bytes(s), stream,
                              s, k_hi, k_lo, draft_tok, draft_len, draft_score, draft_edge_w, used_k, 0, hand);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(s.P); cfg.blockDim = dim3(kFusedThreads);
@@ -2159,7 +2167,7 @@ cudaError_t launch_build_fused(const Dev& s, int k_hi, int k_lo, int32_t* draft_
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr; cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, build_variant(true, s.epochs), s, k_hi, k_lo, draft_tok, draft_len, draft_score, draft_edge_w,
+  return cudaLaunchKernelEx(&cfg, build_variant(true, s.epochs, hand > 0 && s.eps == 0), s, k_hi, k_lo, draft_tok, draft_len, draft_score, draft_edge_w,
                             used_k, (int)s.build_cluster, hand);
 }
 
