@@ -401,6 +401,7 @@ def steady_state(wl, device, iters=20, peak=None, max_matches=0, ks=None, beams=
                 torch.empty((wl.P, max(beams, 1)), dtype=torch.int32, device=dev),
                 torch.empty((wl.P, max(beams, 1)), dtype=torch.float32, device=dev))
     out = {}
+    launches = 0                                                 # of the build that takes most
     for k in (ks or range(1, wl.k_max + 1)):
         for _ in range(3):
             s.build_drafts(k)
@@ -419,6 +420,9 @@ def steady_state(wl, device, iters=20, peak=None, max_matches=0, ks=None, beams=
             s.build_drafts(k)
         split = {n: 1e3 * ms / c for n, (ms, c) in binding.sdms_profile_read(s.ctx).items() if c}
         binding.sdms_profile_enable(s.ctx, False)
+        n0 = binding.sdms_launch_count(s.ctx)
+        s.build_drafts(k)
+        launches = max(launches, binding.sdms_launch_count(s.ctx) - n0)
         off, _ = s.matches()
         m = np.diff(off.numpy())
         modes = s.query_modes()
@@ -455,7 +459,7 @@ def steady_state(wl, device, iters=20, peak=None, max_matches=0, ks=None, beams=
     assert s.status() == 0
     return {"groups": wl.G, "paths_per_group": wl.N, "capacity": wl.L, "max_draft_len": wl.D, "fill": 0.97,
             "max_matches_per_path": max_matches, "index_max_n": index_max_n or wl.k_max,
-            "launches_per_build": 1 if fused else 4, "build_cluster_size": binding.sdms_build_cluster_size(s.ctx), "workspace_bytes": s.workspace_bytes, "build_by_k": out}
+            "launches_per_build": launches, "build_cluster_size": binding.sdms_build_cluster_size(s.ctx), "workspace_bytes": s.workspace_bytes, "build_by_k": out}
 
 
 def scan_at_scale(device, G=64, N=256, L=8192, V=151936):

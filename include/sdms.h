@@ -94,7 +94,8 @@ typedef struct {
   int32_t  epsilon;              /* Eq. 4 edit-distance tolerance of the suffix match: 0 (exact)
                                     or 1.  With 1 there is no index: small prompts (N*L <= 131072
                                     tokens and G*N*N*L <= match_capacity) are scanned by the single-launch
-                                    build, larger ones in two passes (count, then fill)             */
+                                    build, larger ones in one pass that notes what it finds, given a match_capacity of
+                                    three times the matches there are (with less, in two)             */
   int32_t  pool_mode;            /* draft pool: 0 = weighted DAG (the method); the weaker pools of the
                                     paper's ablation: 1 = tree (merge identical prefixes only),
                                     2 = list (no merging: the heaviest single candidate)            */
@@ -152,7 +153,9 @@ int sdms_destroy(sdms_ctx* ctx);
  * the model's log-probability of each of those tokens (the p_theta of Eq. 5 is
  * exp(logprob), stored as round_half_even(exp(logprob) * 2^30) in [0, 2^30]).
  * Rows are `row_width` wide (1 <= row_width; any width, e.g. a prefill chunk).
- * The new positions' n-grams (n = 1..k_max) enter the prompt's hash tables.
+ * The new positions enter the prompt's hash tables: under every n-gram that ends at them (n = 1..index_max_n),
+ * or, where the tables take 16 MiB and more, under the shortest one that still has a place; with epsilon 1
+ * there are none.
  * Clamping: count outside [0, row_width] -> BAD_COUNT; beyond capacity ->
  * CAPACITY, truncated; token outside [0, V) -> BAD_TOKEN, the path keeps the
  * tokens before it.
@@ -249,8 +252,8 @@ int sdms_build_cluster_size(sdms_ctx* ctx, int32_t* paths);
  * those tokens had ever been appended.  d_keep[p] >= the path's length changes
  * nothing; d_keep[p] < 0 raises SDMS_STATUS_BAD_COUNT and changes nothing.
  * The n-gram tables of every prompt with a trimmed path are emptied and filled
- * again from the histories (three launches; cost proportional to the prompt's
- * tokens * k_max), so call it every few hundred steps with a generous cut, not
+ * again from the histories (three launches; cost proportional to the size of the
+ * prompt's tables and its tokens), so call it every few hundred steps with a generous cut, not
  * every step.  Drafts built before the call refer to the old positions: build
  * again before the next sdms_accept.
  */
@@ -314,7 +317,10 @@ int sdms_get_beams(sdms_ctx* ctx, int32_t num_beams, int32_t* d_beam_tok, int32_
 int sdms_debug_read_history(sdms_ctx* ctx, int32_t* d_tok, int32_t* d_pq, int32_t* d_len, void* stream);
 
 /* How each path's query of the last sdms_build_drafts was answered: d_modes [P],
- * 0 = no query or no index entry, 1 = from the index bucket, 2 = by scanning. */
+ * 0 = no query or no index entry, 1 = from index buckets, 2 = by scanning (3: see
+ * sdms_build_drafts_backoff).  Which occurrences of an n-gram are listed depends on the order in
+ * which they came, so where the tables take 16 MiB and more a query may be answered the one way
+ * or the other from run to run.  Matches and drafts are the same. */
 int sdms_debug_read_query_modes(sdms_ctx* ctx, int32_t* d_modes, void* stream);
 
 /* Every wait inside a kernel (such as the copy barriers of the streaming scan) is bounded:

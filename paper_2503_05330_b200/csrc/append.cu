@@ -1,8 +1,9 @@
 // State update and acceptance kernels.
 //
 // append_kernel : one CTA per path; writes tokens and fixed-point probabilities
-//                 into the path store and inserts the n-grams (n = 1..k_max) that
-//                 end at each new position into the prompt's hash tables.
+//                 into the path store and enters each new position into the prompt's
+//                 hash tables: under every n-gram that ends at it, or once in a chained
+//                 index (append_dev.cuh); with tolerance 1 there is no index.
 // append_plan_kernel, append_bulk_kernel : the same for wide rows: how much each
 //                 path takes, then many CTAs per path.
 // accept_kernel : one CTA per path; longest accepted prefix of the draft
@@ -61,6 +62,10 @@ __global__ void __launch_bounds__(128) append_kernel(Dev s, const int32_t* token
 // 2270).  Also measured: four positions of a thread with their reads and claims on their way together, at 1024 threads per SM (32 x 16: 220 us,
 // the lanes' ways through the lengths part), single tokens in a table of their own without hashing (256 x 7800: 155), prompts taken in turn (16 x 128 x 3900
 // without a common token 351 for 302, with many 433 for 417).
+// Small launches wait for the positions with the longest way along their chain, each length a look, a claim and a count.  Reset and append, with an entry
+// per length / chained: 16 x 2200 tokens, lengths up to 8, 97 % full, little in common 18 / 15, a third 21 / 17, mostly the same phrases 19 / 26; a fifth full 11 / 13 and 10 / 21;
+// 64 x 2048, up to 4, 97 % full 32 / 27 and 29 / 27, a fifth full 12 / 15 and 12 / 16.  (The builds behind it take 4 us less where a query has 7 to 12 occurrences.)  Also measured: all further
+// lengths of a position at once, with places given out twice (16 x 2200 26 / 24, but 8 x 16 x 1024 20 / 28, 64 x 2048, up to 16, 42 / 67).
 // Indexes that are cleared have an entry per length, and a CTA each for it: 16 x 1024 17 us.
 constexpr int kPlanThreads = 256;
 constexpr int kBulkThreads = 256;
@@ -278,7 +283,7 @@ __global__ void __launch_bounds__(256) trim_clear_kernel(Dev s) {
     if (s.g_trim[x / per_group]) index[x] = make_uint4(0u, 0u, 0u, 0u);
 }
 
-// Third launch: every n-gram (n = 1..k_max) of every path of those prompts goes into the tables again.
+// Third launch: every position of those prompts goes into the tables again.
 template <int FORM>
 __global__ void __launch_bounds__(kBulkThreads, bulk_ctas(FORM)) trim_reindex_kernel(Dev s, int chunk, int chunks) {
   __shared__ int32_t sh_win[kHalo - 1 + kBulkChunk];

@@ -1,8 +1,8 @@
-// Follower gather, DAG aggregation (Eq. 5) and the greedy walk for queries with many matches on prompts that do not take the
-// single-launch build, spread over the whole device.
+// Follower gather, DAG aggregation (Eq. 5) and the greedy walk for queries with many matches, spread over the whole device: on prompts that do not
+// take the single-launch build, and behind that build or step for its heaviest queries (hand_over_from, dag.cu).
 //
 // One CTA that aggregates a query of thousands of matches by itself takes hundreds of microseconds while the other SMs idle,
-// so dag_kernel hands such queries over (wide_register).  First all CTAs lay the followers of all candidates out layer by layer.
+// so dag_kernel and the single-launch kernels hand such queries over (wide_register).  First all CTAs lay the followers of all candidates out layer by layer.
 // Then (query, layer) pairs are tasks that come from a counter, heavy queries first, each done by one CTA in its shared memory:
 //   sums    followers and probabilities of the layer, summed up per token in a hash table
 //   offers  a second table, by the token of the layer before: the heaviest node among its successors, found in three 32-bit

@@ -88,3 +88,17 @@ def test_inputs_that_another_call_may_still_write_are_not_declared_read_only():
     for kernel in ("append_kernel", "append_plan_kernel", "accept_kernel", "trim_shift_kernel"):
         params = re.search(kernel + r"\(Dev s,([^)]*)\) \{", text).group(1)
         assert "__restrict__" not in params, kernel
+
+
+def test_the_default_table_area_follows_the_configuration(lib):
+    # 16 bytes per layer and match: every 64th position of a prompt for each of its paths (tolerance 1: 16th), at least eight queries of 14336, at most 320 MiB
+    def area(G, N, L, D, **kw):
+        with_it, without = (binding.sdms_workspace_bytes(binding.make_config(G, N, L, 1000, 2, D, wide_table_bytes=w, **kw)) for w in (0, -1))
+        return with_it - without
+
+    for G, N, L, D, kw, matches in ((32, 16, 4096, 12, {}, 32 * 16 * 16 * 4096 // 64), (1, 64, 2048, 8, {}, 64 * 64 * 2048 // 64),
+                                    (1, 16, 4096, 12, {}, 8 * 14336), (8, 32, 1024, 8, dict(epsilon=1), 256 * 32 * 1024 // 16)):
+        lists = area(G, N, L, D, **kw) - 16 * D * matches
+        assert 0 <= lists < 1 << 15                                  # (the pass's list of queries)
+    assert area(2, 256, 512, 32) > 320 << 20 > area(2, 256, 512, 32) - (1 << 15)
+    assert area(1, 16, 1024, 8) == 0                                 # no hand-over, no area
