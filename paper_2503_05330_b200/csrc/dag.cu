@@ -1852,7 +1852,7 @@ __device__ void build_phase(const Dev& s, const Smem& sm, int k_hi, int k_lo, in
   // nobody has before (32 x 16 x 4096: 8 us for 2).  A step knows only its own prompt's paths as they will be.
   const bool at_once = (int)gridDim.x <= s.w_grid;
   const int w0 = own_rec ? g * s.N : 0, w1 = own_rec ? w0 + s.N : s.P;
-  if (WEIGH && at_once) occurrences(s, w0, w1, sh_heavy);
+  if (WEIGH && hand > 0 && at_once) occurrences(s, w0, w1, sh_heavy);
   // the cluster shares its scans (same decision in every CTA of the launch)
   const bool share = SHARE && csize > 1 && k_lo == k_hi && s.eps == 0 && (s.L & 3) == 0 && slice >= kShareMinTokens;
   if (tid == 0) sh_M = 0;
@@ -2033,9 +2033,12 @@ static size_t fused_smem_bytes(const Dev& s) {
 }
 
 namespace {
-// Their instances: a launch runs the one that has the code it needs (after a cold start a step fetches every instruction it may
+// Their instances: a context runs the one that has the code it needs (after a cold start a step fetches every instruction it may
 // run past: 0.15 us of 9.7 with the chained index's code in the step of an index that is not; 0.2 of 15 with that of the exact hand-over in a step
 // that has none; and 32 x 16 x 4096, k = 1, where every CTA scans for itself, 127 to 148 us, with the cluster-shared scan's code 142 to 170).
+// All its launches run the same one, also those that hand nothing over: a session's k = 1 builds would fetch theirs each time (64 x 2048 tokens,
+// 32 steps: 9 us of 735).
+bool weighs(const Dev& s) { return s.w_grid > 0 && s.eps == 0; }
 template <bool WEIGH>
 auto build_variant_of(bool share, bool chained) {
   return share ? (chained ? build_fused_kernel<false, true, true, WEIGH> : build_fused_kernel<false, true, false, WEIGH>)
@@ -2118,7 +2121,7 @@ cudaError_t launch_step(const Dev& s, int k, int k_lo, const int32_t* sampled, c
   cudaLaunchConfig_t cfg; cudaLaunchAttribute attr[2];
   step_launch_config(s, stream, &cfg, attr);
   const bool share = s.eps == 0 && (s.L & 3) == 0 && (long long)s.N * s.L >= kShareMinTokens;       // the prompt is worth sharing its scan
-  return cudaLaunchKernelEx(&cfg, step_variant(share, s.epochs, hand > 0 && s.eps == 0), s, k, k_lo, sampled, sampled_lp, accept_len,
+  return cudaLaunchKernelEx(&cfg, step_variant(share, s.epochs, weighs(s)), s, k, k_lo, sampled, sampled_lp, accept_len,
                             draft_tok, draft_len, draft_score, draft_edge_w, used_k, hand);
 }
 
@@ -2156,7 +2159,7 @@ int build_cluster_size(const Dev& s) {
 cudaError_t launch_build_fused(const Dev& s, int k_hi, int k_lo, int32_t* draft_tok, int32_t* draft_len,
                                float* draft_score, float* draft_edge_w, int32_t* used_k, int hand, cudaStream_t stream) {
   if (s.build_cluster <= 1 || k_lo != k_hi || s.eps > 0)
-    return launch_overlapped(build_variant(false, s.epochs, hand > 0 && s.eps == 0), dim3(s.P), dim3(kFusedThreads), fused_smem_bytes(s), stream,
+    return launch_overlapped(build_variant(false, s.epochs, weighs(s)), dim3(s.P), dim3(kFusedThreads), fused_smem_bytes(s), stream,
                              s, k_hi, k_lo, draft_tok, draft_len, draft_score, draft_edge_w, used_k, 0, hand);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(s.P); cfg.blockDim = dim3(kFusedThreads);
@@ -2167,7 +2170,7 @@ cudaError_t launch_build_fused(const Dev& s, int k_hi, int k_lo, int32_t* draft_
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr; cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, build_variant(true, s.epochs, hand > 0 && s.eps == 0), s, k_hi, k_lo, draft_tok, draft_len, draft_score, draft_edge_w,
+  return cudaLaunchKernelEx(&cfg, build_variant(true, s.epochs, weighs(s)), s, k_hi, k_lo, draft_tok, draft_len, draft_score, draft_edge_w,
                             used_k, (int)s.build_cluster, hand);
 }
 
